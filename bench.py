@@ -181,14 +181,11 @@ def peaks():
 # thread operations) per cycle; scaled by the SM clock sampled during the timed region.
 SMS, SMSP_PER_SM, LANES = 152, 4, 32
 # Thread operations the intersection needs per unit of work (the algorithmic count, not what the
-# compiler emits): per scanned list entry with a stored colour, the colour filter of the larger
-# endpoint's edge -- the ordered key (min, max: 2), the seed xor (2), SplitMix64 (64-bit add 2, three
-# 64-bit xor-shifts 3 x 4, two 64-bit multiplies by constants 2 x 3: 20), the high word of the
-# divisibility test (64-bit subtract 2, multiply 3, funnel shift 1, compare 1: 7) -- plus the entry's
-# id mask, colour extraction and age test (3): 34; per scanned entry without stored colours, the
-# age test and mask (2); per probe, the home-bucket hash and the 4-key compare (8); per counted
+# compiler emits): per scanned list entry, the filter test -- the hash multiply, the shift and the
+# address of the filter word, two rotates and the shift of the second bit's number, two ands and the
+# merge into the lane's mask (9); per probe, the home-bucket hash and the 4-key compare (8); per counted
 # wedge, the colours of both edges (2 x 31) and the three local updates (3): 65.
-OPS_ENTRY_COLOURED, OPS_ENTRY_PLAIN, OPS_PROBE, OPS_WEDGE = 34, 2, 8, 65
+OPS_ENTRY, OPS_PROBE, OPS_WEDGE = 9, 8, 65
 
 
 # --------------------------------------------------------------------------- oracle digests
@@ -261,7 +258,7 @@ def kernel_source_sha16() -> str:
 # DRAM bytes (read + write) per k_intersect launch from an ncu capture, keyed by (workload, c, digest
 # of the kernel sources at capture time).  A figure whose digest no longer matches the sources is not
 # reported (traffic null).
-K3_TRAFFIC: dict = {("rmat_s20", 100, "6093804f85a48125"): 864792474.0}
+K3_TRAFFIC: dict = {}
 
 
 # --------------------------------------------------------------------------- reference arm
@@ -352,11 +349,9 @@ def single_leg(name, m, c, seed, steps, warmup, dev, pg, digests, clock_mhz_hint
         proc_w, _ = rw.counts()
         st = rw.stats()
     assert np.array_equal(proc_w, proc), "work-counter pass disagrees with the timed pass"
-    coloured = (c + m - 1) // m == 1 and 2 <= m <= 256 and s.n_nodes <= (1 << 24)
     edges = T - st["self_loops"]
-    k3_bytes = 24 * edges + 8 * st["small_entries"] + 8 * st["probes"] + 16 * st["counted"]
-    k3_ops = ((OPS_ENTRY_COLOURED if coloured else OPS_ENTRY_PLAIN) * st["small_entries"] +
-              OPS_PROBE * st["probes"] + OPS_WEDGE * st["counted"])
+    k3_bytes = 24 * edges + 4 * st["small_entries"] + 8 * st["probes"] + 16 * st["counted"]
+    k3_ops = OPS_ENTRY * st["small_entries"] + OPS_PROBE * st["probes"] + OPS_WEDGE * st["counted"]
     k3_ms, k3_n = kt["intersect"]
     k3_s = k3_ms / steps * 1e-3
     hbm, hbm_src = peaks()
@@ -372,8 +367,7 @@ def single_leg(name, m, c, seed, steps, warmup, dev, pg, digests, clock_mhz_hint
         "l2": (f"inputs and state larger than L2, no flush: {ws_bytes / 1e9:.2f} GB touched per step (edges, "
                f"node blocks written as they are handed out, per-node arrays cleared at every step's start)"
                if ws_bytes > (129 << 20) else "working set fits in L2 (no flush)"),
-        "k3": {"bytes": k3_bytes, "ops": k3_ops, "seconds": k3_s, "launches": k3_n // max(steps, 1),
-               "coloured": coloured},
+        "k3": {"bytes": k3_bytes, "ops": k3_ops, "seconds": k3_s, "launches": k3_n // max(steps, 1)},
         "hbm_roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
                          "peak_source": hbm_src},
     }

@@ -95,8 +95,8 @@ typedef struct rept_config {
     uint64_t expected_edges; /* sizing hint: edges the stream will carry (0: start small and grow) */
     uint64_t max_batch;      /* sizing hint: largest batch passed to an ingest call (0: 2^20) */
     uint32_t tile_max;       /* tuning: edges whose smaller endpoint holds at most this many entries
-                                (4, 8, 16 or 32; 0: 32) share a warp with other edges, larger ones get a
-                                warp of their own; results do not depend on it */
+                                (4, 8, 16 or 32; 0: 32) share a warp with other edges, the others are
+                                grouped by their larger endpoint; results do not depend on it */
     uint32_t proc_begin;     /* colour sharding: the handle keeps processors [proc_begin, proc_end) only
                                 (stores the edges they keep, counts their semi-triangles); 0, 0: all c.
                                 Processors are independent until the final sums (Algorithm 1), so
@@ -120,15 +120,17 @@ typedef struct rept_stats {
     /* with REPT_FLAG_WORK_COUNTERS, totals over the stream's intersection passes: */
     uint64_t small_entries;  /* entries present in the smaller endpoint's table, summed over edges */
     uint64_t small_slots;    /* slots of those tables read (entries plus empty slots) */
-    uint64_t probes;         /* probes of the larger endpoint's table (small-side entries older than the edge
-                                and, where colours are kept, coloured alike for a kept processor) */
+    uint64_t probes;         /* probes of the larger endpoint's table (small-side entries that its filter or
+                                their colours did not rule out) */
     uint64_t probe_slots;    /* slots read by those probes */
     uint64_t wedges;         /* closed wedges found in the union adjacency (both edges older than the edge) */
     uint64_t counted;        /* (wedge, hash group) pairs counted for some processor */
     uint64_t class_items[6]; /* edges per intersection work class (smaller endpoint with <= 4, 8, 16,
                                 32, 256, more entries) */
     uint64_t class_probes[6];  /* probes issued per work class */
-    uint64_t class_cycles[6];  /* warp-cycles spent per work class (clock64, summed over warps) */
+    uint64_t class_cycles[6];  /* warp-cycles spent (clock64, summed over warps) on edges grouped by a larger
+                                  endpoint of more than 1,024 entries ([5]) and fewer ([4]), and on the
+                                  others ([3]) */
 } rept_stats;
 
 typedef struct rept_state rept_state;
@@ -143,10 +145,11 @@ typedef struct rept_state rept_state;
  * counters (16 + 12 * ceil(c/m) bytes per stream edge).
  * Speed: with one hash group (c <= m, or MASCOT with c == 1) and m >= 2, each
  * stored entry keeps its colour (in the entry's top 8 bits when m <= 256 and
- * n_nodes <= 2^24, else in a word beside it, 25 % more pool), and the
- * intersection tests colours before it looks an edge up, so only about 1/m
- * of the lookups happen; configurations with several hash groups look up
- * every candidate wedge edge (same counts, slower intersection).
+ * n_nodes <= 2^24, else in a word beside it, 25 % more pool), and only
+ * neighbours that two endpoints share with the same colour are looked up;
+ * with several hash groups every shared neighbour is, and its colours are
+ * compared through a stored word (50 % more pool; hashed again where the
+ * groups' colours do not fit 32 bits or the larger pool cannot be had).
  */
 int rept_create(const rept_config* cfg, void* stream, rept_state** out);
 
@@ -270,7 +273,8 @@ int rept_kernel_times(rept_state* s, double* ms, uint64_t* launches, int clear);
  * rept_restore loads such a snapshot into a handle created with the same
  * m, c, seed, n_nodes and flags (REPT_E_INVAL otherwise), replacing its
  * state; ingesting the rest of the stream then gives exactly the counts of
- * an uninterrupted run.  All three synchronise `stream`.
+ * an uninterrupted run.  Snapshots of the library's previous block layout are
+ * read as well (their blocks are rebuilt).  All three synchronise `stream`.
  */
 int rept_snapshot_size(rept_state* s, uint64_t* bytes, void* stream);
 int rept_snapshot(rept_state* s, void* h_buf, uint64_t bytes, void* stream);

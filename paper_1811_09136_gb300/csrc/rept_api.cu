@@ -51,6 +51,7 @@ struct rept_state {
     int device = 0;
     int sm_count = 0;
     uint32_t groups = 1;
+    uint32_t tile_max = 32;
     StreamDev d{};
     unsigned long long max_batch = 0;
     unsigned long long next_t = 0;  // stream index of the next edge
@@ -87,12 +88,11 @@ void dev_free(rept_state* s, void* p, size_t bytes) {
     }
 }
 
-// Pool slots that guarantee no batch can run out: a node's block (table plus list) holds at
-// most 8 slots per entry (12 with colour words: 4 + 4 + 4 at one entry, at most 4 + 2 + 1 per entry
-// beyond), and its successive blocks form a doubling series bounded by twice the last one, so at
-// most 16 (24) slots per stored entry, i.e. 32 (48) slots, 8 (12) quads, per stream edge.
-unsigned long long quads_bound(unsigned long long edges, bool words) {
-    return (words ? 12ull : 8ull) * edges + 64ull;
+// Pool quads that guarantee no batch can run out: a node's block holds at most 2 quads per entry (3 with
+// colour words: at one entry, less beyond), and its successive blocks form a doubling series bounded by
+// twice the last one, so at most 4 (6) quads per stored entry, i.e. 8 (12) per stream edge.
+unsigned long long quads_bound(unsigned long long edges, uint32_t colours) {
+    return (colours == kColWords || colours == kColMulti ? 12ull : 8ull) * edges + 64ull;
 }
 
 int grow_pool(rept_state* s, unsigned long long min_quads, cudaStream_t st) {
@@ -119,6 +119,17 @@ int read_ctrl(rept_state* s, cudaStream_t st) {
     return REPT_OK;
 }
 
+// Shared memory of an intersection launch for c processors.  (cudaFuncSetAttribute lifts the default
+// limit of the kernel; it applies to the current device.)
+size_t intersect_smem(uint32_t colours, uint32_t c) {
+    return ix_words((int)colours, false) * sizeof(uint32_t) + c * sizeof(unsigned long long);
+}
+
+template <class K>
+cudaError_t allow_smem(K* kernel, size_t bytes) {
+    return cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
 int ensure_batch_scratch(rept_state* s, unsigned long long n, cudaStream_t st) {
     if (n <= s->max_batch) return REPT_OK;
     REPT_CUDA(cudaStreamSynchronize(st));
@@ -127,15 +138,17 @@ int ensure_batch_scratch(rept_state* s, unsigned long long n, cudaStream_t st) {
     dev_free(s, s->d.grow_rel, 2 * old * sizeof(uint32_t));
     dev_free(s, s->d.big, 2 * old * sizeof(uint32_t));
     dev_free(s, s->d.rec, old * sizeof(WorkItem));
-    dev_free(s, s->d.srec, old * sizeof(WorkItem));
+    dev_free(s, s->d.units, old * kListBytes);
     s->d.touched = s->d.grow_rel = s->d.big = nullptr;
-    s->d.rec = s->d.srec = nullptr;
+    s->d.rec = nullptr;
+    s->d.units = nullptr;
     int rc = dev_alloc(s, (void**)&s->d.touched, 2 * n * sizeof(uint32_t));
     if (!rc) rc = dev_alloc(s, (void**)&s->d.grow_rel, 2 * n * sizeof(uint32_t));
     if (!rc) rc = dev_alloc(s, (void**)&s->d.big, 2 * n * sizeof(uint32_t));
     if (!rc) rc = dev_alloc(s, (void**)&s->d.rec, n * sizeof(WorkItem));
-    if (!rc) rc = dev_alloc(s, (void**)&s->d.srec, n * sizeof(WorkItem));
+    if (!rc) rc = dev_alloc(s, (void**)&s->d.units, n * kListBytes);
     if (rc) return rc;
+    set_list_pointers(s->d, n);
     s->max_batch = n;
     s->d.big_cap = 2 * n;
     return REPT_OK;
@@ -239,7 +252,7 @@ int launch_batch(rept_state* s, const uint32_t* d_src, const uint32_t* d_dst, un
         const int prc = ensure_pair_capacity(s, s->next_t + n, st);
         if (prc) return prc;
     }
-    BatchDev b{d_src, d_dst, n, s->next_t};
+    const BatchDev b = make_batch(d_src, d_dst, n, s->next_t, s->tile_max);
     const int threads = 256;
     const unsigned long long want_blocks = (n + threads - 1) / threads;
     const int grid = (int)std::min<unsigned long long>(want_blocks, (unsigned long long)s->grid_stream);
@@ -257,7 +270,7 @@ int launch_batch(rept_state* s, const uint32_t* d_src, const uint32_t* d_dst, un
     }
     if ((rc = timed_launch(s, REPT_K_PLAN, st, [&] { k_plan<<<grid, threads, 0, st>>>(s->d); }))) return rc;
     const bool fixed = (s->cfg.flags & REPT_FLAG_FIXED_POOL) != 0;
-    if (!fixed && s->d.pool_quads < quads_bound(s->next_t + n, has_words(s->d))) {
+    if (!fixed && s->d.pool_quads < quads_bound(s->next_t + n, s->d.colours)) {
         // not provably large enough: read this batch's request and grow if needed
         if ((rc = read_ctrl(s, st))) return rc;
         const unsigned long long need = s->h_ctrl->pool_top + s->h_ctrl->need_quads;
@@ -268,29 +281,32 @@ int launch_batch(rept_state* s, const uint32_t* d_src, const uint32_t* d_dst, un
     if ((rc = timed_launch(s, REPT_K_COMMIT, st, [&] {
              k_commit<<<grid, threads, 0, st>>>(s->d);
              k_rehash_big<<<s->sm_count * 4, threads, 0, st>>>(s->d);
-             k_rehash_huge<<<s->sm_count * 2, 1024, 0, st>>>(s->d);
+             k_rehash_huge<<<s->sm_count * 2, 1024, kHugeSmemWords * sizeof(uint32_t), st>>>(s->d);
          }, 3)))
         return rc;
     if ((rc = timed_launch(s, REPT_K_INSERT, st, [&] { k_insert<<<grid, threads, 0, st>>>(s->d, b); }))) return rc;
     if ((rc = timed_launch(s, REPT_K_SORT, st, [&] {
-             k_sort_scan<<<1, 1024, 0, st>>>(s->d);
-             k_sort_scatter<<<grid, threads, 0, st>>>(s->d, b);
+             k_units<<<grid, threads, 0, st>>>(s->d, b);
+             k_order<<<grid, threads, 0, st>>>(s->d, b);
          }, 2)))
         return rc;
-    const unsigned long long want_i = (n * 8 + 255) / 256;  // work is claimed dynamically; >= 1 block
+    const unsigned long long want_i = (n + 31) / 32;  // work is claimed dynamically; >= 1 block
     const int grid_i = (int)std::min<unsigned long long>(want_i, (unsigned long long)s->grid_intersect);
-    const size_t smem = s->cfg.c * sizeof(unsigned long long);
+    const size_t smem = intersect_smem(s->d.colours, s->cfg.c);
     const bool work = (s->cfg.flags & REPT_FLAG_WORK_COUNTERS) != 0;
     rc = timed_launch(s, REPT_K_INTERSECT, st, [&] {
         if (s->d.colours == kColInEntry) {
-            if (work) k_intersect<true><<<grid_i, 256, smem, st>>>(s->d, b);
-            else k_intersect<false><<<grid_i, 256, smem, st>>>(s->d, b);
+            if (work) k_intersect<true><<<grid_i, kIxThreads, smem, st>>>(s->d, b);
+            else k_intersect<false><<<grid_i, kIxThreads, smem, st>>>(s->d, b);
         } else if (s->d.colours == kColWords) {
-            if (work) k_intersect_words<true><<<grid_i, 256, smem, st>>>(s->d, b);
-            else k_intersect_words<false><<<grid_i, 256, smem, st>>>(s->d, b);
+            if (work) k_intersect_words<true><<<grid_i, kIxThreads, smem, st>>>(s->d, b);
+            else k_intersect_words<false><<<grid_i, kIxThreads, smem, st>>>(s->d, b);
+        } else if (s->d.colours == kColMulti) {
+            if (work) k_intersect_multi<true><<<grid_i, kIxThreads, smem, st>>>(s->d, b);
+            else k_intersect_multi<false><<<grid_i, kIxThreads, smem, st>>>(s->d, b);
         } else {
-            if (work) k_intersect_probe<true><<<grid_i, 256, smem, st>>>(s->d, b);
-            else k_intersect_probe<false><<<grid_i, 256, smem, st>>>(s->d, b);
+            if (work) k_intersect_probe<true><<<grid_i, kIxThreads, smem, st>>>(s->d, b);
+            else k_intersect_probe<false><<<grid_i, kIxThreads, smem, st>>>(s->d, b);
         }
     });
     if (rc) return rc;
@@ -366,16 +382,27 @@ int rept_create(const rept_config* cfg, void* stream, rept_state** out) {
     uint32_t cbits = 0;
     while (cbits < 32 && (1ull << cbits) < cfg->m) ++cbits;
     const bool coloured = n_groups == 1 && cfg->m >= 2 && cfg->m <= 256 && cfg->n_nodes <= (1u << kIdBits);
-    // colour words: one group that cannot carry its colour in the entries.  With several groups an
-    // entry would cost a hash per group, which measured slower than probing every entry: the 5-group
-    // Chung-Lu stream's intersection took 404 ms per step with words (scan first, candidate queue)
-    // against 162 ms probing.
+    // colour words: one group that cannot carry its colour in the entries
     const bool words = !coloured && !mascot_flag && cfg->m >= 2 && n_groups == 1;
+    // several groups: their colours in one word, or a bit per group where a group keeps one colour only
+    const bool one_colour = mascot_flag || cfg->m == 1;
+    const bool multi = !coloured && !words && n_groups * (one_colour ? 1ull : cbits) <= 32ull;
+    uint32_t colours = coloured ? kColInEntry : words ? kColWords : multi ? kColMulti : kColNone;
+    const size_t max_smem = intersect_smem(kColMulti, kMaxProcessors);
+    if (allow_smem(k_rehash_huge, kHugeSmemWords * sizeof(uint32_t)) != cudaSuccess ||
+        allow_smem(k_intersect<false>, max_smem) != cudaSuccess || allow_smem(k_intersect<true>, max_smem) != cudaSuccess ||
+        allow_smem(k_intersect_words<false>, max_smem) != cudaSuccess ||
+        allow_smem(k_intersect_words<true>, max_smem) != cudaSuccess ||
+        allow_smem(k_intersect_multi<false>, max_smem) != cudaSuccess ||
+        allow_smem(k_intersect_multi<true>, max_smem) != cudaSuccess ||
+        allow_smem(k_intersect_probe<false>, max_smem) != cudaSuccess ||
+        allow_smem(k_intersect_probe<true>, max_smem) != cudaSuccess)
+        return fail(REPT_E_CUDA);
     const void* k3 = coloured ? (const void*)k_intersect<false>
-                              : words ? (const void*)k_intersect_words<false> : (const void*)k_intersect_probe<false>;
+                     : words ? (const void*)k_intersect_words<false>
+                     : multi ? (const void*)k_intersect_multi<false> : (const void*)k_intersect_probe<false>;
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k3, 256, cfg->c * sizeof(unsigned long long)) !=
-        cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k3, kIxThreads, intersect_smem(colours, cfg->c)) != cudaSuccess)
         return fail(REPT_E_CUDA);
     s->grid_intersect = s->sm_count * std::max(per_sm, 1);
     s->grid_stream = s->sm_count * 8;
@@ -389,24 +416,29 @@ int rept_create(const rept_config* cfg, void* stream, rept_state** out) {
     d.n_nodes = n;
     d.seed = cfg->seed;
     d.fm = make_fastmod(cfg->m);
-    d.tile_max = cfg->tile_max == 0 ? 32u : cfg->tile_max;
+    s->tile_max = cfg->tile_max == 0 ? 32u : cfg->tile_max;
     const unsigned long long mb = cfg->max_batch ? cfg->max_batch : (1ull << 20);
-    unsigned long long quads = quads_bound(cfg->expected_edges ? cfg->expected_edges : mb, words);
-    if (quads > 0xFFFFFFFFull) quads = 0xFFFFFFFFull;
+    auto wanted_quads = [&] {
+        return std::min(quads_bound(cfg->expected_edges ? cfg->expected_edges : mb, colours), 0xFFFFFFFFull);
+    };
+    unsigned long long quads = wanted_quads();
     if ((rc = dev_alloc(s, (void**)&d.meta, (size_t)n * sizeof(uint4)))) return fail(rc);
     if ((rc = dev_alloc(s, (void**)&d.cnt_add, (size_t)n * sizeof(uint32_t)))) return fail(rc);
     if ((rc = dev_alloc(s, (void**)&d.local, (size_t)n * sizeof(unsigned long long)))) return fail(rc);
     if ((rc = dev_alloc(s, (void**)&d.proc, (size_t)cfg->c * sizeof(unsigned long long)))) return fail(rc);
     if ((rc = dev_alloc(s, (void**)&d.ctrl, sizeof(Ctrl)))) return fail(rc);
-    if ((rc = dev_alloc(s, (void**)&d.hist, kSortBuckets * sizeof(uint32_t)))) return fail(rc);
-    if ((rc = dev_alloc(s, (void**)&d.pool, quads * 32ull))) return fail(rc);
+    rc = dev_alloc(s, (void**)&d.pool, quads * 32ull);
+    if (rc == REPT_E_NOMEM && colours == kColMulti) {  // the layout without colour words needs a third less
+        colours = kColNone;
+        quads = wanted_quads();
+        rc = dev_alloc(s, (void**)&d.pool, quads * 32ull);
+    }
+    if (rc) return fail(rc);
     if ((rc = dev_alloc(s, (void**)&s->d_global, sizeof(double)))) return fail(rc);
     d.pool_quads = quads;
-    // one hash group, few colours and ids of at most kIdBits: list entries carry their colour;
-    // several groups whose colours fit 32 bits: a colour word per entry
-    d.colours = coloured ? kColInEntry : words ? kColWords : kColNone;
-    d.cbits = words ? cbits : 0u;
-    d.cmask = words ? (uint32_t)((1ull << cbits) - 1ull) : 0u;
+    d.colours = colours;
+    d.cbits = colours == kColMulti && one_colour ? 1u : cbits;
+    d.cmask = (uint32_t)((1ull << d.cbits) - 1ull);
     d.c1 = mascot || cfg->c <= cfg->m ? cfg->c : cfg->c / cfg->m;
     d.keep = mascot ? 1u : cfg->m;
     d.pstride = mascot ? 1u : cfg->m;
@@ -414,6 +446,7 @@ int rept_create(const rept_config* cfg, void* stream, rept_state** out) {
     d.pcount = sharded ? cfg->proc_end - cfg->proc_begin : cfg->c;
     d.kbeg = d.pbeg / d.pstride;
     d.kend = (d.pbeg + d.pcount - 1u) / d.pstride + 1u;
+    for (uint32_t k = d.kbeg; colours == kColMulti && k < d.kend; ++k) d.ctop |= 1u << ((k + 1u) * d.cbits - 1u);
     if (cfg->flags & REPT_FLAG_LOCAL_PER_PROCESSOR) {
         if ((rc = dev_alloc(s, (void**)&d.local_proc, (size_t)cfg->c * n * sizeof(unsigned long long))))
             return fail(rc);
@@ -615,10 +648,13 @@ struct SnapHeader {
     uint64_t m, c, seed, n_nodes, flags, groups;
     uint64_t next_t, pool_top, self_loops, stored;
     uint64_t proc_begin, proc_end;
+    uint64_t colours;  // version 4: the layout of the blocks (StreamDev::colours)
 };
 constexpr uint64_t kSnapMagic = 0x5245505453544154ull;  // "REPTSTAT"
-// 3: a table bucket holds its 4 ids and then their 4 stream indices (2: ids and indices in two arrays)
-constexpr uint64_t kSnapVersion = 3;
+// 4: lists hold the entry words side by side.  3 (still read): lists of {entry word, stream index}
+// pairs, no kColMulti, a header without `colours`.
+constexpr uint64_t kSnapVersion = 4;
+constexpr size_t kSnapHeader3 = sizeof(SnapHeader) - sizeof(uint64_t);
 
 // The arrays of a snapshot after the header, in order: {device pointer, bytes}.
 struct SnapPart {
@@ -674,7 +710,7 @@ int rept_snapshot(rept_state* s, void* h_buf, uint64_t bytes, void* stream) {
     if (bytes < total) return REPT_E_INVAL;
     SnapHeader h{kSnapMagic, kSnapVersion, s->cfg.m, s->cfg.c, s->cfg.seed, s->cfg.n_nodes, s->cfg.flags, s->groups,
                  s->next_t, s->h_ctrl->pool_top, s->h_ctrl->self_loops, s->h_ctrl->stored,
-                 s->cfg.proc_begin, s->cfg.proc_end};
+                 s->cfg.proc_begin, s->cfg.proc_end, s->d.colours};
     std::memcpy(h_buf, &h, sizeof(h));
     char* out = static_cast<char*>(h_buf) + sizeof(h);
     for (int i = 0; i < np; ++i) {
@@ -686,38 +722,92 @@ int rept_snapshot(rept_state* s, void* h_buf, uint64_t bytes, void* stream) {
 }
 
 int rept_restore(rept_state* s, const void* h_buf, uint64_t bytes, void* stream) {
-    if (!s || !h_buf || bytes < sizeof(SnapHeader)) return REPT_E_INVAL;
+    if (!s || !h_buf || bytes < kSnapHeader3) return REPT_E_INVAL;
     cudaStream_t st = as_stream(stream);
-    SnapHeader h;
-    std::memcpy(&h, h_buf, sizeof(h));
-    if (h.magic != kSnapMagic || h.version != kSnapVersion || h.m != s->cfg.m || h.c != s->cfg.c || h.seed != s->cfg.seed ||
-        h.n_nodes != s->cfg.n_nodes || h.flags != s->cfg.flags || h.groups != s->groups ||
-        h.proc_begin != s->cfg.proc_begin || h.proc_end != s->cfg.proc_end)
+    SnapHeader h{};
+    std::memcpy(&h, h_buf, kSnapHeader3);
+    const bool pairs = h.version == 3;
+    const size_t header = pairs ? kSnapHeader3 : sizeof(SnapHeader);
+    if (h.magic != kSnapMagic || (!pairs && h.version != kSnapVersion) || bytes < header || h.m != s->cfg.m ||
+        h.c != s->cfg.c || h.seed != s->cfg.seed || h.n_nodes != s->cfg.n_nodes || h.flags != s->cfg.flags ||
+        h.groups != s->groups || h.proc_begin != s->cfg.proc_begin || h.proc_end != s->cfg.proc_end)
         return REPT_E_INVAL;
+    if (pairs) h.colours = s->d.colours == kColMulti ? kColNone : s->d.colours;
+    else std::memcpy(&h.colours, static_cast<const char*>(h_buf) + kSnapHeader3, sizeof(h.colours));
+    // another layout can be taken over if its lists hold the stream indices
+    const bool convert = pairs || h.colours != s->d.colours;
+    if (convert && !pairs && (interleaved((uint32_t)h.colours) || interleaved(s->d.colours))) return REPT_E_INVAL;
     int rc = rept_reset(s, stream);
     if (rc) return rc;
-    if (h.pool_top > s->d.pool_quads && (rc = grow_pool(s, h.pool_top, st))) return rc;
+    const size_t n = s->d.n_nodes;
     s->next_t = h.next_t;
     if (s->d.local2 && (rc = ensure_pair_capacity(s, std::max<unsigned long long>(h.next_t, 1), st))) return rc;
     SnapPart parts[16];
     int np = 0;
     snap_parts(s, h.pool_top, parts, &np);
-    unsigned long long total = sizeof(SnapHeader);
+    unsigned long long total = header;
     for (int i = 0; i < np; ++i) total += parts[i].bytes;
     if (bytes < total) return REPT_E_INVAL;
-    const char* in = static_cast<const char*>(h_buf) + sizeof(h);
-    for (int i = 0; i < np; ++i) {
-        if (parts[i].bytes) REPT_CUDA(cudaMemcpyAsync(parts[i].ptr, in, parts[i].bytes, cudaMemcpyHostToDevice, st));
+    const char* in = static_cast<const char*>(h_buf) + header;
+    unsigned long long pool_top = h.pool_top;
+    std::vector<uint4> meta;
+    std::vector<uint32_t> old_off;
+    if (convert) {  // new block offsets, in node order
+        meta.resize(n);
+        old_off.resize(n);
+        std::memcpy(meta.data(), in, n * sizeof(uint4));
+        pool_top = 0;
+        for (size_t x = 0; x < n; ++x) {
+            old_off[x] = meta[x].x;
+            const uint32_t cnt = meta[x].y;
+            meta[x].x = cnt ? (uint32_t)pool_top : 0u;
+            if (cnt) pool_top += block_quads(table_lg(cnt), s->d.colours);
+        }
+    }
+    if (pool_top > s->d.pool_quads) {
+        if ((rc = grow_pool(s, pool_top, st))) return rc;
+        snap_parts(s, h.pool_top, parts, &np);  // the pool moved
+    }
+    void* old_pool = nullptr;
+    uint32_t* d_old_off = nullptr;
+    if (convert) {
+        if (cudaMalloc(&old_pool, std::max<size_t>(parts[3].bytes, 32)) != cudaSuccess ||
+            cudaMalloc((void**)&d_old_off, n * sizeof(uint32_t)) != cudaSuccess) {
+            (void)cudaGetLastError();
+            cudaFree(old_pool);
+            return REPT_E_NOMEM;
+        }
+        parts[3].ptr = old_pool;
+    }
+    cudaError_t err = cudaSuccess;
+    for (int i = 0; i < np && err == cudaSuccess; ++i) {
+        const void* src = convert && i == 0 ? (const void*)meta.data() : in;
+        if (parts[i].bytes) err = cudaMemcpyAsync(parts[i].ptr, src, parts[i].bytes, cudaMemcpyHostToDevice, st);
         in += parts[i].bytes;
     }
     // control block: the pool in use and the tallies; every per-batch counter starts at zero
     Ctrl c{};
-    c.pool_top = h.pool_top;
+    c.pool_top = pool_top;
     c.self_loops = h.self_loops;
     c.stored = h.stored;
     std::memcpy(s->h_ctrl, &c, sizeof(Ctrl));
-    REPT_CUDA(cudaMemcpyAsync(s->d.ctrl, s->h_ctrl, sizeof(Ctrl), cudaMemcpyHostToDevice, st));
-    REPT_CUDA(cudaStreamSynchronize(st));
+    if (err == cudaSuccess) err = cudaMemcpyAsync(s->d.ctrl, s->h_ctrl, sizeof(Ctrl), cudaMemcpyHostToDevice, st);
+    if (convert && err == cudaSuccess) {
+        err = cudaMemcpyAsync(d_old_off, old_off.data(), n * sizeof(uint32_t), cudaMemcpyHostToDevice, st);
+        if (err == cudaSuccess) {
+            k_convert<<<s->sm_count * 8, 256, 0, st>>>(s->d, static_cast<const uint2*>(old_pool), d_old_off,
+                                                       (uint32_t)h.colours, pairs);
+            g_launches.fetch_add(1, std::memory_order_relaxed);
+            err = cudaPeekAtLastError();
+        }
+    }
+    if (err == cudaSuccess) err = cudaStreamSynchronize(st);
+    cudaFree(old_pool);
+    cudaFree(d_old_off);
+    if (err != cudaSuccess) {
+        (void)cudaGetLastError();
+        return REPT_E_CUDA;
+    }
     return REPT_OK;
 }
 
@@ -760,7 +850,7 @@ int rept_get_stats(rept_state* s, rept_stats* out, void* stream) {
     out->probe_slots = s->h_ctrl->probe_slots;
     out->wedges = s->h_ctrl->wedges;
     out->counted = s->h_ctrl->counted;
-    for (int c = 0; c < kBins; ++c) {
+    for (int c = 0; c < kClasses; ++c) {
         out->class_items[c] = s->h_ctrl->class_items[c];
         out->class_probes[c] = s->h_ctrl->class_probes[c];
         out->class_cycles[c] = s->h_ctrl->class_cycles[c];
@@ -802,7 +892,7 @@ void rept_destroy(rept_state* s) {
     cudaFree(d.grow_rel);
     cudaFree(d.big);
     cudaFree(d.rec);
-    cudaFree(d.srec);
+    cudaFree(d.units);
     cudaFree(d.local2);
     cudaFree(d.eta_proc);
     cudaFree(d.eta_local);
@@ -811,7 +901,6 @@ void rept_destroy(rept_state* s) {
     cudaFree(d.pair_evt);
     cudaFree(d.pair_list);
     cudaFree(d.local_proc);
-    cudaFree(d.hist);
     cudaFree(s->stage_src);
     cudaFree(s->stage_dst);
     cudaFree(s->d_global);
@@ -847,7 +936,7 @@ __global__ void k_gather_requests(const StreamDev* __restrict__ ds, uint32_t k, 
 
 struct rept_group {
     uint32_t max_streams = 0, flags = 0;
-    int sm_count = 0, intersect_per_sm = 1;
+    int sm_count = 0, intersect_per_sm[4] = {1, 1, 1, 1};  // group_intersect
     StreamDev* d_sd = nullptr;  // device descriptor arrays read by the _multi kernels
     BatchDev* d_bd = nullptr;
     unsigned long long* d_req = nullptr;
@@ -859,7 +948,7 @@ struct rept_group {
     unsigned long long* h_req = nullptr;
     cudaEvent_t slot_done[2] = {nullptr, nullptr};
     cudaGraphExec_t exec[2] = {nullptr, nullptr};
-    unsigned long long shape[2][6] = {{0}};  // what each slot's graph was captured for
+    unsigned long long shape[2][5] = {{0}};  // what each slot's graph was captured for
     int slot = 0;
     cudaStream_t capture = nullptr;  // private stream the graphs are captured on (the legacy stream cannot be)
     // REPT_GROUP_PERSISTENT: the grid barrier state, its per-launch initial value (pinned), and the
@@ -872,10 +961,28 @@ struct rept_group {
 
 namespace {
 
+// The group intersection for streams that all store colours alike (kColAny: that do not).
+struct GroupIntersect {
+    void (*kernel)(const StreamDev*, const BatchDev*, uint32_t, const unsigned long long*, unsigned long long*);
+    size_t smem;
+    int slot;  // in rept_group::intersect_per_sm
+};
+constexpr int kGroupIntersects = 4;
+template <int MODE>
+constexpr GroupIntersect make_group_intersect(int slot) {
+    return GroupIntersect{k_intersect_group<MODE>, ix_words(MODE, true) * sizeof(uint32_t), slot};
+}
+const GroupIntersect& group_intersect(int colours) {
+    static const GroupIntersect all[kGroupIntersects] = {
+        make_group_intersect<kColAny>(0), make_group_intersect<(int)kColInEntry>(1),
+        make_group_intersect<(int)kColWords>(2), make_group_intersect<(int)kColMulti>(3)};
+    return all[colours == (int)kColInEntry ? 1 : colours == (int)kColWords ? 2 : colours == (int)kColMulti ? 3 : 0];
+}
+
 struct GroupShape {
     uint32_t k;
-    int x_edge, x_big, x_huge, x_int;
-    size_t smem;
+    int colours;  // of every stream, or kColAny
+    int x_edge, x_big, x_huge;
 };
 
 // Enqueue the batch path for all k streams: one launch per step.  With `split`, stop after
@@ -890,13 +997,15 @@ int enqueue_group(rept_group* g, const GroupShape& sh, cudaStream_t st, int part
     if (part != 1) {
         k_commit_multi<<<dim3(sh.x_edge, k), blk, 0, st>>>(g->d_sd, g->d_bd);
         k_rehash_big_multi<<<dim3(sh.x_big, k), blk, 0, st>>>(g->d_sd, g->d_bd);
-        k_rehash_huge_multi<<<dim3(sh.x_huge, k), dim3(1024), 0, st>>>(g->d_sd, g->d_bd);
+        k_rehash_huge_multi<<<dim3(sh.x_huge, k), dim3(1024), kHugeSmemWords * sizeof(uint32_t), st>>>(g->d_sd, g->d_bd);
         k_insert_multi<<<dim3(sh.x_edge, k), blk, 0, st>>>(g->d_sd, g->d_bd);
-        k_sort_scan_multi<<<dim3(1, k), dim3(1024), 0, st>>>(g->d_sd, g->d_bd);
-        k_sort_scatter_multi<<<dim3(sh.x_edge, k), blk, 0, st>>>(g->d_sd, g->d_bd);
+        k_units_multi<<<dim3(sh.x_edge, k), blk, 0, st>>>(g->d_sd, g->d_bd);
+        k_order_multi<<<dim3(sh.x_edge, k), blk, 0, st>>>(g->d_sd, g->d_bd);
         // one grid for all streams' intersection work
         k_group_prefix<<<1, 1024, 0, st>>>(g->d_sd, k, g->d_pref, g->d_cursor);
-        k_intersect_group<<<g->intersect_per_sm * g->sm_count, blk, 0, st>>>(g->d_sd, k, g->d_pref, g->d_cursor);
+        const GroupIntersect& gi = group_intersect(sh.colours);
+        gi.kernel<<<g->intersect_per_sm[gi.slot] * g->sm_count, kIxThreads, gi.smem, st>>>(g->d_sd, g->d_bd, k, g->d_pref,
+                                                                                            g->d_cursor);
     }
     const int launched = part == 1 ? 2 : (part == 2 ? 8 : 10);
     g_launches.fetch_add((unsigned long long)launched, std::memory_order_relaxed);
@@ -951,10 +1060,15 @@ int rept_group_create(uint32_t max_streams, uint32_t flags, rept_group** out) {
     if (cudaGetDevice(&dev) != cudaSuccess) return fail(REPT_E_CUDA);
     if (cudaDeviceGetAttribute(&g->sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return fail(REPT_E_CUDA);
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_intersect_group, 256, 0) != cudaSuccess)
-        return fail(REPT_E_CUDA);
-    g->intersect_per_sm = std::max(per_sm, 1);
+    if (allow_smem(k_rehash_huge_multi, kHugeSmemWords * sizeof(uint32_t)) != cudaSuccess) return fail(REPT_E_CUDA);
+    for (int colours : {kColAny, (int)kColInEntry, (int)kColWords, (int)kColMulti}) {
+        const GroupIntersect& gi = group_intersect(colours);
+        int per_sm = 0;
+        if (allow_smem(gi.kernel, gi.smem) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gi.kernel, kIxThreads, gi.smem) != cudaSuccess)
+            return fail(REPT_E_CUDA);
+        g->intersect_per_sm[gi.slot] = std::max(per_sm, 1);
+    }
     if (cudaMalloc(&g->d_sd, max_streams * sizeof(StreamDev)) != cudaSuccess) return fail(REPT_E_NOMEM);
     if (cudaMalloc(&g->d_bd, max_streams * sizeof(BatchDev)) != cudaSuccess) return fail(REPT_E_NOMEM);
     if (cudaMalloc(&g->d_req, 3ull * max_streams * sizeof(unsigned long long)) != cudaSuccess)
@@ -977,6 +1091,7 @@ int rept_group_create(uint32_t max_streams, uint32_t flags, rept_group** out) {
         int coop = 0, per_sm_p = 0;
         if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop)
             return fail(REPT_E_CUDA);
+        if (allow_smem(k_group_persistent, kPersistSmemWords * sizeof(uint32_t)) != cudaSuccess) return fail(REPT_E_CUDA);
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_p, k_group_persistent, 256,
                                                           kPersistSmemWords * sizeof(uint32_t)) != cudaSuccess ||
             per_sm_p < 1)
@@ -1017,7 +1132,6 @@ int rept_group_ingest(rept_group* g, rept_state* const* hs, const uint32_t* cons
     NvtxRange range("rept group ingest");
     cudaStream_t st = as_stream(stream);
     unsigned long long max_n = 0;
-    uint32_t max_c = 1;
     bool guaranteed = true;
     for (uint32_t i = 0; i < k; ++i) {
         rept_state* s = hs[i];
@@ -1027,9 +1141,8 @@ int rept_group_ingest(rept_group* g, rept_state* const* hs, const uint32_t* cons
         int rc = ensure_batch_scratch(s, std::max<unsigned long long>(n[i], 1ull), st);
         if (rc) return rc;
         max_n = std::max<unsigned long long>(max_n, n[i]);
-        max_c = std::max(max_c, s->cfg.c);
         const bool fixed = (s->cfg.flags & REPT_FLAG_FIXED_POOL) != 0;
-        if (!fixed && s->d.pool_quads < quads_bound(s->next_t + n[i], has_words(s->d))) guaranteed = false;
+        if (!fixed && s->d.pool_quads < quads_bound(s->next_t + n[i], s->d.colours)) guaranteed = false;
     }
     // launch shape: the edge kernels cover the largest batch, the rest share the SMs between streams
     GroupShape sh{};
@@ -1039,8 +1152,9 @@ int rept_group_ingest(rept_group* g, rept_state* const* hs, const uint32_t* cons
     sh.x_edge = (int)std::min<unsigned long long>((pow2 + 255) / 256, (unsigned long long)per_stream_cap);
     sh.x_big = std::max(1, 4 * g->sm_count / (int)k);
     sh.x_huge = std::max(1, 2 * g->sm_count / (int)k);
-    sh.x_int = std::max(1, g->intersect_per_sm * g->sm_count / (int)k);
-    sh.smem = (size_t)max_c * sizeof(unsigned long long);
+    sh.colours = (int)hs[0]->d.colours;
+    for (uint32_t i = 1; i < k; ++i)
+        if ((int)hs[i]->d.colours != sh.colours) sh.colours = kColAny;
 
     const int slot = g->slot;
     g->slot ^= 1;
@@ -1049,7 +1163,7 @@ int rept_group_ingest(rept_group* g, rept_state* const* hs, const uint32_t* cons
     BatchDev* hbd = g->h_bd[slot];
     for (uint32_t i = 0; i < k; ++i) {
         hsd[i] = hs[i]->d;
-        hbd[i] = BatchDev{d_src[i], d_dst[i], n[i], hs[i]->next_t};
+        hbd[i] = make_batch(d_src[i], d_dst[i], n[i], hs[i]->next_t, hs[i]->tile_max);
     }
     auto upload = [&]() -> int {
         REPT_CUDA(cudaMemcpyAsync(g->d_sd, hsd, k * sizeof(StreamDev), cudaMemcpyHostToDevice, st));
@@ -1084,10 +1198,10 @@ int rept_group_ingest(rept_group* g, rept_state* const* hs, const uint32_t* cons
         if ((rc = enqueue_persistent(g, sh, st))) return rc;
     } else if (g->flags & REPT_GROUP_GRAPH) {
         const bool persistent = (g->flags & REPT_GROUP_PERSISTENT) != 0;
-        const unsigned long long key[6] = {k, (unsigned long long)sh.x_edge, (unsigned long long)sh.x_big,
-                                           (unsigned long long)sh.x_huge, (unsigned long long)sh.x_int, sh.smem};
+        const unsigned long long key[5] = {k, (unsigned long long)sh.x_edge, (unsigned long long)sh.x_big,
+                                           (unsigned long long)sh.x_huge, (unsigned long long)sh.colours};
         bool same = g->exec[slot] != nullptr;
-        for (int j = 0; j < 6 && same; ++j) same = g->shape[slot][j] == key[j];
+        for (int j = 0; j < 5 && same; ++j) same = g->shape[slot][j] == key[j];
         if (!same) {
             if (g->exec[slot]) {
                 cudaGraphExecDestroy(g->exec[slot]);
@@ -1121,7 +1235,7 @@ int rept_group_ingest(rept_group* g, rept_state* const* hs, const uint32_t* cons
             }
             if (rc_cap) return rc_cap;
             if (e_end != cudaSuccess || e_inst != cudaSuccess) return REPT_E_CUDA;
-            for (int j = 0; j < 6; ++j) g->shape[slot][j] = key[j];
+            for (int j = 0; j < 5; ++j) g->shape[slot][j] = key[j];
         }
         REPT_CUDA(cudaGraphLaunch(g->exec[slot], st));
         g_launches.fetch_add(persistent ? 1 : 10, std::memory_order_relaxed);

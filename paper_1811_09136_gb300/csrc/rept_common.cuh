@@ -1,30 +1,33 @@
 // Device-side data layout and helpers of the REPT streaming counter.
 //
 // HBM layout of one stream (one rept_state):
-//   meta[n_nodes]   uint4 {off, cnt, add, 0}: node x's block starts at slot
+//   meta[n_nodes]   uint4 {off, cnt, add, grp}: node x's block starts at slot
 //                   4*off of the pool and holds cnt entries; its size is a
 //                   function of cnt alone (table_lg below), so a node's block
 //                   is re-allocated exactly when cnt crosses a power-of-two
 //                   boundary.  add counts the current batch's new entries of x
 //                   (zero between batches); it shares x's 16-byte record so
 //                   that the insert's position counter and the block's place
-//                   sit in one 32-byte sector.  k_classify counts into the
+//                   sit in one 32-byte sector.  grp counts the batch's
+//                   grouped edges whose larger endpoint is x (zero between
+//                   batches).  k_classify counts into the
 //                   compact array cnt_add[n_nodes] first; k_plan moves the
 //                   counts into the records.
-//   pool[]          8-byte slots: per node, an open-addressing (linear probing,
+//   pool[]          32-byte quads: per node, an open-addressing (linear probing,
 //                   4-key buckets) table of 2^lg neighbour ids and their stream
-//                   indices (2^lg slots in all; for streams with stored colours
+//                   indices (for single-group streams with stored colours
 //                   each 32-byte bucket holds its 4 ids and then their 4
 //                   indices, so that an insert or a probe hit touches one
-//                   sector; streams that probe every candidate keep all ids
+//                   sector; the others keep all ids
 //                   first and the indices after them, ids packed densely), then
-//                   the same entries as a packed list of {nbr, eidx} pairs
-//                   (and, for streams with colour words, one word per entry).
+//                   the neighbour ids as a packed list, 4 bytes each, which is
+//                   all that the intersection's scans read (block_quads).
 //                   An entry (w, t) of x is the stored edge {x, w} that
 //                   arrived at stream index t.  Empty keys are all-ones.  The
 //                   tables of all processors share one union adjacency: an
 //                   edge is stored once if any processor keeps it, and which
-//                   processors keep it is recomputed from the hash when needed
+//                   processors keep it is recomputed from the hash or read from
+//                   a stored colour word when needed
 //                   (Section III-A: processor i keeps colour i).
 //   local[n_nodes]  uint64 sum over processors of tau_v^(i)
 //   proc[c]         uint64 tau^(i)
@@ -33,6 +36,7 @@
 // the control block.
 #pragma once
 
+#include <algorithm>
 #include <cstdint>
 #include <cstdio>
 
@@ -41,20 +45,28 @@
 namespace rept {
 
 constexpr uint32_t kEmptyId = 0xFFFFFFFFu;
-constexpr unsigned long long kEmptySlot = 0xFFFFFFFFFFFFFFFFull;
 constexpr uint64_t kGoldenGamma = 0x9E3779B97F4A7C15ull;  // SplitMix64 increment
 constexpr uint32_t kIdBits = 24;                             // node-id bits of a list entry with a colour
 constexpr uint32_t kIdMask = (1u << kIdBits) - 1u;
 constexpr uint32_t kNoGrow = 0xFFFFFFFFu;
 constexpr uint32_t kMaxProcessors = 4096;  // per-block tau^(i) histogram lives in shared memory
-// Number of k_intersect work classes (see bin_of_cnt).
-constexpr int kBins = 6;
-// Within a class, work items are ordered by a hash of the larger endpoint (kKeyBits bits), so that
-// the edges probing the same large table run back to back and find it in L2.
-constexpr int kKeyBits = 13;
-constexpr uint32_t kKeyBuckets = 1u << kKeyBits;
-constexpr uint32_t kSortBuckets = kBins * kKeyBuckets;
-constexpr uint16_t kNoKey = 0xFFFFu;
+// Work kinds of the intersection.  An edge whose smaller endpoint holds at most tile_max entries is
+// small: warps take them straight from the batch, a chunk of edges at a time.  The others are grouped
+// by their larger endpoint l into units of edges of one l; a unit is worked on by a warp when l holds at
+// most kWarpUnitNodes entries, else by a thread block (those of the largest l's, above kBigUnitNodes
+// entries, first).
+constexpr int kBins = 4;
+constexpr int kBinSmall = 0, kBinWarp = 1, kBinBlock = 2, kBinBig = 3;
+constexpr int kClasses = 6;  // work-counter classes (bin_of_cnt)
+constexpr unsigned long long kSmallBatch = 1ull << 15;  // smaller batches: make_batch
+constexpr uint32_t kSmallBatchMax = 256u;
+constexpr uint32_t kWarpUnitItems = 32u;  // edges per warp unit: at most one per lane
+constexpr uint32_t kWarpUnitEntries = 8192u;
+constexpr uint32_t kUnitItems = 64u;      // ... and at most of a block unit
+constexpr uint32_t kWarpUnitNodes = 1024u;
+constexpr uint32_t kBigUnitNodes = 4096u;
+// Marks (StreamDev::mark): node ids are below kSmallEdge (n_nodes < 2^32 - 1)
+constexpr uint32_t kNoWork = 0xFFFFFFFFu, kSmallEdge = 0xFFFFFFFEu;
 
 // status bits (sticky)
 constexpr unsigned kStRange = 1u, kStCapacity = 2u, kStInternal = 4u, kStTimeout = 8u, kStDuplicate = 16u;
@@ -180,11 +192,12 @@ struct Ctrl {
     unsigned int pad;
     // work counters of k_intersect<true> (see rept_stats)
     unsigned long long small_entries, small_slots, probes, probe_slots, wedges, counted;
-    unsigned long long class_items[6], class_probes[6], class_cycles[6];
-    // per-batch work list of k_intersect: class c occupies items[bin_start[c] .. + bin_count[c])
-    unsigned long long bin_start[kBins];
-    unsigned long long bin_count[kBins];
-    unsigned long long bin_next[kBins];
+    unsigned long long class_items[kClasses], class_probes[kClasses], class_cycles[kClasses];
+    // per-batch work lists of the intersection
+    unsigned long long n_groups;           // larger endpoints of grouped edges (glist)
+    unsigned long long n_items;            // grouped edges with a place in order[]
+    unsigned long long bin_count[kBins];   // small chunks and units of each kind
+    unsigned long long bin_next[kBins];    // claimed so far
     unsigned long long n_pairs;  // entries of pair_list this batch
     unsigned long long n_big;   // nodes whose table (32..2048 slots) k_rehash_big moves, a warp each
     unsigned long long n_huge;  // nodes whose table (>= 4096 slots) k_rehash_huge moves, a block each
@@ -192,45 +205,60 @@ struct Ctrl {
     unsigned long long dbg[4];  // REPT_DEBUG_BOUNDS builds: first failed check {site, index, bound}, count
 };
 
-// What k_intersect needs about one arriving edge t = (s, l), s the endpoint with the smaller table:
-// both tables' offsets (in 4-slot units) and sizes, written by k_insert once the batch's tables are
-// final, then moved into sorted order by k_sort_scatter.
+// What the intersection needs about one arriving edge t = (s, l), s the endpoint with the smaller
+// table: both tables' offsets (in 4-slot units) and sizes, written by k_insert once the batch's tables
+// are final.  Record e belongs to the batch's edge e.
 struct __align__(16) WorkItem {
     uint32_t s, l, off_s, off_l;
     uint32_t t;      // stream index of the edge
     uint32_t lgs;    // log2 table sizes: smaller | larger << 8
     uint32_t cnt_s;  // entries of the smaller endpoint
-    uint32_t key;    // work class * kKeyBuckets + hash of l, or kNoKey
+    uint32_t cnt_l;  // entries of the larger endpoint
 };
+
+// Edges order[first .. first + count) of one larger endpoint.
+struct __align__(8) Unit {
+    uint32_t first, count;
+};
+
+// Scratch bytes per batch edge of the work lists beside the records: two unit lists, order, mark,
+// glist.
+constexpr unsigned long long kListBytes = 3ull * sizeof(uint32_t) + 2ull * sizeof(Unit);
 
 // Everything a kernel needs to know about one stream's state.
 struct StreamDev {
     uint32_t m, c, groups, n_nodes;
     uint64_t seed;
     FastMod fm;         // x mod m
-    uint32_t tile_max;  // edges whose smaller endpoint has more entries get a warp (4, 8, 16 or 32)
-    uint4* meta;  // per node {block offset in 4-slot units, entries, this batch's new entries, 0}
+    uint4* meta;  // per node {block offset in 4-slot units, entries, 0, grouped edges of this batch with this
+                  // larger endpoint, then their cursor into order[]}; the last is zero between batches
     uint32_t* cnt_add;  // [n_nodes] new entries per node as k_classify counts them (a compact array, so
-                        // that its atomics stay in L2); k_plan moves each touched node's count into its
-                        // record and clears it, so it is zero between batches
+                        // that its atomics stay in L2); k_plan takes each touched node's count and clears
+                        // it, so it is zero between batches
     uint2* pool;
     unsigned long long pool_quads;
     // How list entries carry their edge's colours (the intersection tests colours before it probes):
-    // kColNone: plain entries; kColInEntry: every list entry {w, t} of node x carries h_0(x, w) in
-    // the top 8 bits of its first word (w itself in the low kIdBits), for one hash group,
-    // 2 <= m <= 256 and n_nodes <= 2^kIdBits; kColWords: a parallel array of 32-bit words beside
-    // the list holds h_k(x, w) of every hash group k in bits [k * cbits, (k + 1) * cbits), for REPT
-    // with groups * cbits <= 32
+    // kColNone: not at all; kColInEntry: every list entry w of node x carries h_0(x, w) in its top 8
+    // bits (w itself in the low kIdBits), for one hash group, 2 <= m <= 256 and n_nodes <= 2^kIdBits;
+    // kColWords: a parallel array of 32-bit words beside the list holds h_0(x, w), for one hash group
+    // otherwise; kColMulti: several hash groups, a 32-bit word beside every stream index in tables and
+    // lists holds h_k(x, w) of every group k in bits [k * cbits, (k + 1) * cbits) or, when a group
+    // keeps colour 0 only (parallel MASCOT), one bit per group that is set if it keeps the edge
     uint32_t colours;
-    uint32_t cbits;  // kColWords: bits per group colour, ceil(log2 m)
+    uint32_t cbits;  // kColWords, kColMulti: bits per group colour
     uint32_t cmask;  // (1 << cbits) - 1
+    uint32_t ctop;   // kColMulti: the top bit of every group's colour (groups of this state only)
     unsigned long long* local;
     unsigned long long* proc;
     uint32_t* touched;
     uint32_t* grow_rel;
-    struct WorkItem* rec;   // [max_batch] work record of each edge (key kNoKey if it closes no wedge)
-    struct WorkItem* srec;  // [max_batch] the records of edges that can close wedges, sorted by key
-    uint32_t* hist;         // [kSortBuckets] counts, then cursors, of the counting sort by key
+    struct WorkItem* rec;   // [max_batch] work record of each edge that can close wedges
+    uint32_t* mark;         // [max_batch] per edge: its larger endpoint (grouped), kSmallEdge or kNoWork
+    uint32_t* order;        // [max_batch] grouped edges, those of one larger endpoint side by side
+    uint32_t* glist;        // [max_batch] larger endpoints with grouped edges
+    struct Unit* units;     // [2 * max_batch] first half: the largest l's block units from the front and
+                            // warp units from the back; second half: the other block units
+    unsigned long long unit_cap;  // max_batch
     uint32_t* big;      // [big_cap] touched-list indices of nodes with a large table to move: the
                         // k_rehash_big list from the front, the k_rehash_huge list from the back
     unsigned long long big_cap;
@@ -253,6 +281,14 @@ struct StreamDev {
     unsigned long long pair_cap;    // stream indices covered by the pair arrays
     unsigned long long* local_proc; // [c * n_nodes] tau_v^(i), processor-major (REPT_FLAG_LOCAL_PER_PROCESSOR)
 };
+
+// The work lists of n edges, one after the other from d.units on (kListBytes * n bytes).
+inline void set_list_pointers(StreamDev& d, unsigned long long n) {
+    d.unit_cap = n;
+    d.order = reinterpret_cast<uint32_t*>(d.units + 2 * n);
+    d.mark = d.order + n;
+    d.glist = d.mark + n;
+}
 
 // The block a batch kernel's body runs as: its index among the nbx blocks that share one stream's
 // work (blockIdx.x and gridDim.x for a launch per stream, or a virtual block of the persistent group
@@ -277,7 +313,19 @@ struct BatchDev {
     const uint32_t* dst;
     unsigned long long n;
     unsigned long long t0;  // stream index of src[0], dst[0]
+    uint32_t small_max;     // edges whose smaller endpoint has more entries are grouped
+    uint32_t chunk;         // edges of a small chunk
 };
+
+// A batch of a stream.  Grouping pays through the lists that share a filter; in a small batch few do, and
+// what counts is the chain of dependent steps, so nearly all edges stay small (`tile_max`: the handle's
+// bound for the others) and are dealt out in smaller chunks.
+inline BatchDev make_batch(const uint32_t* src, const uint32_t* dst, unsigned long long n, unsigned long long t0,
+                           uint32_t tile_max) {
+    const bool few = n < kSmallBatch;
+    return BatchDev{src, dst, n, t0, few ? kSmallBatchMax : tile_max,
+                    few ? std::max((uint32_t)(n >> 10), 4u) : 64u};
+}
 
 // Index checks of the REPT_DEBUG_BOUNDS build (a stand-in for a memory checker): a failed check
 // records {site, index, bound} once, counts, raises kStBounds, and the caller skips the access.
@@ -350,38 +398,25 @@ __device__ __forceinline__ bool kept_by_any(const StreamDev& d, uint32_t u, uint
     return false;
 }
 
-constexpr uint32_t kColNone = 0u, kColInEntry = 1u, kColWords = 2u;
+constexpr uint32_t kColNone = 0u, kColInEntry = 1u, kColWords = 2u, kColMulti = 3u;
 
 // The mask that takes a node id out of the first word of a list entry.
 __host__ __device__ __forceinline__ uint32_t id_mask(const StreamDev& d) {
     return d.colours == kColInEntry ? kIdMask : ~0u;
 }
-__host__ __device__ __forceinline__ bool has_words(const StreamDev& d) { return d.colours == kColWords; }
-// The stream's tables are interleaved (key_word) exactly when it stores colours.
-__host__ __device__ __forceinline__ bool tables_interleaved(const StreamDev& d) { return d.colours != kColNone; }
-
-// With one hash group, a wedge (s, w), (l, w) can count only for the processor of colour
-// js = h_0(s, w), and only if that processor exists and h_0(l, w) = js.  The intersection reads js from
-// s's list entry and asks this of the hash alone before it probes l's table for w, so all but about
-// 1/m of the probes are skipped.
-__device__ __forceinline__ bool wedge_may_count(const StreamDev& d, uint32_t l, uint32_t w, uint32_t js) {
-    // every step evaluated and combined with & (no early exit), so the lanes of a warp never part
-    // ways over it (measured 4 % faster than the short-circuit form).  With one hash group the
-    // processor of colour js is js itself: REPT keeps every colour below m (and js < m), parallel
-    // MASCOT's single sampler keeps colour 0 only (pbeg = 0, pcount = 1), so the shard's range test
-    // alone decides processor_of here.
-    const uint64_t lo = l < w ? l : w, hi = l < w ? w : l;
-    const uint64_t z = splitmix64(((lo << 32) | hi) ^ d.seed);
-    return (js - d.pbeg < d.pcount) & mod_equals_nobranch(z, js, d.fm);
+// Single-group streams with colours keep interleaved tables (key_word).
+__host__ __device__ __forceinline__ bool interleaved(uint32_t colours) {
+    return colours == kColInEntry || colours == kColWords;
 }
 
-// The scans' form of wedge_may_count: a superset test.  It never rejects an entry whose wedge can
-// count, and may pass a few whose wedge cannot; count_wedge decides every queued wedge exactly.
-// z mod m = js implies that m divides z - js, i.e. that r = rotr((z - js) q^-1, k) <= floor((2^64 - 1)
-// / m); only the high words are compared (a pass rate of about 1/m + 2^-32).  The range test of
-// wedge_may_count is left out: every entry of a list carries a kept colour (its edge is stored
-// because this state's processor of that colour keeps it), and z < js, which the exact test
-// excludes, has probability below 2^-56.
+// With one hash group, a wedge (s, w), (l, w) can count only if h_0(s, w) = h_0(l, w) = js for a kept
+// colour js.  js is stored with s's list entry; this asks the same of the hash of {l, w} alone, as a
+// superset test: it never rejects an entry whose wedge can count, and may pass a few whose wedge cannot;
+// count_wedge decides every queued wedge exactly.  z mod m = js implies that m divides z - js, i.e. that
+// r = rotr((z - js) q^-1, k) <= floor((2^64 - 1) / m); only the high words are compared (a pass rate of
+// about 1/m + 2^-32).  Every entry of a list carries a kept colour (its edge is stored because this
+// state's processor of that colour keeps it), and z < js, which the exact test excludes, has
+// probability below 2^-56.
 __device__ __forceinline__ bool colour_may_match(const StreamDev& d, uint32_t l, uint32_t w, uint32_t js) {
     const uint64_t lo = l < w ? l : w, hi = l < w ? w : l;
     const uint64_t z = splitmix64(((lo << 32) | hi) ^ d.seed);
@@ -390,38 +425,20 @@ __device__ __forceinline__ bool colour_may_match(const StreamDev& d, uint32_t l,
     return r_hi <= (uint32_t)(d.fm.lim >> 32);
 }
 
-// With several hash groups (kColWords), a wedge (s, w), (l, w) can count only for a group k whose
-// colour js_k = h_k(s, w) names a kept processor and equals h_k(l, w).  The word cw holds every js_k
-// (read from s's entry); the groups are tried in order and the first that agrees decides, so an
-// entry that counts for no processor costs one hash per group and no probe of l's table.
-__device__ __forceinline__ bool words_may_count(const StreamDev& d, uint32_t l, uint32_t w, uint32_t cw) {
-    const uint64_t lo = l < w ? l : w, hi = l < w ? w : l;
-    const uint64_t key = (lo << 32) | hi;
-    uint64_t sk = group_seed(d.seed, d.kbeg);
-    for (uint32_t k = d.kbeg; k < d.kend; ++k, sk += kGoldenGamma) {
-        const uint32_t js = (cw >> (k * d.cbits)) & d.cmask;
-        uint32_t i;
-        if (processor_of(d, k, js, i) && mod_equals_in_range(splitmix64(key ^ sk), js, d.fm)) return true;
-    }
-    return false;
-}
-
-// The scans' superset form of words_may_count (as colour_may_match is of wedge_may_count): every
-// group of this state is tested, each with the high words of its divisibility test, and the results
-// are combined with | (no early exit, so the lanes of a warp stay together).  Groups whose colour
-// js_k no processor keeps may pass too; count_wedge decides every queued wedge exactly.
-__device__ __forceinline__ bool words_may_match(const StreamDev& d, uint32_t l, uint32_t w, uint32_t cw) {
-    const uint64_t lo = l < w ? l : w, hi = l < w ? w : l;
-    const uint64_t key = (lo << 32) | hi;
-    const uint32_t lim_hi = (uint32_t)(d.fm.lim >> 32);
-    uint64_t sk = group_seed(d.seed, d.kbeg);
+// The colour word of edge {u, v} (kColWords, kColMulti) and, in `kept`, whether some processor keeps it.
+__device__ __forceinline__ uint32_t colour_word(const StreamDev& d, uint32_t u, uint32_t v, bool& kept) {
+    uint32_t cw = 0;
     bool any = false;
+    uint64_t sk = group_seed(d.seed, d.kbeg);
     for (uint32_t k = d.kbeg; k < d.kend; ++k, sk += kGoldenGamma) {
-        const uint32_t js = (cw >> (k * d.cbits)) & d.cmask;
-        const uint64_t y = (splitmix64(key ^ sk) - js) * d.fm.qinv;
-        any |= __funnelshift_r((uint32_t)(y >> 32), (uint32_t)y, d.fm.k) <= lim_hi;
+        uint32_t i;
+        const uint32_t j = colour_of(u, v, sk, d.fm);
+        const bool keeps = processor_of(d, k, j, i);
+        cw |= (d.keep == 1u ? (keeps ? 1u : 0u) : j) << (k * d.cbits);
+        any |= keeps;
     }
-    return any;
+    kept = any;
+    return cw;
 }
 
 // log2 of the table capacity for cnt entries: capacity = max(4, nextpow2(2*cnt)); 0 when empty.
@@ -436,22 +453,22 @@ __host__ __device__ __forceinline__ uint32_t table_lg(uint32_t cnt) {
     return lg < 2u ? 2u : lg;
 }
 
-// A node's block in the pool: its hash table (2^lg slots, probed by neighbour id) followed by its
-// entry list (list_slots(lg) slots, the same entries packed in insertion order, scanned when the
-// node is the smaller endpoint) and, with kColWords, the entries' colour words (one uint32 per list
-// slot, word_slots(lg) slots).  Every part is a multiple of 4 slots (32 bytes).
+// A node's block in the pool, 32-byte aligned, in 32-bit words: its hash table of 2^lg slots
+// (2 words a slot, 3 with kColMulti; key_word, eidx_word), then its list: list_slots(lg) entry words
+// (id and, with kColInEntry, colour) in insertion order, followed by their stream indices (kColNone) or
+// {stream index, colour word} pairs (kColMulti); single-group streams leave that part unused (a
+// candidate's age is looked up in the table) and, with kColWords, keep the colour words after it.
 __host__ __device__ __forceinline__ uint32_t list_slots(uint32_t lg) { return lg >= 3u ? (1u << (lg - 1u)) : 4u; }
 __host__ __device__ __forceinline__ uint32_t word_slots(uint32_t lg) { return lg >= 4u ? (1u << (lg - 2u)) : 4u; }
-__host__ __device__ __forceinline__ uint32_t block_quads(uint32_t lg, bool words) {
-    return ((1u << lg) + list_slots(lg) + (words ? word_slots(lg) : 0u)) >> 2;
+__host__ __device__ __forceinline__ uint32_t block_quads(uint32_t lg, uint32_t colours) {
+    const uint32_t slots = (1u << lg) + list_slots(lg);
+    if (colours == kColMulti) return (3u * slots + 7u) >> 3;
+    return (slots + (colours == kColWords ? word_slots(lg) : 0u)) >> 2;
 }
 
-// k_intersect work class of an edge whose smaller endpoint holds cnt entries: tiles of 4, 8, 16, 32
-// lanes (one entry per lane) up to tile_max entries, then a warp per edge for up to 256 entries and
-// for more.
-__host__ __device__ __forceinline__ int bin_of_cnt(uint32_t cnt, uint32_t tile_max) {
-    if (cnt > tile_max) return cnt <= 256u ? 4 : 5;
-    return cnt <= 4u ? 0 : cnt <= 8u ? 1 : cnt <= 16u ? 2 : 3;
+// Work-counter class of an edge whose smaller endpoint holds cnt entries (rept_stats.class_*).
+__host__ __device__ __forceinline__ int bin_of_cnt(uint32_t cnt) {
+    return cnt <= 4u ? 0 : cnt <= 8u ? 1 : cnt <= 16u ? 2 : cnt <= 32u ? 3 : cnt <= 256u ? 4 : 5;
 }
 
 // Home slot of neighbour w in a table of 2^lg slots: the first slot of a 4-slot (32-byte) bucket
@@ -461,19 +478,19 @@ __device__ __forceinline__ uint32_t home_slot(uint32_t w, uint32_t lg) {
 }
 
 // Word offsets, from the start of a table of 2^lg slots, of slot h's neighbour id and of its stream
-// index.  Interleaved (`inter`): bucket h / 4 occupies words 8 (h / 4) .. 8 (h / 4) + 7, ids first.
-// Split: ids in words 0 .. 2^lg - 1, indices in the next 2^lg words.  key_quad: the 16-byte quad that
-// holds the four ids of the bucket that starts at slot h (h a multiple of 4).
-__host__ __device__ __forceinline__ uint32_t key_word(uint32_t h, bool inter) {
-    return inter ? (((h >> 2) << 3) | (h & 3u)) : h;
+// index.  Interleaved tables: bucket h / 4 occupies words 8 (h / 4) .. 8 (h / 4) + 7, ids first.
+// Others: ids in words 0 .. 2^lg - 1, then the stream indices (with kColMulti, each followed by its
+// colour word).  key_quad: the 16-byte quad that holds the four ids of the bucket that starts at slot h
+// (h a multiple of 4).
+__host__ __device__ __forceinline__ uint32_t key_word(uint32_t h, uint32_t colours) {
+    return interleaved(colours) ? (((h >> 2) << 3) | (h & 3u)) : h;
 }
-__host__ __device__ __forceinline__ uint32_t eidx_word(uint32_t h, uint32_t lg, bool inter) {
-    return inter ? key_word(h, true) + 4u : (1u << lg) + h;
+__host__ __device__ __forceinline__ uint32_t eidx_word(uint32_t h, uint32_t lg, uint32_t colours) {
+    return interleaved(colours) ? key_word(h, colours) + 4u
+                                : (1u << lg) + (colours == kColMulti ? 2u * h : h);
 }
-__host__ __device__ __forceinline__ uint32_t key_quad(uint32_t h, bool inter) { return inter ? h >> 1 : h >> 2; }
-
-__device__ __forceinline__ unsigned long long pack_slot(uint32_t nbr, uint32_t eidx) {
-    return ((unsigned long long)eidx << 32) | nbr;
+__host__ __device__ __forceinline__ uint32_t key_quad(uint32_t h, uint32_t colours) {
+    return interleaved(colours) ? h >> 1 : h >> 2;
 }
 
 // Warp-aggregated atomicAdd: every active lane of the full warp calls it with its own
@@ -491,6 +508,47 @@ __device__ __forceinline__ unsigned long long warp_reserve(unsigned long long* c
     if (lane == 31 && total) base = atomicAdd(ctr, total);
     base = __shfl_sync(0xFFFFFFFFu, base, 31);
     return base + incl - inc;
+}
+
+// The same for lanes that each take one place or none.
+__device__ __forceinline__ unsigned long long warp_reserve_one(unsigned long long* ctr, bool take) {
+    const unsigned lane = threadIdx.x & 31u, mask = __ballot_sync(0xFFFFFFFFu, take);
+    unsigned long long base = 0;
+    if (lane == 0 && mask) base = atomicAdd(ctr, (unsigned long long)__popc(mask));
+    return __shfl_sync(0xFFFFFFFFu, base, 0) + __popc(mask & ((1u << lane) - 1u));
+}
+
+// The same for a thread block (at most 32 warps; every thread calls it): one atomic per block.  The
+// atomics of a grid on one counter follow each other about 1.3 ns apart, so a warp's each for 2^20
+// edges takes 40 us.  `part`: shared memory of the caller, two of them used in turn need no barrier
+// between calls.
+struct BlockReserve {
+    uint32_t warp[32];
+    unsigned long long base;
+};
+__device__ __forceinline__ unsigned long long block_reserve(BlockReserve& part, unsigned long long* ctr, uint32_t inc) {
+    const unsigned lane = threadIdx.x & 31u, wid = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    uint32_t incl = inc;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= (unsigned)o) incl += y;
+    }
+    if (lane == 31) part.warp[wid] = incl;
+    __syncthreads();
+    if (wid == 0) {
+        const uint32_t w = lane < warps ? part.warp[lane] : 0u;
+        uint32_t wi = w;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, wi, o);
+            if (lane >= (unsigned)o) wi += y;
+        }
+        part.warp[lane] = wi - w;
+        if (lane == 31) part.base = wi ? atomicAdd(ctr, (unsigned long long)wi) : 0ull;
+    }
+    __syncthreads();
+    return part.base + part.warp[wid] + incl - inc;
 }
 
 }  // namespace rept

@@ -7,15 +7,15 @@
 //   k_commit    move re-allocated tables (rehash), publish the new counts
 //   k_insert    insert each kept edge (nbr, stream index) into both
 //               endpoints' tables                              (Alg. 1 E^(i) <- E^(i) + {(u,v)})
-//   k_sort_scan, k_sort_scatter
-//               order the edges that can close wedges into work classes by
-//               their smaller endpoint's entry count, grouped by the larger
-//               endpoint
-//   k_intersect for every edge t = (u, v): walk the smaller endpoint's list,
-//               look up the larger endpoint's table (for streams that store
-//               colours, only for entries whose colours may agree), and count
-//               the wedges whose two edges both arrived before t and carry
-//               the same kept colour; tally tau^(i), tau_u, tau_v, tau_w
+//   k_units, k_order
+//               group the edges that can close wedges by their larger endpoint
+//               (those with a short smaller list stay as they are)
+//   k_intersect for every edge t = (s, l), s the endpoint with fewer entries:
+//               scan s's list, let through the entries that a filter of l's list
+//               holds (short lists: whose colours may agree), look those up in
+//               l's table, and count the wedges whose two edges both arrived
+//               before t and carry the same kept colour; tally tau^(i), tau_u,
+//               tau_v, tau_w
 //                                                               (Alg. 1 UpdateTriangleCNT)
 // Counting after inserting is exact because every entry carries its stream
 // index and k_intersect only accepts entries with index < t: the state seen by
@@ -30,34 +30,56 @@ namespace rept {
 // Internal linkage: every translation unit of the library that launches these kernels gets its own copy.
 namespace {
 
-// A node's table of 2^lg slots at pool slot `base` holds 2^lg neighbour ids (keys; probed a 4-key,
-// 16-byte bucket at a time) and their stream indices, interleaved per bucket or split (key_word,
-// eidx_word; `inter`).  Insert (nbr, eidx): claim a key slot with a 32-bit CAS, then store the index
-// (in the same sector when interleaved).
+__device__ __forceinline__ uint32_t* block_at(uint2* pool, unsigned long long off_quads) {
+    return reinterpret_cast<uint32_t*>(pool) + 8ull * off_quads;
+}
+__device__ __forceinline__ const uint32_t* block_at(const uint2* pool, unsigned long long off_quads) {
+    return reinterpret_cast<const uint32_t*>(pool) + 8ull * off_quads;
+}
+// Word offset of the list inside a block with a table of 2^lg slots, of the stream indices or pairs
+// beside it (kColNone, kColMulti), and of its colour words (kColWords).
+__device__ __forceinline__ uint32_t list_at(uint32_t lg, uint32_t colours) {
+    return (colours == kColMulti ? 3u : 2u) << lg;
+}
+__device__ __forceinline__ uint32_t aux_at(uint32_t lg, uint32_t colours) { return list_at(lg, colours) + list_slots(lg); }
+__device__ __forceinline__ uint32_t cw_at(uint32_t lg) { return 2u * ((1u << lg) + list_slots(lg)); }
+
+// A node's table of 2^lg slots at `table` holds 2^lg neighbour ids (keys; probed a 4-key, 16-byte
+// bucket at a time) and, per id, its stream index (and colour word), laid out as key_word and eidx_word
+// say.  Insert (nbr, eidx, cw): claim a key slot with a 32-bit CAS, then store the rest.
 // Returns false only if the table has no empty slot left (impossible while cnt <= capacity / 2).
 // Lookups read whole 4-key buckets, so where a key sits inside its bucket does not matter: an insert
 // tries the slots of a bucket starting from one chosen by other bits of the key, so that keys sharing
 // a home bucket seldom contend for the same slot, and moves to the next bucket only when all four are
 // taken.
-// The slot of its home bucket that an insert of nbr tries first.
-__device__ __forceinline__ uint32_t first_slot(uint32_t nbr, uint32_t lg) {
-    return home_slot(nbr, lg) + ((nbr * 0x85EBCA6Bu) >> 30);
+// The slot of its home bucket, whose ids are q, that an insert of nbr tries first: an empty one if there
+// is one.
+__device__ __forceinline__ uint32_t empty_slot(const uint4& q, uint32_t nbr) {
+    const uint32_t start = (nbr * 0x85EBCA6Bu) >> 30;
+    const uint32_t empty = (q.x == kEmptyId ? 1u : 0u) | (q.y == kEmptyId ? 2u : 0u) | (q.z == kEmptyId ? 4u : 0u) |
+                           (q.w == kEmptyId ? 8u : 0u);
+    const uint32_t from = (empty | (empty << 4)) >> start;  // bit i: slot start + i
+    return empty ? (start + (uint32_t)__ffs((int)from) - 1u) & 3u : start;
 }
 
-// `tried_first`: the caller's CAS on first_slot(nbr, lg) failed already.
-__device__ __forceinline__ bool table_insert(uint2* pool, unsigned long long base, uint32_t lg, uint32_t nbr,
-                                             uint32_t eidx, bool inter, bool tried_first = false) {
-    uint32_t* keys = reinterpret_cast<uint32_t*>(pool + base);
+__device__ __forceinline__ void table_store(uint32_t* table, uint32_t lg, uint32_t h, uint32_t eidx, uint32_t cw,
+                                            uint32_t colours) {
+    uint32_t* at = table + eidx_word(h, lg, colours);
+    if (colours == kColMulti) *reinterpret_cast<uint2*>(at) = make_uint2(eidx, cw);
+    else *at = eidx;
+}
+
+__device__ __forceinline__ bool table_insert(uint32_t* table, uint32_t lg, uint32_t nbr, uint32_t eidx, uint32_t cw,
+                                             uint32_t colours) {
     const uint32_t mask = (1u << lg) - 1u;
     const uint32_t start = (nbr * 0x85EBCA6Bu) >> 30;
     uint32_t b = home_slot(nbr, lg);
     for (uint32_t probe = 0; probe <= mask; probe += 4u) {
 #pragma unroll
         for (uint32_t i = 0; i < 4u; ++i) {
-            if (tried_first && probe == 0u && i == 0u) continue;
             const uint32_t h = b + ((start + i) & 3u);
-            if (atomicCAS(keys + key_word(h, inter), kEmptyId, nbr) == kEmptyId) {
-                keys[eidx_word(h, lg, inter)] = eidx;
+            if (atomicCAS(table + key_word(h, colours), kEmptyId, nbr) == kEmptyId) {
+                table_store(table, lg, h, eidx, cw, colours);
                 return true;
             }
         }
@@ -66,18 +88,29 @@ __device__ __forceinline__ bool table_insert(uint2* pool, unsigned long long bas
     return false;
 }
 
+// Scratch that lives in another step's memory: per edge, its places among the batch's new entries of its
+// two endpoints (k_classify to k_insert, where the units go later); per touched node, the batch's new
+// entries (k_plan to k_commit, where the work records go later).
+__device__ __forceinline__ uint2* edge_ranks(const StreamDev& d) { return reinterpret_cast<uint2*>(d.units); }
+__device__ __forceinline__ uint32_t* touched_adds(const StreamDev& d) { return reinterpret_cast<uint32_t*>(d.rec); }
+
 __device__ __forceinline__ void k_classify_body(const StreamDev& d, const BatchDev& b, const Grid g) {
-    // the previous batch's work list is consumed: clear the counting-sort histogram
-    for (uint32_t i = g.bx * blockDim.x + threadIdx.x; i < kSortBuckets; i += g.nbx * blockDim.x)
-        d.hist[i] = 0u;
-    if (g.bx == 0 && threadIdx.x < kBins) d.ctrl->bin_next[threadIdx.x] = 0ull;
-    if (g.bx == 0 && threadIdx.x == 0) d.ctrl->n_pairs = 0ull;
+    // the previous batch's work lists are consumed
+    if (g.bx == 0 && threadIdx.x < kBins) {
+        d.ctrl->bin_next[threadIdx.x] = 0ull;
+        d.ctrl->bin_count[threadIdx.x] = threadIdx.x == kBinSmall ? (b.n + b.chunk - 1u) / b.chunk : 0ull;
+    }
+    if (g.bx == 0 && threadIdx.x == 0) {
+        d.ctrl->n_pairs = 0ull;
+        d.ctrl->n_groups = 0ull;
+        d.ctrl->n_items = 0ull;
+    }
     if (d.ctrl->status) return;
-    const unsigned lane = threadIdx.x & 31u;
+    __shared__ BlockReserve part[2];
+    uint32_t turn = 0;
     const unsigned long long stride = (unsigned long long)g.nbx * blockDim.x;
-    for (unsigned long long base = (unsigned long long)g.bx * blockDim.x + threadIdx.x - lane; base < b.n;
-         base += stride) {
-        const unsigned long long e = base + lane;
+    for (unsigned long long base = (unsigned long long)g.bx * blockDim.x; base < b.n; base += stride) {
+        const unsigned long long e = base + threadIdx.x;
         const bool valid = e < b.n;
         uint32_t u = 0, v = 0;
         if (valid) { u = b.src[e]; v = b.dst[e]; }
@@ -85,165 +118,133 @@ __device__ __forceinline__ void k_classify_body(const StreamDev& d, const BatchD
         if (valid && !in_range) atomicOr(&d.ctrl->status, kStRange);
         const bool kept = valid && in_range && u != v && kept_by_any(d, u, v);
         bool first_u = false, first_v = false;
-        if (kept) {
-            first_u = atomicAdd(&d.cnt_add[u], 1u) == 0u;
-            first_v = atomicAdd(&d.cnt_add[v], 1u) == 0u;
+        if (kept) {  // the edge's places among the batch's new entries of u and v, for k_insert
+            const uint32_t ru = atomicAdd(&d.cnt_add[u], 1u), rv = atomicAdd(&d.cnt_add[v], 1u);
+            first_u = ru == 0u;
+            first_v = rv == 0u;
+            edge_ranks(d)[e] = make_uint2(ru, rv);
         }
-        unsigned long long o = warp_reserve(&d.ctrl->n_touched, (unsigned)first_u + (unsigned)first_v);
+        unsigned long long o = block_reserve(part[turn], &d.ctrl->n_touched, (first_u ? 1u : 0u) + (first_v ? 1u : 0u));
         if (first_u) d.touched[o++] = u;
         if (first_v) d.touched[o] = v;
+        turn ^= 1u;
     }
 }
 
 __device__ __forceinline__ void k_plan_body(const StreamDev& d, const Grid g) {
     if (d.ctrl->status) return;
-    const unsigned lane = threadIdx.x & 31u;
+    __shared__ BlockReserve part[2];
+    uint32_t turn = 0;
     const unsigned long long n_t = d.ctrl->n_touched;
     const unsigned long long stride = (unsigned long long)g.nbx * blockDim.x;
-    for (unsigned long long base = (unsigned long long)g.bx * blockDim.x + threadIdx.x - lane; base < n_t;
-         base += stride) {
-        const unsigned long long i = base + lane;
+    for (unsigned long long base = (unsigned long long)g.bx * blockDim.x; base < n_t; base += stride) {
+        const unsigned long long i = base + threadIdx.x;
         const bool valid = i < n_t;
-        unsigned long long need = 0;
+        uint32_t need = 0;
         if (valid) {
             const uint32_t x = d.touched[i];
             const uint32_t cnt = d.meta[x].y, add = d.cnt_add[x];
-            d.cnt_add[x] = 0u;     // zero again for the next batch
-            d.meta[x].z = add;     // the count travels with the node's record from here on
+            d.cnt_add[x] = 0u;  // zero again for the next batch
+            touched_adds(d)[i] = add;
             const uint32_t lg_old = table_lg(cnt), lg_new = table_lg(cnt + add);
-            if (lg_new != lg_old) need = block_quads(lg_new, has_words(d));
+            if (lg_new != lg_old) need = block_quads(lg_new, d.colours);
         }
-        const unsigned long long rel = warp_reserve(&d.ctrl->need_quads, need);
+        const unsigned long long rel = block_reserve(part[turn], &d.ctrl->need_quads, need);
         if (valid) d.grow_rel[i] = need ? (uint32_t)rel : kNoGrow;
+        turn ^= 1u;
     }
 }
 
-// REPT_DEBUG_BOUNDS: the block of 2^lg table slots and its list at `off_quads` lies inside the pool.
+// REPT_DEBUG_BOUNDS: the block with a table of 2^lg slots at `off_quads` lies inside the pool.
 __device__ __forceinline__ bool block_fits(const StreamDev& d, unsigned site, unsigned long long off_quads,
                                           uint32_t lg) {
-    return REPT_CHECK(d.ctrl, site, 4ull * (off_quads + block_quads(lg, has_words(d))) - 1ull, 4ull * d.pool_quads);
+    return REPT_CHECK(d.ctrl, site, off_quads + block_quads(lg, d.colours) - 1ull, d.pool_quads);
 }
 
-// The colour words (kColWords) of the list of a block at `off_quads` with a table of 2^lg slots.
-__device__ __forceinline__ uint32_t* list_words(uint2* pool, unsigned long long off_quads, uint32_t lg) {
-    return reinterpret_cast<uint32_t*>(pool + 4ull * off_quads + (1ull << lg) + list_slots(lg));
+// Copy n entries' words from one 16-byte aligned array to another (whole quads: the arrays' capacities
+// are multiples of four words), lanes `rank` of `width`.
+__device__ __forceinline__ void copy_words(uint32_t* to, const uint32_t* from, uint32_t n, uint32_t rank, uint32_t width) {
+    for (uint32_t q = rank; q < (n + 3u) / 4u; q += width)
+        reinterpret_cast<uint4*>(to)[q] = reinterpret_cast<const uint4*>(from)[q];
 }
 
-// Move node x's entries (list of cnt_old entries at old_off) into its new block at new_off: copy the
-// list (and, with `words`, the colour words) and insert each entry's id (`mask` takes it out of the
-// entry) into the new table.  Lanes `rank` of `width` share the work.
-__device__ __forceinline__ bool move_block(uint2* pool, uint32_t mask, bool words, bool inter, uint32_t old_off,
-                                           uint32_t cnt_old, unsigned long long new_off, uint32_t lg_new, uint32_t rank,
-                                           uint32_t width) {
-    const uint32_t lg_old = table_lg(cnt_old);
-    const unsigned long long old_at = 4ull * old_off + (1ull << lg_old);
-    const unsigned long long new_at = 4ull * new_off + (1ull << lg_new);
-    const uint2* old_list = pool + old_at;
-    uint2* new_list = pool + new_at;
-    bool ok = true;
-    for (uint32_t j = rank; j < cnt_old; j += width) {
-        const uint2 e = old_list[j];
-        new_list[j] = e;
-        if (words) list_words(pool, new_off, lg_new)[j] = list_words(pool, old_off, lg_old)[j];
-        ok &= table_insert(pool, 4ull * new_off, lg_new, e.x & mask, e.y, inter);
+// Copy the list of cnt_old entries from the block at `from` (table of 2^lg_old slots) to the new one.
+__device__ __forceinline__ void move_list(uint32_t* to, const uint32_t* from, uint32_t cnt_old, uint32_t lg_old,
+                                          uint32_t lg_new, uint32_t colours, uint32_t rank, uint32_t width) {
+    copy_words(to + list_at(lg_new, colours), from + list_at(lg_old, colours), cnt_old, rank, width);
+    if (colours == kColWords) copy_words(to + cw_at(lg_new), from + cw_at(lg_old), cnt_old, rank, width);
+    if (colours == kColNone || colours == kColMulti)
+        copy_words(to + aux_at(lg_new, colours), from + aux_at(lg_old, colours),
+                   colours == kColMulti ? 2u * cnt_old : cnt_old, rank, width);
+}
+
+// Call put(id, eidx, j) for every entry of the block at `from`: from its table (interleaved tables, whose
+// lists hold no stream indices; j unused) or from its list, whose entry j it is.
+template <class Put>
+__device__ __forceinline__ void each_entry(const uint32_t* from, uint32_t cnt, uint32_t lg, uint32_t colours, uint32_t rank,
+                                           uint32_t width, Put&& put) {
+    if (interleaved(colours)) {
+        if (cnt == 0u) return;
+        const uint4* quads = reinterpret_cast<const uint4*>(from);
+        for (uint32_t b = rank; b < (1u << lg) / 4u; b += width) {
+            const uint4 id = quads[2u * b], t = quads[2u * b + 1u];
+            if (id.x != kEmptyId) put(id.x, t.x, 0u);
+            if (id.y != kEmptyId) put(id.y, t.y, 0u);
+            if (id.z != kEmptyId) put(id.z, t.z, 0u);
+            if (id.w != kEmptyId) put(id.w, t.w, 0u);
+        }
+    } else {
+        const uint32_t *ids = from + list_at(lg, colours), *aux = from + aux_at(lg, colours);
+        const uint32_t step = colours == kColMulti ? 2u : 1u;
+        for (uint32_t j = rank; j < cnt; j += width) put(ids[j], aux[j * step], j);
     }
+}
+
+// Move a node's block of cnt_old entries at `from` into its new block at `to`, whose table keys are
+// empty: copy the list and insert each entry into the new table.  Lanes `rank` of `width` share the work.
+__device__ __forceinline__ bool move_block(uint32_t* to, const uint32_t* from, uint32_t cnt_old, uint32_t lg_new,
+                                           uint32_t colours, uint32_t rank, uint32_t width) {
+    const uint32_t lg_old = table_lg(cnt_old);
+    move_list(to, from, cnt_old, lg_old, lg_new, colours, rank, width);
+    bool ok = true;
+    const uint32_t* aux = from + aux_at(lg_old, colours);
+    each_entry(from, cnt_old, lg_old, colours, rank, width, [&](uint32_t id, uint32_t eidx, uint32_t j) {
+        ok &= table_insert(to, lg_new, id, eidx, colours == kColMulti ? aux[2u * j + 1u] : 0u, colours);
+    });
     return ok;
 }
 
-// Set every key of the new table of 2^lg slots at `off_quads` to empty (lanes `rank` of `width`).  The
+// Set every key of the new table of 2^lg slots at `table` to empty (lanes `rank` of `width`).  The
 // pool is not cleared between streams: a block's table gets its empty keys when the block is handed
 // out, from here or from the shared-memory builds, which write the whole table.  (Stream indices are
 // read only beside a matching key, so they need no initial value.)
-__device__ __forceinline__ void init_table_keys(uint2* pool, unsigned long long off_quads, uint32_t lg, bool inter,
-                                                uint32_t rank, uint32_t width) {
-    uint4* quads = reinterpret_cast<uint4*>(pool + 4ull * off_quads);
+__device__ __forceinline__ void init_table_keys(uint32_t* table, uint32_t lg, uint32_t colours, uint32_t rank,
+                                                uint32_t width) {
+    uint4* quads = reinterpret_cast<uint4*>(table);
     const uint4 empty = make_uint4(kEmptyId, kEmptyId, kEmptyId, kEmptyId);
-    for (uint32_t b = rank; b < (1u << lg) / 4u; b += width) quads[inter ? 2u * b : b] = empty;
+    for (uint32_t b = rank; b < (1u << lg) / 4u; b += width) quads[interleaved(colours) ? 2u * b : b] = empty;
 }
 
 // New tables of at most kMoveSlots slots are rebuilt in shared memory by a warp (k_rehash_big), those
 // of at most kBlockMoveSlots by a thread block (k_rehash_huge); larger ones are built in place.
-constexpr uint32_t kInlineSlots = 32;  // k_commit's own moves (one thread each)
 constexpr uint32_t kMoveSlots = 512;
-constexpr uint32_t kBlockMoveSlots = 4096;
+constexpr uint32_t kBlockMoveSlots = 32768;
+constexpr uint32_t kHugeSmemWords = kBlockMoveSlots / 2u;  // a 16-bit word per slot
 
-// Publish the new entry counts of the touched nodes and move the blocks that were re-allocated.
-// One thread per touched node moves a block of at most 8 entries into a new table of at most
-// kInlineSlots slots; other blocks are left to k_rehash_big (a warp each, new tables of at most
-// kMoveSlots slots) or k_rehash_huge (a thread block each).  meta[x].z
-// keeps the batch's new-entry count for k_insert, which counts it back down to zero; a batch that is not
-// applied clears it here.
-__device__ __forceinline__ void k_commit_body(const StreamDev& d, const Grid g) {
-    const unsigned status = d.ctrl->status;
-    const unsigned long long n_t = d.ctrl->n_touched;
-    const unsigned long long need = d.ctrl->need_quads, top = d.ctrl->pool_top;
-    const bool bad = status != 0u || top + need > d.pool_quads;
-    if (status == 0u && bad && g.bx == 0 && threadIdx.x == 0) atomicOr(&d.ctrl->status, kStCapacity);
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned long long stride = (unsigned long long)g.nbx * blockDim.x;
-    for (unsigned long long base = (unsigned long long)g.bx * blockDim.x + threadIdx.x - lane; base < n_t;
-         base += stride) {
-        const unsigned long long i = base + lane;
-        bool defer = false, huge = false;
-        if (i < n_t) {
-            const uint32_t x = d.touched[i];
-            if (bad) {
-                d.meta[x].z = 0u;
-            } else {
-                const uint4 m = d.meta[x];
-                const uint32_t cnt_new = m.y + m.z;
-                const uint32_t rel = d.grow_rel[i];
-                if (rel == kNoGrow) {
-                    d.meta[x].y = cnt_new;
-                } else if (m.y > 8u || (1u << table_lg(cnt_new)) > kInlineSlots) {
-                    defer = (1u << table_lg(cnt_new)) <= kMoveSlots;
-                    huge = !defer;
-                } else {
-                    const unsigned long long new_off = top + rel;
-                    const bool fits = block_fits(d, 10, m.x, table_lg(m.y)) &&
-                                      block_fits(d, 11, new_off, table_lg(cnt_new));
-                    if (fits) init_table_keys(d.pool, new_off, table_lg(cnt_new), tables_interleaved(d), 0u, 1u);
-                    if (fits && !move_block(d.pool, id_mask(d), has_words(d), tables_interleaved(d), m.x, m.y, new_off,
-                                            table_lg(cnt_new), 0u, 1u))
-                        atomicOr(&d.ctrl->status, kStInternal);
-                    d.meta[x] = make_uint4((uint32_t)new_off, cnt_new, m.z, 0u);
-                }
-            }
-        }
-        const unsigned long long o = warp_reserve(&d.ctrl->n_big, defer ? 1ull : 0ull);
-        if (defer) d.big[o] = (uint32_t)i;
-        const unsigned long long h = warp_reserve(&d.ctrl->n_huge, huge ? 1ull : 0ull);
-        if (huge) d.big[d.big_cap - 1 - h] = (uint32_t)i;
-    }
-}
-
-// move_block with the new table built in shared memory (keys and stream indices of 2^lg_new slots,
-// the same placement rule as table_insert) and then written out with coalesced stores, by the lanes
-// `rank` of `width` of one warp (BLOCK = false) or of one thread block (BLOCK = true).  The new block
-// is the caller's alone until the batch's inserts run.
-template <bool BLOCK, bool INTER>
-__device__ __forceinline__ bool move_block_smem(uint2* pool, uint32_t id_bits, bool words, uint32_t old_off,
-                                                uint32_t cnt_old, unsigned long long new_off, uint32_t lg_new,
-                                                uint32_t* s_keys, uint32_t* s_eidx, uint32_t rank, uint32_t width) {
-    auto sync = [] {
-        if (BLOCK) __syncthreads();
-        else __syncwarp();
-    };
-    const uint32_t cap = 1u << lg_new, mask = cap - 1u;
-    for (uint32_t q = rank; q < cap; q += width) {
-        s_keys[q] = kEmptyId;
-        s_eidx[q] = kEmptyId;
-    }
-    sync();
+// move_block with the new table built in shared memory (keys and, per key, its stream index or with
+// kColMulti its list position; 2^lg_new slots, the same placement rule as table_insert) and then written
+// out with coalesced stores, by the lanes `rank` of `width` of one warp.  The new block is the caller's alone until the batch's inserts run.  Parts of a
+// warp may each move a node at the same time; an inactive part takes part in the barriers only.
+__device__ __forceinline__ bool move_block_smem(uint32_t* to, const uint32_t* from, uint32_t cnt_old, uint32_t lg_new,
+                                                uint32_t colours, uint32_t* s_keys, uint32_t* s_aux, uint32_t rank,
+                                                uint32_t width, bool active = true) {
+    const uint32_t cap = active ? 1u << lg_new : 0u, mask = cap - 1u;
+    for (uint32_t q = rank; q < cap; q += width) s_keys[q] = kEmptyId;
+    __syncwarp();
     const uint32_t lg_old = table_lg(cnt_old);
-    const unsigned long long old_at = 4ull * old_off + (1ull << lg_old);
-    const unsigned long long new_at = 4ull * new_off + cap;
+    move_list(to, from, cnt_old, lg_old, lg_new, colours, rank, width);
     bool ok = true;
-    for (uint32_t j = rank; j < cnt_old; j += width) {
-        const uint2 e = pool[old_at + j];
-        pool[new_at + j] = e;
-        if (words) list_words(pool, new_off, lg_new)[j] = list_words(pool, old_off, lg_old)[j];
-        const uint32_t key = e.x & id_bits;
+    each_entry(from, cnt_old, lg_old, colours, rank, width, [&](uint32_t key, uint32_t eidx, uint32_t j) {
         const uint32_t start = (key * 0x85EBCA6Bu) >> 30;
         uint32_t b = home_slot(key, lg_new);
         bool placed = false;
@@ -251,35 +252,104 @@ __device__ __forceinline__ bool move_block_smem(uint2* pool, uint32_t id_bits, b
             for (uint32_t i = 0; i < 4u && !placed; ++i) {
                 const uint32_t h = b + ((start + i) & 3u);
                 if (atomicCAS(&s_keys[h], kEmptyId, key) == kEmptyId) {
-                    s_eidx[h] = e.y;
+                    s_aux[h] = colours == kColMulti ? j : eidx;
                     placed = true;
                 }
             }
             b = (b + 4u) & mask;
         }
         ok &= placed;
+    });
+    __syncwarp();
+    uint4* quads = reinterpret_cast<uint4*>(to);
+    for (uint32_t b = rank; b < cap / 4u; b += width) {
+        const uint4 id = reinterpret_cast<const uint4*>(s_keys)[b], t = reinterpret_cast<const uint4*>(s_aux)[b];
+        if (interleaved(colours)) {
+            quads[2u * b] = id;
+            quads[2u * b + 1u] = t;
+        } else {
+            quads[b] = id;
+            if (colours == kColNone) quads[cap / 4u + b] = t;
+        }
     }
-    sync();
-    uint32_t* words_out = reinterpret_cast<uint32_t*>(pool + 4ull * new_off);
-    if (INTER) {  // word q of the table: bucket q / 8, an id (q % 8 < 4) or a stream index
-        for (uint32_t q = rank; q < 2u * cap; q += width) {
-            const uint32_t h = ((q >> 3) << 2) | (q & 3u);
-            words_out[q] = (q & 4u) ? s_eidx[h] : s_keys[h];
-        }
-    } else {
-        for (uint32_t q = rank; q < cap; q += width) {
-            words_out[q] = s_keys[q];
-            words_out[cap + q] = s_eidx[q];
-        }
+    if (colours == kColMulti) {  // the pairs of the keys' entries, from the old list
+        const uint2* pairs = reinterpret_cast<const uint2*>(from + aux_at(lg_old, colours));
+        uint2* out = reinterpret_cast<uint2*>(to + cap);
+        for (uint32_t q = rank; q < cap; q += width)
+            if (s_keys[q] != kEmptyId) out[q] = pairs[s_aux[q]];
     }
     return ok;
+}
+
+// Publish the new entry counts of the touched nodes and move the blocks that were re-allocated: those
+// with new tables of at most kPartSlots slots here, four at a time by eight lanes each (a thread per node
+// with global compare-and-swaps paid their latency once per entry); the others are left to k_rehash_big
+// (a warp each, new tables of at most kMoveSlots slots) or k_rehash_huge (a thread block each).  49 batches
+// of 4,096 edges: the three kernels took 2.1 ms with a thread per node, 1.8 ms so.
+// `smem`: kCommitSmemWords words.
+constexpr uint32_t kPartSlots = 64u, kPartLanes = 8u;
+constexpr uint32_t kCommitSmemWords = 2u * (256u / kPartLanes) * kPartSlots;
+__device__ __forceinline__ void k_commit_body(const StreamDev& d, const Grid g, uint32_t* smem) {
+    const unsigned status = d.ctrl->status;
+    const unsigned long long n_t = d.ctrl->n_touched;
+    const unsigned long long need = d.ctrl->need_quads, top = d.ctrl->pool_top;
+    const bool bad = status != 0u || top + need > d.pool_quads;
+    if (status == 0u && bad && g.bx == 0 && threadIdx.x == 0) atomicOr(&d.ctrl->status, kStCapacity);
+    if (bad) return;
+    const unsigned lane = threadIdx.x & 31u, part = lane / kPartLanes, rank = lane % kPartLanes;
+    uint32_t* s_keys = smem + (threadIdx.x / kPartLanes) * 2u * kPartSlots;
+    uint32_t* s_aux = s_keys + kPartSlots;
+    const unsigned long long stride = (unsigned long long)g.nbx * blockDim.x;
+    for (unsigned long long base = (unsigned long long)g.bx * blockDim.x + threadIdx.x - lane; base < n_t;
+         base += stride) {
+        const unsigned long long i = base + lane;
+        bool move = false, defer = false, huge = false;
+        uint32_t off_old = 0, cnt_old = 0, off_new = 0, lg_new = 0;
+        if (i < n_t) {
+            const uint32_t x = d.touched[i];
+            const uint4 m = d.meta[x];
+            const uint32_t cnt_new = m.y + touched_adds(d)[i];
+            const uint32_t rel = d.grow_rel[i];
+            if (rel == kNoGrow) {
+                d.meta[x].y = cnt_new;
+            } else {
+                lg_new = table_lg(cnt_new);
+                off_old = m.x;
+                cnt_old = m.y;
+                off_new = (uint32_t)(top + rel);
+                move = (1u << lg_new) <= kPartSlots;
+                defer = !move && (1u << lg_new) <= kMoveSlots;
+                huge = !move && !defer;
+                if (move) d.meta[x] = make_uint4(off_new, cnt_new, 0u, 0u);
+                if (!(block_fits(d, 10, off_old, table_lg(cnt_old)) && block_fits(d, 11, off_new, lg_new))) move = false;
+            }
+        }
+        const unsigned movers = __ballot_sync(0xFFFFFFFFu, move);
+        const uint32_t n_move = __popc(movers);
+        for (uint32_t r = 0; r < n_move; r += 32u / kPartLanes) {
+            const bool active = r + part < n_move;
+            uint32_t from = 0;  // the lane of the part's node: the (r + part)-th mover
+#pragma unroll
+            for (uint32_t step = 16u; step; step >>= 1)
+                if ((uint32_t)__popc(movers & ((1u << (from + step)) - 1u)) <= r + part) from += step;
+            const uint32_t oo = __shfl_sync(0xFFFFFFFFu, off_old, from), co = __shfl_sync(0xFFFFFFFFu, cnt_old, from),
+                           on = __shfl_sync(0xFFFFFFFFu, off_new, from), ln = __shfl_sync(0xFFFFFFFFu, lg_new, from);
+            if (!move_block_smem(block_at(d.pool, on), block_at(d.pool, oo), active ? co : 0u, ln, d.colours, s_keys,
+                                        s_aux, rank, kPartLanes, active))
+                atomicOr(&d.ctrl->status, kStInternal);
+            __syncwarp();
+        }
+        const unsigned long long o = warp_reserve_one(&d.ctrl->n_big, defer);
+        if (defer) d.big[o] = (uint32_t)i;
+        const unsigned long long h = warp_reserve_one(&d.ctrl->n_huge, huge);
+        if (huge) d.big[d.big_cap - 1 - h] = (uint32_t)i;
+    }
 }
 
 // Move the blocks listed by k_commit whose new table has at most kMoveSlots slots: one warp per node.
 // `smem`: kMoveSmemWords words of shared memory (a key and a stream-index table of kMoveSlots slots
 // for each of the block's 8 warps).
 constexpr uint32_t kMoveSmemWords = 2u * 8u * kMoveSlots;
-static_assert(kMoveSmemWords >= 2u * kBlockMoveSlots, "the block move uses the same shared memory");
 __device__ __forceinline__ void k_rehash_big_body(const StreamDev& d, const Grid g, uint32_t* smem) {
     const unsigned long long n_big = d.ctrl->n_big, top = d.ctrl->pool_top;
     const unsigned lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
@@ -289,34 +359,95 @@ __device__ __forceinline__ void k_rehash_big_body(const StreamDev& d, const Grid
         const uint32_t i = d.big[k];
         const uint32_t x = d.touched[i];
         const uint4 m = d.meta[x];
-        const uint32_t cnt_new = m.y + m.z;
+        const uint32_t cnt_new = m.y + touched_adds(d)[i];
         const unsigned long long new_off = top + d.grow_rel[i];
         const bool fits = block_fits(d, 10, m.x, table_lg(m.y)) && block_fits(d, 11, new_off, table_lg(cnt_new));
         const uint32_t lg_new = table_lg(cnt_new);
+        uint32_t* to = block_at(d.pool, new_off);
+        const uint32_t* from = block_at(d.pool, m.x);
         bool ok = true;
         if (fits && (1u << lg_new) <= kMoveSlots && REPT_CHECK(d.ctrl, 14, wid, 8u))
-            ok = tables_interleaved(d)
-                     ? move_block_smem<false, true>(d.pool, id_mask(d), has_words(d), m.x, m.y, new_off, lg_new,
-                                                    smem + wid * kMoveSlots, smem + (8u + wid) * kMoveSlots, lane, 32u)
-                     : move_block_smem<false, false>(d.pool, id_mask(d), has_words(d), m.x, m.y, new_off, lg_new,
-                                                     smem + wid * kMoveSlots, smem + (8u + wid) * kMoveSlots, lane, 32u);
+            ok = move_block_smem(to, from, m.y, lg_new, d.colours, smem + wid * kMoveSlots,
+                                        smem + (8u + wid) * kMoveSlots, lane, 32u);
         else if (fits) {
-            init_table_keys(d.pool, new_off, lg_new, tables_interleaved(d), lane, 32u);
+            init_table_keys(to, lg_new, d.colours, lane, 32u);
             __syncwarp();
-            ok = move_block(d.pool, id_mask(d), has_words(d), tables_interleaved(d), m.x, m.y, new_off, lg_new, lane, 32u);
+            ok = move_block(to, from, m.y, lg_new, d.colours, lane, 32u);
         }
         if (!ok) atomicOr(&d.ctrl->status, kStInternal);
         __syncwarp();
-        if (lane == 0) d.meta[x] = make_uint4((uint32_t)new_off, cnt_new, m.z, 0u);
+        if (lane == 0) d.meta[x] = make_uint4((uint32_t)new_off, cnt_new, 0u, 0u);
     }
 }
 
+// move_block by one thread block, for tables of at most kBlockMoveSlots slots: the new table is laid out in
+// shared memory as one 16-bit number per slot, 1 + where its entry stands in the old block (table slot or
+// list position), and then written out bucket by bucket.  Built in place instead, with a global
+// compare-and-swap per entry, the moves of R-MAT scale 20 took 1.02 ms, so 0.85 ms.
+__device__ __forceinline__ bool move_block_index(uint32_t* to, const uint32_t* from, uint32_t cnt_old, uint32_t lg_new,
+                                                 uint32_t colours, uint16_t* s_at) {
+    const uint32_t cap = 1u << lg_new, mask = cap - 1u, lg_old = table_lg(cnt_old), rank = threadIdx.x, width = blockDim.x;
+    const bool inter = interleaved(colours);
+    for (uint32_t q = rank; q < cap / 8u; q += width) reinterpret_cast<uint4*>(s_at)[q] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    move_list(to, from, cnt_old, lg_old, lg_new, colours, rank, width);
+    bool ok = true;
+    auto place = [&](uint32_t key, uint32_t at) {
+        const uint32_t start = (key * 0x85EBCA6Bu) >> 30;
+        uint32_t b = home_slot(key, lg_new);
+        for (uint32_t probe = 0; probe <= mask; probe += 4u) {
+            for (uint32_t i = 0; i < 4u; ++i)
+                if (atomicCAS(reinterpret_cast<unsigned short*>(s_at) + b + ((start + i) & 3u), (unsigned short)0,
+                              (unsigned short)(at + 1u)) == 0)
+                    return;
+            b = (b + 4u) & mask;
+        }
+        ok = false;
+    };
+    const uint32_t* ids = from + list_at(lg_old, colours);
+    const uint32_t* aux = from + aux_at(lg_old, colours);
+    if (inter) {
+        for (uint32_t h = rank; cnt_old && h < (1u << lg_old); h += width) {
+            const uint32_t id = from[key_word(h, colours)];
+            if (id != kEmptyId) place(id, h);
+        }
+    } else {
+        for (uint32_t j = rank; j < cnt_old; j += width) place(ids[j], j);
+    }
+    __syncthreads();
+    for (uint32_t b = rank; b < cap / 4u; b += width) {
+        uint32_t id[4], t[4], cw[4];
+        const uint2 at4 = reinterpret_cast<const uint2*>(s_at)[b];
+#pragma unroll
+        for (uint32_t i = 0; i < 4u; ++i) {
+            const uint32_t at = ((i < 2u ? at4.x : at4.y) >> (16u * (i & 1u))) & 0xFFFFu;
+            id[i] = kEmptyId;
+            t[i] = cw[i] = 0u;
+            if (at) {
+                const uint32_t j = at - 1u;
+                id[i] = inter ? from[key_word(j, colours)] : ids[j];
+                t[i] = inter ? from[eidx_word(j, lg_old, colours)] : colours == kColMulti ? aux[2u * j] : aux[j];
+                if (colours == kColMulti) cw[i] = aux[2u * j + 1u];
+            }
+        }
+        uint4* out = reinterpret_cast<uint4*>(to);
+        out[inter ? 2u * b : b] = make_uint4(id[0], id[1], id[2], id[3]);
+        if (inter) {
+            out[2u * b + 1u] = make_uint4(t[0], t[1], t[2], t[3]);
+        } else if (colours == kColNone) {
+            out[cap / 4u + b] = make_uint4(t[0], t[1], t[2], t[3]);
+        } else {
+            out[cap / 4u + 2u * b] = make_uint4(t[0], cw[0], t[1], cw[1]);
+            out[cap / 4u + 2u * b + 1u] = make_uint4(t[2], cw[2], t[3], cw[3]);
+        }
+    }
+    return ok;
+}
+
 // Move the blocks listed by k_commit whose new table has more than kMoveSlots slots: thread blocks
-// claim one node at a time, and build tables of at most kBlockMoveSlots slots in shared memory.
-// `smem`: kMoveSmemWords words of shared memory (a key and a stream-index table of kBlockMoveSlots slots).
-__device__ __forceinline__ void k_rehash_huge_body(const StreamDev& d, const Grid g, uint32_t* smem) {
-    uint32_t* s_keys = smem;
-    uint32_t* s_eidx = smem + kBlockMoveSlots;
+// claim one node at a time, and build tables of at most max_slots slots in shared memory (`smem`: as many
+// 16-bit words), larger ones in place.
+__device__ __forceinline__ void k_rehash_huge_body(const StreamDev& d, const Grid g, uint32_t* smem, uint32_t max_slots) {
     __shared__ unsigned long long s_k;
     __shared__ int s_bad;
     const unsigned long long n_huge = d.ctrl->n_huge, top = d.ctrl->pool_top;
@@ -331,28 +462,25 @@ __device__ __forceinline__ void k_rehash_huge_body(const StreamDev& d, const Gri
         const uint32_t i = d.big[d.big_cap - 1 - k];
         const uint32_t x = d.touched[i];
         const uint4 m = d.meta[x];
-        const uint32_t cnt_new = m.y + m.z;
+        const uint32_t cnt_new = m.y + touched_adds(d)[i];
         const unsigned long long new_off = top + d.grow_rel[i];
         const bool fits = block_fits(d, 10, m.x, table_lg(m.y)) && block_fits(d, 11, new_off, table_lg(cnt_new));
         const uint32_t lg_new = table_lg(cnt_new);
+        uint32_t* to = block_at(d.pool, new_off);
+        const uint32_t* from = block_at(d.pool, m.x);
         bool ok = true;
-        if (fits && (1u << lg_new) <= kBlockMoveSlots)  // uniform over the block
-            ok = tables_interleaved(d)
-                     ? move_block_smem<true, true>(d.pool, id_mask(d), has_words(d), m.x, m.y, new_off, lg_new, s_keys,
-                                                   s_eidx, threadIdx.x, blockDim.x)
-                     : move_block_smem<true, false>(d.pool, id_mask(d), has_words(d), m.x, m.y, new_off, lg_new, s_keys,
-                                                    s_eidx, threadIdx.x, blockDim.x);
+        if (fits && (1u << lg_new) <= max_slots)  // uniform over the block
+            ok = move_block_index(to, from, m.y, lg_new, d.colours, reinterpret_cast<uint16_t*>(smem));
         else if (fits) {  // (uniform over the block) built in place: empty keys first
-            init_table_keys(d.pool, new_off, lg_new, tables_interleaved(d), threadIdx.x, blockDim.x);
+            init_table_keys(to, lg_new, d.colours, threadIdx.x, blockDim.x);
             __syncthreads();
-            ok = move_block(d.pool, id_mask(d), has_words(d), tables_interleaved(d), m.x, m.y, new_off, lg_new,
-                            threadIdx.x, blockDim.x);
+            ok = move_block(to, from, m.y, lg_new, d.colours, threadIdx.x, blockDim.x);
         }
         if (!ok) s_bad = 1;
         __syncthreads();
         if (threadIdx.x == 0) {
             if (s_bad) atomicOr(&d.ctrl->status, kStInternal);
-            d.meta[x] = make_uint4((uint32_t)new_off, cnt_new, m.z, 0u);
+            d.meta[x] = make_uint4((uint32_t)new_off, cnt_new, 0u, 0u);
         }
         __syncthreads();
     }
@@ -371,73 +499,73 @@ __device__ __forceinline__ void k_insert_body(const StreamDev& d, const BatchDev
         ct->huge_next = 0;
     }
     if (status) return;
+    __shared__ BlockReserve part[2];
+    uint32_t turn = 0;
     const unsigned lane = threadIdx.x & 31u;
     const unsigned long long stride = (unsigned long long)g.nbx * blockDim.x;
     unsigned long long n_loops = 0, n_kept = 0;  // this lane's tallies, added once per warp at the end
-    for (unsigned long long base = (unsigned long long)g.bx * blockDim.x + threadIdx.x - lane; base < b.n;
-         base += stride) {
-        const unsigned long long e = base + lane;
+    for (unsigned long long base = (unsigned long long)g.bx * blockDim.x; base < b.n; base += stride) {
+        const unsigned long long e = base + threadIdx.x;
         const bool valid = e < b.n;
         uint32_t u = 0, v = 0;
         if (valid) { u = b.src[e]; v = b.dst[e]; }
         const bool loop = valid && u == v;
-        // with stored colours the edge's colours decide whether it is kept and ride with its list
-        // entries (in the entries' top bits for one hash group, in a word per entry for several): the
-        // same hashes serve both
+        // with stored colours the edge's colours decide whether it is kept and ride with its entries (in
+        // the list entries' top bits or in a word per entry): the same hashes serve both
         uint32_t cj = 0u, cw = 0u;
         bool kept;
         if (d.colours == kColInEntry) {
             uint32_t i;
             const uint32_t j = colour_of(u, v, d.seed, d.fm);
-            kept = valid && u != v && processor_of(d, 0u, j, i);
+            kept = processor_of(d, 0u, j, i);
             cj = j << kIdBits;
-        } else if (has_words(d)) {
-            bool any = false;
-            uint64_t sk = group_seed(d.seed, d.kbeg);
-            for (uint32_t k = d.kbeg; k < d.kend; ++k, sk += kGoldenGamma) {
-                uint32_t i;
-                const uint32_t j = colour_of(u, v, sk, d.fm);
-                cw |= j << (k * d.cbits);
-                any |= processor_of(d, k, j, i);
-            }
-            kept = valid && u != v && any;
+        } else if (d.colours != kColNone) {
+            cw = colour_word(d, u, v, kept);
         } else {
-            kept = valid && u != v && kept_by_any(d, u, v);
+            kept = kept_by_any(d, u, v);
         }
-        uint32_t key = kNoKey;
-        WorkItem it{};
+        kept = kept && valid && u != v;
+        uint32_t mark = kNoWork;
+        bool lead = false;  // the first grouped edge seen with its larger endpoint
         if (valid && u != v) {
-            // list positions: meta[x].z counts this batch's entries of x back down to zero.  The two
-            // counters, the two records and then the first CAS of each table insert are issued
-            // before any result is used, so that their round trips overlap.
-            uint32_t zu = 0u, zv = 0u;
-            if (kept) {
-                zu = atomicSub(&d.meta[u].z, 1u);
-                zv = atomicSub(&d.meta[v].z, 1u);
-            }
+            // list positions: the batch's new entries of a node fill its list from the end.  The two
+            // records, then the first CAS of each table insert are issued before any result is used, so
+            // that their round trips overlap.
+            const uint2 rank = kept ? edge_ranks(d)[e] : make_uint2(0u, 0u);
             const uint4 mu = d.meta[u], mv = d.meta[v];
             if (kept && block_fits(d, 1, mu.x, table_lg(mu.y)) && block_fits(d, 1, mv.x, table_lg(mv.y))) {
                 const uint32_t t = (uint32_t)(b.t0 + e);
                 const uint32_t lu = table_lg(mu.y), lv = table_lg(mv.y);
-                uint32_t* tu = reinterpret_cast<uint32_t*>(d.pool + 4ull * mu.x);
-                uint32_t* tv = reinterpret_cast<uint32_t*>(d.pool + 4ull * mv.x);
-                const bool inter = tables_interleaved(d);
-                const uint32_t hu = first_slot(v, lu), hv = first_slot(u, lv);
-                const uint32_t cu = atomicCAS(tu + key_word(hu, inter), kEmptyId, v);
-                const uint32_t cv = atomicCAS(tv + key_word(hv, inter), kEmptyId, u);
+                uint32_t *tu = block_at(d.pool, mu.x), *tv = block_at(d.pool, mv.x);
+                const uint32_t col = d.colours;
+                // the home buckets are read before the compare-and-swaps: a bucket that is not in L2 is
+                // then fetched by a load, of which many more can be waiting than atomics (R-MAT scale 20,
+                // 15.7M edges: 3.2 ms without, 2.5 ms with)
+                const uint32_t bu = home_slot(v, lu), bv = home_slot(u, lv);
+                const uint4 qu = __ldcg(reinterpret_cast<const uint4*>(tu) + key_quad(bu, col)),
+                            qv = __ldcg(reinterpret_cast<const uint4*>(tv) + key_quad(bv, col));
+                const uint32_t hu = bu + empty_slot(qu, v), hv = bv + empty_slot(qv, u);
+                const uint32_t cu = atomicCAS(tu + key_word(hu, col), kEmptyId, v);
+                const uint32_t cv = atomicCAS(tv + key_word(hv, col), kEmptyId, u);
                 bool ok = true;
-                if (cu == kEmptyId) tu[eidx_word(hu, lu, inter)] = t;
-                else ok = table_insert(d.pool, 4ull * mu.x, lu, v, t, inter, true);
-                if (cv == kEmptyId) tv[eidx_word(hv, lv, inter)] = t;
-                else ok &= table_insert(d.pool, 4ull * mv.x, lv, u, t, inter, true);
+                if (cu == kEmptyId) table_store(tu, lu, hu, t, cw, col);
+                else ok = table_insert(tu, lu, v, t, cw, col);
+                if (cv == kEmptyId) table_store(tv, lv, hv, t, cw, col);
+                else ok &= table_insert(tv, lv, u, t, cw, col);
                 if (!ok) atomicOr(&ct->status, kStInternal);
-                const uint32_t pu = mu.y - zu, pv = mv.y - zv;
+                const uint32_t pu = mu.y - 1u - rank.x, pv = mv.y - 1u - rank.y;
                 if (REPT_CHECK(ct, 2, pu, list_slots(lu)) && REPT_CHECK(ct, 2, pv, list_slots(lv))) {
-                    d.pool[4ull * mu.x + (1ull << lu) + pu] = make_uint2(v | cj, t);
-                    d.pool[4ull * mv.x + (1ull << lv) + pv] = make_uint2(u | cj, t);
-                    if (has_words(d)) {
-                        list_words(d.pool, mu.x, lu)[pu] = cw;
-                        list_words(d.pool, mv.x, lv)[pv] = cw;
+                    tu[list_at(lu, col) + pu] = v | cj;
+                    tv[list_at(lv, col) + pv] = u | cj;
+                    if (col == kColWords) {
+                        tu[cw_at(lu) + pu] = cw;
+                        tv[cw_at(lv) + pv] = cw;
+                    } else if (col == kColNone) {
+                        tu[aux_at(lu, col) + pu] = t;
+                        tv[aux_at(lv, col) + pv] = t;
+                    } else if (col == kColMulti) {
+                        reinterpret_cast<uint2*>(tu + aux_at(lu, col))[pu] = make_uint2(t, cw);
+                        reinterpret_cast<uint2*>(tv + aux_at(lv, col))[pv] = make_uint2(t, cw);
                     }
                 }
                 if (d.edge_ends) d.edge_ends[t] = make_uint2(u, v);
@@ -446,6 +574,7 @@ __device__ __forceinline__ void k_insert_body(const StreamDev& d, const BatchDev
             if (mu.y != 0u && mv.y != 0u) {
                 const bool u_small = mu.y <= mv.y;
                 const uint4 ms = u_small ? mu : mv, ml = u_small ? mv : mu;
+                WorkItem it;
                 it.s = u_small ? u : v;
                 it.l = u_small ? v : u;
                 it.off_s = ms.x;
@@ -453,16 +582,19 @@ __device__ __forceinline__ void k_insert_body(const StreamDev& d, const BatchDev
                 it.t = (uint32_t)(b.t0 + e);
                 it.lgs = table_lg(ms.y) | (table_lg(ml.y) << 8);
                 it.cnt_s = ms.y;
-                key = (uint32_t)bin_of_cnt(ms.y, d.tile_max) * kKeyBuckets + ((it.l * 0x9E3779B1u) >> (32 - kKeyBits));
+                it.cnt_l = ml.y;
+                d.rec[e] = it;
+                mark = kSmallEdge;
+                if (ms.y > b.small_max) {
+                    mark = it.l;
+                    lead = atomicAdd(&d.meta[it.l].w, 1u) == 0u;
+                }
             }
         }
-        it.key = key;
-        if (valid) d.rec[e] = it;
-        {
-            const unsigned peers = __match_any_sync(0xFFFFFFFFu, key);
-            if (key != kNoKey && lane == (unsigned)(__ffs(peers) - 1))
-                atomicAdd(&d.hist[key], (uint32_t)__popc(peers));
-        }
+        if (valid) d.mark[e] = mark;
+        const unsigned long long o = block_reserve(part[turn], &ct->n_groups, lead ? 1u : 0u);
+        if (lead) d.glist[o] = mark;
+        turn ^= 1u;
         n_loops += loop ? 1ull : 0ull;
         n_kept += kept ? 1ull : 0ull;
     }
@@ -476,108 +608,87 @@ __device__ __forceinline__ void k_insert_body(const StreamDev& d, const BatchDev
     }
 }
 
-// Exclusive scan of the counting-sort histogram (one block of 256 or 1024 threads): counts become
-// the first position of each key, and the class boundaries are recorded.  The counters are scanned
-// in chunks of 4 * blockDim, thread t holding counters 4t..4t+3 of a chunk (one coalesced 16-byte
-// load); both block sizes divide the class size.
-__device__ __forceinline__ void k_sort_scan_body(const StreamDev& d, const Grid g) {
-    const uint32_t kChunk = 4u * blockDim.x;
-    static_assert(kKeyBuckets % 4096u == 0 && kSortBuckets % 4096u == 0, "scan chunks");
-    (void)g;
-    __shared__ uint32_t warp_sum[33];
-    if (d.ctrl->status) return;
-    const uint32_t tid = threadIdx.x, lane = tid & 31u, wid = tid >> 5;
-    uint32_t carry = 0;
-    for (uint32_t base = 0; base < kSortBuckets; base += kChunk) {
-        const uint4 v = reinterpret_cast<const uint4*>(d.hist + base)[tid];
-        const uint32_t sum = v.x + v.y + v.z + v.w;
-        uint32_t incl = sum;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-            if (lane >= (uint32_t)o) incl += y;
-        }
-        if (lane == 31) warp_sum[wid] = incl;
-        __syncthreads();
-        if (wid == 0) {
-            const uint32_t w = lane < (blockDim.x >> 5) ? warp_sum[lane] : 0u;
-            uint32_t wi = w;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, wi, o);
-                if (lane >= (uint32_t)o) wi += y;
-            }
-            warp_sum[lane] = wi - w;
-            if (lane == 31) warp_sum[32] = wi;  // the chunk's total
-        }
-        __syncthreads();
-        uint32_t run = carry + warp_sum[wid] + incl - sum;
-        const uint32_t key = base + 4u * tid;
-        if (key % kKeyBuckets == 0u) d.ctrl->bin_start[key / kKeyBuckets] = run;
-        uint4 o;
-        o.x = run;
-        run += v.x;
-        o.y = run;
-        run += v.y;
-        o.z = run;
-        run += v.z;
-        o.w = run;
-        reinterpret_cast<uint4*>(d.hist + base)[tid] = o;
-        carry += warp_sum[32];
-        __syncthreads();  // warp_sum is reused by the next chunk
-    }
-    if (tid == 0) {  // totals (thread 0 wrote every class start): carry is the number of items
-        unsigned long long prev = carry;
-        for (int c = kBins - 1; c >= 0; --c) {
-            d.ctrl->bin_count[c] = prev - d.ctrl->bin_start[c];
-            prev = d.ctrl->bin_start[c];
-        }
-    }
-}
-
-// Scatter each edge that can close a wedge to its place in the sorted work list.
-__device__ __forceinline__ void k_sort_scatter_body(const StreamDev& d, const BatchDev& b, const Grid g) {
-    if (d.ctrl->status) return;
+// Place the grouped edges: every larger endpoint l gets a run of order[] for its edges (its record's
+// cursor starts there), cut into units.  Runs and units are handed out in no particular order.
+__device__ __forceinline__ void k_units_body(const StreamDev& d, const BatchDev& b, const Grid g) {
+    Ctrl* ct = d.ctrl;
+    if (ct->status) return;
     const unsigned lane = threadIdx.x & 31u;
+    const unsigned long long n_g = ct->n_groups;
+    // edges per block unit: fewer in smaller batches, so that there are units for every SM
+    const uint32_t per_block = (uint32_t)min(max(b.n >> 14, 16ull), (unsigned long long)kUnitItems);
     const unsigned long long stride = (unsigned long long)g.nbx * blockDim.x;
-    for (unsigned long long base = (unsigned long long)g.bx * blockDim.x + threadIdx.x - lane; base < b.n;
+    for (unsigned long long base = (unsigned long long)g.bx * blockDim.x + threadIdx.x - lane; base < n_g;
          base += stride) {
-        const unsigned long long e = base + lane;
-        WorkItem it{};
-        it.key = kNoKey;
-        if (e < b.n) it = d.rec[e];
-        const uint32_t key = it.key;
-        const unsigned peers = __match_any_sync(0xFFFFFFFFu, key);
-        const int leader = __ffs(peers) - 1;
-        uint32_t pos = 0;
-        if (key != kNoKey && (int)lane == leader) pos = atomicAdd(&d.hist[key], (uint32_t)__popc(peers));
-        pos = __shfl_sync(0xFFFFFFFFu, pos, leader);
-        if (key != kNoKey) d.srec[pos + __popc(peers & ((1u << lane) - 1u))] = it;
+        const unsigned long long i = base + lane;
+        uint32_t l = 0, count = 0;
+        uint32_t per = 1;
+        int kind = kBinWarp;
+        if (i < n_g) {
+            l = d.glist[i];
+            const uint4 m = d.meta[l];
+            count = m.w;
+            kind = m.y > kBigUnitNodes ? kBinBig : m.y > kWarpUnitNodes ? kBinBlock : kBinWarp;
+            // (an edge's smaller list is no longer than the larger: at most kWarpUnitEntries per warp unit)
+            per = kind == kBinWarp ? min(max(kWarpUnitEntries / m.y, 1u), kWarpUnitItems) : per_block;
+        }
+        const uint32_t first = (uint32_t)warp_reserve(&ct->n_items, count);
+        if (i < n_g) d.meta[l].w = first;
+        const uint32_t n_u = (count + per - 1u) / per;
+        const unsigned long long uw = warp_reserve(&ct->bin_count[kBinWarp], kind == kBinWarp ? n_u : 0u);
+        unsigned long long at = d.unit_cap - 1ull - uw;
+        if (__any_sync(0xFFFFFFFFu, kind != kBinWarp)) {
+            const unsigned long long ub = warp_reserve(&ct->bin_count[kBinBlock], kind == kBinBlock ? n_u : 0u);
+            const unsigned long long ug = warp_reserve(&ct->bin_count[kBinBig], kind == kBinBig ? n_u : 0u);
+            if (kind == kBinBlock) at = d.unit_cap + ub;
+            else if (kind == kBinBig) at = ug;
+        }
+        for (uint32_t k = 0; k < n_u; ++k) {
+            if (!REPT_CHECK(ct, 15, at, 2ull * d.unit_cap)) break;
+            d.units[at] = Unit{first + k * per, min(per, count - k * per)};
+            at += kind == kBinWarp ? -1ll : 1ll;
+        }
     }
 }
 
-// Look neighbour w up in the table of 2^lg slots at `base` (lg >= 2): read 4-key buckets from w's
-// home bucket on until w or an empty key shows up.  Returns w's stream index, or kEmptyId when w is
-// absent; `slots` receives the number of keys read.
-__device__ __forceinline__ uint32_t table_find(const uint2* __restrict__ pool, unsigned long long base, uint32_t lg,
-                                               uint32_t w, uint32_t& slots, bool inter) {
+// Write each grouped edge to its place in order[].
+__device__ __forceinline__ void k_order_body(const StreamDev& d, const BatchDev& b, const Grid g) {
+    if (d.ctrl->status) return;
+    const unsigned long long stride = (unsigned long long)g.nbx * blockDim.x;
+    for (unsigned long long e = (unsigned long long)g.bx * blockDim.x + threadIdx.x; e < b.n; e += stride) {
+        const uint32_t l = d.mark[e];
+        if (l >= kSmallEdge) continue;
+        const uint32_t pos = atomicAdd(&d.meta[l].w, 1u);
+        if (REPT_CHECK(d.ctrl, 16, pos, d.unit_cap)) d.order[pos] = (uint32_t)e;
+    }
+}
+
+// Look neighbour w up in the table of 2^lg slots at `table` (lg >= 2): read 4-key buckets from w's
+// home bucket on until w or an empty key shows up.  Returns w's slot, or kEmptyId when w is absent;
+// `slots` receives the number of keys read.
+__device__ __forceinline__ uint32_t table_slot(const uint32_t* __restrict__ table, uint32_t lg, uint32_t w,
+                                               uint32_t& slots, uint32_t colours) {
     const uint32_t mask = (1u << lg) - 1u;
-    const uint32_t* keys = reinterpret_cast<const uint32_t*>(pool + base);
-    const uint4* buckets = reinterpret_cast<const uint4*>(keys);
+    const uint4* buckets = reinterpret_cast<const uint4*>(table);
     uint32_t h = home_slot(w, lg);
     for (uint32_t probe = 0; probe <= mask; probe += 4u) {  // h: the first slot of a bucket
-        const uint4 k4 = buckets[key_quad(h, inter)];
+        const uint4 k4 = buckets[key_quad(h, colours)];
         slots = probe + 4u;
-        int at = -1;
-        if (k4.x == w) at = 0;
-        else if (k4.y == w) at = 1;
-        else if (k4.z == w) at = 2;
-        else if (k4.w == w) at = 3;
-        if (at >= 0) return keys[eidx_word(h + (uint32_t)at, lg, inter)];
+        if (k4.x == w) return h;
+        if (k4.y == w) return h + 1u;
+        if (k4.z == w) return h + 2u;
+        if (k4.w == w) return h + 3u;
         if (k4.x == kEmptyId || k4.y == kEmptyId || k4.z == kEmptyId || k4.w == kEmptyId) return kEmptyId;
         h = (h + 4u) & mask;
     }
     return kEmptyId;
+}
+
+// w's stream index in that table, or kEmptyId.
+__device__ __forceinline__ uint32_t table_find(const uint32_t* __restrict__ table, uint32_t lg, uint32_t w,
+                                               uint32_t& slots, uint32_t colours) {
+    const uint32_t h = table_slot(table, lg, w, slots, colours);
+    return h == kEmptyId ? kEmptyId : table[eidx_word(h, lg, colours)];
 }
 
 // REPT_FLAG_CHECK_DUPS: before the batch is applied, flag an edge that repeats an earlier stored
@@ -594,7 +705,7 @@ __global__ void k_check_dups(StreamDev d, BatchDev b, unsigned long long mask) {
         if (u == v || u >= d.n_nodes || v >= d.n_nodes) continue;
         const uint4 mu = d.meta[u];
         uint32_t ns;
-        if (mu.y != 0u && table_find(d.pool, 4ull * mu.x, table_lg(mu.y), v, ns, tables_interleaved(d)) != kEmptyId) dup = true;
+        if (mu.y != 0u && table_find(block_at(d.pool, mu.x), table_lg(mu.y), v, ns, d.colours) != kEmptyId) dup = true;
         const unsigned long long key = ((unsigned long long)(u < v ? u : v) << 32) | (u < v ? v : u);
         unsigned long long h = splitmix64(key) & mask;
         for (unsigned long long probe = 0; probe <= mask; ++probe) {
@@ -621,49 +732,32 @@ __device__ __forceinline__ void pair_event(const StreamDev& d, uint32_t t, uint3
     if (atomicAdd(&d.pair_evt[idx], 1u) == 0u) d.pair_list[atomicAdd(&d.ctrl->n_pairs, 1ull)] = (uint32_t)idx;
 }
 
-// MODE: the stream's colour storage (the kernel variant).  DIFF: decide each group's colour agreement
-// from the two hash values' difference (same_colour: one remainder only when they agree), which pays
-// where wedges are counted under several groups (streams without colours in their entries); streams
-// with colours in their entries form both colours, which keeps their registers lower.  INTER: the
-// stream's tables are interleaved (tables_interleaved), i.e. it stores colours.
+// kColAny: the colour storage is read from each stream's descriptor (groups).
+constexpr int kColAny = 8;
 template <int MODE>
-__device__ __forceinline__ uint32_t count_wedge(const StreamDev& d, uint32_t s, uint32_t l, uint32_t w,
-                                                unsigned long long* s_proc) {
-    constexpr bool DIFF = MODE != (int)kColInEntry, INTER = MODE != (int)kColNone;
-    if (!REPT_CHECK(d.ctrl, 9, max(w, max(s, l)), d.n_nodes)) return 0u;
-    uint32_t found = 0, found2 = 0;
-    uint32_t t_sw = kEmptyId, t_lw = kEmptyId;
-    for (uint32_t k = d.kbeg; k < d.kend; ++k) {
-        uint32_t js, i;
-        bool agree;
-        if (DIFF) {
-            agree = same_colour(s, l, w, group_seed(d.seed, k), d.fm, js) && processor_of(d, k, js, i);
-        } else {
-            const uint64_t sk = group_seed(d.seed, k);
-            js = colour_of(s, w, sk, d.fm);
-            agree = processor_of(d, k, js, i) && colour_of(l, w, sk, d.fm) == js;
-        }
-        if (agree) {
-            atomicAdd(&s_proc[i], 1ull);
-            if (d.local2 && k >= d.c1) ++found2; else ++found;
-            if (d.local_proc) {
-                unsigned long long* lp = d.local_proc + (unsigned long long)i * d.n_nodes;
-                atomicAdd(&lp[s], 1ull);
-                atomicAdd(&lp[l], 1ull);
-                atomicAdd(&lp[w], 1ull);
-            }
-            if (d.pair_tau) {
-                if (t_sw == kEmptyId) {  // the wedge's two stream indices, looked up once
-                    uint32_t ns;
-                    const uint4 ms = d.meta[s], ml = d.meta[l];
-                    t_sw = table_find(d.pool, 4ull * ms.x, table_lg(ms.y), w, ns, INTER);
-                    t_lw = table_find(d.pool, 4ull * ml.x, table_lg(ml.y), w, ns, INTER);
-                }
-                pair_event(d, t_sw, k);
-                pair_event(d, t_lw, k);
-            }
-        }
-    }
+__device__ __forceinline__ uint32_t colours_of(const StreamDev& d) {
+    return MODE == kColAny ? d.colours : (uint32_t)MODE;
+}
+
+// Where closed wedges are tallied: a single stream's blocks keep tau^(i) in shared memory, as a low and a
+// high 32-bit half (processor i: words 2i, 2i + 1; 64-bit shared atomics are compare-and-swap loops); a
+// group's go straight to global memory (half == nullptr).
+__device__ __forceinline__ void tally(const StreamDev& d, uint32_t* half, uint32_t i) {
+    if (half == nullptr) atomicAdd(&d.proc[i], 1ull);
+    else if (atomicAdd(&half[2u * i], 1u) == 0xFFFFFFFFu) atomicAdd(&half[2u * i + 1u], 1u);
+}
+
+// Processor i counted the wedge (s, w), (l, w): its own tau_v^(i), when kept.
+__device__ __forceinline__ void count_local_proc(const StreamDev& d, uint32_t i, uint32_t s, uint32_t l, uint32_t w) {
+    unsigned long long* lp = d.local_proc + (unsigned long long)i * d.n_nodes;
+    atomicAdd(&lp[s], 1ull);
+    atomicAdd(&lp[l], 1ull);
+    atomicAdd(&lp[w], 1ull);
+}
+
+// `found` groups counted it for the local sums, `found2` for Algorithm 2's partial group.
+__device__ __forceinline__ void count_locals(const StreamDev& d, uint32_t found, uint32_t found2, uint32_t s, uint32_t l,
+                                             uint32_t w) {
     if (found) {
         atomicAdd(&d.local[w], (unsigned long long)found);
         atomicAdd(&d.local[s], (unsigned long long)found);
@@ -674,507 +768,734 @@ __device__ __forceinline__ uint32_t count_wedge(const StreamDev& d, uint32_t s, 
         atomicAdd(&d.local2[s], (unsigned long long)found2);
         atomicAdd(&d.local2[l], (unsigned long long)found2);
     }
+}
+
+// The wedge's colours from the hashes.  Single-group streams with colours in their entries form both
+// colours, which keeps registers low; the others decide each group's agreement from the two hash values'
+// difference (same_colour: one remainder only when they agree).
+template <int MODE>
+__device__ __forceinline__ uint32_t count_wedge(const StreamDev& d, uint32_t* half, uint32_t s, uint32_t l, uint32_t w) {
+    if (!REPT_CHECK(d.ctrl, 9, max(w, max(s, l)), d.n_nodes)) return 0u;
+    uint32_t found = 0, found2 = 0;
+    uint32_t t_sw = kEmptyId, t_lw = kEmptyId;
+    for (uint32_t k = d.kbeg; k < d.kend; ++k) {
+        uint32_t js, i;
+        bool agree;
+        if (MODE != (int)kColInEntry) {
+            agree = same_colour(s, l, w, group_seed(d.seed, k), d.fm, js) && processor_of(d, k, js, i);
+        } else {
+            const uint64_t sk = group_seed(d.seed, k);
+            js = colour_of(s, w, sk, d.fm);
+            agree = processor_of(d, k, js, i) && colour_of(l, w, sk, d.fm) == js;
+        }
+        if (agree) {
+            tally(d, half, i);
+            if (d.local2 && k >= d.c1) ++found2; else ++found;
+            if (d.local_proc) count_local_proc(d, i, s, l, w);
+            if (d.pair_tau) {
+                if (t_sw == kEmptyId) {  // the wedge's two stream indices, looked up once
+                    uint32_t ns;
+                    const uint4 ms = d.meta[s], ml = d.meta[l];
+                    t_sw = table_find(block_at(d.pool, ms.x), table_lg(ms.y), w, ns, kColNone);
+                    t_lw = table_find(block_at(d.pool, ml.x), table_lg(ml.y), w, ns, kColNone);
+                }
+                pair_event(d, t_sw, k);
+                pair_event(d, t_lw, k);
+            }
+        }
+    }
+    count_locals(d, found, found2, s, l, w);
     return found + found2;
 }
 
-// Per-warp queue of closed wedges (s, l, w) in shared memory.  Wedges are pushed as the probes find
-// them and coloured 32 at a time, so that the hash work runs on full warps.  `n` is warp-uniform.
-constexpr int kMatchQ = 64;
-struct MatchQueue {
-    uint32_t* s;
-    uint32_t* l;
-    uint32_t* w;
-    uint32_t n;
+// The groups in which two edges with the stored colour words cs, cl (kColMulti) have the same colour: bit
+// (k + 1) cbits - 1 for group k, found for all groups at once (a field of cs ^ cl is zero); where a group
+// keeps one colour only, the groups that keep both edges.
+__device__ __forceinline__ uint32_t agreeing_groups(const StreamDev& d, uint32_t cs, uint32_t cl) {
+    if (d.keep == 1u) return cs & cl;
+    const uint32_t x = cs ^ cl, low = ~d.ctop;
+    return ~(((x & low) + low) | x) & d.ctop;
+}
+
+// Count the wedge (s, w), (l, w) in those groups, where a processor keeps the colour (cs, of {s, w}).
+__device__ __forceinline__ uint32_t count_groups(const StreamDev& d, uint32_t* half, uint32_t s, uint32_t l, uint32_t w,
+                                                 uint32_t groups, uint32_t cs) {
+    if (!REPT_CHECK(d.ctrl, 9, max(w, max(s, l)), d.n_nodes)) return 0u;
+    uint32_t found = 0, found2 = 0;
+    uint32_t t_sw = kEmptyId, t_lw = kEmptyId;
+    for (; groups; groups &= groups - 1u) {
+        const uint32_t top = (uint32_t)__ffs((int)groups), k = top / d.cbits - 1u;
+        uint32_t i;
+        const uint32_t js = d.keep == 1u ? 0u : (cs >> (top - d.cbits)) & d.cmask;
+        if (!processor_of(d, k, js, i)) continue;
+        tally(d, half, i);
+        if (d.local2 && k >= d.c1) ++found2; else ++found;
+        if (d.local_proc) count_local_proc(d, i, s, l, w);
+        if (d.pair_tau) {
+            if (t_sw == kEmptyId) {  // the wedge's two stream indices, looked up once
+                uint32_t ns;
+                const uint4 ms = d.meta[s], ml = d.meta[l];
+                t_sw = table_find(block_at(d.pool, ms.x), table_lg(ms.y), w, ns, kColMulti);
+                t_lw = table_find(block_at(d.pool, ml.x), table_lg(ml.y), w, ns, kColMulti);
+            }
+            pair_event(d, t_sw, k);
+            pair_event(d, t_lw, k);
+        }
+    }
+    count_locals(d, found, found2, s, l, w);
+    return found + found2;
+}
+
+// ---------------------------------------------------------------------------------------------
+// The intersection.  An edge t = (s, l) closes the wedges {s, w}, {l, w} of entries w that both lists
+// hold.  Few entries of s's list do (with the same colour in both, about 0.1 % on the R-MAT streams), so
+// the work is to reject the others cheaply.  A filter of l's list is built in shared memory -- a Bloom
+// filter of two bits per entry, both in one 32-bit word, keyed by the entry's id and stored colour --
+// and the lists of l's grouped edges are scanned against it: nine instructions and one shared-memory
+// read per entry, where hashing the larger endpoint's edge for its colour takes 58.  Grouping by l makes
+// one filter serve all edges of l (R-MAT scale 20, late batches: 14 to 26 times as many entries are
+// scanned as inserted).  Entries that pass (0.6 % there; with several groups the common neighbours, 14 %
+// on the 4M-node stream) join the warp's candidate queue and are looked up in l's table, which decides
+// exactly.  R-MAT scale 20, m = c = 100: 8.83 ms per stream with a hash per entry, 5.51 ms so; the 4M-node
+// stream with five groups: 157 ms with a probe per entry, 122 ms so, of which the scans alone are 18 ms.
+// What bounds it: instruction issue (57 % of the slots) in the scans, the latency of the candidates'
+// dependent loads where many pass.
+
+constexpr int kIxThreads = 256;
+constexpr int kIxBlocks = 4;  // per SM: 4 x 48 KB of shared memory
+constexpr uint32_t kIxWarps = kIxThreads / 32;
+constexpr uint32_t kFilterLg = 13;  // words of a block's filter (32 KB); a warp's share serves warp units
+constexpr uint32_t kFilterWords = 1u << kFilterLg;
+constexpr uint32_t kWarpFilterLg = 10;
+static_assert(kIxWarps << kWarpFilterLg <= kFilterWords, "warp filters share the block's");
+static_assert(kUnitItems == 64, "two records per lane of the first warp");
+
+// A warp's two queues, arrays of kCandQ and kMatchQ words.  Candidates: the position in the smaller endpoint's list
+// of an entry that passed a filter or colour test, its edge and, for groups, the stream.  Closed wedges:
+// the neighbour, the edge, the agreeing groups and the colour word (kColMulti) and, for groups, the
+// stream; they are counted
+// 32 at a time so that the work runs on full warps.
+struct WarpQueues {
+    uint32_t* base;      // candidates, then closed wedges
+    uint32_t n, closed;  // how many of each are waiting (warp-uniform)
+};
+constexpr uint32_t kCandQ = 96, kMatchQ = 96;  // 63 + 32 candidates; 31 + 2 x 32 wedges
+// Arrays of closed wedges before the streams'.
+constexpr uint32_t match_arrays(int mode) { return mode == (int)kColMulti || mode == kColAny ? 4u : 2u; }
+constexpr uint32_t queue_words(int mode, bool group) {
+    return (group ? 3u : 2u) * kCandQ + (match_arrays(mode) + (group ? 1u : 0u)) * kMatchQ;
+}
+
+// Shared memory of one intersection block, in words: the filter, the records of the unit's edges and the
+// warps' queues.
+constexpr uint32_t ix_words(int mode, bool group) {
+    return kFilterWords + 4u * kUnitItems + kIxWarps * queue_words(mode, group);
+}
+
+// The streams an intersection works on: one, passed by value to the kernel, with its block's counters
+// (tally), or a group's array.
+struct OneStream {
+    static constexpr bool kGroup = false;
+    const StreamDev& d;
+    uint32_t* half;
+    __device__ __forceinline__ const StreamDev& at(uint32_t) const { return d; }
+};
+struct ManyStreams {
+    static constexpr bool kGroup = true;
+    const StreamDev* __restrict__ ds;
+    static constexpr uint32_t* half = nullptr;
+    __device__ __forceinline__ const StreamDev& at(uint32_t sid) const { return ds[sid]; }
 };
 
-template <bool WORK, int MODE>
-__device__ __forceinline__ void mq_flush(const StreamDev& d, MatchQueue& q, uint32_t take,
-                                         unsigned long long* s_proc, Work& wk) {
+// Count `take` closed wedges from the end of the queue (n waiting).
+template <bool WORK, int MODE, class S>
+__device__ __forceinline__ void count_closed(const S& st, const uint32_t* mq, uint32_t n, uint32_t take, Work& wk) {
+    constexpr bool GROUP = S::kGroup;
     const unsigned lane = threadIdx.x & 31u;
     if (lane < take) {
-        const uint32_t i = q.n - take + lane;
-        const uint32_t f = count_wedge<MODE>(d, q.s[i], q.l[i], q.w[i], s_proc);
+        const uint32_t i = n - take + lane, w = mq[i];
+        const StreamDev& d = st.at(GROUP ? mq[match_arrays(MODE) * kMatchQ + i] : 0u);
+        const uint2 sl = *reinterpret_cast<const uint2*>(d.rec + mq[kMatchQ + i]);
+        uint32_t f = 0;
+        if (match_arrays(MODE) == 4u && colours_of<MODE>(d) == kColMulti)
+            f = count_groups(d, st.half, sl.x, sl.y, w, mq[2u * kMatchQ + i], mq[3u * kMatchQ + i]);
+        else
+            f = count_wedge<MODE>(d, st.half, sl.x, sl.y, w);
         if (WORK) wk.counted += f;
     }
-    q.n -= take;
     __syncwarp();
 }
 
-template <bool WORK, int MODE>
-__device__ __forceinline__ void mq_push(const StreamDev& d, MatchQueue& q, bool has, uint32_t s, uint32_t l,
-                                        uint32_t w, unsigned long long* s_proc, Work& wk) {
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned mask = __ballot_sync(0xFFFFFFFFu, has);
-    if (!REPT_CHECK(d.ctrl, 13, q.n + __popc(mask), (unsigned long long)kMatchQ + 1ull)) return;
-    if (has) {
-        const uint32_t i = q.n + __popc(mask & ((1u << lane) - 1u));
-        q.s[i] = s;
-        q.l[i] = l;
-        q.w[i] = w;
-        if (WORK) ++wk.wedges;
-    }
-    q.n += __popc(mask);
-    __syncwarp();
-    if (q.n >= 32u) mq_flush<WORK, MODE>(d, q, 32u, s_proc, wk);
-}
-
-// Edges whose smaller endpoint has at most TILE entries: one tile of TILE lanes per edge, one list
-// entry per lane.
-template <int TILE, bool WORK, int MODE>
-__device__ __forceinline__ void intersect_tile(const StreamDev& d, const WorkItem& x, bool valid,
-                                               unsigned long long* s_proc, MatchQueue& mq, Work& wk) {
-    const unsigned lane = threadIdx.x & 31u, j = lane & (TILE - 1);
-    bool has = false;
-    uint32_t w = 0;
-    if (valid && j < x.cnt_s) {
-        const unsigned long long at = 4ull * x.off_s + (1ull << (x.lgs & 0xFFu)) + j;
-        const bool fits = REPT_CHECK(d.ctrl, 3, at, 4ull * d.pool_quads) && block_fits(d, 4, x.off_l, x.lgs >> 8);
-        const uint2 es = fits ? d.pool[at] : make_uint2(kEmptyId, kEmptyId);
-        if (WORK && j == 0) { wk.entries += x.cnt_s; wk.slots += x.cnt_s; }
-        const uint32_t ws = es.x & id_mask(d);
-        bool pass = es.y < x.t;
-        if (d.colours == kColInEntry) pass = pass & wedge_may_count(d, x.l, ws, es.x >> kIdBits);
-        else if (pass && has_words(d) && block_fits(d, 12, x.off_s, x.lgs & 0xFFu))
-            pass = words_may_count(d, x.l, ws, list_words(d.pool, x.off_s, x.lgs & 0xFFu)[j]);
-        if (pass) {
-            uint32_t nslots = 0;
-            // the single-stream kernels' streams: split tables exactly in the probe variant
-            const uint32_t tl = table_find(d.pool, 4ull * x.off_l, x.lgs >> 8, ws, nslots, MODE != (int)kColNone);
-            if (WORK) { ++wk.probes; wk.pslots += nslots; }
-            has = tl < x.t;  // kEmptyId (absent) is never < t
-            w = ws;
+// Probe candidates 0 .. take - 1 (take <= 64) of the queue at `cq`, two per lane.  A hit whose two edges are
+// older than the candidate's edge is a closed wedge.  `closed` wedges were waiting; returns how many
+// are now (`all`: none, everything is counted).
+template <bool WORK, int MODE, class S>
+__device__ __forceinline__ uint32_t cand_probe(const S& st, const uint32_t* cq, uint32_t* mq, uint32_t take,
+                                               uint32_t closed, bool all, Work& wk) {
+    constexpr bool GROUP = S::kGroup;
+    const unsigned lane = threadIdx.x & 31u, below = (1u << lane) - 1u;
+    if (take) {
+        // every stage loads for both candidates before either is used; lanes past the end repeat the last one
+        uint32_t item[2], sd[2], pos[2], w[2], h[2], lgs[2], lgl[2], t[2], slot[2];
+        uint2 off[2];  // blocks of the smaller and the larger endpoint
+        uint4 bk[2];
+        uint2 as[2], al[2];  // stream index and colour word of the smaller and the larger side's entry
+        bool v[2];
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            const uint32_t k = min(32u * p + lane, take - 1u);
+            v[p] = 32u * p + lane < take;
+            pos[p] = cq[k];
+            item[p] = cq[kCandQ + k];
+            sd[p] = GROUP ? cq[2u * kCandQ + k] : 0u;
         }
-    }
-    mq_push<WORK, MODE>(d, mq, has, x.s, x.l, w, s_proc, wk);
-}
-
-// Edges whose smaller endpoint has more entries, streams without stored colours: a warp per edge.
-// Each pass reads 128 entries of the smaller endpoint's list (two 16-byte loads per lane) and packs
-// those older than the edge into the warp's shared-memory key queue.  The queue is probed with all 32
-// lanes, kProbesPerLane keys per lane, whenever it holds a full round; a partial round waits for the
-// next pass, so sparse candidates share round trips.
-#ifndef REPT_GRAB_MID
-#define REPT_GRAB_MID 4
-#endif
-#ifndef REPT_GRAB_HUB
-#define REPT_GRAB_HUB 1
-#endif
-constexpr uint32_t kGrabMid = REPT_GRAB_MID;  // class 4 items (33..256 entries) claimed per atomic
-constexpr uint32_t kGrabHub = REPT_GRAB_HUB;  // class 5 items (more entries) claimed per atomic
-// The scan-first path's claims: its items cost less each (about 1/m of the entries are probed), so
-// a warp takes more of them per atomic on the class cursor.
-#ifndef REPT_SCAN_GRAB_MID
-#define REPT_SCAN_GRAB_MID 8
-#endif
-#ifndef REPT_SCAN_GRAB_HUB
-#define REPT_SCAN_GRAB_HUB 2
-#endif
-constexpr uint32_t kScanGrabMid = REPT_SCAN_GRAB_MID;
-constexpr uint32_t kScanGrabHub = REPT_SCAN_GRAB_HUB;
-constexpr int kQueue = 192;  // one partial round (< 64 keys) + 128 new keys
-
-#ifndef REPT_PROBES_PER_LANE
-#define REPT_PROBES_PER_LANE 2
-#endif
-constexpr int kProbesPerLane = REPT_PROBES_PER_LANE;  // probes each lane keeps in flight (warp path)
-#ifndef REPT_WORDS_BLOCKS
-#define REPT_WORDS_BLOCKS 6
-#endif
-
-// Streams without stored colours (MODE kColNone): every entry older than the edge is probed, so the
-// path is probe-bound and runs with fewer registers and more warps per SM.  Streams that store
-// colours take the scan-first path (drain_warp_bin_coloured) instead.
-// `push(has, w)` (warp-collective) takes each probed key w and whether it closed a wedge.
-template <bool WORK, int MODE, class Push>
-__device__ __forceinline__ void intersect_warp(const StreamDev& d, const WorkItem& x, uint32_t* queue, Work& wk,
-                                               Push&& push) {
-    static_assert(MODE == (int)kColNone, "streams that store colours take the scan-first path");
-    constexpr uint32_t kRound = 32u * kProbesPerLane;
-    static_assert(kRound - 1 + 128 <= kQueue, "key queue too small");
-    const unsigned lane = threadIdx.x & 31u;
-    const uint32_t lg_l = x.lgs >> 8, n_s = x.cnt_s;
-    const unsigned long long base_l = 4ull * x.off_l;
-    if (WORK && lane == 0) { wk.entries += n_s; wk.slots += n_s; }
-    if (!(block_fits(d, 5, x.off_s, x.lgs & 0xFFu) && REPT_CHECK(d.ctrl, 6, n_s, list_slots(x.lgs & 0xFFu) + 1u) &&
-          block_fits(d, 7, x.off_l, lg_l)))
-        return;  // (uniform over the warp: x is)
-    // the smaller endpoint's entry list (32-byte aligned), read 128 entries per pass, two per 16-byte
-    // load
-    const unsigned long long at_s = 4ull * x.off_s + (1ull << (x.lgs & 0xFFu));
-    const uint4* list = reinterpret_cast<const uint4*>(d.pool + at_s);
-    const uint32_t mask = id_mask(d);
-    const uint32_t* keys_l = reinterpret_cast<const uint32_t*>(d.pool + base_l);
-    const uint4* buckets_l = reinterpret_cast<const uint4*>(keys_l);
-    const bool inter = false;  // these streams keep split tables
-    const unsigned below = (1u << lane) - 1u;
-    uint4 nq[2];
-    auto load_pass = [&](uint32_t j0) {
 #pragma unroll
-        for (uint32_t half = 0; half < 2; ++half) {
-            const uint32_t jj = j0 + 64u * half + 2u * lane;
-            nq[half] = make_uint4(kEmptyId, kEmptyId, kEmptyId, kEmptyId);
-            if (jj < n_s) nq[half] = list[jj >> 1];
-        }
-    };
-    uint32_t n_q = 0;
-
-    for (uint32_t j0 = 0; j0 < n_s; j0 += 128u) {
-        if (!REPT_CHECK(d.ctrl, 8, n_q, kRound)) break;
-        load_pass(j0);
-        const uint4 cq[2] = {nq[0], nq[1]};
-#pragma unroll
-        for (uint32_t half = 0; half < 2; ++half) {
-            if (j0 + 64u * half >= n_s) break;  // an empty half (short lists, last passes): uniform skip
-            const uint32_t jj = j0 + 64u * half + 2u * lane;
-            const uint4 q = cq[half];
-            const uint32_t w1 = q.x & mask, w2 = q.z & mask;
-            const bool a1 = jj < n_s && q.y < x.t, a2 = jj + 1u < n_s && q.w < x.t;
-            const unsigned m1 = __ballot_sync(0xFFFFFFFFu, a1), m2 = __ballot_sync(0xFFFFFFFFu, a2);
-            if (a1) queue[n_q + __popc(m1 & below)] = w1;
-            n_q += __popc(m1);
-            if (a2) queue[n_q + __popc(m2 & below)] = w2;
-            n_q += __popc(m2);
-        }
-        __syncwarp();
-        const bool last = j0 + 128u >= n_s;
-        // full rounds now, everything after the last pass: kProbesPerLane queued keys per lane, all
-        // their home buckets loaded before any is examined, then the stream indices of the hits
-        uint32_t k0 = 0;
-        for (; last ? k0 < n_q : k0 + kRound <= n_q; k0 += kRound) {
-            uint32_t w[kProbesPerLane], h[kProbesPerLane], r[kProbesPerLane];
-            uint4 bk[kProbesPerLane];
-#pragma unroll
-            for (int p = 0; p < kProbesPerLane; ++p) {
-                const bool v = k0 + 32u * p + lane < n_q;
-                w[p] = v ? queue[k0 + 32u * p + lane] : kEmptyId;
-                h[p] = home_slot(w[p], lg_l);
-                bk[p] = make_uint4(kEmptyId, kEmptyId, kEmptyId, kEmptyId);
-                if (v) bk[p] = __ldg(&buckets_l[key_quad(h[p], inter)]);
-            }
-#pragma unroll
-            for (int p = 0; p < kProbesPerLane; ++p) {
-                const uint4 b = bk[p];
-                const int at = b.x == w[p] ? 0 : b.y == w[p] ? 1 : b.z == w[p] ? 2 : b.w == w[p] ? 3 : -1;
-                r[p] = kEmptyId;
-                if (w[p] != kEmptyId) {
-                    uint32_t ns = 4u;
-                    if (at >= 0) {
-                        r[p] = __ldg(&keys_l[eidx_word(h[p] + (uint32_t)at, lg_l, inter)]);
-                    } else if (b.x != kEmptyId && b.y != kEmptyId && b.z != kEmptyId && b.w != kEmptyId) {
-                        r[p] = table_find(d.pool, base_l, lg_l, w[p], ns, inter);  // rare: the bucket is full
-                    }
-                    if (WORK) { ++wk.probes; wk.pslots += ns; }
+        for (int p = 0; p < 2; ++p) {  // WorkItem: {s, l, off_s, off_l}, {t, lgs, cnt_s, cnt_l}
+            const uint2* rec = reinterpret_cast<const uint2*>(st.at(sd[p]).rec + item[p]);
+            off[p] = rec[1];
+            const uint2 r = rec[2];
+            t[p] = r.x;
+            lgs[p] = r.y & 0xFFu;
+            lgl[p] = r.y >> 8;
+            if (WORK) {
+                const uint32_t cls = v[p] ? (uint32_t)bin_of_cnt(rec[3].x) : 6u;
+                for (uint32_t c = 0; c < 6u; ++c) {
+                    const unsigned of = __ballot_sync(0xFFFFFFFFu, cls == c);
+                    if (of && lane == 0) atomicAdd(&st.at(0u).ctrl->class_probes[c], (unsigned long long)__popc(of));
                 }
             }
-#pragma unroll
-            for (int p = 0; p < kProbesPerLane; ++p)
-                push(w[p] != kEmptyId && r[p] < x.t, w[p]);
         }
-        __syncwarp();
-        if (last) break;
-        if (k0) {  // move the unprobed rest (< kRound <= k0 keys) to the front; the ranges are disjoint
-            const uint32_t rest = n_q - k0;
-            for (uint32_t r = lane; r < rest; r += 32u) queue[r] = queue[k0 + r];
-            n_q = rest;
-            __syncwarp();
-        }
-    }
-}
-
-// Streams that store colours (kColInEntry, kColWords), warp classes: scan first, probe later.  A warp
-// reads an item's smaller-endpoint list kScanPass entries per pass (kScanLoads 16-byte loads per
-// lane, two entries each) and tests every entry's colour against the larger endpoint by hash alone.
-// The few entries that pass (about 1/m) join the warp's candidate queue together with the index of
-// their work item; the queue is probed 64 candidates at a time, whatever items they come from, so
-// that an item with a handful of candidates does not pay for a probe round of its own.
-#ifndef REPT_SCAN_LOADS
-#define REPT_SCAN_LOADS 4
-#endif
-#ifndef REPT_SCAN_FULL
-#define REPT_SCAN_FULL 1
-#endif
-constexpr uint32_t kScanLoads = REPT_SCAN_LOADS;  // 16-byte loads per lane and pass
-constexpr uint32_t kScanPass = 64u * kScanLoads;  // entries per pass
-constexpr bool kScanFull = REPT_SCAN_FULL != 0;  // passes inside the list skip the position checks
-constexpr uint32_t kCandQ = 64u + kScanPass;       // candidate queue slots per warp
-struct CandQueue {
-    uint32_t* w;     // [kCandQ] candidate neighbour w
-    uint32_t* item;  // [kCandQ] its work item, an index into srec
-    uint32_t n;      // warp-uniform
-};
-
-// Probe candidates k0 .. k0 + take - 1 (take <= 64), two per lane: both items' records and then both
-// home buckets are loaded before either is examined.  A hit older than its edge is a closed wedge.
-template <bool WORK, int MODE>
-__device__ __forceinline__ void cand_probe(const StreamDev& d, const CandQueue& cq, uint32_t k0, uint32_t take,
-                                           unsigned long long* s_proc, MatchQueue& mq, Work& wk) {
-    const unsigned lane = threadIdx.x & 31u;
-    uint32_t w[2], h[2], lg[2], tt[2], ss[2], ll[2];
-    unsigned long long base[2];
-    uint4 bk[2];
 #pragma unroll
-    for (int p = 0; p < 2; ++p) {
-        const uint32_t k = 32u * p + lane;
-        bool v = k < take;
-        w[p] = kEmptyId;
-        lg[p] = 2u;
-        base[p] = 0ull;
-        tt[p] = ss[p] = ll[p] = 0u;
-        bk[p] = make_uint4(kEmptyId, kEmptyId, kEmptyId, kEmptyId);
-        if (v) {
-            const uint4* rec = reinterpret_cast<const uint4*>(d.srec + cq.item[k0 + k]);
-            const uint4 r0 = rec[0], r1 = rec[1];  // {s, l, off_s, off_l}, {t, lgs, cnt_s, key}
-            w[p] = cq.w[k0 + k];
-            ss[p] = r0.x;
-            ll[p] = r0.y;
-            base[p] = 4ull * r0.w;
-            tt[p] = r1.x;
-            lg[p] = r1.y >> 8;
-            if (!block_fits(d, 7, r0.w, lg[p])) {
-                v = false;
-                w[p] = kEmptyId;
+        for (int p = 0; p < 2; ++p) {
+            const StreamDev& d = st.at(sd[p]);
+            const uint32_t col = colours_of<MODE>(d);
+            as[p] = make_uint2(0u, 0u);
+            w[p] = 0u;
+            if (block_fits(d, 5, off[p].x, lgs[p]) && block_fits(d, 7, off[p].y, lgl[p]) &&
+                REPT_CHECK(d.ctrl, 3, pos[p], list_slots(lgs[p]))) {
+                const uint32_t* block_s = block_at(d.pool, off[p].x);
+                w[p] = block_s[list_at(lgs[p], col) + pos[p]] & id_mask(d);
+                if (col == kColNone) as[p].x = block_s[aux_at(lgs[p], col) + pos[p]];
+                if (col == kColMulti) as[p] = reinterpret_cast<const uint2*>(block_s + aux_at(lgs[p], col))[pos[p]];
+            } else {
+                v[p] = false;
+                lgl[p] = 2u;
             }
         }
-        h[p] = home_slot(w[p], lg[p]);
-        if (v) bk[p] = __ldg(reinterpret_cast<const uint4*>(d.pool + base[p]) + key_quad(h[p], true));
-    }
 #pragma unroll
-    for (int p = 0; p < 2; ++p) {
-        const uint4 b = bk[p];
-        const int at = b.x == w[p] ? 0 : b.y == w[p] ? 1 : b.z == w[p] ? 2 : b.w == w[p] ? 3 : -1;
-        uint32_t r = kEmptyId;
-        if (w[p] != kEmptyId) {
+        for (int p = 0; p < 2; ++p) {
+            const StreamDev& d = st.at(sd[p]);
+            const uint32_t col = colours_of<MODE>(d);
+            h[p] = home_slot(w[p], lgl[p]);
+            bk[p] = make_uint4(kEmptyId, kEmptyId, kEmptyId, kEmptyId);
+            if (REPT_CHECK(d.ctrl, 7, off[p].y, d.pool_quads))
+                bk[p] = __ldg(reinterpret_cast<const uint4*>(block_at(d.pool, off[p].y)) + key_quad(h[p], col));
+        }
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            const uint4 b = bk[p];
+            slot[p] = b.x == w[p] ? h[p] : b.y == w[p] ? h[p] + 1u : b.z == w[p] ? h[p] + 2u : b.w == w[p] ? h[p] + 3u : kEmptyId;
             uint32_t ns = 4u;
-            if (at >= 0)
-                r = __ldg(reinterpret_cast<const uint32_t*>(d.pool + base[p]) + eidx_word(h[p] + (uint32_t)at, lg[p], true));
-            else if (b.x != kEmptyId && b.y != kEmptyId && b.z != kEmptyId && b.w != kEmptyId)
-                r = table_find(d.pool, base[p], lg[p], w[p], ns, true);  // rare: the bucket is full
-            if (WORK) { ++wk.probes; wk.pslots += ns; }
+            if (v[p] && slot[p] == kEmptyId && b.x != kEmptyId && b.y != kEmptyId && b.z != kEmptyId && b.w != kEmptyId) {
+                const StreamDev& d = st.at(sd[p]);  // rare: the home bucket is full
+                slot[p] = table_slot(block_at(d.pool, off[p].y), lgl[p], w[p], ns, colours_of<MODE>(d));
+            }
+            if (!v[p]) slot[p] = kEmptyId;
+            if (WORK && v[p]) { ++wk.probes; wk.pslots += ns; }
         }
-        mq_push<WORK, MODE>(d, mq, w[p] != kEmptyId && r < tt[p], ss[p], ll[p], w[p], s_proc, wk);
-    }
-}
-
-// Probe the queue's full rounds of 64 (`all`: everything) and move the rest to the front.
-template <bool WORK, int MODE>
-__device__ __forceinline__ void cand_flush(const StreamDev& d, CandQueue& cq, bool all, unsigned long long* s_proc,
-                                           MatchQueue& mq, Work& wk) {
-    __syncwarp();
-    uint32_t k0 = 0;
-    for (; all ? k0 < cq.n : k0 + 64u <= cq.n; k0 += 64u)
-        cand_probe<WORK, MODE>(d, cq, k0, cq.n - k0 < 64u ? cq.n - k0 : 64u, s_proc, mq, wk);
-    if (all) {
-        cq.n = 0;
-    } else if (k0) {  // the rest (< 64 <= k0 candidates): source and destination ranges are disjoint
-        const uint32_t rest = cq.n - k0;
-        const unsigned lane = threadIdx.x & 31u;
-        for (uint32_t r = lane; r < rest; r += 32u) {
-            cq.w[r] = cq.w[k0 + r];
-            cq.item[r] = cq.item[k0 + r];
-        }
-        cq.n = rest;
-    }
-    __syncwarp();
-}
-
-// `t0`: the batch's first stream index.  A list holds the entries of earlier batches first (appends
-// and block moves keep list order), so a pass whose last entry is older than t0 holds only entries
-// older than every edge of the batch, and its entries skip the age test.
-template <bool WORK, int MODE>
-__device__ __forceinline__ void drain_warp_bin_coloured(const StreamDev& d, int cls, uint32_t grab,
-                                                        unsigned long long* s_proc, CandQueue& cq, MatchQueue& mq,
-                                                        Work& wk, uint32_t t0) {
-    static_assert(63 + kScanPass <= kCandQ, "candidate queue too small");  // flushed at 64 after a pass
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned below = (1u << lane) - 1u;
-    const unsigned long long count = d.ctrl->bin_count[cls];
-    const uint32_t first = (uint32_t)d.ctrl->bin_start[cls];
-    const WorkItem* items = d.srec + first;
-    for (;;) {
-        unsigned long long i0 = 0;
-        if (lane == 0) i0 = atomicAdd(&d.ctrl->bin_next[cls], (unsigned long long)grab);
-        i0 = __shfl_sync(0xFFFFFFFFu, i0, 0);
-        if (i0 >= count) break;
-        const unsigned long long i1 = i0 + grab < count ? i0 + grab : count;
-        for (unsigned long long i = i0; i < i1; ++i) {
-            const WorkItem x = items[i];
-            const uint32_t n_s = x.cnt_s, l = x.l, t = x.t, lgs = x.lgs & 0xFFu;
-            if (WORK && lane == 0) { wk.entries += n_s; wk.slots += n_s; }
-            if (!(block_fits(d, 5, x.off_s, lgs) && REPT_CHECK(d.ctrl, 6, n_s, list_slots(lgs) + 1u) &&
-                  block_fits(d, 7, x.off_l, x.lgs >> 8)))
-                continue;  // (uniform over the warp: x is)
-            // the list (32-byte aligned), two entries per 16-byte load; a lane past the end re-reads
-            // the last pair, and its entries are masked off by position
-            const uint4* list = reinterpret_cast<const uint4*>(d.pool + 4ull * x.off_s + (1ull << lgs));
-            const uint32_t last_pair = (n_s - 1u) >> 1;
-            const uint32_t item = first + (uint32_t)i;
-            // kColWords: the entries' colour words, two per 8-byte load beside each entry pair
-            const uint2* words = reinterpret_cast<const uint2*>(list_words(d.pool, x.off_s, lgs));
-            // the tests of one pass on loaded entries q (and words cw); FULL: inside the list (no
-            // position test); OLD: every entry older than the batch (no age test)
-            auto test = [&](const uint4 (&q)[kScanLoads], const uint2 (&cw)[kScanLoads], uint32_t j0, auto full,
-                            auto old) {
-                constexpr bool FULL = decltype(full)::value, OLD = decltype(old)::value;
 #pragma unroll
-                for (uint32_t h = 0; h < kScanLoads; ++h) {
-                    if (!FULL && j0 + 64u * h >= n_s) break;  // an empty part: uniform skip
-                    const uint32_t jj = j0 + 64u * h + 2u * lane;
-                    const bool words_mode = MODE == (int)kColWords;
-                    const uint32_t w1 = words_mode ? q[h].x : q[h].x & kIdMask;
-                    const uint32_t w2 = words_mode ? q[h].z : q[h].z & kIdMask;
-                    const bool c1 = words_mode ? words_may_match(d, l, w1, cw[h].x) : colour_may_match(d, l, w1, q[h].x >> kIdBits);
-                    const bool c2 = words_mode ? words_may_match(d, l, w2, cw[h].y) : colour_may_match(d, l, w2, q[h].z >> kIdBits);
-                    const bool a1 = (FULL || jj < n_s) & (OLD || q[h].y < t) & c1;
-                    const bool a2 = (FULL || jj + 1u < n_s) & (OLD || q[h].w < t) & c2;
-                    const unsigned m1 = __ballot_sync(0xFFFFFFFFu, a1), m2 = __ballot_sync(0xFFFFFFFFu, a2);
-                    if (m1 | m2) {  // rare (about 1/m of the entries pass): uniform
-                        if (a1) {
-                            const uint32_t k = cq.n + __popc(m1 & below);
-                            cq.w[k] = w1;
-                            cq.item[k] = item;
-                        }
-                        cq.n += __popc(m1);
-                        if (a2) {
-                            const uint32_t k = cq.n + __popc(m2 & below);
-                            cq.w[k] = w2;
-                            cq.item[k] = item;
-                        }
-                        cq.n += __popc(m2);
+        for (int p = 0; p < 2; ++p) {
+            const StreamDev& d = st.at(sd[p]);
+            const uint32_t col = colours_of<MODE>(d);
+            al[p] = make_uint2(kEmptyId, 0u);  // absent: never older
+            if (slot[p] != kEmptyId) {
+                const uint32_t* a = block_at(d.pool, off[p].y) + eidx_word(slot[p], lgl[p], col);
+                if (col == kColMulti) al[p] = *reinterpret_cast<const uint2*>(a);
+                else al[p].x = *a;
+            }
+        }
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            const StreamDev& d = st.at(sd[p]);
+            const uint32_t col = colours_of<MODE>(d);
+            bool has = al[p].x < t[p];
+            if (interleaved(col) && has) {
+                uint32_t ns;
+                as[p].x = table_find(block_at(d.pool, off[p].x), lgs[p], w[p], ns, col);
+            }
+            has = has && as[p].x < t[p];
+            if (WORK && has) ++wk.wedges;
+            uint32_t groups = 0;
+            if (col == kColMulti) {
+                groups = agreeing_groups(d, as[p].y, al[p].y);
+                has = has && groups != 0u;
+            }
+            const unsigned m = __ballot_sync(0xFFFFFFFFu, has);
+            if (m && REPT_CHECK(st.at(0u).ctrl, 13, closed + __popc(m), (unsigned long long)kMatchQ + 1ull)) {
+                if (has) {
+                    const uint32_t k = closed + __popc(m & below);
+                    mq[k] = w[p];
+                    mq[kMatchQ + k] = item[p];
+                    if (match_arrays(MODE) == 4u) {
+                        mq[2u * kMatchQ + k] = groups;
+                        mq[3u * kMatchQ + k] = as[p].y;
+                    }
+                    if (GROUP) mq[match_arrays(MODE) * kMatchQ + k] = sd[p];
+                }
+                closed += __popc(m);
+            }
+        }
+        __syncwarp();
+    }
+#pragma unroll 1
+    while (closed >= 32u || (all && closed)) {
+        const uint32_t n = min(closed, 32u);
+        count_closed<WORK, MODE>(st, mq, closed, n, wk);
+        closed -= n;
+    }
+    return closed;
+}
+
+// Probe the first 64 candidates (fewer when `all`, which also counts every closed wedge) and move the
+// rest to the front.
+template <bool WORK, int MODE, class S>
+__device__ __forceinline__ void cand_flush(const S& st, WarpQueues& q, Work& wk, bool all) {
+    const unsigned lane = threadIdx.x & 31u;
+    const uint32_t take = min(q.n, 64u), rest = q.n - take;
+    __syncwarp();
+    q.closed = cand_probe<WORK, MODE>(st, q.base, q.base + (S::kGroup ? 3u : 2u) * kCandQ, take, q.closed, all, wk);
+    if (lane < rest) {  // rest < 32
+#pragma unroll
+        for (uint32_t a = 0; a < (S::kGroup ? 3u : 2u); ++a) q.base[a * kCandQ + lane] = q.base[a * kCandQ + 64u + lane];
+    }
+    q.n = rest;
+    __syncwarp();
+}
+
+// Filter hash of a list entry: `word` holds its id and, with kColInEntry, its colour; `cw` its colour
+// word with kColWords.  Equal entries hash alike; the filter only needs that.
+template <int MODE>
+__device__ __forceinline__ uint32_t filter_hash(uint32_t word, uint32_t cw) {
+    return (MODE == (int)kColWords || MODE == kColAny ? word + cw * 0x85EBCA6Bu : word) * 0x9E3779B1u;
+}
+// The product's top bits choose the word, its low bits and some from the middle the two bits.
+__device__ __forceinline__ void filter_set(uint32_t* filter, uint32_t lg, uint32_t h) {
+    atomicOr(filter + (h >> (32u - lg)), (1u << (h & 31u)) | (1u << ((h >> 9) & 31u)));
+}
+// 1 if both bits are set, else 0.
+__device__ __forceinline__ uint32_t filter_test(const uint32_t* filter, uint32_t lg, uint32_t h) {
+    const uint32_t v = filter[h >> (32u - lg)];
+    return __funnelshift_r(v, v, h) & __funnelshift_r(v, v, h >> 9) & 1u;
+}
+// log2 of the filter words for n entries: one word (32 bits) per entry, at least 32 words.
+__device__ __forceinline__ uint32_t filter_lg(uint32_t n, uint32_t max_lg) {
+    const uint32_t lg = n <= 32u ? 5u : 32u - __clz(n - 1u);
+    return lg < max_lg ? lg : max_lg;
+}
+
+// Clear the filter; lanes `rank` of `width`.
+__device__ __forceinline__ void filter_clear(uint32_t* filter, uint32_t lg, uint32_t rank, uint32_t width) {
+    for (uint32_t i = rank; i < (1u << lg) / 4u; i += width)
+        reinterpret_cast<uint4*>(filter)[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
+// Set the n entries of the block at off_quads in the (cleared) filter; lanes `rank` of `width`.
+template <int MODE>
+__device__ __forceinline__ void filter_build(const StreamDev& d, uint32_t* filter, uint32_t lg, uint32_t off, uint32_t n,
+                                             uint32_t rank, uint32_t width) {
+    const uint32_t lgt = table_lg(n), col = colours_of<MODE>(d);
+    if (!(block_fits(d, 7, off, lgt) && REPT_CHECK(d.ctrl, 6, n, list_slots(lgt) + 1u))) return;
+    const uint32_t* block = block_at(d.pool, off);
+    const uint4* list = reinterpret_cast<const uint4*>(block + list_at(lgt, col));
+    const uint4* words = reinterpret_cast<const uint4*>(block + cw_at(lgt));
+    const uint32_t last = (n - 1u) >> 2;
+    for (uint32_t i = rank; i <= last; i += 2u * width) {
+        uint4 q[2], cw[2];
+#pragma unroll
+        for (uint32_t j = 0; j < 2u; ++j) {  // past the end: the last quad again (setting bits twice is harmless)
+            const uint32_t at = min(i + j * width, last);
+            q[j] = list[at];
+            cw[j] = make_uint4(0u, 0u, 0u, 0u);
+            if (col == kColWords) cw[j] = words[at];
+        }
+#pragma unroll
+        for (uint32_t j = 0; j < 2u; ++j) {
+            const uint32_t at = 4u * min(i + j * width, last);
+            filter_set(filter, lg, filter_hash<MODE>(q[j].x, cw[j].x));
+            if (at + 1u < n) filter_set(filter, lg, filter_hash<MODE>(q[j].y, cw[j].y));
+            if (at + 2u < n) filter_set(filter, lg, filter_hash<MODE>(q[j].z, cw[j].z));
+            if (at + 3u < n) filter_set(filter, lg, filter_hash<MODE>(q[j].w, cw[j].w));
+        }
+    }
+}
+
+// One step's passing entries join the warp's queue: bit b of a lane's m is the entry at position
+// base + 128 (b / 4) + b % 4 of edge `item`'s list of n entries (positions past its end are repeats of its
+// last quad).  One entry a lane at a time; a full round of 64 is probed.
+template <bool WORK, int MODE, class S>
+__device__ __forceinline__ void queue_step(const S& st, WarpQueues& wq, uint32_t m, uint32_t base, uint32_t n,
+                                           uint32_t item, uint32_t sid, Work& wk) {
+    while (__any_sync(0xFFFFFFFFu, m != 0u)) {
+        const uint32_t b = (uint32_t)__ffs((int)m) - 1u;  // (unused where m is 0)
+        const uint32_t at = base + ((b >> 2) << 7) + (b & 3u);
+        const bool has = m != 0u && at < n;
+        const unsigned mask = __ballot_sync(0xFFFFFFFFu, has);
+        m &= m - 1u;
+        if (!S::kGroup && !REPT_CHECK(st.at(0u).ctrl, 13, wq.n + __popc(mask), (unsigned long long)kCandQ + 1ull)) return;
+        if (has) {
+            uint32_t* to = wq.base + wq.n + __popc(mask & ((1u << (threadIdx.x & 31u)) - 1u));
+            to[0] = at;
+            to[kCandQ] = item;
+            if (S::kGroup) to[2u * kCandQ] = sid;
+        }
+        wq.n += __popc(mask);
+        if (wq.n >= 64u) cand_flush<WORK, MODE>(st, wq, wk, false);
+    }
+}
+
+// The four entries of a quad against the filter: bit i is set if entry i passes.
+template <int MODE>
+__device__ __forceinline__ uint32_t test_quad(const uint32_t* filter, uint32_t lg, const uint4& q, const uint4& cw) {
+    return filter_test(filter, lg, filter_hash<MODE>(q.x, cw.x)) | (filter_test(filter, lg, filter_hash<MODE>(q.y, cw.y)) << 1) |
+           (filter_test(filter, lg, filter_hash<MODE>(q.z, cw.z)) << 2) | (filter_test(filter, lg, filter_hash<MODE>(q.w, cw.w)) << 3);
+}
+// Scan rows j0 .. j1 - 1 (32 quads, one per lane) of a list of n entries: four rows per step.  A lane past
+// the list's end reads its last quad again.
+template <bool WORK, int MODE, class S>
+__device__ __forceinline__ void scan_rows(const S& st, uint32_t sid, const uint32_t* filter, uint32_t lg, uint32_t off_s,
+                                          uint32_t n, uint32_t item, uint32_t j0, uint32_t j1, WarpQueues& wq, Work& wk) {
+    const StreamDev& d = st.at(sid);
+    const unsigned lane = threadIdx.x & 31u;
+    const uint32_t col = colours_of<MODE>(d), lgs = table_lg(n), last = (n - 1u) >> 2;
+    const bool has_cw = MODE == (int)kColWords || (MODE == kColAny && col == kColWords);
+    const uint32_t* block = block_at(d.pool, off_s);
+    const uint4* list = reinterpret_cast<const uint4*>(block + list_at(lgs, col));
+    const uint4* words = reinterpret_cast<const uint4*>(block + cw_at(lgs));
+#pragma unroll 1
+    for (uint32_t j = j0; j < j1; j += 4u) {
+        uint4 q[4], cw[4];
+#pragma unroll
+        for (uint32_t h = 0; h < 4u; ++h) {
+            cw[h] = make_uint4(0u, 0u, 0u, 0u);
+            if (h == 0u || j + h < j1) {  // (uniform)
+                const uint32_t at = min(32u * (j + h) + lane, last);
+                q[h] = list[at];
+                if (has_cw) cw[h] = words[at];
+            }
+        }
+        uint32_t m = 0;
+#pragma unroll
+        for (uint32_t h = 0; h < 4u; ++h)
+            if (h == 0u || j + h < j1) m |= test_quad<MODE>(filter, lg, q[h], cw[h]) << (4u * h);
+        queue_step<WORK, MODE>(st, wq, m, 4u * (32u * j + lane), n, item, sid, wk);
+    }
+}
+// Rows of a list of n entries.
+__device__ __forceinline__ uint32_t list_rows(uint32_t n) { return (n + 127u) >> 7; }
+
+// Shorter lists, one per lane (n entries of the block at off_s, edge e; n == 0: none): their quads are laid
+// end to end and dealt to the lanes, two per lane and step, so that no lane idles at a list's end.
+template <bool WORK, int MODE, class S>
+__device__ __forceinline__ void scan_short(const S& st, uint32_t sid, const uint32_t* filter, uint32_t lg, uint32_t off_s,
+                                           uint32_t n, uint32_t e, WarpQueues& wq, Work& wk) {
+    const StreamDev& d = st.at(sid);
+    const unsigned lane = threadIdx.x & 31u;
+    const uint32_t col = colours_of<MODE>(d), lgs = table_lg(n);
+    const bool has_cw = MODE == (int)kColWords || (MODE == kColAny && col == kColWords);
+    const uint32_t list_off = off_s + (list_at(lgs, col) >> 3);  // in 32-byte units (n > 4: a whole number)
+    const uint32_t quads = (n + 3u) >> 2;
+    uint32_t incl = quads;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= (uint32_t)o) incl += y;
+    }
+    const uint32_t total = __shfl_sync(0xFFFFFFFFu, incl, 31), excl = incl - quads;
+#pragma unroll 1
+    for (uint32_t f = 0; f < total; f += 64u) {
+        uint4 q[2], cw[2];
+        uint32_t own[2], pos[2], m[2];
+#pragma unroll
+        for (uint32_t p = 0; p < 2u; ++p) {
+            const uint32_t at = min(f + 32u * p + lane, total - 1u);
+            uint32_t o = 0;  // the lane whose quads cover position `at`: the first with incl > at
+#pragma unroll
+            for (uint32_t step = 16u; step; step >>= 1)
+                if (__shfl_sync(0xFFFFFFFFu, incl, o + step - 1u) <= at) o += step;
+            own[p] = o;
+            pos[p] = at - __shfl_sync(0xFFFFFFFFu, excl, o);
+            q[p] = reinterpret_cast<const uint4*>(block_at(d.pool, __shfl_sync(0xFFFFFFFFu, list_off, o)))[pos[p]];
+            cw[p] = make_uint4(0u, 0u, 0u, 0u);
+            if (has_cw) {
+                const uint32_t oo = __shfl_sync(0xFFFFFFFFu, off_s, o), on = __shfl_sync(0xFFFFFFFFu, n, o);
+                cw[p] = reinterpret_cast<const uint4*>(block_at(d.pool, oo) + cw_at(table_lg(on)))[pos[p]];
+            }
+        }
+#pragma unroll
+        for (uint32_t p = 0; p < 2u; ++p) {
+            m[p] = test_quad<MODE>(filter, lg, q[p], cw[p]);
+            if (f + 32u * p + lane >= total) m[p] = 0u;
+        }
+        if (__any_sync(0xFFFFFFFFu, (m[0] | m[1]) != 0u)) {
+#pragma unroll 1
+            for (uint32_t p = 0; p < 2u; ++p) {
+                const uint32_t mp = p ? m[1] : m[0], o = p ? own[1] : own[0], at = 4u * (p ? pos[1] : pos[0]);
+                const uint32_t on = __shfl_sync(0xFFFFFFFFu, n, o), oe = __shfl_sync(0xFFFFFFFFu, e, o);
+                queue_step<WORK, MODE>(st, wq, mp, at, on, oe, sid, wk);
+            }
+        }
+    }
+}
+
+// A block unit as its first thread claims it: the edges order[first .. first + count) of stream sid and
+// the larger endpoint's block (n entries at off).
+struct UnitClaim {
+    uint32_t ok, sid, first, count, off, n;
+};
+__device__ __forceinline__ UnitClaim claimed_unit(const StreamDev& d, uint32_t sid, unsigned long long at) {
+    const Unit u = d.units[at];
+    const WorkItem x = d.rec[d.order[u.first]];
+    d.meta[x.l].w = 0u;  // the record's cursor has served
+    return UnitClaim{1u, sid, u.first, min(u.count, kUnitItems), x.off_l, x.cnt_l};
+}
+
+// Work through the block units: the block builds the larger endpoint's filter while its first warp cuts
+// the lists of the unit's edges into pieces of at most kPieceRows rows, which the warps then take in turn,
+// so that they finish together.  `claim` (first thread only) yields the next unit, while the other warps
+// scan.
+constexpr uint32_t kPieceRows = 8u;  // 1,024 entries
+template <bool WORK, int MODE, class S, class Claim>
+__device__ __forceinline__ void run_block_units(const S& st, uint32_t* filter, uint4* items, WarpQueues& wq, Work& wk,
+                                                Claim&& claim) {
+    __shared__ UnitClaim s_claim;
+    __shared__ uint32_t s_taken;  // pieces taken
+    const unsigned lane = threadIdx.x & 31u;
+    if (threadIdx.x == 0) s_claim = claim();
+    __syncthreads();
+    for (;;) {
+        const UnitClaim u = s_claim;
+        if (!u.ok) break;
+        const StreamDev& d = st.at(u.sid);
+        const uint32_t lg = filter_lg(2u * u.n, kFilterLg);
+        filter_clear(filter, lg, threadIdx.x, blockDim.x);
+        if (threadIdx.x == 0) s_taken = 0u;
+        __syncthreads();
+        if (threadIdx.x < 32u) {  // items[i] = {block offset, entries, edge, pieces of lists 0 .. i}
+            uint32_t carry = 0;
+#pragma unroll
+            for (uint32_t h = 0; h < 2u; ++h) {
+                const uint32_t i = 32u * h + lane;
+                uint4 x = make_uint4(0u, 0u, 0u, 0u);
+                if (i < u.count) {
+                    const uint32_t e = d.order[u.first + i];
+                    const WorkItem r = d.rec[e];
+                    const uint32_t lgs = table_lg(r.cnt_s);
+                    x = make_uint4(r.off_s, r.cnt_s, e, 0u);
+                    if (!(block_fits(d, 5, x.x, lgs) && REPT_CHECK(d.ctrl, 6, x.y, list_slots(lgs) + 1u))) x.y = 0u;
+                    if (WORK && x.y) {
+                        wk.entries += x.y;
+                        wk.slots += x.y;
+                        atomicAdd(&d.ctrl->class_items[bin_of_cnt(x.y)], 1ull);
                     }
                 }
-                if (cq.n >= 64u) cand_flush<WORK, MODE>(d, cq, false, s_proc, mq, wk);
-            };
-            auto pass = [&](uint32_t j0, auto full) {
-                constexpr bool FULL = decltype(full)::value;
-                uint4 q[kScanLoads];
-                uint2 cw[kScanLoads];
+                uint32_t incl = (list_rows(x.y) + kPieceRows - 1u) / kPieceRows;
 #pragma unroll
-                for (uint32_t h = 0; h < kScanLoads; ++h) {
-                    const uint32_t pr = (j0 >> 1) + 32u * h + lane;
-                    const uint32_t at = FULL || pr < last_pair ? pr : last_pair;
-                    q[h] = list[at];
-                    cw[h] = make_uint2(0u, 0u);
-                    if (MODE == (int)kColWords) cw[h] = words[at];
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+                    if (lane >= (uint32_t)o) incl += y;
                 }
-                if (FULL && __shfl_sync(0xFFFFFFFFu, q[kScanLoads - 1].w, 31) < t0)
-                    test(q, cw, j0, full, std::true_type{});
-                else
-                    test(q, cw, j0, full, std::false_type{});
-            };
-            uint32_t j0 = 0;
-            if (kScanFull)
-                for (; j0 + kScanPass <= n_s; j0 += kScanPass) pass(j0, std::true_type{});
-            for (; j0 < n_s; j0 += kScanPass) pass(j0, std::false_type{});
+                x.w = incl + carry;
+                carry += __shfl_sync(0xFFFFFFFFu, incl, 31);
+                items[i] = x;
+            }
         }
+        filter_build<MODE>(d, filter, lg, u.off, u.n, threadIdx.x, blockDim.x);
+        __syncthreads();
+        if (threadIdx.x == 0) s_claim = claim();
+        __syncwarp();
+        const uint32_t total = items[kUnitItems - 1u].w;
+        for (;;) {
+            uint32_t i = 0;
+            if (lane == 0) i = atomicAdd(&s_taken, 1u);
+            i = __shfl_sync(0xFFFFFFFFu, i, 0);
+            if (i >= total) break;
+            // the list that piece i belongs to: as many lists end before it
+            const uint32_t at = __popc(__ballot_sync(0xFFFFFFFFu, items[lane].w <= i)) +
+                                __popc(__ballot_sync(0xFFFFFFFFu, items[32u + lane].w <= i));
+            const uint4 x = items[at];
+            const uint32_t rows = list_rows(x.y), pieces = (rows + kPieceRows - 1u) / kPieceRows;
+            const uint32_t j0 = (i + pieces - x.w) * kPieceRows;
+            scan_rows<WORK, MODE>(st, u.sid, filter, lg, x.x, x.y, x.z, j0, min(j0 + kPieceRows, rows), wq, wk);
+        }
+        __syncthreads();
     }
 }
 
-template <int TILE, bool WORK, int MODE>
-__device__ __forceinline__ void drain_tile_bin(const StreamDev& d, int cls, unsigned long long* s_proc,
-                                               MatchQueue& mq, Work& wk) {
-    constexpr uint32_t kPerWarp = 32 / TILE, kRounds = 4, kGrab = kPerWarp * kRounds;
+// Lists of at most kShortList entries are scanned end to end in warp units.
+constexpr uint32_t kShortList = 128u;
+
+// One warp unit: the warp builds l's filter in its share of the shared memory and scans the unit's lists.
+template <bool WORK, int MODE, class S>
+__device__ __forceinline__ void run_warp_unit(const S& st, uint32_t sid, Unit u, uint32_t* filter, WarpQueues& wq,
+                                              Work& wk) {
+    const StreamDev& d = st.at(sid);
     const unsigned lane = threadIdx.x & 31u;
-    const unsigned long long count = d.ctrl->bin_count[cls];
-    const WorkItem* items = d.srec + d.ctrl->bin_start[cls];
-    for (;;) {
-        unsigned long long base = 0;
-        if (lane == 0) base = atomicAdd(&d.ctrl->bin_next[cls], (unsigned long long)kGrab);
-        base = __shfl_sync(0xFFFFFFFFu, base, 0);
-        if (base >= count) break;
+    WorkItem x{};
+    uint32_t e = 0;
+    if (lane < min(u.count, kWarpUnitItems)) {
+        e = d.order[u.first + lane];
+        x = d.rec[e];
+    }
+    const uint32_t off_l = __shfl_sync(0xFFFFFFFFu, x.off_l, 0), n_l = __shfl_sync(0xFFFFFFFFu, x.cnt_l, 0);
+    const uint32_t lg = filter_lg(n_l, kWarpFilterLg);
+    filter_clear(filter, lg, lane, 32u);
+    if (lane == 0) d.meta[x.l].w = 0u;  // the record's cursor has served
+    __syncwarp();
+    filter_build<MODE>(d, filter, lg, off_l, n_l, lane, 32u);
+    __syncwarp();
+    // lists of more than a row one by one, the others end to end
+    uint32_t n = x.cnt_s;
+    if (n && !(block_fits(d, 5, x.off_s, table_lg(n)) && REPT_CHECK(d.ctrl, 6, n, list_slots(table_lg(n)) + 1u))) n = 0u;
+    if (WORK && n) {
+        wk.entries += n;
+        wk.slots += n;
+        atomicAdd(&d.ctrl->class_items[bin_of_cnt(n)], 1ull);
+    }
+    for (unsigned lng = __ballot_sync(0xFFFFFFFFu, n > kShortList); lng; lng &= lng - 1u) {
+        const int i = __ffs((int)lng) - 1;
+        const uint32_t oi = __shfl_sync(0xFFFFFFFFu, x.off_s, i), ni = __shfl_sync(0xFFFFFFFFu, n, i),
+                       ei = __shfl_sync(0xFFFFFFFFu, e, i);
+        scan_rows<WORK, MODE>(st, sid, filter, lg, oi, ni, ei, 0u, list_rows(ni), wq, wk);
+    }
+    scan_short<WORK, MODE>(st, sid, filter, lg, x.off_s, n > kShortList ? 0u : n, e, wq, wk);
+    __syncwarp();  // the filter is rebuilt by the next unit
+}
+
+// The small edges among edges e0 .. e1 - 1 of the batch: 32 edges at a time, their lists'
+// entries laid end to end and dealt to the lanes, two per lane and round.  With one group's stored
+// colours an entry passes if its colour may agree with the larger endpoint's edge (one hash); else every
+// entry passes.
+template <bool WORK, int MODE, class S>
+__device__ __forceinline__ void run_small_chunk(const S& st, uint32_t sid, uint32_t e0, uint32_t e1, WarpQueues& wq,
+                                                Work& wk) {
+    const StreamDev& d = st.at(sid);
+    const unsigned lane = threadIdx.x & 31u;
+    const uint32_t col = colours_of<MODE>(d), mask = id_mask(d);
 #pragma unroll 1
-        for (uint32_t r = 0; r < kRounds; ++r) {
-            const unsigned long long i = base + r * kPerWarp + lane / TILE;
-            const bool valid = i < count;
-            WorkItem x{};
-            if (valid) x = items[i];
-            intersect_tile<TILE, WORK, MODE>(d, x, valid, s_proc, mq, wk);
+    for (uint32_t eb = e0; eb < e1; eb += 32u) {
+        const uint32_t e = eb + lane;
+        uint32_t cnt = 0, off_s = 0, l = 0;
+        if (e < e1 && d.mark[e] == kSmallEdge) {
+            const WorkItem x = d.rec[e];
+            cnt = x.cnt_s;
+            off_s = x.off_s;
+            l = x.l;
+            if (!(block_fits(d, 5, off_s, table_lg(cnt)) && REPT_CHECK(d.ctrl, 4, cnt, kSmallBatchMax + 1u))) cnt = 0u;
+            if (WORK && cnt) {
+                wk.entries += cnt;
+                wk.slots += cnt;
+                atomicAdd(&d.ctrl->class_items[bin_of_cnt(cnt)], 1ull);
+            }
+        }
+        uint32_t incl = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= (uint32_t)o) incl += y;
+        }
+        const uint32_t total = __shfl_sync(0xFFFFFFFFu, incl, 31), excl = incl - cnt;
+#pragma unroll 1
+        for (uint32_t f = 0; f < total; f += 64u) {
+            uint32_t word[2], cw[2], own[2], ol[2], pos[2];
+            bool v[2];
+#pragma unroll
+            for (uint32_t p = 0; p < 2u; ++p) {
+                const uint32_t at = f + 32u * p + lane;
+                v[p] = at < total;
+                uint32_t o = 0;  // the lane whose entries cover position `at`: the first with incl > at
+#pragma unroll
+                for (uint32_t step = 16u; step; step >>= 1)
+                    if (__shfl_sync(0xFFFFFFFFu, incl, o + step - 1u) <= at) o += step;
+                own[p] = o;
+                pos[p] = at - __shfl_sync(0xFFFFFFFFu, excl, o);
+                const uint32_t oo = __shfl_sync(0xFFFFFFFFu, off_s, o), oc = __shfl_sync(0xFFFFFFFFu, cnt, o);
+                ol[p] = __shfl_sync(0xFFFFFFFFu, l, o);
+                word[p] = cw[p] = 0u;
+                if (v[p] && interleaved(col)) {
+                    const uint32_t lgs = table_lg(oc);
+                    const uint32_t* block = block_at(d.pool, oo);
+                    word[p] = block[list_at(lgs, col) + pos[p]];
+                    if (col == kColWords) cw[p] = block[cw_at(lgs) + pos[p]];
+                }
+            }
+            if (interleaved(col)) {
+#pragma unroll
+                for (uint32_t p = 0; p < 2u; ++p)
+                    v[p] = v[p] & colour_may_match(d, ol[p], word[p] & mask, col == kColWords ? cw[p] : word[p] >> kIdBits);
+            }
+#pragma unroll 1
+            for (uint32_t p = 0; p < 2u; ++p)
+                queue_step<WORK, MODE>(st, wq, (p ? v[1] : v[0]) ? 1u : 0u, p ? pos[1] : pos[0], kEmptyId,
+                                       eb + (p ? own[1] : own[0]), sid, wk);
         }
     }
 }
 
-// Warp classes: a warp claims `grab` consecutive items per atomic on the class cursor (one cursor is
-// shared by every warp of the grid, so claiming one item at a time serialises on it).
-template <bool WORK, int MODE>
-__device__ __forceinline__ void drain_warp_bin(const StreamDev& d, int cls, uint32_t grab, unsigned long long* s_proc,
-                                               uint32_t* queue, MatchQueue& mq, Work& wk) {
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned long long count = d.ctrl->bin_count[cls];
-    const WorkItem* items = d.srec + d.ctrl->bin_start[cls];
-    for (;;) {
-        unsigned long long i0 = 0;
-        if (lane == 0) i0 = atomicAdd(&d.ctrl->bin_next[cls], (unsigned long long)grab);
-        i0 = __shfl_sync(0xFFFFFFFFu, i0, 0);
-        if (i0 >= count) break;
-        const unsigned long long i1 = i0 + grab < count ? i0 + grab : count;
-        for (unsigned long long i = i0; i < i1; ++i) {
-            const WorkItem x = items[i];
-            intersect_warp<WORK, MODE>(d, x, queue, wk, [&](bool has, uint32_t w) {
-                mq_push<WORK, MODE>(d, mq, has, x.s, x.l, w, s_proc, wk);
-            });
-        }
-    }
-}
-
-// UpdateTriangleCNT for every edge of the batch.  The edges were sorted into work classes by
-// k_insert; warps claim work dynamically, largest class first.  Dynamic shared memory: c uint64
-// counters (tau^(i) of this block).  WORK = true also tallies the table reads.
+// UpdateTriangleCNT for every edge of the batch: block units, then warp units and small edges (odd warps
+// the other way round, so that the two kinds overlap in small batches), each claimed dynamically.
+// Dynamic shared memory: ix_words(MODE, false) words, then 2 c words of counters (tau^(i) of this block).
+// WORK = true also tallies the table reads.
 template <bool WORK, int MODE>
 __device__ __forceinline__ void k_intersect_body(const StreamDev& d, const BatchDev& b) {
-    extern __shared__ unsigned long long s_proc[];
-    // the scan-first warp path (candidate queue): streams that store colours
-    constexpr bool CAND = MODE == (int)kColInEntry || MODE == (int)kColWords;
-    __shared__ uint32_t s_queue[CAND ? 1 : 256 / 32][kQueue];  // intersect_warp's key queue
-    __shared__ uint32_t s_cand[CAND ? 256 / 32 : 1][2][kCandQ];
-    __shared__ uint32_t s_match[256 / 32][3][kMatchQ];
-    for (uint32_t i = threadIdx.x; i < d.c; i += blockDim.x) s_proc[i] = 0ull;
-    __syncthreads();
+    extern __shared__ __align__(16) uint32_t ix_smem[];
+    uint32_t* filter = ix_smem;
+    uint4* items = reinterpret_cast<uint4*>(filter + kFilterWords);
+    uint32_t* half = ix_smem + ix_words(MODE, false);
+    for (uint32_t i = threadIdx.x; i < 2u * d.c; i += blockDim.x) half[i] = 0u;
     const unsigned lane = threadIdx.x & 31u;
     const unsigned wid = threadIdx.x >> 5;
-    uint32_t* queue = s_queue[CAND ? 0 : wid];
-    MatchQueue mq{s_match[wid][0], s_match[wid][1], s_match[wid][2], 0u};
-    CandQueue cq{s_cand[CAND ? wid : 0][0], s_cand[CAND ? wid : 0][1], 0u};
+    WarpQueues wq{filter + kFilterWords + 4u * kUnitItems + wid * queue_words(MODE, false), 0u, 0u};
+    const OneStream st{d, half};
     Work wk;
-    if (d.ctrl->status == 0u) {
-        // WORK: per class, the probes issued and the warp-cycles spent (clock64 around each drain)
-        long long t0 = WORK ? clock64() : 0;
-        unsigned long long p0 = wk.probes;
+    Ctrl* ct = d.ctrl;
+    __syncthreads();
+    if (ct->status == 0u) {
+        // WORK: warp-cycles of block units, warp units and small edges, kept under classes 5, 4 and 3
+        long long c0 = WORK ? clock64() : 0;
         auto mark = [&](int cls) {
-            if (WORK) {
-                const long long t1 = clock64();
-                const unsigned long long p1 = wk.probes;
-                unsigned long long pr = p1 - p0;
-                for (int o = 16; o > 0; o >>= 1) pr += __shfl_down_sync(0xFFFFFFFFu, pr, o);
-                if (lane == 0) {
-                    atomicAdd(&d.ctrl->class_cycles[cls], (unsigned long long)(t1 - t0));
-                    atomicAdd(&d.ctrl->class_probes[cls], pr);
-                }
-                t0 = t1;
-                p0 = p1;
+            if (WORK && lane == 0) {
+                const long long c1 = clock64();
+                atomicAdd(&ct->class_cycles[cls], (unsigned long long)(c1 - c0));
+                c0 = c1;
             }
         };
-        if constexpr (CAND) {
-            drain_warp_bin_coloured<WORK, MODE>(d, 5, kScanGrabHub, s_proc, cq, mq, wk, (uint32_t)b.t0);
-            mark(5);
-            drain_warp_bin_coloured<WORK, MODE>(d, 4, kScanGrabMid, s_proc, cq, mq, wk, (uint32_t)b.t0);
-            if (cq.n) cand_flush<WORK, MODE>(d, cq, true, s_proc, mq, wk);
-            mark(4);
-        } else {
-            drain_warp_bin<WORK, MODE>(d, 5, kGrabHub, s_proc, queue, mq, wk);
-            mark(5);
-            drain_warp_bin<WORK, MODE>(d, 4, kGrabMid, s_proc, queue, mq, wk);
-            mark(4);
+        int kind = kBinBig;
+        run_block_units<WORK, MODE>(st, filter, items, wq, wk, [&]() -> UnitClaim {
+            for (; kind >= kBinBlock; --kind) {
+                if (ct->bin_count[kind] == 0ull) continue;
+                const unsigned long long i = atomicAdd(&ct->bin_next[kind], 1ull);
+                if (i < ct->bin_count[kind]) return claimed_unit(d, 0u, kind == kBinBig ? i : d.unit_cap + i);
+            }
+            return UnitClaim{0u, 0u, 0u, 0u, 0u, 0u};
+        });
+        mark(5);
+#pragma unroll 1
+        for (uint32_t part = 0; part < 2u; ++part) {
+            const int bin = (part ^ wid) & 1u ? kBinSmall : kBinWarp;
+            const unsigned long long count = ct->bin_count[bin];
+            for (;;) {
+                unsigned long long i = 0;
+                if (lane == 0) i = atomicAdd(&ct->bin_next[bin], 1ull);
+                i = __shfl_sync(0xFFFFFFFFu, i, 0);
+                if (i >= count) break;
+                if (bin == kBinWarp)
+                    run_warp_unit<WORK, MODE>(st, 0u, d.units[d.unit_cap - 1ull - i], filter + (wid << kWarpFilterLg), wq, wk);
+                else
+                    run_small_chunk<WORK, MODE>(st, 0u, (uint32_t)i * b.chunk, (uint32_t)min((i + 1ull) * b.chunk, b.n), wq, wk);
+            }
+            mark(bin == kBinWarp ? 4 : 3);
         }
-        drain_tile_bin<32, WORK, MODE>(d, 3, s_proc, mq, wk);
-        mark(3);
-        drain_tile_bin<16, WORK, MODE>(d, 2, s_proc, mq, wk);
-        mark(2);
-        drain_tile_bin<8, WORK, MODE>(d, 1, s_proc, mq, wk);
-        mark(1);
-        drain_tile_bin<4, WORK, MODE>(d, 0, s_proc, mq, wk);
-        mark(0);
-        if (mq.n) mq_flush<WORK, MODE>(d, mq, mq.n, s_proc, wk);
-        if (WORK && blockIdx.x == 0 && threadIdx.x < kBins)
-            d.ctrl->class_items[threadIdx.x] += d.ctrl->bin_count[threadIdx.x];
+        cand_flush<WORK, MODE>(st, wq, wk, true);
     }
     if (WORK) {
         for (int o = 16; o > 0; o >>= 1) {
@@ -1195,18 +1516,19 @@ __device__ __forceinline__ void k_intersect_body(const StreamDev& d, const Batch
         }
     }
     __syncthreads();
-    for (uint32_t i = threadIdx.x; i < d.c; i += blockDim.x)
-        if (s_proc[i]) atomicAdd(&d.proc[i], s_proc[i]);
+    for (uint32_t i = threadIdx.x; i < d.c; i += blockDim.x) {
+        const unsigned long long n = ((unsigned long long)half[2u * i + 1u] << 32) | half[2u * i];
+        if (n) atomicAdd(&d.proc[i], n);
+    }
 }
 
 // ---------------------------------------------------------------------------------------------
-// Intersection for a group of streams with one grid: every warp may work on any stream.  The
-// per-class work lists of the k streams are concatenated (k_group_prefix writes, per class, the
-// prefix of the streams' item counts); warps claim ranges of the concatenation with one cursor per
-// class and find each item's stream from the prefix.  Closed wedges carry their stream in the
-// match queue and tau^(i) goes straight to global memory.
+// Intersection for a group of streams with one grid: every block and warp may work on any stream.  The
+// streams' lists of each kind of work are concatenated (k_group_prefix writes, per kind, the prefix of
+// the streams' counts); claims come from one cursor per kind, and each finds its stream from the prefix.
+// Candidates and closed wedges carry their stream and tau^(i) goes straight to global memory.
 
-// Per class c: pref[c * (k + 1) + i] = sum of the item counts of streams < i; cursors reset.  One
+// Per kind c: pref[c * (k + 1) + i] = sum of the counts of streams < i; cursors reset.  One
 // block of any multiple of 32 threads up to 1024.
 __device__ __forceinline__ void group_prefix_body(const StreamDev* __restrict__ ds, uint32_t k,
                                                   unsigned long long* __restrict__ pref,
@@ -1257,64 +1579,7 @@ __global__ void __launch_bounds__(1024) k_group_prefix(const StreamDev* __restri
     group_prefix_body(ds, k, pref, cursor);
 }
 
-struct GroupQueue {
-    uint32_t* sid;
-    uint32_t* s;
-    uint32_t* l;
-    uint32_t* w;
-    uint32_t n;
-};
-
-__device__ __forceinline__ void gq_flush(const StreamDev* __restrict__ ds, GroupQueue& q, uint32_t take) {
-    const unsigned lane = threadIdx.x & 31u;
-    if (lane < take) {
-        const uint32_t i = q.n - take + lane;
-        const StreamDev& d = ds[q.sid[i]];
-        const uint32_t s = q.s[i], l = q.l[i], w = q.w[i];
-        uint32_t found = 0;
-        for (uint32_t k = d.kbeg; k < d.kend; ++k) {
-            const uint64_t sk = group_seed(d.seed, k);
-            const uint32_t js = colour_of(s, w, sk, d.fm);
-            uint32_t i;
-            if (processor_of(d, k, js, i) && colour_of(l, w, sk, d.fm) == js) {
-                ++found;
-                atomicAdd(&d.proc[i], 1ull);
-            }
-        }
-        if (found) {
-            atomicAdd(&d.local[w], (unsigned long long)found);
-            atomicAdd(&d.local[s], (unsigned long long)found);
-            atomicAdd(&d.local[l], (unsigned long long)found);
-        }
-    }
-    q.n -= take;
-    __syncwarp();
-}
-
-__device__ __forceinline__ void gq_push(const StreamDev* __restrict__ ds, GroupQueue& q, bool has, uint32_t sid,
-                                        uint32_t s, uint32_t l, uint32_t w) {
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned mask = __ballot_sync(0xFFFFFFFFu, has);
-    if (has) {
-        const uint32_t i = q.n + __popc(mask & ((1u << lane) - 1u));
-        q.sid[i] = sid;
-        q.s[i] = s;
-        q.l[i] = l;
-        q.w[i] = w;
-    }
-    q.n += __popc(mask);
-    __syncwarp();
-    if (q.n >= 32u) gq_flush(ds, q, 32u);
-}
-
-// Stream of item `i` of class c: the last stream whose prefix is <= i, searched from `from`.
-__device__ __forceinline__ uint32_t group_stream_of(const unsigned long long* __restrict__ pc, uint32_t k,
-                                                    unsigned long long i, uint32_t from) {
-    uint32_t sidx = from;
-    while (sidx + 1 < k && pc[sidx + 1] <= i) ++sidx;
-    return sidx;
-}
-
+// Stream of item `i`: the last stream whose prefix is <= i.
 __device__ __forceinline__ uint32_t group_stream_search(const unsigned long long* __restrict__ pc, uint32_t k,
                                                         unsigned long long i) {
     uint32_t lo = 0, hi = k - 1;  // pc[0] = 0 <= i
@@ -1325,239 +1590,60 @@ __device__ __forceinline__ uint32_t group_stream_search(const unsigned long long
     return lo;
 }
 
-__device__ __forceinline__ WorkItem group_item(const StreamDev& d, int cls, unsigned long long local) {
-    return d.srec[d.ctrl->bin_start[cls] + local];
-}
-
-template <int TILE>
-__device__ __forceinline__ void group_drain_tiles(const StreamDev* __restrict__ ds, uint32_t k, int cls,
-                                                  const unsigned long long* __restrict__ pref,
-                                                  unsigned long long* __restrict__ cursor, GroupQueue& q) {
-    constexpr uint32_t kPerWarp = 32 / TILE, kRounds = 4, kGrab = kPerWarp * kRounds;
-    const unsigned lane = threadIdx.x & 31u, j = lane & (TILE - 1);
-    const unsigned long long* pc = pref + cls * (k + 1);
-    const unsigned long long total = pc[k];
-    for (;;) {
-        unsigned long long base = 0;
-        if (lane == 0) base = atomicAdd(&cursor[cls], (unsigned long long)kGrab);
-        base = __shfl_sync(0xFFFFFFFFu, base, 0);
-        if (base >= total) break;
-        const uint32_t s0 = group_stream_search(pc, k, base);
-#pragma unroll 1
-        for (uint32_t r = 0; r < kRounds; ++r) {
-            const unsigned long long i = base + r * kPerWarp + lane / TILE;
-            const bool valid = i < total;
-            bool has = false;
-            uint32_t sid = 0, w = 0;
-            WorkItem x{};
-            if (valid) {
-                sid = group_stream_of(pc, k, i, s0);
-                const StreamDev& d = ds[sid];
-                x = group_item(d, cls, i - pc[sid]);
-                if (j < x.cnt_s) {
-                    const unsigned long long at = 4ull * x.off_s + (1ull << (x.lgs & 0xFFu)) + j;
-                    const bool fits = REPT_CHECK(d.ctrl, 3, at, 4ull * d.pool_quads) &&
-                                      block_fits(d, 4, x.off_l, x.lgs >> 8);
-                    const uint2 es = fits ? d.pool[at] : make_uint2(kEmptyId, kEmptyId);
-                    const uint32_t ws = es.x & id_mask(d);
-                    if (es.y < x.t && (d.colours != kColInEntry || wedge_may_count(d, x.l, ws, es.x >> kIdBits))) {
-                        uint32_t nslots = 0;
-                        has = table_find(d.pool, 4ull * x.off_l, x.lgs >> 8, ws, nslots, tables_interleaved(d)) < x.t;
-                        w = ws;
-                    }
-                }
-            }
-            gq_push(ds, q, has, sid, x.s, x.l, w);
-        }
-    }
-}
-
-// Warp classes of a group: the scan-first scheme of drain_warp_bin_coloured over all streams of the
-// group, a candidate also naming its stream.  A stream without colours in its entries passes every
-// entry older than the edge to the probes.
-struct GroupCand {
-    uint32_t* w;     // [kCandQ] candidate neighbour w
-    uint32_t* item;  // [kCandQ] its work item, an index into its stream's srec
-    uint32_t* sid;   // [kCandQ] its stream
-    uint32_t n;      // warp-uniform
-};
-
-__device__ __forceinline__ void gcand_probe(const StreamDev* __restrict__ ds, const GroupCand& cq, uint32_t k0,
-                                            uint32_t take, GroupQueue& q) {
-    const unsigned lane = threadIdx.x & 31u;
-    uint32_t w[2], h[2], lg[2], tt[2], ss[2], ll[2], sd[2];
-    const uint2* pool[2];
-    bool inter[2];
-    unsigned long long base[2];
-    uint4 bk[2];
-#pragma unroll
-    for (int p = 0; p < 2; ++p) {
-        const uint32_t k = 32u * p + lane;
-        bool v = k < take;
-        w[p] = kEmptyId;
-        lg[p] = 2u;
-        base[p] = 0ull;
-        tt[p] = ss[p] = ll[p] = sd[p] = 0u;
-        pool[p] = nullptr;
-        inter[p] = true;
-        bk[p] = make_uint4(kEmptyId, kEmptyId, kEmptyId, kEmptyId);
-        if (v) {
-            sd[p] = cq.sid[k0 + k];
-            const StreamDev& d = ds[sd[p]];
-            const uint4* rec = reinterpret_cast<const uint4*>(d.srec + cq.item[k0 + k]);
-            const uint4 r0 = rec[0], r1 = rec[1];  // {s, l, off_s, off_l}, {t, lgs, cnt_s, key}
-            w[p] = cq.w[k0 + k];
-            ss[p] = r0.x;
-            ll[p] = r0.y;
-            base[p] = 4ull * r0.w;
-            tt[p] = r1.x;
-            lg[p] = r1.y >> 8;
-            pool[p] = d.pool;
-            inter[p] = tables_interleaved(d);
-            if (!block_fits(d, 7, r0.w, lg[p])) {
-                v = false;
-                w[p] = kEmptyId;
-            }
-        }
-        h[p] = home_slot(w[p], lg[p]);
-        if (v) bk[p] = __ldg(reinterpret_cast<const uint4*>(pool[p] + base[p]) + key_quad(h[p], inter[p]));
-    }
-#pragma unroll
-    for (int p = 0; p < 2; ++p) {
-        const uint4 b = bk[p];
-        const int at = b.x == w[p] ? 0 : b.y == w[p] ? 1 : b.z == w[p] ? 2 : b.w == w[p] ? 3 : -1;
-        uint32_t r = kEmptyId;
-        if (w[p] != kEmptyId) {
-            uint32_t ns = 4u;
-            if (at >= 0)
-                r = __ldg(reinterpret_cast<const uint32_t*>(pool[p] + base[p]) +
-                          eidx_word(h[p] + (uint32_t)at, lg[p], inter[p]));
-            else if (b.x != kEmptyId && b.y != kEmptyId && b.z != kEmptyId && b.w != kEmptyId)
-                r = table_find(pool[p], base[p], lg[p], w[p], ns, inter[p]);  // rare: the bucket is full
-        }
-        gq_push(ds, q, w[p] != kEmptyId && r < tt[p], sd[p], ss[p], ll[p], w[p]);
-    }
-}
-
-__device__ __forceinline__ void gcand_flush(const StreamDev* __restrict__ ds, GroupCand& cq, bool all, GroupQueue& q) {
-    __syncwarp();
-    uint32_t k0 = 0;
-    for (; all ? k0 < cq.n : k0 + 64u <= cq.n; k0 += 64u) gcand_probe(ds, cq, k0, cq.n - k0 < 64u ? cq.n - k0 : 64u, q);
-    if (all) {
-        cq.n = 0;
-    } else if (k0) {  // the rest (< 64 <= k0 candidates): source and destination ranges are disjoint
-        const uint32_t rest = cq.n - k0;
-        const unsigned lane = threadIdx.x & 31u;
-        for (uint32_t r = lane; r < rest; r += 32u) {
-            cq.w[r] = cq.w[k0 + r];
-            cq.item[r] = cq.item[k0 + r];
-            cq.sid[r] = cq.sid[k0 + r];
-        }
-        cq.n = rest;
-    }
-    __syncwarp();
-}
-
-__device__ __forceinline__ void group_drain_warps_cand(const StreamDev* __restrict__ ds, uint32_t k, int cls,
-                                                       uint32_t grab, const unsigned long long* __restrict__ pref,
-                                                       unsigned long long* __restrict__ cursor, GroupCand& cq,
-                                                       GroupQueue& q) {
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned below = (1u << lane) - 1u;
-    const unsigned long long* pc = pref + cls * (k + 1);
-    const unsigned long long total = pc[k];
-    for (;;) {
-        unsigned long long i0 = 0;
-        if (lane == 0) i0 = atomicAdd(&cursor[cls], (unsigned long long)grab);
-        i0 = __shfl_sync(0xFFFFFFFFu, i0, 0);
-        if (i0 >= total) break;
-        const unsigned long long i1 = i0 + grab < total ? i0 + grab : total;
-        uint32_t sid = group_stream_search(pc, k, i0);
-        for (unsigned long long i = i0; i < i1; ++i) {
-            sid = group_stream_of(pc, k, i, sid);
-            const StreamDev& d = ds[sid];
-            const uint32_t item = (uint32_t)(d.ctrl->bin_start[cls] + (i - pc[sid]));
-            const WorkItem x = d.srec[item];
-            const uint32_t n_s = x.cnt_s, l = x.l, t = x.t, lgs = x.lgs & 0xFFu;
-            if (!(block_fits(d, 5, x.off_s, lgs) && REPT_CHECK(d.ctrl, 6, n_s, list_slots(lgs) + 1u) &&
-                  block_fits(d, 7, x.off_l, x.lgs >> 8)))
-                continue;  // (uniform over the warp: x is)
-            const uint4* list = reinterpret_cast<const uint4*>(d.pool + 4ull * x.off_s + (1ull << lgs));
-            const uint32_t last_pair = (n_s - 1u) >> 1;
-            const uint32_t mask = id_mask(d);
-            const bool open = d.colours != kColInEntry;  // no colour test: every older entry is probed
-            auto pass = [&](uint32_t j0, auto full) {
-                constexpr bool FULL = decltype(full)::value;
-                uint4 qv[kScanLoads];
-#pragma unroll
-                for (uint32_t hh = 0; hh < kScanLoads; ++hh) {
-                    const uint32_t pr = (j0 >> 1) + 32u * hh + lane;
-                    qv[hh] = list[FULL || pr < last_pair ? pr : last_pair];
-                }
-#pragma unroll
-                for (uint32_t hh = 0; hh < kScanLoads; ++hh) {
-                    if (!FULL && j0 + 64u * hh >= n_s) break;  // an empty part: uniform skip
-                    const uint32_t jj = j0 + 64u * hh + 2u * lane;
-                    const uint32_t w1 = qv[hh].x & mask, w2 = qv[hh].z & mask;
-                    const bool a1 = (FULL || jj < n_s) & (qv[hh].y < t) &
-                                    (open | colour_may_match(d, l, w1, qv[hh].x >> kIdBits));
-                    const bool a2 = (FULL || jj + 1u < n_s) & (qv[hh].w < t) &
-                                    (open | colour_may_match(d, l, w2, qv[hh].z >> kIdBits));
-                    const unsigned m1 = __ballot_sync(0xFFFFFFFFu, a1), m2 = __ballot_sync(0xFFFFFFFFu, a2);
-                    if (m1 | m2) {
-                        if (a1) {
-                            const uint32_t kk = cq.n + __popc(m1 & below);
-                            cq.w[kk] = w1;
-                            cq.item[kk] = item;
-                            cq.sid[kk] = sid;
-                        }
-                        cq.n += __popc(m1);
-                        if (a2) {
-                            const uint32_t kk = cq.n + __popc(m2 & below);
-                            cq.w[kk] = w2;
-                            cq.item[kk] = item;
-                            cq.sid[kk] = sid;
-                        }
-                        cq.n += __popc(m2);
-                    }
-                }
-                if (cq.n >= 64u) gcand_flush(ds, cq, false, q);
-            };
-            uint32_t j0 = 0;
-            if (kScanFull)
-                for (; j0 + kScanPass <= n_s; j0 += kScanPass) pass(j0, std::true_type{});
-            for (; j0 < n_s; j0 += kScanPass) pass(j0, std::false_type{});
-        }
-    }
-}
-
-// Shared memory of the group intersection, per block of 8 warps: a candidate queue of three arrays
-// (w, item, stream) and a match queue of four arrays (stream, s, l, w) per warp.
-constexpr uint32_t kGroupSmemWords = 8u * 3u * kCandQ + 8u * 4u * kMatchQ;
-
-__device__ __forceinline__ void intersect_group_body(const StreamDev* __restrict__ ds, uint32_t k,
-                                                     const unsigned long long* __restrict__ pref,
+// MODE: the colour storage of every stream, or kColAny.
+template <int MODE>
+__device__ __forceinline__ void intersect_group_body(const StreamDev* __restrict__ ds, const BatchDev* __restrict__ bs,
+                                                     uint32_t k, const unsigned long long* __restrict__ pref,
                                                      unsigned long long* __restrict__ cursor, uint32_t* smem) {
-    const unsigned wid = threadIdx.x >> 5;
-    uint32_t* cw = smem + wid * 3u * kCandQ;
-    uint32_t* mq = smem + 8u * 3u * kCandQ + wid * 4u * kMatchQ;
-    GroupQueue q{mq, mq + kMatchQ, mq + 2u * kMatchQ, mq + 3u * kMatchQ, 0u};
-    GroupCand cq{cw, cw + kCandQ, cw + 2u * kCandQ, 0u};
-    group_drain_warps_cand(ds, k, 5, kGrabHub, pref, cursor, cq, q);
-    group_drain_warps_cand(ds, k, 4, kGrabMid, pref, cursor, cq, q);
-    if (cq.n) gcand_flush(ds, cq, true, q);
-    group_drain_tiles<32>(ds, k, 3, pref, cursor, q);
-    group_drain_tiles<16>(ds, k, 2, pref, cursor, q);
-    group_drain_tiles<8>(ds, k, 1, pref, cursor, q);
-    group_drain_tiles<4>(ds, k, 0, pref, cursor, q);
-    if (q.n) gq_flush(ds, q, q.n);
+    const unsigned lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
+    uint32_t* filter = smem;
+    uint4* items = reinterpret_cast<uint4*>(filter + kFilterWords);
+    WarpQueues wq{filter + kFilterWords + 4u * kUnitItems + wid * queue_words(MODE, true), 0u, 0u};
+    const ManyStreams st{ds};
+    Work wk;
+    int kind = kBinBig;
+    run_block_units<false, MODE>(st, filter, items, wq, wk, [&]() -> UnitClaim {
+        for (; kind >= kBinBlock; --kind) {
+            const unsigned long long* pc = pref + kind * (k + 1);
+            if (pc[k] == 0ull) continue;
+            const unsigned long long i = atomicAdd(&cursor[kind], 1ull);
+            if (i < pc[k]) {
+                const uint32_t sid = group_stream_search(pc, k, i);
+                return claimed_unit(ds[sid], sid, i - pc[sid] + (kind == kBinBig ? 0ull : ds[sid].unit_cap));
+            }
+        }
+        return UnitClaim{0u, 0u, 0u, 0u, 0u, 0u};
+    });
+#pragma unroll 1
+    for (uint32_t part = 0; part < 2u; ++part) {
+        const int bin = (part ^ wid) & 1u ? kBinSmall : kBinWarp;
+        const unsigned long long* pc = pref + bin * (k + 1);
+        for (;;) {
+            unsigned long long i = 0;
+            if (lane == 0) i = atomicAdd(&cursor[bin], 1ull);
+            i = __shfl_sync(0xFFFFFFFFu, i, 0);
+            if (i >= pc[k]) break;
+            const uint32_t sid = group_stream_search(pc, k, i);
+            i -= pc[sid];
+            if (bin == kBinWarp)
+                run_warp_unit<false, MODE>(st, sid, ds[sid].units[ds[sid].unit_cap - 1ull - i],
+                                              filter + (wid << kWarpFilterLg), wq, wk);
+            else
+                run_small_chunk<false, MODE>(st, sid, (uint32_t)i * bs[sid].chunk,
+                                                (uint32_t)min((i + 1ull) * bs[sid].chunk, bs[sid].n), wq, wk);
+        }
+    }
+    cand_flush<false, MODE>(st, wq, wk, true);
 }
 
-__global__ void __launch_bounds__(256, 4) k_intersect_group(const StreamDev* __restrict__ ds, uint32_t k,
-                                                            const unsigned long long* __restrict__ pref,
-                                                            unsigned long long* __restrict__ cursor) {
-    __shared__ uint32_t smem[kGroupSmemWords];
-    intersect_group_body(ds, k, pref, cursor, smem);
+// Dynamic shared memory: ix_words(MODE, true) words.
+template <int MODE>
+__global__ void __launch_bounds__(kIxThreads, kIxBlocks) k_intersect_group(const StreamDev* __restrict__ ds,
+                                                                           const BatchDev* __restrict__ bs, uint32_t k,
+                                                                           const unsigned long long* __restrict__ pref,
+                                                                           unsigned long long* __restrict__ cursor) {
+    extern __shared__ __align__(16) uint32_t ix_smem[];
+    intersect_group_body<MODE>(ds, bs, k, pref, cursor, ix_smem);
 }
 
 // Algorithm 2's triangle-pair counters, folded in after the intersection.  Edge e of group k was a
@@ -1656,18 +1742,22 @@ __global__ void k_plan_multi(const StreamDev* __restrict__ ds, const BatchDev* _
     k_plan_body(sd, launch_grid());
 }
 
-__global__ void k_commit(StreamDev d) { k_commit_body(d, launch_grid()); }
+__global__ void __launch_bounds__(256) k_commit(StreamDev d) {
+    __shared__ __align__(16) uint32_t smem[kCommitSmemWords];
+    k_commit_body(d, launch_grid(), smem);
+}
 
-__global__ void k_commit_multi(const StreamDev* __restrict__ ds, const BatchDev* __restrict__ bs) {
+__global__ void __launch_bounds__(256) k_commit_multi(const StreamDev* __restrict__ ds, const BatchDev* __restrict__ bs) {
     (void)bs;
+    __shared__ __align__(16) uint32_t smem[kCommitSmemWords];
     __shared__ StreamDev sd;
     if (threadIdx.x == 0) sd = ds[blockIdx.y];
     __syncthreads();
-    k_commit_body(sd, launch_grid());
+    k_commit_body(sd, launch_grid(), smem);
 }
 
 __global__ void __launch_bounds__(256) k_rehash_big(StreamDev d) {
-    __shared__ uint32_t smem[kMoveSmemWords];
+    __shared__ __align__(16) uint32_t smem[kMoveSmemWords];
     k_rehash_big_body(d, launch_grid(), smem);
 }
 
@@ -1675,30 +1765,30 @@ __global__ void __launch_bounds__(256) k_rehash_big_multi(const StreamDev* __res
                                                             const BatchDev* __restrict__ bs) {
     (void)bs;
     __shared__ StreamDev sd;
-    __shared__ uint32_t smem[kMoveSmemWords];
+    __shared__ __align__(16) uint32_t smem[kMoveSmemWords];
     if (threadIdx.x == 0) sd = ds[blockIdx.y];
     __syncthreads();
     k_rehash_big_body(sd, launch_grid(), smem);
 }
 
-// Two blocks of 1024 threads per SM (32 registers a thread), so that the whole grid is resident.
+// Two blocks of 1024 threads per SM (32 registers a thread), so that the whole grid is resident.  Dynamic
+// shared memory: kHugeSmemWords words.
 __global__ void __launch_bounds__(1024, 2) k_rehash_huge(StreamDev d) {
-    __shared__ uint32_t smem[kMoveSmemWords];
-    k_rehash_huge_body(d, launch_grid(), smem);
+    extern __shared__ __align__(16) uint32_t hsmem[];
+    k_rehash_huge_body(d, launch_grid(), hsmem, kBlockMoveSlots);
 }
 
 __global__ void __launch_bounds__(1024, 2) k_rehash_huge_multi(const StreamDev* __restrict__ ds,
                                                               const BatchDev* __restrict__ bs) {
     (void)bs;
+    extern __shared__ __align__(16) uint32_t hsmem[];
     __shared__ StreamDev sd;
-    __shared__ uint32_t smem[kMoveSmemWords];
     if (threadIdx.x == 0) sd = ds[blockIdx.y];
     __syncthreads();
-    k_rehash_huge_body(sd, launch_grid(), smem);
+    k_rehash_huge_body(sd, launch_grid(), hsmem, kBlockMoveSlots);
 }
 
-// 5 blocks of 256 threads per SM (48 registers): 2.79 against 2.93 ms per headline step at 56
-// registers and 4 blocks; at 6 blocks (40 registers) it spills.
+// 5 blocks of 256 threads per SM (48 registers).
 __global__ void __launch_bounds__(256, 5) k_insert(StreamDev d, BatchDev b) { k_insert_body(d, b, launch_grid()); }
 
 __global__ void k_insert_multi(const StreamDev* __restrict__ ds, const BatchDev* __restrict__ bs) {
@@ -1712,20 +1802,9 @@ __global__ void k_insert_multi(const StreamDev* __restrict__ ds, const BatchDev*
     k_insert_body(sd, sb, launch_grid());
 }
 
-__global__ void __launch_bounds__(1024) k_sort_scan(StreamDev d) { k_sort_scan_body(d, launch_grid()); }
+__global__ void __launch_bounds__(256) k_units(StreamDev d, BatchDev b) { k_units_body(d, b, launch_grid()); }
 
-__global__ void __launch_bounds__(1024) k_sort_scan_multi(const StreamDev* __restrict__ ds,
-                                                           const BatchDev* __restrict__ bs) {
-    (void)bs;
-    __shared__ StreamDev sd;
-    if (threadIdx.x == 0) sd = ds[blockIdx.y];
-    __syncthreads();
-    k_sort_scan_body(sd, launch_grid());
-}
-
-__global__ void k_sort_scatter(StreamDev d, BatchDev b) { k_sort_scatter_body(d, b, launch_grid()); }
-
-__global__ void k_sort_scatter_multi(const StreamDev* __restrict__ ds, const BatchDev* __restrict__ bs) {
+__global__ void __launch_bounds__(256) k_units_multi(const StreamDev* __restrict__ ds, const BatchDev* __restrict__ bs) {
     __shared__ StreamDev sd;
     __shared__ BatchDev sb;
     if (threadIdx.x == 0) {
@@ -1733,7 +1812,20 @@ __global__ void k_sort_scatter_multi(const StreamDev* __restrict__ ds, const Bat
         sb = bs[blockIdx.y];
     }
     __syncthreads();
-    k_sort_scatter_body(sd, sb, launch_grid());
+    k_units_body(sd, sb, launch_grid());
+}
+
+__global__ void __launch_bounds__(256) k_order(StreamDev d, BatchDev b) { k_order_body(d, b, launch_grid()); }
+
+__global__ void __launch_bounds__(256) k_order_multi(const StreamDev* __restrict__ ds, const BatchDev* __restrict__ bs) {
+    __shared__ StreamDev sd;
+    __shared__ BatchDev sb;
+    if (threadIdx.x == 0) {
+        sd = ds[blockIdx.y];
+        sb = bs[blockIdx.y];
+    }
+    __syncthreads();
+    k_order_body(sd, sb, launch_grid());
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1792,7 +1884,8 @@ struct PersistShape {
 
 // Dynamic shared memory of the persistent kernel: the larger of the block moves' and the group
 // intersection's needs.
-constexpr uint32_t kPersistSmemWords = kMoveSmemWords > kGroupSmemWords ? kMoveSmemWords : kGroupSmemWords;
+static_assert(ix_words(kColAny, true) * 2u >= kBlockMoveSlots / 2u, "the block moves fit");
+constexpr uint32_t kPersistSmemWords = kMoveSmemWords > ix_words(kColAny, true) ? kMoveSmemWords : ix_words(kColAny, true);
 
 __global__ void __launch_bounds__(256, 3) k_group_persistent(const StreamDev* __restrict__ ds,
                                                            const BatchDev* __restrict__ bs, uint32_t k,
@@ -1827,22 +1920,22 @@ __global__ void __launch_bounds__(256, 3) k_group_persistent(const StreamDev* __
     ok = ok && grid_barrier(gs, wait_ns);
     if (ok) step(sh.x_edge, [&](Grid g) { k_plan_body(sd, g); });
     ok = ok && grid_barrier(gs, wait_ns);
-    if (ok) step(sh.x_edge, [&](Grid g) { k_commit_body(sd, g); });
+    if (ok) step(sh.x_edge, [&](Grid g) { k_commit_body(sd, g, psmem); });
     ok = ok && grid_barrier(gs, wait_ns);
     if (ok) step(sh.x_big, [&](Grid g) { k_rehash_big_body(sd, g, psmem); });
     ok = ok && grid_barrier(gs, wait_ns);
-    if (ok) step(sh.x_huge, [&](Grid g) { k_rehash_huge_body(sd, g, psmem); });
+    if (ok) step(sh.x_huge, [&](Grid g) { k_rehash_huge_body(sd, g, psmem, kBlockMoveSlots / 2u); });
     ok = ok && grid_barrier(gs, wait_ns);
     if (ok) step(sh.x_edge, [&](Grid g) { k_insert_body(sd, sb, g); });
     ok = ok && grid_barrier(gs, wait_ns);
-    if (ok) step(1u, [&](Grid g) { k_sort_scan_body(sd, g); });
+    if (ok) step(sh.x_edge, [&](Grid g) { k_units_body(sd, sb, g); });
     ok = ok && grid_barrier(gs, wait_ns);
-    if (ok) step(sh.x_edge, [&](Grid g) { k_sort_scatter_body(sd, sb, g); });
+    if (ok) step(sh.x_edge, [&](Grid g) { k_order_body(sd, sb, g); });
     ok = ok && grid_barrier(gs, wait_ns);
     if (ok && blockIdx.x == 0) group_prefix_body(ds, k, pref, cursor);
     ok = ok && grid_barrier(gs, wait_ns);
     if (ok) {
-        intersect_group_body(ds, k, pref, cursor, psmem);
+        intersect_group_body<kColAny>(ds, bs, k, pref, cursor, psmem);
         return;
     }
     // a wait ran out: the round is not applied for any stream (every step checks the status first)
@@ -1850,28 +1943,67 @@ __global__ void __launch_bounds__(256, 3) k_group_persistent(const StreamDev* __
         for (uint32_t i = blockIdx.x; i < k; i += gridDim.x) atomicOr(&ds[i].ctrl->status, kStTimeout);
 }
 
-// Streams whose entries carry their colour (one hash group, m <= 256): 5 blocks of 256 threads per SM.
-#ifndef REPT_COLOURED_BLOCKS
-#define REPT_COLOURED_BLOCKS 5
-#endif
+// Streams whose entries carry their colour (one hash group, m <= 256).
 template <bool WORK>
-__global__ void __launch_bounds__(256, REPT_COLOURED_BLOCKS) k_intersect(StreamDev d, BatchDev b) {
+__global__ void __launch_bounds__(kIxThreads, kIxBlocks) k_intersect(StreamDev d, BatchDev b) {
     k_intersect_body<WORK, (int)kColInEntry>(d, b);
 }
 
 // Streams whose entries have colour words (one hash group whose colour does not fit the entry: m > 256
-// or more than 2^24 nodes): the scan-first path with one hash per entry, and probes for about 1/m of
-// the entries.
+// or more than 2^24 nodes).
 template <bool WORK>
-__global__ void __launch_bounds__(256, REPT_WORDS_BLOCKS) k_intersect_words(StreamDev d, BatchDev b) {
+__global__ void __launch_bounds__(kIxThreads, kIxBlocks) k_intersect_words(StreamDev d, BatchDev b) {
     k_intersect_body<WORK, (int)kColWords>(d, b);
 }
 
-// Streams without stored colours (parallel MASCOT with several samplers, or too many groups for a
-// word): every probe is issued, so the kernel waits on memory and wants every warp an SM can hold.
+// Streams of several hash groups, with a colour word beside every stream index.
 template <bool WORK>
-__global__ void __launch_bounds__(256, 8) k_intersect_probe(StreamDev d, BatchDev b) {
+__global__ void __launch_bounds__(kIxThreads, kIxBlocks) k_intersect_multi(StreamDev d, BatchDev b) {
+    k_intersect_body<WORK, (int)kColMulti>(d, b);
+}
+
+// Streams without stored colours (too many hash groups for a word, or too little memory for one).
+template <bool WORK>
+__global__ void __launch_bounds__(kIxThreads, kIxBlocks) k_intersect_probe(StreamDev d, BatchDev b) {
     k_intersect_body<WORK, (int)kColNone>(d, b);
+}
+
+// Rebuild every node's block from a pool of another layout: `from_colours`, with pair lists of version 3
+// when `pairs`.  meta holds the new block offsets, old_off those in `old`; a warp per node.
+__global__ void __launch_bounds__(256) k_convert(StreamDev d, const uint2* __restrict__ old,
+                                                 const uint32_t* __restrict__ old_off, uint32_t from_colours, bool pairs) {
+    const unsigned lane = threadIdx.x & 31u;
+    const uint32_t col = d.colours, mask = id_mask(d);
+    for (uint32_t x = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < d.n_nodes; x += (gridDim.x * blockDim.x) >> 5) {
+        const uint4 m = d.meta[x];
+        const uint32_t cnt = m.y, lg = table_lg(cnt);
+        if (cnt == 0u || !block_fits(d, 10, m.x, lg)) continue;
+        const uint32_t* from = block_at(old, old_off[x]);
+        uint32_t* to = block_at(d.pool, m.x);
+        init_table_keys(to, lg, col, lane, 32u);
+        __syncwarp();
+        bool ok = true;
+        for (uint32_t j = lane; j < cnt; j += 32u) {
+            uint32_t word, t, cw = 0u;
+            if (pairs) {
+                word = from[(2u << lg) + 2u * j];
+                t = from[(2u << lg) + 2u * j + 1u];
+            } else {
+                word = from[list_at(lg, from_colours) + j];
+                t = from[aux_at(lg, from_colours) + (from_colours == kColMulti ? 2u * j : j)];
+            }
+            bool kept;
+            if (col == kColWords) cw = from[cw_at(lg) + j];
+            if (col == kColMulti) cw = colour_word(d, x, word, kept);
+            to[list_at(lg, col) + j] = word;
+            if (col == kColWords) to[cw_at(lg) + j] = cw;
+            if (col == kColNone) to[aux_at(lg, col) + j] = t;
+            if (col == kColMulti) reinterpret_cast<uint2*>(to + aux_at(lg, col))[j] = make_uint2(t, cw);
+            ok &= table_insert(to, lg, word & mask, t, cw, col);
+        }
+        if (!ok) atomicOr(&d.ctrl->status, kStInternal);
+        __syncwarp();
+    }
 }
 
 // tau_hat_v = f * sum_i tau_v^(i), f formed in double on the host.

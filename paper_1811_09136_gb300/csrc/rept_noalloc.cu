@@ -25,7 +25,7 @@ inline unsigned long long align256(unsigned long long x) { return (x + 255ull) &
 
 // Offsets of the state inside the scratch area for n nodes and E edges.
 struct Layout {
-    unsigned long long meta, cnt_add, touched, grow_rel, big, rec, srec, hist, ctrl, pool, end;
+    unsigned long long meta, cnt_add, touched, grow_rel, big, rec, lists, ctrl, pool, end;
     unsigned long long pool_quads;
 };
 
@@ -38,8 +38,7 @@ Layout layout_for(unsigned long long n, unsigned long long E) {
     L.grow_rel = o; o = align256(o + 2 * E * sizeof(uint32_t));
     L.big = o;      o = align256(o + 2 * E * sizeof(uint32_t));
     L.rec = o;      o = align256(o + E * sizeof(WorkItem));
-    L.srec = o;     o = align256(o + E * sizeof(WorkItem));
-    L.hist = o;     o = align256(o + kSortBuckets * sizeof(uint32_t));
+    L.lists = o;    o = align256(o + E * kListBytes);
     L.ctrl = o;     o = align256(o + sizeof(Ctrl));
     // From an empty state every node's block (table plus list) is allocated once, with at most 8
     // slots per entry: at most 16 slots (4 quads) per edge.
@@ -115,7 +114,6 @@ extern "C" int rept_count_noalloc(const uint32_t* d_src, const uint32_t* d_dst, 
     d.n_nodes = n_nodes;
     d.seed = seed;
     d.fm = make_fastmod(m);
-    d.tile_max = 32u;
     d.meta = reinterpret_cast<uint4*>(sc + L.meta);
     d.cnt_add = reinterpret_cast<uint32_t*>(sc + L.cnt_add);
     d.touched = reinterpret_cast<uint32_t*>(sc + L.touched);
@@ -123,8 +121,8 @@ extern "C" int rept_count_noalloc(const uint32_t* d_src, const uint32_t* d_dst, 
     d.big = reinterpret_cast<uint32_t*>(sc + L.big);
     d.big_cap = 2 * (n_edges ? n_edges : 1);
     d.rec = reinterpret_cast<WorkItem*>(sc + L.rec);
-    d.srec = reinterpret_cast<WorkItem*>(sc + L.srec);
-    d.hist = reinterpret_cast<uint32_t*>(sc + L.hist);
+    d.units = reinterpret_cast<Unit*>(sc + L.lists);
+    set_list_pointers(d, n_edges);
     d.ctrl = reinterpret_cast<Ctrl*>(sc + L.ctrl);
     d.pool = reinterpret_cast<uint2*>(sc + L.pool);
     d.pool_quads = L.pool_quads;
@@ -143,7 +141,7 @@ extern "C" int rept_count_noalloc(const uint32_t* d_src, const uint32_t* d_dst, 
         int dev = 0, sms = 0;
         NA_CUDA(cudaGetDevice(&dev));
         NA_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        const BatchDev b{d_src, d_dst, n_edges, 0ull};
+        const BatchDev b = make_batch(d_src, d_dst, n_edges, 0ull, 32u);
         const int threads = 256;
         const unsigned long long blocks = (n_edges + threads - 1) / threads;
         const int grid = (int)(blocks < (unsigned long long)sms * 8 ? blocks : (unsigned long long)sms * 8);
@@ -151,13 +149,17 @@ extern "C" int rept_count_noalloc(const uint32_t* d_src, const uint32_t* d_dst, 
         k_plan<<<grid, threads, 0, st>>>(d);
         k_commit<<<grid, threads, 0, st>>>(d);
         k_rehash_big<<<sms * 4, threads, 0, st>>>(d);
-        k_rehash_huge<<<sms * 2, 1024, 0, st>>>(d);
+        NA_CUDA(cudaFuncSetAttribute(k_rehash_huge, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)(kHugeSmemWords * sizeof(uint32_t))));
+        k_rehash_huge<<<sms * 2, 1024, kHugeSmemWords * sizeof(uint32_t), st>>>(d);
         k_insert<<<grid, threads, 0, st>>>(d, b);
-        k_sort_scan<<<1, 1024, 0, st>>>(d);
-        k_sort_scatter<<<grid, threads, 0, st>>>(d, b);
-        const unsigned long long want_i = (n_edges * 8 + 255) / 256;
+        k_units<<<grid, threads, 0, st>>>(d, b);
+        k_order<<<grid, threads, 0, st>>>(d, b);
+        const unsigned long long want_i = (n_edges + 31) / 32;
         const int grid_i = (int)(want_i < (unsigned long long)sms * 4 ? want_i : (unsigned long long)sms * 4);
-        k_intersect_probe<false><<<grid_i, 256, c * sizeof(unsigned long long), st>>>(d, b);
+        const size_t smem = ix_words((int)kColNone, false) * sizeof(uint32_t) + c * sizeof(unsigned long long);
+        NA_CUDA(cudaFuncSetAttribute(k_intersect_probe<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        k_intersect_probe<false><<<grid_i, kIxThreads, smem, st>>>(d, b);
         NA_CUDA(cudaPeekAtLastError());
     }
     if (d_global) {
