@@ -165,6 +165,11 @@ cudaEvent_t take_event(rept_state* s) {
     return e;
 }
 
+// Batches of at most this many edges run their steps in one launch (k_state).  Per batch, all launches of it
+// included, on a 20,000-node power-law stream (launch per step against k_state): 1,024 edges 82 and 60 us,
+// 4,096 92 and 70, 8,192 94 and 81, 16,384 109 and 124: one cluster's 8,192 threads are then too few.
+constexpr unsigned long long kStateBatch = 1ull << 13;
+
 // NVTX range names of the phases (seen by profilers that record NVTX, e.g. ncu --nvtx); the
 // ranges cost a check of a function pointer when no tool is attached.
 const char* const kPhaseNames[] = {"rept classify", "rept plan", "rept commit", "rept insert",
@@ -247,15 +252,9 @@ int ensure_pair_capacity(rept_state* s, unsigned long long edges, cudaStream_t s
     return REPT_OK;
 }
 
-int launch_batch(rept_state* s, const uint32_t* d_src, const uint32_t* d_dst, unsigned long long n, cudaStream_t st) {
-    if (s->d.pair_tau) {
-        const int prc = ensure_pair_capacity(s, s->next_t + n, st);
-        if (prc) return prc;
-    }
-    const BatchDev b = make_batch(d_src, d_dst, n, s->next_t, s->tile_max);
-    const int threads = 256;
-    const unsigned long long want_blocks = (n + threads - 1) / threads;
-    const int grid = (int)std::min<unsigned long long>(want_blocks, (unsigned long long)s->grid_stream);
+// The steps of a batch before its intersection, a launch or more each.  Without `pool_safe` the batch's
+// request is read after k_plan, and the pool grown if need be.
+int launch_steps(rept_state* s, const BatchDev& b, int grid, int threads, bool pool_safe, cudaStream_t st) {
     int rc = REPT_OK;
     if ((rc = timed_launch(s, REPT_K_CLASSIFY, st, [&] { k_classify<<<grid, threads, 0, st>>>(s->d, b); })))
         return rc;
@@ -263,14 +262,13 @@ int launch_batch(rept_state* s, const uint32_t* d_src, const uint32_t* d_dst, un
         // the set of this batch's edge keys: a power of two >= 2n slots of 8 bytes in the work-record
         // scratch (32 bytes per batch edge, so at most half of it)
         unsigned long long cap = 1;
-        while (cap < 2 * n) cap <<= 1;
+        while (cap < 2 * b.n) cap <<= 1;
         REPT_CUDA(cudaMemsetAsync(s->d.rec, 0xFF, cap * sizeof(unsigned long long), st));
         if ((rc = timed_launch(s, REPT_K_CLASSIFY, st, [&] { k_check_dups<<<grid, threads, 0, st>>>(s->d, b, cap - 1); })))
             return rc;
     }
     if ((rc = timed_launch(s, REPT_K_PLAN, st, [&] { k_plan<<<grid, threads, 0, st>>>(s->d); }))) return rc;
-    const bool fixed = (s->cfg.flags & REPT_FLAG_FIXED_POOL) != 0;
-    if (!fixed && s->d.pool_quads < quads_bound(s->next_t + n, s->d.colours)) {
+    if (!pool_safe) {
         // not provably large enough: read this batch's request and grow if needed
         if ((rc = read_ctrl(s, st))) return rc;
         const unsigned long long need = s->h_ctrl->pool_top + s->h_ctrl->need_quads;
@@ -290,6 +288,28 @@ int launch_batch(rept_state* s, const uint32_t* d_src, const uint32_t* d_dst, un
              k_order<<<grid, threads, 0, st>>>(s->d, b);
          }, 2)))
         return rc;
+    return REPT_OK;
+}
+
+int launch_batch(rept_state* s, const uint32_t* d_src, const uint32_t* d_dst, unsigned long long n, cudaStream_t st) {
+    if (s->d.pair_tau) {
+        const int prc = ensure_pair_capacity(s, s->next_t + n, st);
+        if (prc) return prc;
+    }
+    const BatchDev b = make_batch(d_src, d_dst, n, s->next_t, s->tile_max);
+    const int threads = 256;
+    const unsigned long long want_blocks = (n + threads - 1) / threads;
+    const int grid = (int)std::min<unsigned long long>(want_blocks, (unsigned long long)s->grid_stream);
+    int rc = REPT_OK;
+    const bool fixed = (s->cfg.flags & REPT_FLAG_FIXED_POOL) != 0;
+    const bool pool_safe = fixed || s->d.pool_quads >= quads_bound(s->next_t + n, s->d.colours);
+    if (n <= kStateBatch && pool_safe && !(s->cfg.flags & (REPT_FLAG_PROFILE | REPT_FLAG_CHECK_DUPS))) {
+        NvtxRange range("rept state");
+        k_state<<<kStateBlocks, kStateThreads, kStateSmemWords * sizeof(uint32_t), st>>>(s->d, b);
+        REPT_LAUNCHED();
+    } else if ((rc = launch_steps(s, b, grid, threads, pool_safe, st))) {
+        return rc;
+    }
     const unsigned long long want_i = (n + 31) / 32;  // work is claimed dynamically; >= 1 block
     const int grid_i = (int)std::min<unsigned long long>(want_i, (unsigned long long)s->grid_intersect);
     const size_t smem = intersect_smem(s->d.colours, s->cfg.c);
@@ -389,7 +409,8 @@ int rept_create(const rept_config* cfg, void* stream, rept_state** out) {
     const bool multi = !coloured && !words && n_groups * (one_colour ? 1ull : cbits) <= 32ull;
     uint32_t colours = coloured ? kColInEntry : words ? kColWords : multi ? kColMulti : kColNone;
     const size_t max_smem = intersect_smem(kColMulti, kMaxProcessors);
-    if (allow_smem(k_rehash_huge, kHugeSmemWords * sizeof(uint32_t)) != cudaSuccess ||
+    if (allow_smem(k_state, kStateSmemWords * sizeof(uint32_t)) != cudaSuccess ||
+        allow_smem(k_rehash_huge, kHugeSmemWords * sizeof(uint32_t)) != cudaSuccess ||
         allow_smem(k_intersect<false>, max_smem) != cudaSuccess || allow_smem(k_intersect<true>, max_smem) != cudaSuccess ||
         allow_smem(k_intersect_words<false>, max_smem) != cudaSuccess ||
         allow_smem(k_intersect_words<true>, max_smem) != cudaSuccess ||

@@ -88,6 +88,16 @@ __device__ __forceinline__ bool table_insert(uint32_t* table, uint32_t lg, uint3
     return false;
 }
 
+// Has an earlier step failed?  The answer is the same for the whole block (another block may be setting
+// the status meanwhile), so that its threads meet at the same barriers.
+__device__ __forceinline__ bool block_failed(const Ctrl* c) {
+    __shared__ unsigned s_status;
+    __syncthreads();
+    if (threadIdx.x == 0) s_status = c->status;
+    __syncthreads();
+    return s_status != 0u;
+}
+
 // Scratch that lives in another step's memory: per edge, its places among the batch's new entries of its
 // two endpoints (k_classify to k_insert, where the units go later); per touched node, the batch's new
 // entries (k_plan to k_commit, where the work records go later).
@@ -105,7 +115,7 @@ __device__ __forceinline__ void k_classify_body(const StreamDev& d, const BatchD
         d.ctrl->n_groups = 0ull;
         d.ctrl->n_items = 0ull;
     }
-    if (d.ctrl->status) return;
+    if (block_failed(d.ctrl)) return;
     __shared__ BlockReserve part[2];
     uint32_t turn = 0;
     const unsigned long long stride = (unsigned long long)g.nbx * blockDim.x;
@@ -132,7 +142,7 @@ __device__ __forceinline__ void k_classify_body(const StreamDev& d, const BatchD
 }
 
 __device__ __forceinline__ void k_plan_body(const StreamDev& d, const Grid g) {
-    if (d.ctrl->status) return;
+    if (block_failed(d.ctrl)) return;
     __shared__ BlockReserve part[2];
     uint32_t turn = 0;
     const unsigned long long n_t = d.ctrl->n_touched;
@@ -347,8 +357,8 @@ __device__ __forceinline__ void k_commit_body(const StreamDev& d, const Grid g, 
 }
 
 // Move the blocks listed by k_commit whose new table has at most kMoveSlots slots: one warp per node.
-// `smem`: kMoveSmemWords words of shared memory (a key and a stream-index table of kMoveSlots slots
-// for each of the block's 8 warps).
+// `smem`: a key and a stream-index table of kMoveSlots slots for each of the block's warps (kMoveSmemWords
+// words for 8).
 constexpr uint32_t kMoveSmemWords = 2u * 8u * kMoveSlots;
 __device__ __forceinline__ void k_rehash_big_body(const StreamDev& d, const Grid g, uint32_t* smem) {
     const unsigned long long n_big = d.ctrl->n_big, top = d.ctrl->pool_top;
@@ -366,9 +376,9 @@ __device__ __forceinline__ void k_rehash_big_body(const StreamDev& d, const Grid
         uint32_t* to = block_at(d.pool, new_off);
         const uint32_t* from = block_at(d.pool, m.x);
         bool ok = true;
-        if (fits && (1u << lg_new) <= kMoveSlots && REPT_CHECK(d.ctrl, 14, wid, 8u))
-            ok = move_block_smem(to, from, m.y, lg_new, d.colours, smem + wid * kMoveSlots,
-                                        smem + (8u + wid) * kMoveSlots, lane, 32u);
+        if (fits && (1u << lg_new) <= kMoveSlots && REPT_CHECK(d.ctrl, 14, wid, 32u))
+            ok = move_block_smem(to, from, m.y, lg_new, d.colours, smem + wid * 2u * kMoveSlots,
+                                 smem + (wid * 2u + 1u) * kMoveSlots, lane, 32u);
         else if (fits) {
             init_table_keys(to, lg_new, d.colours, lane, 32u);
             __syncwarp();
@@ -488,17 +498,17 @@ __device__ __forceinline__ void k_rehash_huge_body(const StreamDev& d, const Gri
 
 __device__ __forceinline__ void k_insert_body(const StreamDev& d, const BatchDev& b, const Grid g) {
     Ctrl* ct = d.ctrl;
-    const unsigned status = ct->status;
+    const bool failed = block_failed(ct);
     if (g.bx == 0 && threadIdx.x == 0) {
         // the batch's table space is now in use; reset the per-batch counters
-        if (status == 0u) ct->pool_top += ct->need_quads;
+        if (!failed) ct->pool_top += ct->need_quads;
         ct->need_quads = 0;
         ct->n_touched = 0;
         ct->n_big = 0;
         ct->n_huge = 0;
         ct->huge_next = 0;
     }
-    if (status) return;
+    if (failed) return;
     __shared__ BlockReserve part[2];
     uint32_t turn = 0;
     const unsigned lane = threadIdx.x & 31u;
@@ -1826,6 +1836,39 @@ __global__ void __launch_bounds__(256) k_order_multi(const StreamDev* __restrict
     }
     __syncthreads();
     k_order_body(sd, sb, launch_grid());
+}
+
+// Every step of a small batch before its intersection in one launch: a single cluster of thread blocks runs
+// them in turn, with the cluster's hardware barrier between them (its release and acquire order global
+// memory as well), so that a batch of a few thousand edges pays for two launches instead of nine.
+// Dynamic shared memory: kStateSmemWords words.
+constexpr uint32_t kStateBlocks = 8, kStateThreads = 1024;
+constexpr uint32_t kStateSmemWords = 2u * (kStateThreads / 32u) * kMoveSlots;
+static_assert(kStateSmemWords >= kHugeSmemWords && kStateSmemWords >= kCommitSmemWords * (kStateThreads / 256u),
+              "the steps share the memory");
+
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__global__ void __cluster_dims__(kStateBlocks, 1, 1) __launch_bounds__(kStateThreads, 1) k_state(StreamDev d, BatchDev b) {
+    extern __shared__ __align__(16) uint32_t hsmem[];
+    const Grid g = launch_grid();
+    k_classify_body(d, b, g);
+    cluster_barrier();
+    k_plan_body(d, g);
+    cluster_barrier();
+    k_commit_body(d, g, hsmem);
+    cluster_barrier();
+    k_rehash_big_body(d, g, hsmem);
+    __syncthreads();
+    k_rehash_huge_body(d, g, hsmem, kBlockMoveSlots);
+    cluster_barrier();
+    k_insert_body(d, b, g);
+    cluster_barrier();
+    k_units_body(d, b, g);
+    cluster_barrier();
+    k_order_body(d, b, g);
 }
 
 // ---------------------------------------------------------------------------------------------
