@@ -55,12 +55,17 @@ struct rept_state {
     StreamDev d{};
     unsigned long long max_batch = 0;
     unsigned long long next_t = 0;  // stream index of the next edge
-    Ctrl* h_ctrl = nullptr;         // pinned mirror of the control block
+    // One allocation holds what a reset clears: node records, counters, then the results (Results) that a
+    // query copies to the host at once.
+    void* core = nullptr;
+    size_t core_bytes = 0;
+    unsigned char* h_results = nullptr;  // pinned mirror of the results: tau_hat, control block, tau^(i)
+    Ctrl* h_ctrl = nullptr;              // ... its control block
     uint32_t* stage_src = nullptr;  // device staging for rept_ingest_host
     uint32_t* stage_dst = nullptr;
     unsigned long long stage_cap = 0;
     double* d_global = nullptr;
-    double* h_global = nullptr;  // pinned
+    double* h_global = nullptr;  // ... and tau_hat
     double* d_local_tmp = nullptr;
     int grid_stream = 0;     // blocks for edge/node-parallel kernels
     int grid_intersect = 0;  // blocks for k_intersect
@@ -105,7 +110,6 @@ int grow_pool(rept_state* s, unsigned long long min_quads, cudaStream_t st) {
     REPT_CUDA(cudaStreamSynchronize(st));
     const unsigned long long used = s->h_ctrl->pool_top;
     if (s->d.pool && used) REPT_CUDA(cudaMemcpyAsync(np, s->d.pool, used * 32ull, cudaMemcpyDeviceToDevice, st));
-    REPT_CUDA(cudaMemsetAsync((char*)np + used * 32ull, 0xFF, (want - used) * 32ull, st));
     REPT_CUDA(cudaStreamSynchronize(st));
     dev_free(s, s->d.pool, s->d.pool_quads * 32ull);
     s->d.pool = np;
@@ -113,11 +117,18 @@ int grow_pool(rept_state* s, unsigned long long min_quads, cudaStream_t st) {
     return REPT_OK;
 }
 
-int read_ctrl(rept_state* s, cudaStream_t st) {
-    REPT_CUDA(cudaMemcpyAsync(s->h_ctrl, s->d.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, st));
+// The results part of the core allocation, and its mirror: tau_hat, the control block, c counters.
+constexpr size_t kResultsCtrl = 16, kResultsProc = kResultsCtrl + (sizeof(Ctrl) + 15) / 16 * 16;
+
+// Copy the control block, tau_hat and (`proc`) the counters to the pinned mirror and wait for them.
+int read_results(rept_state* s, bool proc, cudaStream_t st) {
+    const size_t bytes = proc ? kResultsProc + s->cfg.c * sizeof(uint64_t) : kResultsProc;
+    REPT_CUDA(cudaMemcpyAsync(s->h_results, s->d_global, bytes, cudaMemcpyDeviceToHost, st));
     REPT_CUDA(cudaStreamSynchronize(st));
     return REPT_OK;
 }
+
+int read_ctrl(rept_state* s, cudaStream_t st) { return read_results(s, false, st); }
 
 // Shared memory of an intersection launch for c processors.  (cudaFuncSetAttribute lifts the default
 // limit of the kernel; it applies to the current device.)
@@ -345,19 +356,22 @@ double estimate_factor(const rept_config& c) {
     return md / (double)(c.c / c.m);
 }
 
-// tau_hat into s->d_global: Section III-A / III-B.1 factor, or Algorithm 2's combination.
-int enqueue_global_estimate(rept_state* s, cudaStream_t st) {
-    if (s->d.local2)
-        return timed_launch(s, REPT_K_ESTIMATE, st, [&] {
-            k_global_estimate_partial<<<1, 32, 0, st>>>(s->d.proc, s->d.eta_proc, s->cfg.m, s->cfg.c, s->d_global);
-        });
-    const double f = estimate_factor(s->cfg);
-    return timed_launch(s, REPT_K_ESTIMATE, st,
-                        [&] { k_global_estimate<<<1, 256, 0, st>>>(s->d.proc, s->cfg.c, f, s->d_global); });
+// tau_hat into s->d_global and (d_local) the local estimates: Section III-A / III-B.1 factor, or
+// Algorithm 2's combination.
+int enqueue_estimates(rept_state* s, double* d_local, cudaStream_t st) {
+    const int grid = d_local ? (int)std::min<unsigned long long>((s->d.n_nodes + 255ull) / 256, s->sm_count * 4ull) : 1;
+    return timed_launch(s, REPT_K_ESTIMATE, st, [&] {
+        if (s->d.local2)
+            k_estimates_partial<<<grid, 256, 0, st>>>(s->d.proc, s->d.eta_proc, s->d.local, s->d.local2, s->d.eta_local,
+                                                      s->d.n_nodes, s->cfg.m, s->cfg.c, s->d_global, d_local);
+        else
+            k_estimates<<<grid, 256, 0, st>>>(s->d.proc, s->cfg.c, s->d.local, s->d.n_nodes, estimate_factor(s->cfg),
+                                              s->d_global, d_local);
+    });
 }
 
-int sync_status(rept_state* s, cudaStream_t st) {
-    int rc = read_ctrl(s, st);
+int sync_status(rept_state* s, cudaStream_t st, bool proc = false) {
+    int rc = read_results(s, proc, st);
     if (rc) return rc;
 #ifdef REPT_DEBUG_BOUNDS
     report_failed_check(s->h_ctrl->dbg);
@@ -443,11 +457,26 @@ int rept_create(const rept_config* cfg, void* stream, rept_state** out) {
         return std::min(quads_bound(cfg->expected_edges ? cfg->expected_edges : mb, colours), 0xFFFFFFFFull);
     };
     unsigned long long quads = wanted_quads();
-    if ((rc = dev_alloc(s, (void**)&d.meta, (size_t)n * sizeof(uint4)))) return fail(rc);
-    if ((rc = dev_alloc(s, (void**)&d.cnt_add, (size_t)n * sizeof(uint32_t)))) return fail(rc);
-    if ((rc = dev_alloc(s, (void**)&d.local, (size_t)n * sizeof(unsigned long long)))) return fail(rc);
-    if ((rc = dev_alloc(s, (void**)&d.proc, (size_t)cfg->c * sizeof(unsigned long long)))) return fail(rc);
-    if ((rc = dev_alloc(s, (void**)&d.ctrl, sizeof(Ctrl)))) return fail(rc);
+    {
+        size_t at = 0;
+        auto carve = [&](size_t bytes) {
+            const size_t o = at;
+            at = (at + bytes + 255) / 256 * 256;
+            return o;
+        };
+        const size_t meta = carve((size_t)n * sizeof(uint4)), local = carve((size_t)n * sizeof(unsigned long long)),
+                     add = carve((size_t)n * sizeof(uint32_t)),
+                     results = carve(kResultsProc + (size_t)cfg->c * sizeof(unsigned long long));
+        s->core_bytes = at;
+        if ((rc = dev_alloc(s, &s->core, at))) return fail(rc);
+        unsigned char* p = static_cast<unsigned char*>(s->core);
+        d.meta = reinterpret_cast<uint4*>(p + meta);
+        d.local = reinterpret_cast<unsigned long long*>(p + local);
+        d.cnt_add = reinterpret_cast<uint32_t*>(p + add);
+        s->d_global = reinterpret_cast<double*>(p + results);
+        d.ctrl = reinterpret_cast<Ctrl*>(p + results + kResultsCtrl);
+        d.proc = reinterpret_cast<unsigned long long*>(p + results + kResultsProc);
+    }
     rc = dev_alloc(s, (void**)&d.pool, quads * 32ull);
     if (rc == REPT_E_NOMEM && colours == kColMulti) {  // the layout without colour words needs a third less
         colours = kColNone;
@@ -455,7 +484,6 @@ int rept_create(const rept_config* cfg, void* stream, rept_state** out) {
         rc = dev_alloc(s, (void**)&d.pool, quads * 32ull);
     }
     if (rc) return fail(rc);
-    if ((rc = dev_alloc(s, (void**)&s->d_global, sizeof(double)))) return fail(rc);
     d.pool_quads = quads;
     d.colours = colours;
     d.cbits = colours == kColMulti && one_colour ? 1u : cbits;
@@ -480,40 +508,23 @@ int rept_create(const rept_config* cfg, void* stream, rept_state** out) {
         if ((rc = ensure_pair_capacity(s, std::max<unsigned long long>(cfg->expected_edges, mb), st))) return fail(rc);
     }
     if ((rc = ensure_batch_scratch(s, mb, st))) return fail(rc);
-    if (cudaMallocHost((void**)&s->h_ctrl, sizeof(Ctrl)) != cudaSuccess) return fail(REPT_E_NOMEM);
-    if (cudaMallocHost((void**)&s->h_global, sizeof(double)) != cudaSuccess) return fail(REPT_E_NOMEM);
-    memset(s->h_ctrl, 0, sizeof(Ctrl));
-    if (cudaMemsetAsync(d.ctrl, 0, sizeof(Ctrl), st) != cudaSuccess) return fail(REPT_E_CUDA);
-    if (cudaMemsetAsync(d.pool, 0xFF, quads * 32ull, st) != cudaSuccess) return fail(REPT_E_CUDA);
+    if (cudaMallocHost((void**)&s->h_results, kResultsProc + (size_t)cfg->c * sizeof(uint64_t)) != cudaSuccess)
+        return fail(REPT_E_NOMEM);
+    s->h_global = reinterpret_cast<double*>(s->h_results);
+    s->h_ctrl = reinterpret_cast<Ctrl*>(s->h_results + kResultsCtrl);
     if ((rc = rept_reset(s, stream))) return fail(rc);
     if (cudaStreamSynchronize(st) != cudaSuccess) return fail(REPT_E_CUDA);
     *out = s;
     return REPT_OK;
 }
 
-// The pool itself is not cleared: blocks are handed out again from its start, and each new table
+// The pool itself is never cleared: blocks are handed out again from its start, and each new table
 // gets its empty keys when its block is handed out (init_table_keys and the shared-memory builds).
 int rept_reset(rept_state* s, void* stream) {
     if (!s) return REPT_E_INVAL;
-    cudaStream_t st = as_stream(stream);
-    StreamDev& d = s->d;
-    const size_t n = d.n_nodes;
-    REPT_CUDA(cudaMemsetAsync(d.meta, 0, n * sizeof(uint4), st));
-    REPT_CUDA(cudaMemsetAsync(d.cnt_add, 0, n * sizeof(uint32_t), st));
-    REPT_CUDA(cudaMemsetAsync(d.local, 0, n * sizeof(unsigned long long), st));
-    REPT_CUDA(cudaMemsetAsync(d.proc, 0, (size_t)d.c * sizeof(unsigned long long), st));
-    if (d.local2) REPT_CUDA(cudaMemsetAsync(d.local2, 0, n * sizeof(unsigned long long), st));
-    if (d.eta_local) REPT_CUDA(cudaMemsetAsync(d.eta_local, 0, n * sizeof(unsigned long long), st));
-    if (d.eta_proc) REPT_CUDA(cudaMemsetAsync(d.eta_proc, 0, (size_t)d.c * sizeof(unsigned long long), st));
-    if (d.pair_tau) {
-        REPT_CUDA(cudaMemsetAsync(d.pair_tau, 0, d.pair_cap * s->groups * sizeof(uint32_t), st));
-        REPT_CUDA(cudaMemsetAsync(d.pair_evt, 0, d.pair_cap * s->groups * sizeof(uint32_t), st));
-    }
-    if (d.local_proc) REPT_CUDA(cudaMemsetAsync(d.local_proc, 0, (size_t)d.c * n * sizeof(unsigned long long), st));
-    REPT_CUDA(cudaMemsetAsync(d.ctrl, 0, sizeof(Ctrl), st));
-    memset(s->h_ctrl, 0, sizeof(Ctrl));
-    s->next_t = 0;
-    return REPT_OK;
+    int rc = rept_reset_async(s, s->cfg.seed, stream);
+    if (!rc) memset(s->h_ctrl, 0, sizeof(Ctrl));
+    return rc;
 }
 
 int rept_reset_async(rept_state* s, uint64_t seed, void* stream) {
@@ -523,10 +534,7 @@ int rept_reset_async(rept_state* s, uint64_t seed, void* stream) {
     s->cfg.seed = seed;
     d.seed = seed;
     const size_t n = d.n_nodes;
-    REPT_CUDA(cudaMemsetAsync(d.meta, 0, n * sizeof(uint4), st));
-    REPT_CUDA(cudaMemsetAsync(d.cnt_add, 0, n * sizeof(uint32_t), st));
-    REPT_CUDA(cudaMemsetAsync(d.local, 0, n * sizeof(unsigned long long), st));
-    REPT_CUDA(cudaMemsetAsync(d.proc, 0, (size_t)d.c * sizeof(unsigned long long), st));
+    REPT_CUDA(cudaMemsetAsync(s->core, 0, s->core_bytes, st));
     if (d.local2) REPT_CUDA(cudaMemsetAsync(d.local2, 0, n * sizeof(unsigned long long), st));
     if (d.eta_local) REPT_CUDA(cudaMemsetAsync(d.eta_local, 0, n * sizeof(unsigned long long), st));
     if (d.eta_proc) REPT_CUDA(cudaMemsetAsync(d.eta_proc, 0, (size_t)d.c * sizeof(unsigned long long), st));
@@ -535,7 +543,6 @@ int rept_reset_async(rept_state* s, uint64_t seed, void* stream) {
         REPT_CUDA(cudaMemsetAsync(d.pair_evt, 0, d.pair_cap * s->groups * sizeof(uint32_t), st));
     }
     if (d.local_proc) REPT_CUDA(cudaMemsetAsync(d.local_proc, 0, (size_t)d.c * n * sizeof(unsigned long long), st));
-    REPT_CUDA(cudaMemsetAsync(d.ctrl, 0, sizeof(Ctrl), st));
     s->next_t = 0;
     return REPT_OK;
 }
@@ -589,24 +596,9 @@ int rept_ingest_host(rept_state* s, const uint32_t* h_src, const uint32_t* h_dst
 int rept_estimates(rept_state* s, double* h_global, double* d_local, void* stream) {
     if (!s || !h_global) return REPT_E_INVAL;
     cudaStream_t st = as_stream(stream);
-    int rc0 = enqueue_global_estimate(s, st);
-    if (rc0) return rc0;
-    if (d_local) {
-        if (s->d.local2) {
-            rc0 = timed_launch(s, REPT_K_ESTIMATE, st, [&] {
-                k_local_estimates_partial<<<s->sm_count * 4, 256, 0, st>>>(s->d.local, s->d.local2, s->d.eta_local,
-                                                                           s->d.n_nodes, s->cfg.m, s->cfg.c, d_local);
-            });
-        } else {
-            const double f = estimate_factor(s->cfg);
-            rc0 = timed_launch(s, REPT_K_ESTIMATE, st, [&] {
-                k_local_estimates<<<s->sm_count * 4, 256, 0, st>>>(s->d.local, s->d.n_nodes, f, d_local);
-            });
-        }
-        if (rc0) return rc0;
-    }
-    REPT_CUDA(cudaMemcpyAsync(s->h_global, s->d_global, sizeof(double), cudaMemcpyDeviceToHost, st));
-    int rc = sync_status(s, st);
+    int rc = enqueue_estimates(s, d_local, st);
+    if (rc) return rc;
+    rc = sync_status(s, st);
     *h_global = *s->h_global;
     return rc;
 }
@@ -614,7 +606,7 @@ int rept_estimates(rept_state* s, double* h_global, double* d_local, void* strea
 int rept_estimates_async(rept_state* s, double* h_global, uint64_t* h_proc, uint32_t* h_status, void* stream) {
     if (!s || !h_global || !h_status) return REPT_E_INVAL;
     cudaStream_t st = as_stream(stream);
-    int rc = enqueue_global_estimate(s, st);
+    int rc = enqueue_estimates(s, nullptr, st);
     if (rc) return rc;
     REPT_CUDA(cudaMemcpyAsync(h_global, s->d_global, sizeof(double), cudaMemcpyDeviceToHost, st));
     if (h_proc)
@@ -646,9 +638,6 @@ int rept_estimates_host(rept_state* s, double* h_global, double* h_local, void* 
 int rept_counts(rept_state* s, uint64_t* h_proc, uint64_t* d_local, void* stream) {
     if (!s) return REPT_E_INVAL;
     cudaStream_t st = as_stream(stream);
-    if (h_proc)
-        REPT_CUDA(cudaMemcpyAsync(h_proc, s->d.proc, (size_t)s->cfg.c * sizeof(uint64_t), cudaMemcpyDeviceToHost,
-                                  st));
     if (d_local) {
         if (s->d.local2) {
             k_add_local<<<s->sm_count * 4, 256, 0, st>>>(s->d.local, s->d.local2, s->d.n_nodes,
@@ -659,7 +648,9 @@ int rept_counts(rept_state* s, uint64_t* h_proc, uint64_t* d_local, void* stream
                                       cudaMemcpyDeviceToDevice, st));
         }
     }
-    return sync_status(s, st);
+    const int rc = sync_status(s, st, h_proc != nullptr);
+    if (h_proc && rc != REPT_E_CUDA) std::memcpy(h_proc, s->h_results + kResultsProc, (size_t)s->cfg.c * sizeof(uint64_t));
+    return rc;
 }
 
 namespace {
@@ -903,11 +894,7 @@ void rept_destroy(rept_state* s) {
     if (!s) return;
     cudaDeviceSynchronize();
     StreamDev& d = s->d;
-    cudaFree(d.meta);
-    cudaFree(d.cnt_add);
-    cudaFree(d.local);
-    cudaFree(d.proc);
-    cudaFree(d.ctrl);
+    cudaFree(s->core);
     cudaFree(d.pool);
     cudaFree(d.touched);
     cudaFree(d.grow_rel);
@@ -924,15 +911,13 @@ void rept_destroy(rept_state* s) {
     cudaFree(d.local_proc);
     cudaFree(s->stage_src);
     cudaFree(s->stage_dst);
-    cudaFree(s->d_global);
     cudaFree(s->d_local_tmp);
     for (auto& t : s->timed) {
         cudaEventDestroy(t.start);
         cudaEventDestroy(t.stop);
     }
     for (auto e : s->spare_events) cudaEventDestroy(e);
-    if (s->h_ctrl) cudaFreeHost(s->h_ctrl);
-    if (s->h_global) cudaFreeHost(s->h_global);
+    if (s->h_results) cudaFreeHost(s->h_results);
     delete s;
 }
 
@@ -1316,8 +1301,9 @@ int rept_estimates_from_counts(uint32_t m, uint32_t c, uint32_t flags, const uin
         int dev = 0, sms = 0;
         REPT_CUDA(cudaGetDevice(&dev));
         REPT_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        k_local_estimates<<<sms * 4, 256, 0, as_stream(stream)>>>(reinterpret_cast<const unsigned long long*>(d_local),
-                                                                   n_nodes, f, d_local_est);
+        k_estimates<<<sms * 4, 256, 0, as_stream(stream)>>>(nullptr, 0u,
+                                                             reinterpret_cast<const unsigned long long*>(d_local), n_nodes,
+                                                             f, nullptr, d_local_est);
         REPT_LAUNCHED();
     }
     return REPT_OK;

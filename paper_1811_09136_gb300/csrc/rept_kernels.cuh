@@ -292,12 +292,12 @@ __device__ __forceinline__ bool move_block_smem(uint32_t* to, const uint32_t* fr
 }
 
 // Publish the new entry counts of the touched nodes and move the blocks that were re-allocated: those
-// with new tables of at most kPartSlots slots here, four at a time by eight lanes each (a thread per node
+// with new tables of at most kPartSlots slots here, eight at a time by four lanes each (a thread per node
 // with global compare-and-swaps paid their latency once per entry); the others are left to k_rehash_big
 // (a warp each, new tables of at most kMoveSlots slots) or k_rehash_huge (a thread block each).  49 batches
 // of 4,096 edges: the three kernels took 2.1 ms with a thread per node, 1.8 ms so.
 // `smem`: kCommitSmemWords words.
-constexpr uint32_t kPartSlots = 64u, kPartLanes = 8u;
+constexpr uint32_t kPartSlots = 64u, kPartLanes = 4u;
 constexpr uint32_t kCommitSmemWords = 2u * (256u / kPartLanes) * kPartSlots;
 __device__ __forceinline__ void k_commit_body(const StreamDev& d, const Grid g, uint32_t* smem) {
     const unsigned status = d.ctrl->status;
@@ -1690,28 +1690,31 @@ __device__ __forceinline__ double combine_estimates(double t1, double t2, double
     return (w1 + w2 > 0.0) ? (w2 * t1 + w1 * t2) / (w1 + w2) : t1;
 }
 
-__global__ void k_global_estimate_partial(const unsigned long long* __restrict__ proc,
-                                          const unsigned long long* __restrict__ eta, uint32_t m, uint32_t c,
-                                          double* __restrict__ out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    const uint32_t c1 = c / m, c2 = c % m;
-    unsigned long long s1 = 0, s2 = 0, se = 0;
-    for (uint32_t i = 0; i < c1 * m; ++i) s1 += proc[i];
-    for (uint32_t i = c1 * m; i < c; ++i) s2 += proc[i];
-    for (uint32_t i = 0; i < c; ++i) se += eta[i];
-    const double md = (double)m;
-    const double t1 = (double)s1 * (md / (double)c1), t2 = (double)s2 * (md * md / (double)c2);
-    const double eta_hat = (double)se * (md * md * md / (double)c);
-    *out = combine_estimates(t1, t2, eta_hat, md, (double)c1, (double)c2);
-}
-
-__global__ void k_local_estimates_partial(const unsigned long long* __restrict__ l1,
-                                          const unsigned long long* __restrict__ l2,
-                                          const unsigned long long* __restrict__ el, uint32_t n, uint32_t m,
-                                          uint32_t c, double* __restrict__ out) {
+// tau_hat into *global (the first warp of the first block) and, with `out`, the local estimates.
+__global__ void k_estimates_partial(const unsigned long long* __restrict__ proc, const unsigned long long* __restrict__ eta,
+                                    const unsigned long long* __restrict__ l1, const unsigned long long* __restrict__ l2,
+                                    const unsigned long long* __restrict__ el, uint32_t n, uint32_t m, uint32_t c,
+                                    double* __restrict__ global, double* __restrict__ out) {
     const uint32_t c1 = c / m, c2 = c % m;
     const double md = (double)m;
-    for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
+    if (blockIdx.x == 0 && threadIdx.x < 32u) {
+        unsigned long long s1 = 0, s2 = 0, se = 0;
+        for (uint32_t i = threadIdx.x; i < c; i += 32u) {
+            if (i < c1 * m) s1 += proc[i]; else s2 += proc[i];
+            se += eta[i];
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            s1 += __shfl_down_sync(0xFFFFFFFFu, s1, o);
+            s2 += __shfl_down_sync(0xFFFFFFFFu, s2, o);
+            se += __shfl_down_sync(0xFFFFFFFFu, se, o);
+        }
+        if (threadIdx.x == 0) {
+            const double t1 = (double)s1 * (md / (double)c1), t2 = (double)s2 * (md * md / (double)c2);
+            const double eta_hat = (double)se * (md * md * md / (double)c);
+            *global = combine_estimates(t1, t2, eta_hat, md, (double)c1, (double)c2);
+        }
+    }
+    for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; out && v < n; v += gridDim.x * blockDim.x) {
         const double a1 = (double)l1[v] * (md / (double)c1), a2 = (double)l2[v] * (md * md / (double)c2);
         const double eh = (double)el[v] * (md * md * md / (double)c);
         out[v] = combine_estimates(a1, a2, eh, md, (double)c1, (double)c2);
@@ -2049,27 +2052,26 @@ __global__ void __launch_bounds__(256) k_convert(StreamDev d, const uint2* __res
     }
 }
 
-// tau_hat_v = f * sum_i tau_v^(i), f formed in double on the host.
-__global__ void k_local_estimates(const unsigned long long* __restrict__ local, uint32_t n, double f,
-                                  double* __restrict__ out) {
-    for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x)
-        out[v] = (double)local[v] * f;
-}
-
-// tau_hat = f * sum_{i < c_used} tau^(i); one block.
-__global__ void k_global_estimate(const unsigned long long* __restrict__ proc, uint32_t c_used, double f,
-                                  double* __restrict__ out) {
-    __shared__ unsigned long long part[32];
-    unsigned long long s = 0;
-    for (uint32_t i = threadIdx.x; i < c_used; i += blockDim.x) s += proc[i];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xFFFFFFFFu, s, o);
-    if ((threadIdx.x & 31u) == 0) part[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        s = threadIdx.x < (blockDim.x >> 5) ? part[threadIdx.x] : 0ull;
+// tau_hat = f * sum_{i < c_used} tau^(i) into *global (first block) and tau_hat_v = f * sum_i tau_v^(i) into
+// out, f formed in double on the host; either output may be NULL.
+__global__ void k_estimates(const unsigned long long* __restrict__ proc, uint32_t c_used,
+                            const unsigned long long* __restrict__ local, uint32_t n, double f,
+                            double* __restrict__ global, double* __restrict__ out) {
+    if (blockIdx.x == 0 && global) {
+        __shared__ unsigned long long part[32];
+        unsigned long long s = 0;
+        for (uint32_t i = threadIdx.x; i < c_used; i += blockDim.x) s += proc[i];
         for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xFFFFFFFFu, s, o);
-        if (threadIdx.x == 0) *out = (double)s * f;
+        if ((threadIdx.x & 31u) == 0) part[threadIdx.x >> 5] = s;
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            s = threadIdx.x < (blockDim.x >> 5) ? part[threadIdx.x] : 0ull;
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xFFFFFFFFu, s, o);
+            if (threadIdx.x == 0) *global = (double)s * f;
+        }
     }
+    for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; out && v < n; v += gridDim.x * blockDim.x)
+        out[v] = (double)local[v] * f;
 }
 
 }  // namespace

@@ -165,7 +165,7 @@ extern "C" int rept_count_noalloc(const uint32_t* d_src, const uint32_t* d_dst, 
     if (d_global) {
         const double md = (double)m;
         const double f = c <= m ? md * md / (double)c : md / (double)(c / m);
-        k_global_estimate<<<1, 256, 0, st>>>(d.proc, c, f, d_global);
+        k_estimates<<<1, 256, 0, st>>>(d.proc, c, nullptr, 0u, f, d_global, nullptr);
         NA_CUDA(cudaPeekAtLastError());
     }
     unsigned int status = 0;
