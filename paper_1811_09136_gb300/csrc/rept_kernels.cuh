@@ -867,7 +867,7 @@ __device__ __forceinline__ uint32_t count_groups(const StreamDev& d, uint32_t* h
 // scanned as inserted).  Entries that pass (0.6 % there; with several groups the common neighbours, 14 %
 // on the 4M-node stream) join the warp's candidate queue and are looked up in l's table, which decides
 // exactly.  R-MAT scale 20, m = c = 100: 8.83 ms per stream with a hash per entry, 5.51 ms so; the 4M-node
-// stream with five groups: 157 ms with a probe per entry, 122 ms so, of which the scans alone are 18 ms.
+// stream with five groups: 157 ms with a probe per entry, 114 ms so, of which the scans alone are 18 ms.
 // What bounds it: instruction issue (57 % of the slots) in the scans, the latency of the candidates'
 // dependent loads where many pass.
 
@@ -880,8 +880,10 @@ constexpr uint32_t kWarpFilterLg = 10;
 static_assert(kIxWarps << kWarpFilterLg <= kFilterWords, "warp filters share the block's");
 static_assert(kUnitItems == 64, "two records per lane of the first warp");
 
-// A warp's two queues, arrays of kCandQ and kMatchQ words.  Candidates: the position in the smaller endpoint's list
-// of an entry that passed a filter or colour test, its edge and, for groups, the stream.  Closed wedges:
+// A warp's two queues, arrays of kCandQ and kMatchQ words.  Candidates: the neighbour of an entry of the
+// smaller endpoint's list that passed a filter or colour test (queued as scanned, so that the probe need not
+// read the list again before it can form its address: five groups, 4M nodes, 122 to 114 ms), its edge, its
+// position in the list (where the stream index stands beside the list) and, for groups, the stream.  Closed wedges:
 // the neighbour, the edge, the agreeing groups and the colour word (kColMulti) and, for groups, the
 // stream; they are counted
 // 32 at a time so that the work runs on full warps.
@@ -892,8 +894,10 @@ struct WarpQueues {
 constexpr uint32_t kCandQ = 96, kMatchQ = 96;  // 63 + 32 candidates; 31 + 2 x 32 wedges
 // Arrays of closed wedges before the streams'.
 constexpr uint32_t match_arrays(int mode) { return mode == (int)kColMulti || mode == kColAny ? 4u : 2u; }
+// Arrays of candidates before the streams'.
+constexpr uint32_t cand_arrays(int mode) { return mode == (int)kColInEntry || mode == (int)kColWords ? 2u : 3u; }
 constexpr uint32_t queue_words(int mode, bool group) {
-    return (group ? 3u : 2u) * kCandQ + (match_arrays(mode) + (group ? 1u : 0u)) * kMatchQ;
+    return (cand_arrays(mode) + (group ? 1u : 0u)) * kCandQ + (match_arrays(mode) + (group ? 1u : 0u)) * kMatchQ;
 }
 
 // Shared memory of one intersection block, in words: the filter, the records of the unit's edges and the
@@ -955,9 +959,10 @@ __device__ __forceinline__ uint32_t cand_probe(const S& st, const uint32_t* cq, 
         for (int p = 0; p < 2; ++p) {
             const uint32_t k = min(32u * p + lane, take - 1u);
             v[p] = 32u * p + lane < take;
-            pos[p] = cq[k];
+            w[p] = cq[k];
             item[p] = cq[kCandQ + k];
-            sd[p] = GROUP ? cq[2u * kCandQ + k] : 0u;
+            pos[p] = cand_arrays(MODE) == 3u ? cq[2u * kCandQ + k] : 0u;
+            sd[p] = GROUP ? cq[cand_arrays(MODE) * kCandQ + k] : 0u;
         }
 #pragma unroll
         for (int p = 0; p < 2; ++p) {  // WorkItem: {s, l, off_s, off_l}, {t, lgs, cnt_s, cnt_l}
@@ -980,26 +985,18 @@ __device__ __forceinline__ uint32_t cand_probe(const S& st, const uint32_t* cq, 
             const StreamDev& d = st.at(sd[p]);
             const uint32_t col = colours_of<MODE>(d);
             as[p] = make_uint2(0u, 0u);
-            w[p] = 0u;
+            bk[p] = make_uint4(kEmptyId, kEmptyId, kEmptyId, kEmptyId);
+            h[p] = 0u;
             if (block_fits(d, 5, off[p].x, lgs[p]) && block_fits(d, 7, off[p].y, lgl[p]) &&
                 REPT_CHECK(d.ctrl, 3, pos[p], list_slots(lgs[p]))) {
-                const uint32_t* block_s = block_at(d.pool, off[p].x);
-                w[p] = block_s[list_at(lgs[p], col) + pos[p]] & id_mask(d);
-                if (col == kColNone) as[p].x = block_s[aux_at(lgs[p], col) + pos[p]];
-                if (col == kColMulti) as[p] = reinterpret_cast<const uint2*>(block_s + aux_at(lgs[p], col))[pos[p]];
+                h[p] = home_slot(w[p], lgl[p]);
+                bk[p] = __ldg(reinterpret_cast<const uint4*>(block_at(d.pool, off[p].y)) + key_quad(h[p], col));
+                const uint32_t* aux_s = block_at(d.pool, off[p].x) + aux_at(lgs[p], col);
+                if (col == kColNone) as[p].x = aux_s[pos[p]];
+                if (col == kColMulti) as[p] = reinterpret_cast<const uint2*>(aux_s)[pos[p]];
             } else {
                 v[p] = false;
-                lgl[p] = 2u;
             }
-        }
-#pragma unroll
-        for (int p = 0; p < 2; ++p) {
-            const StreamDev& d = st.at(sd[p]);
-            const uint32_t col = colours_of<MODE>(d);
-            h[p] = home_slot(w[p], lgl[p]);
-            bk[p] = make_uint4(kEmptyId, kEmptyId, kEmptyId, kEmptyId);
-            if (REPT_CHECK(d.ctrl, 7, off[p].y, d.pool_quads))
-                bk[p] = __ldg(reinterpret_cast<const uint4*>(block_at(d.pool, off[p].y)) + key_quad(h[p], col));
         }
 #pragma unroll
         for (int p = 0; p < 2; ++p) {
@@ -1073,10 +1070,10 @@ __device__ __forceinline__ void cand_flush(const S& st, WarpQueues& q, Work& wk,
     const unsigned lane = threadIdx.x & 31u;
     const uint32_t take = min(q.n, 64u), rest = q.n - take;
     __syncwarp();
-    q.closed = cand_probe<WORK, MODE>(st, q.base, q.base + (S::kGroup ? 3u : 2u) * kCandQ, take, q.closed, all, wk);
+    q.closed = cand_probe<WORK, MODE>(st, q.base, q.base + (cand_arrays(MODE) + (S::kGroup ? 1u : 0u)) * kCandQ, take, q.closed, all, wk);
     if (lane < rest) {  // rest < 32
 #pragma unroll
-        for (uint32_t a = 0; a < (S::kGroup ? 3u : 2u); ++a) q.base[a * kCandQ + lane] = q.base[a * kCandQ + 64u + lane];
+        for (uint32_t a = 0; a < cand_arrays(MODE) + (S::kGroup ? 1u : 0u); ++a) q.base[a * kCandQ + lane] = q.base[a * kCandQ + 64u + lane];
     }
     q.n = rest;
     __syncwarp();
@@ -1141,10 +1138,10 @@ __device__ __forceinline__ void filter_build(const StreamDev& d, uint32_t* filte
 
 // One step's passing entries join the warp's queue: bit b of a lane's m is the entry at position
 // base + 128 (b / 4) + b % 4 of edge `item`'s list of n entries (positions past its end are repeats of its
-// last quad).  One entry a lane at a time; a full round of 64 is probed.
-template <bool WORK, int MODE, class S>
+// last quad); word(b) yields its list word.  One entry a lane at a time; a full round of 64 is probed.
+template <bool WORK, int MODE, class S, class Word>
 __device__ __forceinline__ void queue_step(const S& st, WarpQueues& wq, uint32_t m, uint32_t base, uint32_t n,
-                                           uint32_t item, uint32_t sid, Work& wk) {
+                                           uint32_t item, uint32_t sid, Work& wk, Word&& word) {
     while (__any_sync(0xFFFFFFFFu, m != 0u)) {
         const uint32_t b = (uint32_t)__ffs((int)m) - 1u;  // (unused where m is 0)
         const uint32_t at = base + ((b >> 2) << 7) + (b & 3u);
@@ -1154,9 +1151,10 @@ __device__ __forceinline__ void queue_step(const S& st, WarpQueues& wq, uint32_t
         if (!S::kGroup && !REPT_CHECK(st.at(0u).ctrl, 13, wq.n + __popc(mask), (unsigned long long)kCandQ + 1ull)) return;
         if (has) {
             uint32_t* to = wq.base + wq.n + __popc(mask & ((1u << (threadIdx.x & 31u)) - 1u));
-            to[0] = at;
+            to[0] = word(b) & id_mask(st.at(sid));
             to[kCandQ] = item;
-            if (S::kGroup) to[2u * kCandQ] = sid;
+            if (cand_arrays(MODE) == 3u) to[2u * kCandQ] = at;
+            if (S::kGroup) to[cand_arrays(MODE) * kCandQ] = sid;
         }
         wq.n += __popc(mask);
         if (wq.n >= 64u) cand_flush<WORK, MODE>(st, wq, wk, false);
@@ -1168,6 +1166,10 @@ template <int MODE>
 __device__ __forceinline__ uint32_t test_quad(const uint32_t* filter, uint32_t lg, const uint4& q, const uint4& cw) {
     return filter_test(filter, lg, filter_hash<MODE>(q.x, cw.x)) | (filter_test(filter, lg, filter_hash<MODE>(q.y, cw.y)) << 1) |
            (filter_test(filter, lg, filter_hash<MODE>(q.z, cw.z)) << 2) | (filter_test(filter, lg, filter_hash<MODE>(q.w, cw.w)) << 3);
+}
+// Word b % 4 of a quad.
+__device__ __forceinline__ uint32_t quad_word(const uint4& q, uint32_t b) {
+    return b & 2u ? (b & 1u ? q.w : q.z) : (b & 1u ? q.y : q.x);
 }
 // Scan rows j0 .. j1 - 1 (32 quads, one per lane) of a list of n entries: four rows per step.  A lane past
 // the list's end reads its last quad again.
@@ -1186,7 +1188,7 @@ __device__ __forceinline__ void scan_rows(const S& st, uint32_t sid, const uint3
         uint4 q[4], cw[4];
 #pragma unroll
         for (uint32_t h = 0; h < 4u; ++h) {
-            cw[h] = make_uint4(0u, 0u, 0u, 0u);
+            q[h] = cw[h] = make_uint4(0u, 0u, 0u, 0u);
             if (h == 0u || j + h < j1) {  // (uniform)
                 const uint32_t at = min(32u * (j + h) + lane, last);
                 q[h] = list[at];
@@ -1197,7 +1199,10 @@ __device__ __forceinline__ void scan_rows(const S& st, uint32_t sid, const uint3
 #pragma unroll
         for (uint32_t h = 0; h < 4u; ++h)
             if (h == 0u || j + h < j1) m |= test_quad<MODE>(filter, lg, q[h], cw[h]) << (4u * h);
-        queue_step<WORK, MODE>(st, wq, m, 4u * (32u * j + lane), n, item, sid, wk);
+        queue_step<WORK, MODE>(st, wq, m, 4u * (32u * j + lane), n, item, sid, wk, [&](uint32_t b) {
+            const uint32_t w0 = quad_word(q[0], b), w1 = quad_word(q[1], b), w2 = quad_word(q[2], b), w3 = quad_word(q[3], b);
+            return b & 8u ? (b & 4u ? w3 : w2) : (b & 4u ? w1 : w0);
+        });
     }
 }
 // Rows of a list of n entries.
@@ -1251,7 +1256,8 @@ __device__ __forceinline__ void scan_short(const S& st, uint32_t sid, const uint
             for (uint32_t p = 0; p < 2u; ++p) {
                 const uint32_t mp = p ? m[1] : m[0], o = p ? own[1] : own[0], at = 4u * (p ? pos[1] : pos[0]);
                 const uint32_t on = __shfl_sync(0xFFFFFFFFu, n, o), oe = __shfl_sync(0xFFFFFFFFu, e, o);
-                queue_step<WORK, MODE>(st, wq, mp, at, on, oe, sid, wk);
+                const uint4 qp = p ? q[1] : q[0];
+                queue_step<WORK, MODE>(st, wq, mp, at, on, oe, sid, wk, [&](uint32_t b) { return quad_word(qp, b); });
             }
         }
     }
@@ -1431,7 +1437,7 @@ __device__ __forceinline__ void run_small_chunk(const S& st, uint32_t sid, uint3
                 const uint32_t oo = __shfl_sync(0xFFFFFFFFu, off_s, o), oc = __shfl_sync(0xFFFFFFFFu, cnt, o);
                 ol[p] = __shfl_sync(0xFFFFFFFFu, l, o);
                 word[p] = cw[p] = 0u;
-                if (v[p] && interleaved(col)) {
+                if (v[p]) {
                     const uint32_t lgs = table_lg(oc);
                     const uint32_t* block = block_at(d.pool, oo);
                     word[p] = block[list_at(lgs, col) + pos[p]];
@@ -1446,7 +1452,8 @@ __device__ __forceinline__ void run_small_chunk(const S& st, uint32_t sid, uint3
 #pragma unroll 1
             for (uint32_t p = 0; p < 2u; ++p)
                 queue_step<WORK, MODE>(st, wq, (p ? v[1] : v[0]) ? 1u : 0u, p ? pos[1] : pos[0], kEmptyId,
-                                       eb + (p ? own[1] : own[0]), sid, wk);
+                                       eb + (p ? own[1] : own[0]), sid, wk,
+                                       [&](uint32_t) { return p ? word[1] : word[0]; });
         }
     }
 }
