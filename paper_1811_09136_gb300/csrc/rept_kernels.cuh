@@ -88,6 +88,14 @@ __device__ __forceinline__ bool table_insert(uint32_t* table, uint32_t lg, uint3
     return false;
 }
 
+// First statement of every kernel of a single stream's batch.  Each but k_classify is launched as the programmatic
+// dependent of the one before it on its stream: its blocks may be set up while that one's last blocks still
+// run, and wait here until it (and so all that it waited for) has ended and its writes are visible.
+__device__ __forceinline__ void follow_previous() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // Has an earlier step failed?  The answer is the same for the whole block (another block may be setting
 // the status meanwhile), so that its threads meet at the same barriers.
 __device__ __forceinline__ bool block_failed(const Ctrl* c) {
@@ -1739,7 +1747,10 @@ __global__ void k_add_local(const unsigned long long* __restrict__ a, const unsi
 // descriptors are read from device arrays; blockIdx.x / gridDim.x then range over that stream's blocks).
 __device__ __forceinline__ Grid launch_grid() { return Grid{blockIdx.x, gridDim.x}; }
 
-__global__ void k_classify(StreamDev d, BatchDev b) { k_classify_body(d, b, launch_grid()); }
+__global__ void k_classify(StreamDev d, BatchDev b) {
+    follow_previous();
+    k_classify_body(d, b, launch_grid());
+}
 
 __global__ void k_classify_multi(const StreamDev* __restrict__ ds, const BatchDev* __restrict__ bs) {
     __shared__ StreamDev sd;
@@ -1752,7 +1763,10 @@ __global__ void k_classify_multi(const StreamDev* __restrict__ ds, const BatchDe
     k_classify_body(sd, sb, launch_grid());
 }
 
-__global__ void k_plan(StreamDev d) { k_plan_body(d, launch_grid()); }
+__global__ void k_plan(StreamDev d) {
+    follow_previous();
+    k_plan_body(d, launch_grid());
+}
 
 __global__ void k_plan_multi(const StreamDev* __restrict__ ds, const BatchDev* __restrict__ bs) {
     (void)bs;
@@ -1763,6 +1777,7 @@ __global__ void k_plan_multi(const StreamDev* __restrict__ ds, const BatchDev* _
 }
 
 __global__ void __launch_bounds__(256) k_commit(StreamDev d) {
+    follow_previous();
     __shared__ __align__(16) uint32_t smem[kCommitSmemWords];
     k_commit_body(d, launch_grid(), smem);
 }
@@ -1777,6 +1792,7 @@ __global__ void __launch_bounds__(256) k_commit_multi(const StreamDev* __restric
 }
 
 __global__ void __launch_bounds__(256) k_rehash_big(StreamDev d) {
+    follow_previous();
     __shared__ __align__(16) uint32_t smem[kMoveSmemWords];
     k_rehash_big_body(d, launch_grid(), smem);
 }
@@ -1794,6 +1810,7 @@ __global__ void __launch_bounds__(256) k_rehash_big_multi(const StreamDev* __res
 // Two blocks of 1024 threads per SM (32 registers a thread), so that the whole grid is resident.  Dynamic
 // shared memory: kHugeSmemWords words.
 __global__ void __launch_bounds__(1024, 2) k_rehash_huge(StreamDev d) {
+    follow_previous();
     extern __shared__ __align__(16) uint32_t hsmem[];
     k_rehash_huge_body(d, launch_grid(), hsmem, kBlockMoveSlots);
 }
@@ -1809,7 +1826,10 @@ __global__ void __launch_bounds__(1024, 2) k_rehash_huge_multi(const StreamDev* 
 }
 
 // 5 blocks of 256 threads per SM (48 registers).
-__global__ void __launch_bounds__(256, 5) k_insert(StreamDev d, BatchDev b) { k_insert_body(d, b, launch_grid()); }
+__global__ void __launch_bounds__(256, 5) k_insert(StreamDev d, BatchDev b) {
+    follow_previous();
+    k_insert_body(d, b, launch_grid());
+}
 
 __global__ void k_insert_multi(const StreamDev* __restrict__ ds, const BatchDev* __restrict__ bs) {
     __shared__ StreamDev sd;
@@ -1822,7 +1842,10 @@ __global__ void k_insert_multi(const StreamDev* __restrict__ ds, const BatchDev*
     k_insert_body(sd, sb, launch_grid());
 }
 
-__global__ void __launch_bounds__(256) k_units(StreamDev d, BatchDev b) { k_units_body(d, b, launch_grid()); }
+__global__ void __launch_bounds__(256) k_units(StreamDev d, BatchDev b) {
+    follow_previous();
+    k_units_body(d, b, launch_grid());
+}
 
 __global__ void __launch_bounds__(256) k_units_multi(const StreamDev* __restrict__ ds, const BatchDev* __restrict__ bs) {
     __shared__ StreamDev sd;
@@ -1835,7 +1858,10 @@ __global__ void __launch_bounds__(256) k_units_multi(const StreamDev* __restrict
     k_units_body(sd, sb, launch_grid());
 }
 
-__global__ void __launch_bounds__(256) k_order(StreamDev d, BatchDev b) { k_order_body(d, b, launch_grid()); }
+__global__ void __launch_bounds__(256) k_order(StreamDev d, BatchDev b) {
+    follow_previous();
+    k_order_body(d, b, launch_grid());
+}
 
 __global__ void __launch_bounds__(256) k_order_multi(const StreamDev* __restrict__ ds, const BatchDev* __restrict__ bs) {
     __shared__ StreamDev sd;
@@ -1862,6 +1888,7 @@ __device__ __forceinline__ void cluster_barrier() {
 }
 
 __global__ void __cluster_dims__(kStateBlocks, 1, 1) __launch_bounds__(kStateThreads, 1) k_state(StreamDev d, BatchDev b) {
+    follow_previous();
     extern __shared__ __align__(16) uint32_t hsmem[];
     const Grid g = launch_grid();
     k_classify_body(d, b, g);
@@ -1999,6 +2026,7 @@ __global__ void __launch_bounds__(256, 3) k_group_persistent(const StreamDev* __
 // Streams whose entries carry their colour (one hash group, m <= 256).
 template <bool WORK>
 __global__ void __launch_bounds__(kIxThreads, kIxBlocks) k_intersect(StreamDev d, BatchDev b) {
+    follow_previous();
     k_intersect_body<WORK, (int)kColInEntry>(d, b);
 }
 
@@ -2006,18 +2034,21 @@ __global__ void __launch_bounds__(kIxThreads, kIxBlocks) k_intersect(StreamDev d
 // or more than 2^24 nodes).
 template <bool WORK>
 __global__ void __launch_bounds__(kIxThreads, kIxBlocks) k_intersect_words(StreamDev d, BatchDev b) {
+    follow_previous();
     k_intersect_body<WORK, (int)kColWords>(d, b);
 }
 
 // Streams of several hash groups, with a colour word beside every stream index.
 template <bool WORK>
 __global__ void __launch_bounds__(kIxThreads, kIxBlocks) k_intersect_multi(StreamDev d, BatchDev b) {
+    follow_previous();
     k_intersect_body<WORK, (int)kColMulti>(d, b);
 }
 
 // Streams without stored colours (too many hash groups for a word, or too little memory for one).
 template <bool WORK>
 __global__ void __launch_bounds__(kIxThreads, kIxBlocks) k_intersect_probe(StreamDev d, BatchDev b) {
+    follow_previous();
     k_intersect_body<WORK, (int)kColNone>(d, b);
 }
 
