@@ -189,7 +189,7 @@ struct Ctrl {
     unsigned long long self_loops;
     unsigned long long stored;      // stored (kept) edges
     unsigned int status;
-    unsigned int pad;
+    unsigned int n_giant;  // nodes whose table k_rehash_huge moves in pieces, many blocks each
     // work counters of k_intersect<true> (see rept_stats)
     unsigned long long small_entries, small_slots, probes, probe_slots, wedges, counted;
     unsigned long long class_items[kClasses], class_probes[kClasses], class_cycles[kClasses];
@@ -199,8 +199,8 @@ struct Ctrl {
     unsigned long long bin_count[kBins];   // small chunks and units of each kind
     unsigned long long bin_next[kBins];    // claimed so far
     unsigned long long n_pairs;  // entries of pair_list this batch
-    unsigned long long n_big;   // nodes whose table (32..2048 slots) k_rehash_big moves, a warp each
-    unsigned long long n_huge;  // nodes whose table (>= 4096 slots) k_rehash_huge moves, a block each
+    unsigned long long n_big;   // nodes whose table k_rehash_big moves, a warp each
+    unsigned long long n_huge;  // nodes whose table k_rehash_huge moves, a block each
     unsigned long long huge_next;
     unsigned long long dbg[4];  // REPT_DEBUG_BOUNDS builds: first failed check {site, index, bound}, count
 };

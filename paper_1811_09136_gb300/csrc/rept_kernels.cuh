@@ -244,15 +244,21 @@ __device__ __forceinline__ void init_table_keys(uint32_t* table, uint32_t lg, ui
 }
 
 // New tables of at most kMoveSlots slots are rebuilt in shared memory by a warp (k_rehash_big), those
-// of at most kBlockMoveSlots by a thread block (k_rehash_huge); larger ones are built in place.
+// of at most kBlockMoveSlots by a thread block (k_rehash_huge); larger ones are built in place, each by
+// kGiantPieces thread blocks, for a table that one block moves is longer under way than the rest of a
+// batch's moves together.  Commit and moves, one block for each table against so: R-MAT scale 20 1.73 and
+// 1.62 ms (15 batches), 1.5M edges in batches of 65,536 1.19 and 0.92 ms, 2M edges with hubs of 170,000 0.86
+// and 0.41 ms (with the limit at 16,384 slots 1.60, 0.95 and 0.44; at 32,768 1.60, 1.04 and 0.50).
 constexpr uint32_t kMoveSlots = 512;
-constexpr uint32_t kBlockMoveSlots = 32768;
+constexpr uint32_t kBlockMoveSlots = 8192;
+constexpr uint32_t kGiantPieces = 16;
 constexpr uint32_t kHugeSmemWords = kBlockMoveSlots / 2u;  // a 16-bit word per slot
 
 // move_block with the new table built in shared memory (keys and, per key, its stream index or with
 // kColMulti its list position; 2^lg_new slots, the same placement rule as table_insert) and then written
-// out with coalesced stores, by the lanes `rank` of `width` of one warp.  The new block is the caller's alone until the batch's inserts run.  Parts of a
-// warp may each move a node at the same time; an inactive part takes part in the barriers only.
+// out with coalesced stores, by the lanes `rank` of `width` of one warp.  The new block is the caller's alone
+// until the batch's inserts run.  Parts of a warp may each move a node at the same time; an inactive part
+// takes part in the barriers only.
 __device__ __forceinline__ bool move_block_smem(uint32_t* to, const uint32_t* from, uint32_t cnt_old, uint32_t lg_new,
                                                 uint32_t colours, uint32_t* s_keys, uint32_t* s_aux, uint32_t rank,
                                                 uint32_t width, bool active = true) {
@@ -359,9 +365,44 @@ __device__ __forceinline__ void k_commit_body(const StreamDev& d, const Grid g, 
         }
         const unsigned long long o = warp_reserve_one(&d.ctrl->n_big, defer);
         if (defer) d.big[o] = (uint32_t)i;
+        if (huge && (1u << lg_new) > kBlockMoveSlots) {
+            // listed in the memory that the batch's larger endpoints and their edges use later; what does not
+            // fit there (batches of a few edges) is moved by one block
+            const uint32_t k = atomicAdd(&d.ctrl->n_giant, 1u);
+            if (k < d.unit_cap) {
+                d.glist[k] = (uint32_t)i;
+                d.order[k] = 0u;  // pieces that are done
+                huge = false;
+            }
+        }
         const unsigned long long h = warp_reserve_one(&d.ctrl->n_huge, huge);
         if (huge) d.big[d.big_cap - 1 - h] = (uint32_t)i;
     }
+}
+
+// The move of the i-th touched node's block.
+struct Move {
+    uint32_t x, cnt_old, cnt_new, lg_new, off_new;
+    uint32_t *to, *from;
+    bool fits;
+};
+__device__ __forceinline__ Move move_of(const StreamDev& d, uint32_t i, unsigned long long top) {
+    Move mv;
+    mv.x = d.touched[i];
+    const uint4 m = d.meta[mv.x];
+    const unsigned long long off = top + d.grow_rel[i];
+    mv.cnt_old = m.y;
+    mv.cnt_new = m.y + touched_adds(d)[i];
+    mv.lg_new = table_lg(mv.cnt_new);
+    mv.off_new = (uint32_t)off;
+    mv.fits = block_fits(d, 10, m.x, table_lg(m.y)) && block_fits(d, 11, off, mv.lg_new);
+    mv.to = block_at(d.pool, off);
+    mv.from = block_at(d.pool, m.x);
+    return mv;
+}
+// Nodes listed for moves in pieces.
+__device__ __forceinline__ unsigned long long n_giants(const StreamDev& d) {
+    return min((unsigned long long)d.ctrl->n_giant, (unsigned long long)d.unit_cap);
 }
 
 // Move the blocks listed by k_commit whose new table has at most kMoveSlots slots: one warp per node.
@@ -370,31 +411,30 @@ __device__ __forceinline__ void k_commit_body(const StreamDev& d, const Grid g, 
 constexpr uint32_t kMoveSmemWords = 2u * 8u * kMoveSlots;
 __device__ __forceinline__ void k_rehash_big_body(const StreamDev& d, const Grid g, uint32_t* smem) {
     const unsigned long long n_big = d.ctrl->n_big, top = d.ctrl->pool_top;
+    // the tables that k_rehash_huge builds in place start with empty keys
+    for (unsigned long long p = g.bx; p < n_giants(d) * kGiantPieces; p += g.nbx) {
+        const Move mv = move_of(d, d.glist[p / kGiantPieces], top);
+        if (mv.fits)
+            init_table_keys(mv.to, mv.lg_new, d.colours, (uint32_t)(p % kGiantPieces) * blockDim.x + threadIdx.x,
+                            kGiantPieces * blockDim.x);
+    }
     const unsigned lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
     const unsigned long long warps = ((unsigned long long)g.nbx * blockDim.x) >> 5;
     for (unsigned long long k = ((unsigned long long)g.bx * blockDim.x + threadIdx.x) >> 5; k < n_big;
          k += warps) {
-        const uint32_t i = d.big[k];
-        const uint32_t x = d.touched[i];
-        const uint4 m = d.meta[x];
-        const uint32_t cnt_new = m.y + touched_adds(d)[i];
-        const unsigned long long new_off = top + d.grow_rel[i];
-        const bool fits = block_fits(d, 10, m.x, table_lg(m.y)) && block_fits(d, 11, new_off, table_lg(cnt_new));
-        const uint32_t lg_new = table_lg(cnt_new);
-        uint32_t* to = block_at(d.pool, new_off);
-        const uint32_t* from = block_at(d.pool, m.x);
+        const Move mv = move_of(d, d.big[k], top);
         bool ok = true;
-        if (fits && (1u << lg_new) <= kMoveSlots && REPT_CHECK(d.ctrl, 14, wid, 32u))
-            ok = move_block_smem(to, from, m.y, lg_new, d.colours, smem + wid * 2u * kMoveSlots,
+        if (mv.fits && (1u << mv.lg_new) <= kMoveSlots && REPT_CHECK(d.ctrl, 14, wid, 32u))
+            ok = move_block_smem(mv.to, mv.from, mv.cnt_old, mv.lg_new, d.colours, smem + wid * 2u * kMoveSlots,
                                  smem + (wid * 2u + 1u) * kMoveSlots, lane, 32u);
-        else if (fits) {
-            init_table_keys(to, lg_new, d.colours, lane, 32u);
+        else if (mv.fits) {
+            init_table_keys(mv.to, mv.lg_new, d.colours, lane, 32u);
             __syncwarp();
-            ok = move_block(to, from, m.y, lg_new, d.colours, lane, 32u);
+            ok = move_block(mv.to, mv.from, mv.cnt_old, mv.lg_new, d.colours, lane, 32u);
         }
         if (!ok) atomicOr(&d.ctrl->status, kStInternal);
         __syncwarp();
-        if (lane == 0) d.meta[x] = make_uint4((uint32_t)new_off, cnt_new, 0u, 0u);
+        if (lane == 0) d.meta[mv.x] = make_uint4(mv.off_new, mv.cnt_new, 0u, 0u);
     }
 }
 
@@ -463,12 +503,13 @@ __device__ __forceinline__ bool move_block_index(uint32_t* to, const uint32_t* f
 }
 
 // Move the blocks listed by k_commit whose new table has more than kMoveSlots slots: thread blocks
-// claim one node at a time, and build tables of at most max_slots slots in shared memory (`smem`: as many
-// 16-bit words), larger ones in place.
+// claim pieces of the largest, then one node at a time, and build tables of at most max_slots slots in
+// shared memory (`smem`: as many 16-bit words), larger ones in place.
 __device__ __forceinline__ void k_rehash_huge_body(const StreamDev& d, const Grid g, uint32_t* smem, uint32_t max_slots) {
     __shared__ unsigned long long s_k;
     __shared__ int s_bad;
-    const unsigned long long n_huge = d.ctrl->n_huge, top = d.ctrl->pool_top;
+    const unsigned long long pieces = n_giants(d) * kGiantPieces;
+    const unsigned long long n_work = pieces + d.ctrl->n_huge, top = d.ctrl->pool_top;
     for (;;) {
         if (threadIdx.x == 0) {
             s_k = atomicAdd(&d.ctrl->huge_next, 1ull);
@@ -476,29 +517,27 @@ __device__ __forceinline__ void k_rehash_huge_body(const StreamDev& d, const Gri
         }
         __syncthreads();
         const unsigned long long k = s_k;
-        if (k >= n_huge) break;
-        const uint32_t i = d.big[d.big_cap - 1 - k];
-        const uint32_t x = d.touched[i];
-        const uint4 m = d.meta[x];
-        const uint32_t cnt_new = m.y + touched_adds(d)[i];
-        const unsigned long long new_off = top + d.grow_rel[i];
-        const bool fits = block_fits(d, 10, m.x, table_lg(m.y)) && block_fits(d, 11, new_off, table_lg(cnt_new));
-        const uint32_t lg_new = table_lg(cnt_new);
-        uint32_t* to = block_at(d.pool, new_off);
-        const uint32_t* from = block_at(d.pool, m.x);
+        if (k >= n_work) break;
+        const uint32_t giant = (uint32_t)(k / kGiantPieces);
+        const Move mv = move_of(d, k < pieces ? d.glist[giant] : d.big[d.big_cap - 1 - (k - pieces)], top);
         bool ok = true;
-        if (fits && (1u << lg_new) <= max_slots)  // uniform over the block
-            ok = move_block_index(to, from, m.y, lg_new, d.colours, reinterpret_cast<uint16_t*>(smem));
-        else if (fits) {  // (uniform over the block) built in place: empty keys first
-            init_table_keys(to, lg_new, d.colours, threadIdx.x, blockDim.x);
+        if (mv.fits && k < pieces) {  // (uniform over the block)
+            ok = move_block(mv.to, mv.from, mv.cnt_old, mv.lg_new, d.colours,
+                            (uint32_t)(k % kGiantPieces) * blockDim.x + threadIdx.x, kGiantPieces * blockDim.x);
+        } else if (mv.fits && (1u << mv.lg_new) <= max_slots) {
+            ok = move_block_index(mv.to, mv.from, mv.cnt_old, mv.lg_new, d.colours, reinterpret_cast<uint16_t*>(smem));
+        } else if (mv.fits) {  // built in place: empty keys first
+            init_table_keys(mv.to, mv.lg_new, d.colours, threadIdx.x, blockDim.x);
             __syncthreads();
-            ok = move_block(to, from, m.y, lg_new, d.colours, threadIdx.x, blockDim.x);
+            ok = move_block(mv.to, mv.from, mv.cnt_old, mv.lg_new, d.colours, threadIdx.x, blockDim.x);
         }
         if (!ok) s_bad = 1;
         __syncthreads();
         if (threadIdx.x == 0) {
             if (s_bad) atomicOr(&d.ctrl->status, kStInternal);
-            d.meta[x] = make_uint4((uint32_t)new_off, cnt_new, 0u, 0u);
+            // the record changes when every piece has read it
+            if (k >= pieces || atomicAdd(&d.order[giant], 1u) == kGiantPieces - 1u)
+                d.meta[mv.x] = make_uint4(mv.off_new, mv.cnt_new, 0u, 0u);
         }
         __syncthreads();
     }
@@ -514,6 +553,7 @@ __device__ __forceinline__ void k_insert_body(const StreamDev& d, const BatchDev
         ct->n_touched = 0;
         ct->n_big = 0;
         ct->n_huge = 0;
+        ct->n_giant = 0;
         ct->huge_next = 0;
     }
     if (failed) return;
@@ -1964,7 +2004,7 @@ struct PersistShape {
 
 // Dynamic shared memory of the persistent kernel: the larger of the block moves' and the group
 // intersection's needs.
-static_assert(ix_words(kColAny, true) * 2u >= kBlockMoveSlots / 2u, "the block moves fit");
+static_assert(ix_words(kColAny, true) >= kHugeSmemWords, "the block moves fit");
 constexpr uint32_t kPersistSmemWords = kMoveSmemWords > ix_words(kColAny, true) ? kMoveSmemWords : ix_words(kColAny, true);
 
 __global__ void __launch_bounds__(256, 3) k_group_persistent(const StreamDev* __restrict__ ds,
@@ -2004,7 +2044,7 @@ __global__ void __launch_bounds__(256, 3) k_group_persistent(const StreamDev* __
     ok = ok && grid_barrier(gs, wait_ns);
     if (ok) step(sh.x_big, [&](Grid g) { k_rehash_big_body(sd, g, psmem); });
     ok = ok && grid_barrier(gs, wait_ns);
-    if (ok) step(sh.x_huge, [&](Grid g) { k_rehash_huge_body(sd, g, psmem, kBlockMoveSlots / 2u); });
+    if (ok) step(sh.x_huge, [&](Grid g) { k_rehash_huge_body(sd, g, psmem, kBlockMoveSlots); });
     ok = ok && grid_barrier(gs, wait_ns);
     if (ok) step(sh.x_edge, [&](Grid g) { k_insert_body(sd, sb, g); });
     ok = ok && grid_barrier(gs, wait_ns);
