@@ -6,8 +6,9 @@
 
 The stream is ingested once in batches of --batch edges into a handle whose pool grows as needed, so
 that the device holds little beyond the state the stream needs.  Kernel launches per batch follow
-the library's launch order (classify, plan, commit, two block-move kernels, insert, two sort
-kernels, intersect), which is what a profiler's launch skip count (-s) refers to.  With --mix N the
+the library's launch order (classify, plan, commit, two block-move kernels, insert, units, order,
+intersect; batches of at most 8,192 edges into a pool known to be large enough: one state kernel, intersect),
+which is what a profiler's launch skip count (-s) refers to.  With --mix N the
 first N streams of the batched workload's mix (seed 1000) are counted instead, each with its own
 m = c and hash seed, through one rept_group (--mode group: one launch per step for all streams;
 persistent: one cooperative launch per round) or one stream after the other (--mode plain).
