@@ -334,7 +334,7 @@ int launch_batch(rept_state* s, const uint32_t* d_src, const uint32_t* d_dst, un
         const int prc = ensure_pair_capacity(s, s->next_t + n, st);
         if (prc) return prc;
     }
-    const BatchDev b = make_batch(d_src, d_dst, n, s->next_t, s->tile_max);
+    const BatchDev b = make_batch(d_src, d_dst, n, s->next_t, s->tile_max, n);
     const int threads = 256;
     const unsigned long long want_blocks = (n + threads - 1) / threads;
     const int grid = (int)std::min<unsigned long long>(want_blocks, (unsigned long long)s->grid_stream);
@@ -1166,6 +1166,7 @@ int rept_group_ingest(rept_group* g, rept_state* const* hs, const uint32_t* cons
     cudaStream_t st = as_stream(stream);
     unsigned long long max_n = 0;
     bool guaranteed = true;
+    unsigned long long round = 0;
     for (uint32_t i = 0; i < k; ++i) {
         rept_state* s = hs[i];
         if (!s || s->d.local2) return REPT_E_INVAL;  // c mod m != 0 is served by the single-stream path
@@ -1174,6 +1175,7 @@ int rept_group_ingest(rept_group* g, rept_state* const* hs, const uint32_t* cons
         int rc = ensure_batch_scratch(s, std::max<unsigned long long>(n[i], 1ull), st);
         if (rc) return rc;
         max_n = std::max<unsigned long long>(max_n, n[i]);
+        round += n[i];
         const bool fixed = (s->cfg.flags & REPT_FLAG_FIXED_POOL) != 0;
         if (!fixed && s->d.pool_quads < quads_bound(s->next_t + n[i], s->d.colours)) guaranteed = false;
     }
@@ -1196,7 +1198,7 @@ int rept_group_ingest(rept_group* g, rept_state* const* hs, const uint32_t* cons
     BatchDev* hbd = g->h_bd[slot];
     for (uint32_t i = 0; i < k; ++i) {
         hsd[i] = hs[i]->d;
-        hbd[i] = make_batch(d_src[i], d_dst[i], n[i], hs[i]->next_t, hs[i]->tile_max);
+        hbd[i] = make_batch(d_src[i], d_dst[i], n[i], hs[i]->next_t, hs[i]->tile_max, round);
     }
     auto upload = [&]() -> int {
         REPT_CUDA(cudaMemcpyAsync(g->d_sd, hsd, k * sizeof(StreamDev), cudaMemcpyHostToDevice, st));

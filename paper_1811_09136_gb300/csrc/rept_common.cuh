@@ -315,16 +315,20 @@ struct BatchDev {
     unsigned long long t0;  // stream index of src[0], dst[0]
     uint32_t small_max;     // edges whose smaller endpoint has more entries are grouped
     uint32_t chunk;         // edges of a small chunk
+    uint32_t unit_edges;    // edges of a block unit
 };
 
 // A batch of a stream.  Grouping pays through the lists that share a filter; in a small batch few do, and
 // what counts is the chain of dependent steps, so nearly all edges stay small (`tile_max`: the handle's
-// bound for the others) and are dealt out in smaller chunks.
+// bound for the others) and are dealt out in smaller chunks.  Block units hold fewer edges in smaller
+// batches, so that there are units for every SM; the batches of a group's round (`round` edges together) fill
+// the GPU together and so share their filters among more (48 streams, 65,536 edges each a round: 48.3 ms with
+// units by the stream's own batch, 46.7 ms so).
 inline BatchDev make_batch(const uint32_t* src, const uint32_t* dst, unsigned long long n, unsigned long long t0,
-                           uint32_t tile_max) {
+                           uint32_t tile_max, unsigned long long round) {
     const bool few = n < kSmallBatch;
-    return BatchDev{src, dst, n, t0, few ? kSmallBatchMax : tile_max,
-                    few ? std::max((uint32_t)(n >> 10), 4u) : 64u};
+    return BatchDev{src, dst, n, t0, few ? kSmallBatchMax : tile_max, few ? std::max((uint32_t)(n >> 10), 4u) : 64u,
+                    (uint32_t)std::min(std::max(round >> 14, 16ull), (unsigned long long)kUnitItems)};
 }
 
 // Index checks of the REPT_DEBUG_BOUNDS build (a stand-in for a memory checker): a failed check

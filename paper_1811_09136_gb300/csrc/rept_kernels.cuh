@@ -673,8 +673,6 @@ __device__ __forceinline__ void k_units_body(const StreamDev& d, const BatchDev&
     if (ct->status) return;
     const unsigned lane = threadIdx.x & 31u;
     const unsigned long long n_g = ct->n_groups;
-    // edges per block unit: fewer in smaller batches, so that there are units for every SM
-    const uint32_t per_block = (uint32_t)min(max(b.n >> 14, 16ull), (unsigned long long)kUnitItems);
     const unsigned long long stride = (unsigned long long)g.nbx * blockDim.x;
     for (unsigned long long base = (unsigned long long)g.bx * blockDim.x + threadIdx.x - lane; base < n_g;
          base += stride) {
@@ -688,7 +686,7 @@ __device__ __forceinline__ void k_units_body(const StreamDev& d, const BatchDev&
             count = m.w;
             kind = m.y > kBigUnitNodes ? kBinBig : m.y > kWarpUnitNodes ? kBinBlock : kBinWarp;
             // (an edge's smaller list is no longer than the larger: at most kWarpUnitEntries per warp unit)
-            per = kind == kBinWarp ? min(max(kWarpUnitEntries / m.y, 1u), kWarpUnitItems) : per_block;
+            per = kind == kBinWarp ? min(max(kWarpUnitEntries / m.y, 1u), kWarpUnitItems) : b.unit_edges;
         }
         const uint32_t first = (uint32_t)warp_reserve(&ct->n_items, count);
         if (i < n_g) d.meta[l].w = first;

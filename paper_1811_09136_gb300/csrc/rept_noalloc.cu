@@ -141,7 +141,7 @@ extern "C" int rept_count_noalloc(const uint32_t* d_src, const uint32_t* d_dst, 
         int dev = 0, sms = 0;
         NA_CUDA(cudaGetDevice(&dev));
         NA_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        const BatchDev b = make_batch(d_src, d_dst, n_edges, 0ull, 32u);
+        const BatchDev b = make_batch(d_src, d_dst, n_edges, 0ull, 32u, n_edges);
         const int threads = 256;
         const unsigned long long blocks = (n_edges + threads - 1) / threads;
         const int grid = (int)(blocks < (unsigned long long)sms * 8 ? blocks : (unsigned long long)sms * 8);
