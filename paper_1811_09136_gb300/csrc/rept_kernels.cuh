@@ -1936,7 +1936,7 @@ __global__ void __cluster_dims__(kStateBlocks, 1, 1) __launch_bounds__(kStateThr
     k_commit_body(d, g, hsmem);
     cluster_barrier();
     k_rehash_big_body(d, g, hsmem);
-    __syncthreads();
+    cluster_barrier();  // the tables that k_rehash_huge builds in place are emptied by every block, and filled by any
     k_rehash_huge_body(d, g, hsmem, kBlockMoveSlots);
     cluster_barrier();
     k_insert_body(d, b, g);
