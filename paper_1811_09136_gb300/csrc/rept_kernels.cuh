@@ -1921,8 +1921,10 @@ constexpr uint32_t kStateSmemWords = 2u * (kStateThreads / 32u) * kMoveSlots;
 static_assert(kStateSmemWords >= kHugeSmemWords && kStateSmemWords >= kCommitSmemWords * (kStateThreads / 256u),
               "the steps share the memory");
 
+// (not the .aligned forms: the steps end in code that the lanes of a warp leave at different times, and those
+// forms are undefined for a warp that has not met again)
 __device__ __forceinline__ void cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
 __global__ void __cluster_dims__(kStateBlocks, 1, 1) __launch_bounds__(kStateThreads, 1) k_state(StreamDev d, BatchDev b) {

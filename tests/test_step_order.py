@@ -37,3 +37,9 @@ def test_all_blocks_meet_between_the_steps_of_one_launch(kernel, barrier):
     for step, following in zip(STEPS, STEPS[1:]):
         between = order[order.index(step) + 1:order.index(following)]
         assert between == [barrier], f"{kernel}: {step} and {following} are separated by {between}"
+
+
+def test_cluster_barrier_takes_warps_that_have_not_met():
+    """The steps end in divergent code; the .aligned barrier is undefined for such a warp."""
+    body = function_body(kernels_source(), "cluster_barrier")
+    assert "barrier.cluster.arrive.release;" in body and "barrier.cluster.wait.acquire;" in body
