@@ -722,7 +722,7 @@ __device__ __forceinline__ void k_order_body(const StreamDev& d, const BatchDev&
 // Look neighbour w up in the table of 2^lg slots at `table` (lg >= 2): read 4-key buckets from w's
 // home bucket on until w or an empty key shows up.  Returns w's slot, or kEmptyId when w is absent;
 // `slots` receives the number of keys read.
-__device__ __forceinline__ uint32_t table_slot(const uint32_t* __restrict__ table, uint32_t lg, uint32_t w,
+__device__ __forceinline__ uint32_t table_slot(const uint32_t* table, uint32_t lg, uint32_t w,
                                                uint32_t& slots, uint32_t colours) {
     const uint32_t mask = (1u << lg) - 1u;
     const uint4* buckets = reinterpret_cast<const uint4*>(table);
@@ -741,7 +741,7 @@ __device__ __forceinline__ uint32_t table_slot(const uint32_t* __restrict__ tabl
 }
 
 // w's stream index in that table, or kEmptyId.
-__device__ __forceinline__ uint32_t table_find(const uint32_t* __restrict__ table, uint32_t lg, uint32_t w,
+__device__ __forceinline__ uint32_t table_find(const uint32_t* table, uint32_t lg, uint32_t w,
                                                uint32_t& slots, uint32_t colours) {
     const uint32_t h = table_slot(table, lg, w, slots, colours);
     return h == kEmptyId ? kEmptyId : table[eidx_word(h, lg, colours)];
@@ -1036,7 +1036,9 @@ __device__ __forceinline__ uint32_t cand_probe(const S& st, const uint32_t* cq, 
             if (block_fits(d, 5, off[p].x, lgs[p]) && block_fits(d, 7, off[p].y, lgl[p]) &&
                 REPT_CHECK(d.ctrl, 3, pos[p], list_slots(lgs[p]))) {
                 h[p] = home_slot(w[p], lgl[p]);
-                bk[p] = __ldg(reinterpret_cast<const uint4*>(block_at(d.pool, off[p].y)) + key_quad(h[p], col));
+                // (a plain load: this kernel may be set up while the inserts still write the pool, and a group's
+                // persistent launch writes it itself, so the read-only path is not open to it)
+                bk[p] = reinterpret_cast<const uint4*>(block_at(d.pool, off[p].y))[key_quad(h[p], col)];
                 const uint32_t* aux_s = block_at(d.pool, off[p].x) + aux_at(lgs[p], col);
                 if (col == kColNone) as[p].x = aux_s[pos[p]];
                 if (col == kColMulti) as[p] = reinterpret_cast<const uint2*>(aux_s)[pos[p]];
@@ -1594,8 +1596,7 @@ __device__ __forceinline__ void k_intersect_body(const StreamDev& d, const Batch
 // Per kind c: pref[c * (k + 1) + i] = sum of the counts of streams < i; cursors reset.  One
 // block of any multiple of 32 threads up to 1024.
 __device__ __forceinline__ void group_prefix_body(const StreamDev* __restrict__ ds, uint32_t k,
-                                                  unsigned long long* __restrict__ pref,
-                                                  unsigned long long* __restrict__ cursor) {
+                                                  unsigned long long* pref, unsigned long long* cursor) {
     __shared__ unsigned long long warp_sum[32];
     __shared__ unsigned long long carry;
     const uint32_t tid = threadIdx.x, lane = tid & 31u, wid = tid >> 5, warps = blockDim.x >> 5;
@@ -1643,7 +1644,7 @@ __global__ void __launch_bounds__(1024) k_group_prefix(const StreamDev* __restri
 }
 
 // Stream of item `i`: the last stream whose prefix is <= i.
-__device__ __forceinline__ uint32_t group_stream_search(const unsigned long long* __restrict__ pc, uint32_t k,
+__device__ __forceinline__ uint32_t group_stream_search(const unsigned long long* pc, uint32_t k,
                                                         unsigned long long i) {
     uint32_t lo = 0, hi = k - 1;  // pc[0] = 0 <= i
     while (lo < hi) {
@@ -1656,8 +1657,8 @@ __device__ __forceinline__ uint32_t group_stream_search(const unsigned long long
 // MODE: the colour storage of every stream, or kColAny.
 template <int MODE>
 __device__ __forceinline__ void intersect_group_body(const StreamDev* __restrict__ ds, const BatchDev* __restrict__ bs,
-                                                     uint32_t k, const unsigned long long* __restrict__ pref,
-                                                     unsigned long long* __restrict__ cursor, uint32_t* smem) {
+                                                     uint32_t k, const unsigned long long* pref,
+                                                     unsigned long long* cursor, uint32_t* smem) {
     const unsigned lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
     uint32_t* filter = smem;
     uint4* items = reinterpret_cast<uint4*>(filter + kFilterWords);
@@ -2013,8 +2014,8 @@ constexpr uint32_t kPersistSmemWords = kMoveSmemWords > ix_words(kColAny, true) 
 
 __global__ void __launch_bounds__(256, 3) k_group_persistent(const StreamDev* __restrict__ ds,
                                                            const BatchDev* __restrict__ bs, uint32_t k,
-                                                           PersistShape sh, unsigned long long* __restrict__ pref,
-                                                           unsigned long long* __restrict__ cursor, GroupSync* gs,
+                                                           PersistShape sh, unsigned long long* pref,
+                                                           unsigned long long* cursor, GroupSync* gs,
                                                            unsigned long long wait_ns) {
     extern __shared__ __align__(16) uint32_t psmem[];
     __shared__ StreamDev sd;

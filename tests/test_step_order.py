@@ -43,3 +43,16 @@ def test_cluster_barrier_takes_warps_that_have_not_met():
     """The steps end in divergent code; the .aligned barrier is undefined for such a warp."""
     body = function_body(kernels_source(), "cluster_barrier")
     assert "barrier.cluster.arrive.release;" in body and "barrier.cluster.wait.acquire;" in body
+
+
+def test_memory_that_a_launch_writes_is_not_read_through_the_read_only_path():
+    """The intersection may be resident while the inserts write the pool, and the persistent kernel writes the
+    pool and the prefixes itself: neither may be read with loads for data that stays unwritten throughout."""
+    source = kernels_source()
+    assert not re.search(r"__ldg\b|\.global\.nc", source)
+    for name in ("table_slot", "table_find", "group_prefix_body", "intersect_group_body", "group_stream_search",
+                 "k_group_persistent"):
+        params = re.search(r"\b%s\((.*?)\)\s*\{" % name, source, re.S).group(1)
+        for param in params.split(","):
+            if re.search(r"\b(table|pref|cursor|pc)$", param):
+                assert "__restrict__" not in param, f"{name}: {param.strip()}"
