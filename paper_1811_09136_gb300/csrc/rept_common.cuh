@@ -525,27 +525,29 @@ __device__ __forceinline__ unsigned long long warp_reserve_one(unsigned long lon
 // The same for a thread block (at most 32 warps; every thread calls it): one atomic per block.  The
 // atomics of a grid on one counter follow each other about 1.3 ns apart, so a warp's each for 2^20
 // edges takes 40 us.  `part`: shared memory of the caller, two of them used in turn need no barrier
-// between calls.
+// between calls.  Sum: wide enough for the sum of a block's requests.
+template <class Sum>
 struct BlockReserve {
-    uint32_t warp[32];
+    Sum warp[32];
     unsigned long long base;
 };
-__device__ __forceinline__ unsigned long long block_reserve(BlockReserve& part, unsigned long long* ctr, uint32_t inc) {
+template <class Sum>
+__device__ __forceinline__ unsigned long long block_reserve(BlockReserve<Sum>& part, unsigned long long* ctr, uint32_t inc) {
     const unsigned lane = threadIdx.x & 31u, wid = threadIdx.x >> 5, warps = blockDim.x >> 5;
-    uint32_t incl = inc;
+    Sum incl = inc;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        const Sum y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
         if (lane >= (unsigned)o) incl += y;
     }
     if (lane == 31) part.warp[wid] = incl;
     __syncthreads();
     if (wid == 0) {
-        const uint32_t w = lane < warps ? part.warp[lane] : 0u;
-        uint32_t wi = w;
+        const Sum w = lane < warps ? part.warp[lane] : 0u;
+        Sum wi = w;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, wi, o);
+            const Sum y = __shfl_up_sync(0xFFFFFFFFu, wi, o);
             if (lane >= (unsigned)o) wi += y;
         }
         part.warp[lane] = wi - w;

@@ -124,7 +124,7 @@ __device__ __forceinline__ void k_classify_body(const StreamDev& d, const BatchD
         d.ctrl->n_items = 0ull;
     }
     if (block_failed(d.ctrl)) return;
-    __shared__ BlockReserve part[2];
+    __shared__ BlockReserve<uint32_t> part[2];
     uint32_t turn = 0;
     const unsigned long long stride = (unsigned long long)g.nbx * blockDim.x;
     for (unsigned long long base = (unsigned long long)g.bx * blockDim.x; base < b.n; base += stride) {
@@ -151,7 +151,8 @@ __device__ __forceinline__ void k_classify_body(const StreamDev& d, const BatchD
 
 __device__ __forceinline__ void k_plan_body(const StreamDev& d, const Grid g) {
     if (block_failed(d.ctrl)) return;
-    __shared__ BlockReserve part[2];
+    // (whole block sizes: those of a few hundred large hubs together pass 2^32 quads)
+    __shared__ BlockReserve<unsigned long long> part[2];
     uint32_t turn = 0;
     const unsigned long long n_t = d.ctrl->n_touched;
     const unsigned long long stride = (unsigned long long)g.nbx * blockDim.x;
@@ -557,7 +558,7 @@ __device__ __forceinline__ void k_insert_body(const StreamDev& d, const BatchDev
         ct->huge_next = 0;
     }
     if (failed) return;
-    __shared__ BlockReserve part[2];
+    __shared__ BlockReserve<uint32_t> part[2];
     uint32_t turn = 0;
     const unsigned lane = threadIdx.x & 31u;
     const unsigned long long stride = (unsigned long long)g.nbx * blockDim.x;
