@@ -466,9 +466,20 @@ __host__ __device__ __forceinline__ uint32_t list_slots(uint32_t lg) { return lg
 __host__ __device__ __forceinline__ uint32_t word_slots(uint32_t lg) { return lg >= 4u ? (1u << (lg - 2u)) : 4u; }
 __host__ __device__ __forceinline__ uint32_t block_quads(uint32_t lg, uint32_t colours) {
     const uint32_t slots = (1u << lg) + list_slots(lg);
-    if (colours == kColMulti) return (3u * slots + 7u) >> 3;
+    if (colours == kColMulti) return (uint32_t)((3ull * slots + 7ull) >> 3);
     return (slots + (colours == kColWords ? word_slots(lg) : 0u)) >> 2;
 }
+
+// Word offset of the list inside a block with a table of 2^lg slots, of the stream indices or pairs beside
+// it (kColNone, kColMulti), and of its colour words (kColWords).  In 64 bits, like every offset that passes
+// a table's keys: a block of 2^30 slots (a node of more than 2^28 entries) is longer than 2^32 words.
+__host__ __device__ __forceinline__ uint64_t list_at(uint32_t lg, uint32_t colours) {
+    return (colours == kColMulti ? 3ull : 2ull) << lg;
+}
+__host__ __device__ __forceinline__ uint64_t aux_at(uint32_t lg, uint32_t colours) {
+    return list_at(lg, colours) + list_slots(lg);
+}
+__host__ __device__ __forceinline__ uint64_t cw_at(uint32_t lg) { return 2ull * ((1u << lg) + list_slots(lg)); }
 
 // Work-counter class of an edge whose smaller endpoint holds cnt entries (rept_stats.class_*).
 __host__ __device__ __forceinline__ int bin_of_cnt(uint32_t cnt) {
@@ -489,9 +500,9 @@ __device__ __forceinline__ uint32_t home_slot(uint32_t w, uint32_t lg) {
 __host__ __device__ __forceinline__ uint32_t key_word(uint32_t h, uint32_t colours) {
     return interleaved(colours) ? (((h >> 2) << 3) | (h & 3u)) : h;
 }
-__host__ __device__ __forceinline__ uint32_t eidx_word(uint32_t h, uint32_t lg, uint32_t colours) {
+__host__ __device__ __forceinline__ uint64_t eidx_word(uint32_t h, uint32_t lg, uint32_t colours) {
     return interleaved(colours) ? key_word(h, colours) + 4u
-                                : (1u << lg) + (colours == kColMulti ? 2u * h : h);
+                                : (1u << lg) + (colours == kColMulti ? 2ull * h : h);
 }
 __host__ __device__ __forceinline__ uint32_t key_quad(uint32_t h, uint32_t colours) {
     return interleaved(colours) ? h >> 1 : h >> 2;

@@ -36,13 +36,6 @@ __device__ __forceinline__ uint32_t* block_at(uint2* pool, unsigned long long of
 __device__ __forceinline__ const uint32_t* block_at(const uint2* pool, unsigned long long off_quads) {
     return reinterpret_cast<const uint32_t*>(pool) + 8ull * off_quads;
 }
-// Word offset of the list inside a block with a table of 2^lg slots, of the stream indices or pairs
-// beside it (kColNone, kColMulti), and of its colour words (kColWords).
-__device__ __forceinline__ uint32_t list_at(uint32_t lg, uint32_t colours) {
-    return (colours == kColMulti ? 3u : 2u) << lg;
-}
-__device__ __forceinline__ uint32_t aux_at(uint32_t lg, uint32_t colours) { return list_at(lg, colours) + list_slots(lg); }
-__device__ __forceinline__ uint32_t cw_at(uint32_t lg) { return 2u * ((1u << lg) + list_slots(lg)); }
 
 // A node's table of 2^lg slots at `table` holds 2^lg neighbour ids (keys; probed a 4-key, 16-byte
 // bucket at a time) and, per id, its stream index (and colour word), laid out as key_word and eidx_word
@@ -1266,7 +1259,7 @@ __device__ __forceinline__ void scan_short(const S& st, uint32_t sid, const uint
     const unsigned lane = threadIdx.x & 31u;
     const uint32_t col = colours_of<MODE>(d), lgs = table_lg(n);
     const bool has_cw = MODE == (int)kColWords || (MODE == kColAny && col == kColWords);
-    const uint32_t list_off = off_s + (list_at(lgs, col) >> 3);  // in 32-byte units (n > 4: a whole number)
+    const uint32_t list_off = off_s + (uint32_t)(list_at(lgs, col) >> 3);  // in 32-byte units (n > 4: a whole number)
     const uint32_t quads = (n + 3u) >> 2;
     uint32_t incl = quads;
 #pragma unroll
