@@ -148,8 +148,13 @@ typedef struct rept_state rept_state;
  * n_nodes <= 2^24, else in a word beside it, 25 % more pool), and only
  * neighbours that two endpoints share with the same colour are looked up;
  * with several hash groups every shared neighbour is, and its colours are
- * compared through a stored word (50 % more pool; hashed again where the
- * groups' colours do not fit 32 bits or the larger pool cannot be had).
+ * compared through a stored word (50 % more pool).  The groups' colours are
+ * hashed again instead where they do not fit 32 bits, where the pool for
+ * expected_edges is beyond the 2^32 - 1 blocks of 32 bytes that offsets span
+ * with the words (about 357 million edges; 536 million without) or the memory
+ * for it cannot be had, and from the batch on that takes a growing pool past
+ * either limit (or past 3/7 of the memory that it could have): the blocks are
+ * then rebuilt without words, once, and stay so.
  */
 int rept_create(const rept_config* cfg, void* stream, rept_state** out);
 

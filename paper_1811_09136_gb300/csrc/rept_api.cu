@@ -52,6 +52,7 @@ struct rept_state {
     int sm_count = 0;
     uint32_t groups = 1;
     uint32_t tile_max = 32;
+    uint32_t wide = kColNone;  // widest_colours of the configuration; d.colours is that or, for kColMulti, kColNone
     StreamDev d{};
     unsigned long long max_batch = 0;
     unsigned long long next_t = 0;  // stream index of the next edge
@@ -80,7 +81,20 @@ struct rept_state {
 
 namespace {
 
+// The quads of a pool and the bytes of a handle, at most: the bounds-checked build, which the tests use, takes
+// smaller limits from the environment.
+unsigned long long limit(const char* name, unsigned long long most) {
+#ifdef REPT_DEBUG_BOUNDS
+    if (const char* v = std::getenv(name)) return std::strtoull(v, nullptr, 10);
+#endif
+    (void)name;
+    return most;
+}
+unsigned long long max_quads() { return limit("REPT_DEBUG_MAX_QUADS", kMaxQuads); }
+unsigned long long max_bytes() { return limit("REPT_DEBUG_MAX_BYTES", ~0ull); }
+
 int dev_alloc(rept_state* s, void** p, size_t bytes) {
+    if (s->device_bytes + bytes > max_bytes()) return REPT_E_NOMEM;
     REPT_CUDA(cudaMalloc(p, bytes));
     s->device_bytes += bytes;
     return REPT_OK;
@@ -93,16 +107,8 @@ void dev_free(rept_state* s, void* p, size_t bytes) {
     }
 }
 
-// Pool quads that guarantee no batch can run out: a node's block holds at most 2 quads per entry (3 with
-// colour words: at one entry, less beyond), and its successive blocks form a doubling series bounded by
-// twice the last one, so at most 4 (6) quads per stored entry, i.e. 8 (12) per stream edge.
-unsigned long long quads_bound(unsigned long long edges, uint32_t colours) {
-    return (colours == kColWords || colours == kColMulti ? 12ull : 8ull) * edges + 64ull;
-}
-
 int grow_pool(rept_state* s, unsigned long long min_quads, cudaStream_t st) {
-    unsigned long long want = std::max(min_quads, 2ull * s->d.pool_quads);
-    if (want > 0xFFFFFFFFull) want = 0xFFFFFFFFull;  // offsets are 32-bit quads
+    const unsigned long long want = std::min(std::max(min_quads, 2ull * s->d.pool_quads), max_quads());
     if (want < min_quads) return REPT_E_CAPACITY;
     uint2* np = nullptr;
     int rc = dev_alloc(s, (void**)&np, want * 32ull);
@@ -139,6 +145,70 @@ size_t intersect_smem(uint32_t colours, uint32_t c) {
 template <class K>
 cudaError_t allow_smem(K* kernel, size_t bytes) {
     return cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+// The intersection grid: as many blocks as fit at once, for the variant this stream uses.
+int set_intersect_grid(rept_state* s) {
+    const uint32_t col = s->d.colours;
+    const void* k3 = col == kColInEntry ? (const void*)k_intersect<false>
+                     : col == kColWords ? (const void*)k_intersect_words<false>
+                     : col == kColMulti ? (const void*)k_intersect_multi<false> : (const void*)k_intersect_probe<false>;
+    int per_sm = 0;
+    REPT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k3, kIxThreads, intersect_smem(col, s->cfg.c)));
+    s->grid_intersect = s->sm_count * std::max(per_sm, 1);
+    return REPT_OK;
+}
+
+// Take the handle's blocks over into a pool of at least `least` quads (as far as offsets reach) in the layout
+// `to`, kColNone or kColMulti, with half as much again as they and the batch under way need.  Between a
+// batch's k_plan and its k_commit, whose requests are made again, or between batches.  Synchronises.  When it
+// fails between batches, the handle is as it was.
+int relayout(rept_state* s, uint32_t to, unsigned long long least, cudaStream_t st) {
+    const StreamDev old = s->d;
+    StreamDev& d = s->d;
+    REPT_CUDA(cudaMemsetAsync(&d.ctrl->need_quads, 0, sizeof(d.ctrl->need_quads), st));
+    REPT_CUDA(cudaMemsetAsync(&d.ctrl->layout_quads, 0, sizeof(d.ctrl->layout_quads), st));
+    d.colours = to;
+    k_plan_again<<<s->grid_stream, 256, 0, st>>>(d);
+    REPT_LAUNCHED();
+    k_layout_quads<<<s->grid_stream, 256, 0, st>>>(d);
+    REPT_LAUNCHED();
+    int rc = read_ctrl(s, st);
+    const unsigned long long need = s->h_ctrl->layout_quads + s->h_ctrl->need_quads;
+    const unsigned long long want = std::min(std::max(need + need / 2 + 1024, least), max_quads());
+    uint2* np = nullptr;
+    if (!rc && want < need) rc = REPT_E_CAPACITY;
+    if (!rc) rc = dev_alloc(s, (void**)&np, want * 32ull);
+    if (rc) {
+        d = old;
+        return rc;
+    }
+    d.pool = np;
+    d.pool_quads = want;
+    REPT_CUDA(cudaMemsetAsync(&d.ctrl->pool_top, 0, sizeof(d.ctrl->pool_top), st));
+    k_relayout<<<s->grid_stream, 256, 0, st>>>(d, old.pool, old.pool_quads, old.colours);
+    REPT_LAUNCHED();
+    REPT_CUDA(cudaStreamSynchronize(st));
+    dev_free(s, old.pool, old.pool_quads * 32ull);
+    return set_intersect_grid(s);
+}
+
+// Make room for a batch whose new blocks take `need` quads beyond the `top` that are in use (after its
+// k_plan, with the stream idle).  Blocks with the colour words of several groups give them up rather than be
+// refused a larger pool (words_fit).
+int make_room(rept_state* s, unsigned long long top, unsigned long long need, cudaStream_t st) {
+    const unsigned long long min_quads = top + need + (top + need) / 2 + 1024;
+    s->h_ctrl->pool_top = top;
+    if (s->d.colours != kColMulti) return grow_pool(s, min_quads, st);
+    size_t free_bytes = 0, all_bytes = 0;
+    REPT_CUDA(cudaMemGetInfo(&free_bytes, &all_bytes));
+    const unsigned long long own = s->d.pool_quads * 32ull;
+    const unsigned long long memory = std::min<unsigned long long>(free_bytes, max_bytes() - s->device_bytes) + own;
+    if (words_fit(std::max(min_quads, 2ull * s->d.pool_quads), memory, max_quads())) {
+        const int rc = grow_pool(s, min_quads, st);
+        if (rc != REPT_E_NOMEM) return rc;
+    }
+    return relayout(s, kColNone, s->d.pool_quads / 3ull * 4ull, st);
 }
 
 int ensure_batch_scratch(rept_state* s, unsigned long long n, cudaStream_t st) {
@@ -309,7 +379,7 @@ int launch_steps(rept_state* s, const BatchDev& b, int grid, int threads, bool p
         if ((rc = read_ctrl(s, st))) return rc;
         const unsigned long long need = s->h_ctrl->pool_top + s->h_ctrl->need_quads;
         if (s->h_ctrl->status == 0u && need > s->d.pool_quads) {
-            if ((rc = grow_pool(s, need + need / 2 + 1024, st))) return rc;
+            if ((rc = make_room(s, s->h_ctrl->pool_top, s->h_ctrl->need_quads, st))) return rc;
         }
     }
     if ((rc = timed_launch(s, REPT_K_COMMIT, st, [&] {
@@ -406,24 +476,9 @@ int sync_status(rept_state* s, cudaStream_t st, bool proc = false) {
     return status_to_code(s->h_ctrl->status);
 }
 
-
-}  // namespace
-
-extern "C" {
-
-int rept_create(const rept_config* cfg, void* stream, rept_state** out) {
-    if (!cfg || !out) return REPT_E_INVAL;
-    *out = nullptr;
-    if (cfg->m == 0 || cfg->c == 0 || cfg->n_nodes == 0 || cfg->n_nodes == 0xFFFFFFFFu) return REPT_E_INVAL;
-    if (cfg->c > kMaxProcessors) return REPT_E_INVAL;
-    if (cfg->tile_max != 0 && cfg->tile_max != 4 && cfg->tile_max != 8 && cfg->tile_max != 16 &&
-        cfg->tile_max != 32)
-        return REPT_E_INVAL;
-    if (cfg->reserved != 0 || cfg->reserved2 != 0) return REPT_E_INVAL;
+// Makes the handle; without `words` a stream of several groups stores no colour words.
+int create_state(const rept_config* cfg, void* stream, bool words, rept_state** out) {
     const bool sharded = cfg->proc_begin != 0 || cfg->proc_end != 0;
-    if (sharded && (cfg->proc_begin >= cfg->proc_end || cfg->proc_end > cfg->c)) return REPT_E_INVAL;
-    if (sharded && !(cfg->flags & REPT_FLAG_MASCOT) && cfg->c > cfg->m && cfg->c % cfg->m != 0)
-        return REPT_E_INVAL;  // Algorithm 2's combination needs every processor's counts
     cudaStream_t st = as_stream(stream);
     rept_state* s = new (std::nothrow) rept_state();
     if (!s) return REPT_E_NOMEM;
@@ -436,19 +491,13 @@ int rept_create(const rept_config* cfg, void* stream, rept_state** out) {
     if (cudaGetDevice(&s->device) != cudaSuccess) return fail(REPT_E_CUDA);
     if (cudaDeviceGetAttribute(&s->sm_count, cudaDevAttrMultiProcessorCount, s->device) != cudaSuccess)
         return fail(REPT_E_CUDA);
-    // how list entries carry colours, and the intersection grid: as many blocks as fit at once, for
-    // the variant this stream uses
-    const bool mascot_flag = (cfg->flags & REPT_FLAG_MASCOT) != 0;
-    const uint32_t n_groups = mascot_flag ? cfg->c : (cfg->c + cfg->m - 1) / cfg->m;
+    const unsigned long long mb = cfg->max_batch ? cfg->max_batch : (1ull << 20);
+    const unsigned long long sized_for = cfg->expected_edges ? cfg->expected_edges : mb;
     uint32_t cbits = 0;
-    while (cbits < 32 && (1ull << cbits) < cfg->m) ++cbits;
-    const bool coloured = n_groups == 1 && cfg->m >= 2 && cfg->m <= 256 && cfg->n_nodes <= (1u << kIdBits);
-    // colour words: one group that cannot carry its colour in the entries
-    const bool words = !coloured && !mascot_flag && cfg->m >= 2 && n_groups == 1;
-    // several groups: their colours in one word, or a bit per group where a group keeps one colour only
-    const bool one_colour = mascot_flag || cfg->m == 1;
-    const bool multi = !coloured && !words && n_groups * (one_colour ? 1ull : cbits) <= 32ull;
-    uint32_t colours = coloured ? kColInEntry : words ? kColWords : multi ? kColMulti : kColNone;
+    s->wide = widest_colours(cfg->m, cfg->c, cfg->n_nodes, (cfg->flags & REPT_FLAG_MASCOT) != 0, cbits);
+    // a pool with room for the stream that offsets do not span is made without the words
+    const bool spanned = quads_bound(sized_for, kColMulti) <= max_quads();
+    const uint32_t colours = s->wide != kColMulti || (words && spanned) ? s->wide : kColNone;
     const size_t max_smem = intersect_smem(kColMulti, kMaxProcessors);
     if (allow_smem(k_state, kStateSmemWords * sizeof(uint32_t)) != cudaSuccess ||
         allow_smem(k_rehash_huge, kHugeSmemWords * sizeof(uint32_t)) != cudaSuccess ||
@@ -460,13 +509,6 @@ int rept_create(const rept_config* cfg, void* stream, rept_state** out) {
         allow_smem(k_intersect_probe<false>, max_smem) != cudaSuccess ||
         allow_smem(k_intersect_probe<true>, max_smem) != cudaSuccess)
         return fail(REPT_E_CUDA);
-    const void* k3 = coloured ? (const void*)k_intersect<false>
-                     : words ? (const void*)k_intersect_words<false>
-                     : multi ? (const void*)k_intersect_multi<false> : (const void*)k_intersect_probe<false>;
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k3, kIxThreads, intersect_smem(colours, cfg->c)) != cudaSuccess)
-        return fail(REPT_E_CUDA);
-    s->grid_intersect = s->sm_count * std::max(per_sm, 1);
     s->grid_stream = s->sm_count * 8;
     const bool mascot = (cfg->flags & REPT_FLAG_MASCOT) != 0;
     s->groups = mascot ? cfg->c : cfg->c <= cfg->m ? 1u : (cfg->c + cfg->m - 1) / cfg->m;
@@ -479,11 +521,7 @@ int rept_create(const rept_config* cfg, void* stream, rept_state** out) {
     d.seed = cfg->seed;
     d.fm = make_fastmod(cfg->m);
     s->tile_max = cfg->tile_max == 0 ? 32u : cfg->tile_max;
-    const unsigned long long mb = cfg->max_batch ? cfg->max_batch : (1ull << 20);
-    auto wanted_quads = [&] {
-        return std::min(quads_bound(cfg->expected_edges ? cfg->expected_edges : mb, colours), 0xFFFFFFFFull);
-    };
-    unsigned long long quads = wanted_quads();
+    const unsigned long long quads = std::min(quads_bound(sized_for, colours), max_quads());
     {
         size_t at = 0;
         auto carve = [&](size_t bytes) {
@@ -504,17 +542,12 @@ int rept_create(const rept_config* cfg, void* stream, rept_state** out) {
         d.ctrl = reinterpret_cast<Ctrl*>(p + results + kResultsCtrl);
         d.proc = reinterpret_cast<unsigned long long*>(p + results + kResultsProc);
     }
-    rc = dev_alloc(s, (void**)&d.pool, quads * 32ull);
-    if (rc == REPT_E_NOMEM && colours == kColMulti) {  // the layout without colour words needs a third less
-        colours = kColNone;
-        quads = wanted_quads();
-        rc = dev_alloc(s, (void**)&d.pool, quads * 32ull);
-    }
-    if (rc) return fail(rc);
+    if ((rc = dev_alloc(s, (void**)&d.pool, quads * 32ull))) return fail(rc);
     d.pool_quads = quads;
     d.colours = colours;
-    d.cbits = colours == kColMulti && one_colour ? 1u : cbits;
-    d.cmask = (uint32_t)((1ull << d.cbits) - 1ull);
+    d.cbits = cbits;
+    d.cmask = (uint32_t)((1ull << cbits) - 1ull);
+    if ((rc = set_intersect_grid(s))) return fail(rc);
     d.c1 = mascot || cfg->c <= cfg->m ? cfg->c : cfg->c / cfg->m;
     d.keep = mascot ? 1u : cfg->m;
     d.pstride = mascot ? 1u : cfg->m;
@@ -522,7 +555,7 @@ int rept_create(const rept_config* cfg, void* stream, rept_state** out) {
     d.pcount = sharded ? cfg->proc_end - cfg->proc_begin : cfg->c;
     d.kbeg = d.pbeg / d.pstride;
     d.kend = (d.pbeg + d.pcount - 1u) / d.pstride + 1u;
-    for (uint32_t k = d.kbeg; colours == kColMulti && k < d.kend; ++k) d.ctop |= 1u << ((k + 1u) * d.cbits - 1u);
+    for (uint32_t k = d.kbeg; s->wide == kColMulti && k < d.kend; ++k) d.ctop |= 1u << ((k + 1u) * d.cbits - 1u);
     if (cfg->flags & REPT_FLAG_LOCAL_PER_PROCESSOR) {
         if ((rc = dev_alloc(s, (void**)&d.local_proc, (size_t)cfg->c * n * sizeof(unsigned long long))))
             return fail(rc);
@@ -543,6 +576,29 @@ int rept_create(const rept_config* cfg, void* stream, rept_state** out) {
     if (cudaStreamSynchronize(st) != cudaSuccess) return fail(REPT_E_CUDA);
     *out = s;
     return REPT_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+int rept_create(const rept_config* cfg, void* stream, rept_state** out) {
+    if (!cfg || !out) return REPT_E_INVAL;
+    *out = nullptr;
+    if (cfg->m == 0 || cfg->c == 0 || cfg->n_nodes == 0 || cfg->n_nodes == 0xFFFFFFFFu) return REPT_E_INVAL;
+    if (cfg->c > kMaxProcessors) return REPT_E_INVAL;
+    if (cfg->tile_max != 0 && cfg->tile_max != 4 && cfg->tile_max != 8 && cfg->tile_max != 16 &&
+        cfg->tile_max != 32)
+        return REPT_E_INVAL;
+    if (cfg->reserved != 0 || cfg->reserved2 != 0) return REPT_E_INVAL;
+    const bool sharded = cfg->proc_begin != 0 || cfg->proc_end != 0, mascot = (cfg->flags & REPT_FLAG_MASCOT) != 0;
+    if (sharded && (cfg->proc_begin >= cfg->proc_end || cfg->proc_end > cfg->c)) return REPT_E_INVAL;
+    if (sharded && !mascot && cfg->c > cfg->m && cfg->c % cfg->m != 0)
+        return REPT_E_INVAL;  // Algorithm 2's combination needs every processor's counts
+    const int rc = create_state(cfg, stream, true, out);
+    uint32_t bits;
+    if (rc != REPT_E_NOMEM || widest_colours(cfg->m, cfg->c, cfg->n_nodes, mascot, bits) != kColMulti) return rc;
+    return create_state(cfg, stream, false, out);  // the layout without colour words needs a third less
 }
 
 // The pool itself is never cleared: blocks are handed out again from its start, and each new table
@@ -1187,9 +1243,12 @@ int rept_group_ingest(rept_group* g, rept_state* const* hs, const uint32_t* cons
     sh.x_edge = (int)std::min<unsigned long long>((pow2 + 255) / 256, (unsigned long long)per_stream_cap);
     sh.x_big = std::max(1, 4 * g->sm_count / (int)k);
     sh.x_huge = std::max(1, 2 * g->sm_count / (int)k);
-    sh.colours = (int)hs[0]->d.colours;
-    for (uint32_t i = 1; i < k; ++i)
-        if ((int)hs[i]->d.colours != sh.colours) sh.colours = kColAny;
+    auto common_colours = [&] {
+        for (uint32_t i = 1; i < k; ++i)
+            if (hs[i]->d.colours != hs[0]->d.colours) return kColAny;
+        return (int)hs[0]->d.colours;
+    };
+    sh.colours = common_colours();
 
     const int slot = g->slot;
     g->slot ^= 1;
@@ -1220,13 +1279,13 @@ int rept_group_ingest(rept_group* g, rept_state* const* hs, const uint32_t* cons
             const unsigned long long top = g->h_req[3 * i], need = g->h_req[3 * i + 1];
             const bool fixed = (s->cfg.flags & REPT_FLAG_FIXED_POOL) != 0;
             if (!fixed && g->h_req[3 * i + 2] == 0 && top + need > s->d.pool_quads) {
-                s->h_ctrl->pool_top = top;
-                if ((rc = grow_pool(s, top + need + (top + need) / 2 + 1024, st))) return rc;
+                if ((rc = make_room(s, top, need, st))) return rc;
                 hsd[i] = s->d;
                 grew = true;
             }
         }
         if (grew) REPT_CUDA(cudaMemcpyAsync(g->d_sd, hsd, k * sizeof(StreamDev), cudaMemcpyHostToDevice, st));
+        sh.colours = common_colours();
         if ((rc = enqueue_group(g, sh, st, 2))) return rc;
     } else if ((g->flags & REPT_GROUP_PERSISTENT) && !((g->flags & REPT_GROUP_GRAPH) && g->persist_graph_ok)) {
         if ((rc = upload())) return rc;

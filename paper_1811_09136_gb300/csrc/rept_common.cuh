@@ -202,6 +202,7 @@ struct Ctrl {
     unsigned long long n_big;   // nodes whose table k_rehash_big moves, a warp each
     unsigned long long n_huge;  // nodes whose table k_rehash_huge moves, a block each
     unsigned long long huge_next;
+    unsigned long long layout_quads;  // quads of all blocks in the layout that k_layout_quads was asked for
     unsigned long long dbg[4];  // REPT_DEBUG_BOUNDS builds: first failed check {site, index, bound}, count
 };
 
@@ -468,6 +469,38 @@ __host__ __device__ __forceinline__ uint32_t block_quads(uint32_t lg, uint32_t c
     const uint32_t slots = (1u << lg) + list_slots(lg);
     if (colours == kColMulti) return (uint32_t)((3ull * slots + 7ull) >> 3);
     return (slots + (colours == kColWords ? word_slots(lg) : 0u)) >> 2;
+}
+
+// Offsets of blocks are 32-bit quads.
+constexpr unsigned long long kMaxQuads = 0xFFFFFFFFull;
+
+// Pool quads that guarantee no batch can run out: a node's block holds at most 2 quads per entry (3 with
+// colour words: at one entry, less beyond), and its successive blocks form a doubling series bounded by
+// twice the last one, so at most 4 (6) quads per stored entry, i.e. 8 (12) per stream edge.
+inline unsigned long long quads_bound(unsigned long long edges, uint32_t colours) {
+    return (colours == kColWords || colours == kColMulti ? 12ull : 8ull) * edges + 64ull;
+}
+
+// How a configuration stores its colours (StreamDev::colours) where the pool has room, and the bits of a
+// colour word that each hash group takes.  kColMulti is the one layout that a handle may do without.
+inline uint32_t widest_colours(uint32_t m, uint32_t c, uint32_t n_nodes, bool mascot, uint32_t& bits) {
+    const uint64_t groups = mascot ? c : ((uint64_t)c + m - 1u) / m;
+    bits = 0;
+    while (bits < 32u && (1ull << bits) < m) ++bits;
+    if (groups == 1u && m >= 2u) {
+        if (m <= 256u && n_nodes <= (1u << kIdBits)) return kColInEntry;
+        if (!mascot) return kColWords;
+    }
+    if (mascot || m == 1u) bits = 1u;  // a bit per group that keeps the edge
+    return groups * bits <= 32u ? kColMulti : kColNone;
+}
+
+// May a pool of `quads` quads hold the colour words of several groups, when its handle can have `memory` bytes
+// and blocks can start at `most` quads at most?  The words make the pool half as large again, and a stream
+// that outgrows it with them is taken over into a pool without them, which for twice the entries is 4/3 as
+// large: both have to fit side by side.
+inline bool words_fit(unsigned long long quads, unsigned long long memory, unsigned long long most) {
+    return quads <= most && quads <= memory / 32ull && 7ull * 32ull * quads / 3ull <= memory;
 }
 
 // Word offset of the list inside a block with a table of 2^lg slots, of the stream indices or pairs beside

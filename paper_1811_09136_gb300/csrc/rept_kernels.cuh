@@ -142,6 +142,8 @@ __device__ __forceinline__ void k_classify_body(const StreamDev& d, const BatchD
     }
 }
 
+// AGAIN: the batch's new entries have been taken by an earlier pass (the blocks' layout has changed since).
+template <bool AGAIN = false>
 __device__ __forceinline__ void k_plan_body(const StreamDev& d, const Grid g) {
     if (block_failed(d.ctrl)) return;
     // (whole block sizes: those of a few hundred large hubs together pass 2^32 quads)
@@ -155,9 +157,11 @@ __device__ __forceinline__ void k_plan_body(const StreamDev& d, const Grid g) {
         uint32_t need = 0;
         if (valid) {
             const uint32_t x = d.touched[i];
-            const uint32_t cnt = d.meta[x].y, add = d.cnt_add[x];
-            d.cnt_add[x] = 0u;  // zero again for the next batch
-            touched_adds(d)[i] = add;
+            const uint32_t cnt = d.meta[x].y, add = AGAIN ? touched_adds(d)[i] : d.cnt_add[x];
+            if (!AGAIN) {
+                d.cnt_add[x] = 0u;  // zero again for the next batch
+                touched_adds(d)[i] = add;
+            }
             const uint32_t lg_old = table_lg(cnt), lg_new = table_lg(cnt + add);
             if (lg_new != lg_old) need = block_quads(lg_new, d.colours);
         }
@@ -2089,6 +2093,65 @@ template <bool WORK>
 __global__ void __launch_bounds__(kIxThreads, kIxBlocks) k_intersect_probe(StreamDev d, BatchDev b) {
     follow_previous();
     k_intersect_body<WORK, (int)kColNone>(d, b);
+}
+
+// A handle's change of layout, between a batch's k_plan and its k_commit or between batches: the batch's
+// requests again, the quads that all blocks take, then every block into the new pool.
+__global__ void k_plan_again(StreamDev d) { k_plan_body<true>(d, launch_grid()); }
+
+__global__ void __launch_bounds__(256) k_layout_quads(StreamDev d) {
+    unsigned long long sum = 0;
+    for (unsigned long long x = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; x < d.n_nodes;
+         x += (unsigned long long)gridDim.x * blockDim.x) {
+        const uint32_t cnt = d.meta[x].y;
+        if (cnt) sum += block_quads(table_lg(cnt), d.colours);
+    }
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xFFFFFFFFu, sum, o);
+    if ((threadIdx.x & 31u) == 0 && sum) atomicAdd(&d.ctrl->layout_quads, sum);
+}
+
+// From kColMulti to kColNone or back, a block of the grid per node: both keep split tables whose keys stand
+// alike, so that everything is copied in place order (colour words are formed anew).  pool_top starts at 0
+// and hands out the new places.
+__global__ void __launch_bounds__(256) k_relayout(StreamDev d, const uint2* __restrict__ old, unsigned long long old_quads,
+                                                  uint32_t from_colours) {
+    __shared__ unsigned long long s_off;
+    const uint32_t col = d.colours;
+    for (unsigned long long x = blockIdx.x; x < d.n_nodes; x += gridDim.x) {
+        const uint4 m = d.meta[x];
+        const uint32_t cnt = m.y, lg = table_lg(cnt), quads = block_quads(lg, col);
+        if (cnt == 0u) continue;
+        if (threadIdx.x == 0) s_off = atomicAdd(&d.ctrl->pool_top, (unsigned long long)quads);
+        __syncthreads();
+        const unsigned long long off = s_off;
+        // (the pool has room for k_layout_quads' sum, and blocks lie in the old one: checked all the same)
+        if (off + quads <= d.pool_quads && (unsigned long long)m.x + block_quads(lg, from_colours) <= old_quads) {
+            const uint32_t* from = block_at(old, m.x);
+            uint32_t* to = block_at(d.pool, off);
+            for (uint32_t h = threadIdx.x; h < 1u << lg; h += blockDim.x) {
+                const uint32_t id = from[h];
+                bool kept;
+                to[h] = id;
+                if (id != kEmptyId)
+                    table_store(to, lg, h, from[eidx_word(h, lg, from_colours)],
+                                col == kColMulti ? colour_word(d, (uint32_t)x, id, kept) : 0u, col);
+            }
+            const uint32_t *ids = from + list_at(lg, from_colours), *aux = from + aux_at(lg, from_colours);
+            for (uint32_t j = threadIdx.x; j < cnt; j += blockDim.x) {
+                const uint32_t id = ids[j], t = aux[from_colours == kColMulti ? 2ull * j : j];
+                bool kept;
+                to[list_at(lg, col) + j] = id;
+                if (col == kColMulti)
+                    reinterpret_cast<uint2*>(to + aux_at(lg, col))[j] = make_uint2(t, colour_word(d, (uint32_t)x, id, kept));
+                else
+                    to[aux_at(lg, col) + j] = t;
+            }
+        } else if (threadIdx.x == 0) {
+            atomicOr(&d.ctrl->status, kStInternal);
+        }
+        __syncthreads();  // every thread has read the record
+        if (threadIdx.x == 0) d.meta[x].x = (uint32_t)off;
+    }
 }
 
 // Rebuild every node's block from a pool of another layout: `from_colours`, with pair lists of version 3
