@@ -459,7 +459,7 @@ __host__ __device__ __forceinline__ uint32_t table_lg(uint32_t cnt) {
 }
 
 // A node's block in the pool, 32-byte aligned, in 32-bit words: its hash table of 2^lg slots
-// (2 words a slot, 3 with kColMulti; key_word, eidx_word), then its list: list_slots(lg) entry words
+// (2 words a slot, 3 with kColMulti; key_word, eidx_of), then its list: list_slots(lg) entry words
 // (id and, with kColInEntry, colour) in insertion order, followed by their stream indices (kColNone) or
 // {stream index, colour word} pairs (kColMulti); single-group streams leave that part unused (a
 // candidate's age is looked up in the table) and, with kColWords, keep the colour words after it.
@@ -503,16 +503,23 @@ inline bool words_fit(unsigned long long quads, unsigned long long memory, unsig
     return quads <= most && quads <= memory / 32ull && 7ull * 32ull * quads / 3ull <= memory;
 }
 
-// Word offset of the list inside a block with a table of 2^lg slots, of the stream indices or pairs beside
-// it (kColNone, kColMulti), and of its colour words (kColWords).  In 64 bits, like every offset that passes
-// a table's keys: a block of 2^30 slots (a node of more than 2^28 entries) is longer than 2^32 words.
-__host__ __device__ __forceinline__ uint64_t list_at(uint32_t lg, uint32_t colours) {
-    return (colours == kColMulti ? 3ull : 2ull) << lg;
+// Where the list of a block with a table of 2^lg slots starts, the stream indices or pairs beside it (kColNone,
+// kColMulti), and its colour words (kColWords).  A block of 2^30 slots (a node of more than 2^28 entries)
+// is longer than 2^32 words, so the offsets are 64 bits wide.  (32-bit offsets, which wrap there: intersection of
+// partial groups, 2M edges, 1.23 ms and 1.25 ms so, R-MAT scale 20 5.48 and 5.48; counted in 16-byte
+// units in 32 bits 1.26 and 5.51.)
+template <class Word>
+__host__ __device__ __forceinline__ Word* list_of(Word* block, uint32_t lg, uint32_t colours) {
+    return block + ((colours == kColMulti ? 3ull : 2ull) << lg);
 }
-__host__ __device__ __forceinline__ uint64_t aux_at(uint32_t lg, uint32_t colours) {
-    return list_at(lg, colours) + list_slots(lg);
+template <class Word>
+__host__ __device__ __forceinline__ Word* aux_of(Word* block, uint32_t lg, uint32_t colours) {
+    return list_of(block, lg, colours) + list_slots(lg);
 }
-__host__ __device__ __forceinline__ uint64_t cw_at(uint32_t lg) { return 2ull * ((1u << lg) + list_slots(lg)); }
+template <class Word>
+__host__ __device__ __forceinline__ Word* cw_of(Word* block, uint32_t lg) {
+    return block + 2ull * ((1u << lg) + list_slots(lg));
+}
 
 // Work-counter class of an edge whose smaller endpoint holds cnt entries (rept_stats.class_*).
 __host__ __device__ __forceinline__ int bin_of_cnt(uint32_t cnt) {
@@ -525,17 +532,18 @@ __device__ __forceinline__ uint32_t home_slot(uint32_t w, uint32_t lg) {
     return ((w * 0x9E3779B1u) >> (32u - lg)) & ~3u;
 }
 
-// Word offsets, from the start of a table of 2^lg slots, of slot h's neighbour id and of its stream
-// index.  Interleaved tables: bucket h / 4 occupies words 8 (h / 4) .. 8 (h / 4) + 7, ids first.
+// The word offset, from the start of a table of 2^lg slots, of slot h's neighbour id, and the place of its
+// stream index.  Interleaved tables: bucket h / 4 occupies words 8 (h / 4) .. 8 (h / 4) + 7, ids first.
 // Others: ids in words 0 .. 2^lg - 1, then the stream indices (with kColMulti, each followed by its
 // colour word).  key_quad: the 16-byte quad that holds the four ids of the bucket that starts at slot h
 // (h a multiple of 4).
 __host__ __device__ __forceinline__ uint32_t key_word(uint32_t h, uint32_t colours) {
     return interleaved(colours) ? (((h >> 2) << 3) | (h & 3u)) : h;
 }
-__host__ __device__ __forceinline__ uint64_t eidx_word(uint32_t h, uint32_t lg, uint32_t colours) {
-    return interleaved(colours) ? key_word(h, colours) + 4u
-                                : (1u << lg) + (colours == kColMulti ? 2ull * h : h);
+template <class Word>
+__host__ __device__ __forceinline__ Word* eidx_of(Word* table, uint32_t h, uint32_t lg, uint32_t colours) {
+    if (interleaved(colours)) return table + (key_word(h, colours) + 4u);
+    return colours == kColMulti ? table + (1u << lg) + 2ull * h : table + ((1u << lg) + h);
 }
 __host__ __device__ __forceinline__ uint32_t key_quad(uint32_t h, uint32_t colours) {
     return interleaved(colours) ? h >> 1 : h >> 2;

@@ -38,7 +38,7 @@ __device__ __forceinline__ const uint32_t* block_at(const uint2* pool, unsigned 
 }
 
 // A node's table of 2^lg slots at `table` holds 2^lg neighbour ids (keys; probed a 4-key, 16-byte
-// bucket at a time) and, per id, its stream index (and colour word), laid out as key_word and eidx_word
+// bucket at a time) and, per id, its stream index (and colour word), laid out as key_word and eidx_of
 // say.  Insert (nbr, eidx, cw): claim a key slot with a 32-bit CAS, then store the rest.
 // Returns false only if the table has no empty slot left (impossible while cnt <= capacity / 2).
 // Lookups read whole 4-key buckets, so where a key sits inside its bucket does not matter: an insert
@@ -57,7 +57,7 @@ __device__ __forceinline__ uint32_t empty_slot(const uint4& q, uint32_t nbr) {
 
 __device__ __forceinline__ void table_store(uint32_t* table, uint32_t lg, uint32_t h, uint32_t eidx, uint32_t cw,
                                             uint32_t colours) {
-    uint32_t* at = table + eidx_word(h, lg, colours);
+    uint32_t* at = eidx_of(table, h, lg, colours);
     if (colours == kColMulti) *reinterpret_cast<uint2*>(at) = make_uint2(eidx, cw);
     else *at = eidx;
 }
@@ -187,10 +187,10 @@ __device__ __forceinline__ void copy_words(uint32_t* to, const uint32_t* from, u
 // Copy the list of cnt_old entries from the block at `from` (table of 2^lg_old slots) to the new one.
 __device__ __forceinline__ void move_list(uint32_t* to, const uint32_t* from, uint32_t cnt_old, uint32_t lg_old,
                                           uint32_t lg_new, uint32_t colours, uint32_t rank, uint32_t width) {
-    copy_words(to + list_at(lg_new, colours), from + list_at(lg_old, colours), cnt_old, rank, width);
-    if (colours == kColWords) copy_words(to + cw_at(lg_new), from + cw_at(lg_old), cnt_old, rank, width);
+    copy_words(list_of(to, lg_new, colours), list_of(from, lg_old, colours), cnt_old, rank, width);
+    if (colours == kColWords) copy_words(cw_of(to, lg_new), cw_of(from, lg_old), cnt_old, rank, width);
     if (colours == kColNone || colours == kColMulti)
-        copy_words(to + aux_at(lg_new, colours), from + aux_at(lg_old, colours),
+        copy_words(aux_of(to, lg_new, colours), aux_of(from, lg_old, colours),
                    colours == kColMulti ? 2u * cnt_old : cnt_old, rank, width);
 }
 
@@ -210,7 +210,7 @@ __device__ __forceinline__ void each_entry(const uint32_t* from, uint32_t cnt, u
             if (id.w != kEmptyId) put(id.w, t.w, 0u);
         }
     } else {
-        const uint32_t *ids = from + list_at(lg, colours), *aux = from + aux_at(lg, colours);
+        const uint32_t *ids = list_of(from, lg, colours), *aux = aux_of(from, lg, colours);
         const uint32_t step = colours == kColMulti ? 2u : 1u;
         for (uint32_t j = rank; j < cnt; j += width) put(ids[j], aux[j * step], j);
     }
@@ -223,7 +223,7 @@ __device__ __forceinline__ bool move_block(uint32_t* to, const uint32_t* from, u
     const uint32_t lg_old = table_lg(cnt_old);
     move_list(to, from, cnt_old, lg_old, lg_new, colours, rank, width);
     bool ok = true;
-    const uint32_t* aux = from + aux_at(lg_old, colours);
+    const uint32_t* aux = aux_of(from, lg_old, colours);
     each_entry(from, cnt_old, lg_old, colours, rank, width, [&](uint32_t id, uint32_t eidx, uint32_t j) {
         ok &= table_insert(to, lg_new, id, eidx, colours == kColMulti ? aux[2u * j + 1u] : 0u, colours);
     });
@@ -295,7 +295,7 @@ __device__ __forceinline__ bool move_block_smem(uint32_t* to, const uint32_t* fr
         }
     }
     if (colours == kColMulti) {  // the pairs of the keys' entries, from the old list
-        const uint2* pairs = reinterpret_cast<const uint2*>(from + aux_at(lg_old, colours));
+        const uint2* pairs = reinterpret_cast<const uint2*>(aux_of(from, lg_old, colours));
         uint2* out = reinterpret_cast<uint2*>(to + cap);
         for (uint32_t q = rank; q < cap; q += width)
             if (s_keys[q] != kEmptyId) out[q] = pairs[s_aux[q]];
@@ -460,8 +460,8 @@ __device__ __forceinline__ bool move_block_index(uint32_t* to, const uint32_t* f
         }
         ok = false;
     };
-    const uint32_t* ids = from + list_at(lg_old, colours);
-    const uint32_t* aux = from + aux_at(lg_old, colours);
+    const uint32_t* ids = list_of(from, lg_old, colours);
+    const uint32_t* aux = aux_of(from, lg_old, colours);
     if (inter) {
         for (uint32_t h = rank; cnt_old && h < (1u << lg_old); h += width) {
             const uint32_t id = from[key_word(h, colours)];
@@ -482,7 +482,7 @@ __device__ __forceinline__ bool move_block_index(uint32_t* to, const uint32_t* f
             if (at) {
                 const uint32_t j = at - 1u;
                 id[i] = inter ? from[key_word(j, colours)] : ids[j];
-                t[i] = inter ? from[eidx_word(j, lg_old, colours)] : colours == kColMulti ? aux[2u * j] : aux[j];
+                t[i] = inter ? *eidx_of(from, j, lg_old, colours) : colours == kColMulti ? aux[2u * j] : aux[j];
                 if (colours == kColMulti) cw[i] = aux[2u * j + 1u];
             }
         }
@@ -611,17 +611,17 @@ __device__ __forceinline__ void k_insert_body(const StreamDev& d, const BatchDev
                 if (!ok) atomicOr(&ct->status, kStInternal);
                 const uint32_t pu = mu.y - 1u - rank.x, pv = mv.y - 1u - rank.y;
                 if (REPT_CHECK(ct, 2, pu, list_slots(lu)) && REPT_CHECK(ct, 2, pv, list_slots(lv))) {
-                    tu[list_at(lu, col) + pu] = v | cj;
-                    tv[list_at(lv, col) + pv] = u | cj;
+                    list_of(tu, lu, col)[pu] = v | cj;
+                    list_of(tv, lv, col)[pv] = u | cj;
                     if (col == kColWords) {
-                        tu[cw_at(lu) + pu] = cw;
-                        tv[cw_at(lv) + pv] = cw;
+                        cw_of(tu, lu)[pu] = cw;
+                        cw_of(tv, lv)[pv] = cw;
                     } else if (col == kColNone) {
-                        tu[aux_at(lu, col) + pu] = t;
-                        tv[aux_at(lv, col) + pv] = t;
+                        aux_of(tu, lu, col)[pu] = t;
+                        aux_of(tv, lv, col)[pv] = t;
                     } else if (col == kColMulti) {
-                        reinterpret_cast<uint2*>(tu + aux_at(lu, col))[pu] = make_uint2(t, cw);
-                        reinterpret_cast<uint2*>(tv + aux_at(lv, col))[pv] = make_uint2(t, cw);
+                        reinterpret_cast<uint2*>(aux_of(tu, lu, col))[pu] = make_uint2(t, cw);
+                        reinterpret_cast<uint2*>(aux_of(tv, lv, col))[pv] = make_uint2(t, cw);
                     }
                 }
                 if (d.edge_ends) d.edge_ends[t] = make_uint2(u, v);
@@ -742,7 +742,7 @@ __device__ __forceinline__ uint32_t table_slot(const uint32_t* table, uint32_t l
 __device__ __forceinline__ uint32_t table_find(const uint32_t* table, uint32_t lg, uint32_t w,
                                                uint32_t& slots, uint32_t colours) {
     const uint32_t h = table_slot(table, lg, w, slots, colours);
-    return h == kEmptyId ? kEmptyId : table[eidx_word(h, lg, colours)];
+    return h == kEmptyId ? kEmptyId : *eidx_of(table, h, lg, colours);
 }
 
 // REPT_FLAG_CHECK_DUPS: before the batch is applied, flag an edge that repeats an earlier stored
@@ -1037,7 +1037,7 @@ __device__ __forceinline__ uint32_t cand_probe(const S& st, const uint32_t* cq, 
                 // (a plain load: this kernel may be set up while the inserts still write the pool, and a group's
                 // persistent launch writes it itself, so the read-only path is not open to it)
                 bk[p] = reinterpret_cast<const uint4*>(block_at(d.pool, off[p].y))[key_quad(h[p], col)];
-                const uint32_t* aux_s = block_at(d.pool, off[p].x) + aux_at(lgs[p], col);
+                const uint32_t* aux_s = aux_of(block_at(d.pool, off[p].x), lgs[p], col);
                 if (col == kColNone) as[p].x = aux_s[pos[p]];
                 if (col == kColMulti) as[p] = reinterpret_cast<const uint2*>(aux_s)[pos[p]];
             } else {
@@ -1062,7 +1062,7 @@ __device__ __forceinline__ uint32_t cand_probe(const S& st, const uint32_t* cq, 
             const uint32_t col = colours_of<MODE>(d);
             al[p] = make_uint2(kEmptyId, 0u);  // absent: never older
             if (slot[p] != kEmptyId) {
-                const uint32_t* a = block_at(d.pool, off[p].y) + eidx_word(slot[p], lgl[p], col);
+                const uint32_t* a = eidx_of(block_at(d.pool, off[p].y), slot[p], lgl[p], col);
                 if (col == kColMulti) al[p] = *reinterpret_cast<const uint2*>(a);
                 else al[p].x = *a;
             }
@@ -1159,8 +1159,8 @@ __device__ __forceinline__ void filter_build(const StreamDev& d, uint32_t* filte
     const uint32_t lgt = table_lg(n), col = colours_of<MODE>(d);
     if (!(block_fits(d, 7, off, lgt) && REPT_CHECK(d.ctrl, 6, n, list_slots(lgt) + 1u))) return;
     const uint32_t* block = block_at(d.pool, off);
-    const uint4* list = reinterpret_cast<const uint4*>(block + list_at(lgt, col));
-    const uint4* words = reinterpret_cast<const uint4*>(block + cw_at(lgt));
+    const uint4* list = reinterpret_cast<const uint4*>(list_of(block, lgt, col));
+    const uint4* words = reinterpret_cast<const uint4*>(cw_of(block, lgt));
     const uint32_t last = (n - 1u) >> 2;
     for (uint32_t i = rank; i <= last; i += 2u * width) {
         uint4 q[2], cw[2];
@@ -1227,8 +1227,8 @@ __device__ __forceinline__ void scan_rows(const S& st, uint32_t sid, const uint3
     const uint32_t col = colours_of<MODE>(d), lgs = table_lg(n), last = (n - 1u) >> 2;
     const bool has_cw = MODE == (int)kColWords || (MODE == kColAny && col == kColWords);
     const uint32_t* block = block_at(d.pool, off_s);
-    const uint4* list = reinterpret_cast<const uint4*>(block + list_at(lgs, col));
-    const uint4* words = reinterpret_cast<const uint4*>(block + cw_at(lgs));
+    const uint4* list = reinterpret_cast<const uint4*>(list_of(block, lgs, col));
+    const uint4* words = reinterpret_cast<const uint4*>(cw_of(block, lgs));
 #pragma unroll 1
     for (uint32_t j = j0; j < j1; j += 4u) {
         uint4 q[4], cw[4];
@@ -1263,7 +1263,7 @@ __device__ __forceinline__ void scan_short(const S& st, uint32_t sid, const uint
     const unsigned lane = threadIdx.x & 31u;
     const uint32_t col = colours_of<MODE>(d), lgs = table_lg(n);
     const bool has_cw = MODE == (int)kColWords || (MODE == kColAny && col == kColWords);
-    const uint32_t list_off = off_s + (uint32_t)(list_at(lgs, col) >> 3);  // in 32-byte units (n > 4: a whole number)
+    const uint32_t list_off = off_s + (((col == kColMulti ? 3u : 2u) << lgs) >> 3);  // in 32-byte units (n > 4: a whole number)
     const uint32_t quads = (n + 3u) >> 2;
     uint32_t incl = quads;
 #pragma unroll
@@ -1289,7 +1289,7 @@ __device__ __forceinline__ void scan_short(const S& st, uint32_t sid, const uint
             cw[p] = make_uint4(0u, 0u, 0u, 0u);
             if (has_cw) {
                 const uint32_t oo = __shfl_sync(0xFFFFFFFFu, off_s, o), on = __shfl_sync(0xFFFFFFFFu, n, o);
-                cw[p] = reinterpret_cast<const uint4*>(block_at(d.pool, oo) + cw_at(table_lg(on)))[pos[p]];
+                cw[p] = reinterpret_cast<const uint4*>(cw_of(block_at(d.pool, oo), table_lg(on)))[pos[p]];
             }
         }
 #pragma unroll
@@ -1486,8 +1486,8 @@ __device__ __forceinline__ void run_small_chunk(const S& st, uint32_t sid, uint3
                 if (v[p]) {
                     const uint32_t lgs = table_lg(oc);
                     const uint32_t* block = block_at(d.pool, oo);
-                    word[p] = block[list_at(lgs, col) + pos[p]];
-                    if (col == kColWords) cw[p] = block[cw_at(lgs) + pos[p]];
+                    word[p] = list_of(block, lgs, col)[pos[p]];
+                    if (col == kColWords) cw[p] = cw_of(block, lgs)[pos[p]];
                 }
             }
             if (interleaved(col)) {
@@ -2133,18 +2133,18 @@ __global__ void __launch_bounds__(256) k_relayout(StreamDev d, const uint2* __re
                 bool kept;
                 to[h] = id;
                 if (id != kEmptyId)
-                    table_store(to, lg, h, from[eidx_word(h, lg, from_colours)],
+                    table_store(to, lg, h, *eidx_of(from, h, lg, from_colours),
                                 col == kColMulti ? colour_word(d, (uint32_t)x, id, kept) : 0u, col);
             }
-            const uint32_t *ids = from + list_at(lg, from_colours), *aux = from + aux_at(lg, from_colours);
+            const uint32_t *ids = list_of(from, lg, from_colours), *aux = aux_of(from, lg, from_colours);
             for (uint32_t j = threadIdx.x; j < cnt; j += blockDim.x) {
                 const uint32_t id = ids[j], t = aux[from_colours == kColMulti ? 2ull * j : j];
                 bool kept;
-                to[list_at(lg, col) + j] = id;
+                list_of(to, lg, col)[j] = id;
                 if (col == kColMulti)
-                    reinterpret_cast<uint2*>(to + aux_at(lg, col))[j] = make_uint2(t, colour_word(d, (uint32_t)x, id, kept));
+                    reinterpret_cast<uint2*>(aux_of(to, lg, col))[j] = make_uint2(t, colour_word(d, (uint32_t)x, id, kept));
                 else
-                    to[aux_at(lg, col) + j] = t;
+                    aux_of(to, lg, col)[j] = t;
             }
         } else if (threadIdx.x == 0) {
             atomicOr(&d.ctrl->status, kStInternal);
@@ -2175,16 +2175,16 @@ __global__ void __launch_bounds__(256) k_convert(StreamDev d, const uint2* __res
                 word = from[(2u << lg) + 2u * j];
                 t = from[(2u << lg) + 2u * j + 1u];
             } else {
-                word = from[list_at(lg, from_colours) + j];
-                t = from[aux_at(lg, from_colours) + (from_colours == kColMulti ? 2u * j : j)];
+                word = list_of(from, lg, from_colours)[j];
+                t = aux_of(from, lg, from_colours)[from_colours == kColMulti ? 2ull * j : j];
             }
             bool kept;
-            if (col == kColWords) cw = from[cw_at(lg) + j];
+            if (col == kColWords) cw = cw_of(from, lg)[j];
             if (col == kColMulti) cw = colour_word(d, x, word, kept);
-            to[list_at(lg, col) + j] = word;
-            if (col == kColWords) to[cw_at(lg) + j] = cw;
-            if (col == kColNone) to[aux_at(lg, col) + j] = t;
-            if (col == kColMulti) reinterpret_cast<uint2*>(to + aux_at(lg, col))[j] = make_uint2(t, cw);
+            list_of(to, lg, col)[j] = word;
+            if (col == kColWords) cw_of(to, lg)[j] = cw;
+            if (col == kColNone) aux_of(to, lg, col)[j] = t;
+            if (col == kColMulti) reinterpret_cast<uint2*>(aux_of(to, lg, col))[j] = make_uint2(t, cw);
             ok &= table_insert(to, lg, word & mask, t, cw, col);
         }
         if (!ok) atomicOr(&d.ctrl->status, kStInternal);

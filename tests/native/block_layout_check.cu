@@ -1,4 +1,4 @@
-// Host-only check of the block layouts (block_quads, key_word, eidx_word, list_at, aux_at, cw_at) at every table
+// Host-only check of the block layouts (block_quads, key_word, eidx_of, list_of, aux_of, cw_of) at every table
 // size up to 2^31 slots: the table, the list and what stands beside it follow one another inside the block,
 // none reaching into the next.  Exit code 0: they do.
 #include <cstdint>
@@ -19,11 +19,13 @@ int main() {
             const uint64_t block = 8ull * block_quads(lg, colours);
             const uint32_t last = (uint32_t)(slots - 1u);
             bool ok = block >= end + words && block < end + words + 8u;
-            ok = ok && list_at(lg, colours) == table && aux_at(lg, colours) == table + entries;
-            if (colours == kColWords) ok = ok && cw_at(lg) == end;
+            const uint32_t* at = nullptr;
+            auto words_to = [&](const uint32_t* p) { return (uint64_t)(reinterpret_cast<uintptr_t>(p) / 4u); };
+            ok = ok && words_to(list_of(at, lg, colours)) == table && words_to(aux_of(at, lg, colours)) == table + entries;
+            if (colours == kColWords) ok = ok && words_to(cw_of(at, lg)) == end;
             ok = ok && key_word(0u, colours) == 0u && key_word(last, colours) < table;
-            ok = ok && eidx_word(last, lg, colours) + (colours == kColMulti ? 2u : 1u) == table;
-            ok = ok && eidx_word(0u, lg, colours) == (interleaved(colours) ? 4u : slots);
+            ok = ok && words_to(eidx_of(at, last, lg, colours)) + (colours == kColMulti ? 2u : 1u) == table;
+            ok = ok && words_to(eidx_of(at, 0u, lg, colours)) == (interleaved(colours) ? 4u : slots);
             if (!ok) std::printf("layout %u: tables of 2^%u slots\n", colours, lg);
             bad += !ok;
         }
