@@ -193,6 +193,15 @@ int relayout(rept_state* s, uint32_t to, unsigned long long least, cudaStream_t 
     return set_intersect_grid(s);
 }
 
+// words_fit for a pool of `quads` quads in place of the handle's.
+int pool_may_hold_words(rept_state* s, unsigned long long quads, bool* fits) {
+    size_t free_bytes = 0, all_bytes = 0;
+    REPT_CUDA(cudaMemGetInfo(&free_bytes, &all_bytes));
+    const unsigned long long left = max_bytes() - std::min<unsigned long long>(max_bytes(), s->device_bytes);
+    *fits = words_fit(quads, std::min<unsigned long long>(free_bytes, left) + s->d.pool_quads * 32ull, max_quads());
+    return REPT_OK;
+}
+
 // Make room for a batch whose new blocks take `need` quads beyond the `top` that are in use (after its
 // k_plan, with the stream idle).  Blocks with the colour words of several groups give them up rather than be
 // refused a larger pool (words_fit).
@@ -200,14 +209,10 @@ int make_room(rept_state* s, unsigned long long top, unsigned long long need, cu
     const unsigned long long min_quads = top + need + (top + need) / 2 + 1024;
     s->h_ctrl->pool_top = top;
     if (s->d.colours != kColMulti) return grow_pool(s, min_quads, st);
-    size_t free_bytes = 0, all_bytes = 0;
-    REPT_CUDA(cudaMemGetInfo(&free_bytes, &all_bytes));
-    const unsigned long long own = s->d.pool_quads * 32ull;
-    const unsigned long long memory = std::min<unsigned long long>(free_bytes, max_bytes() - s->device_bytes) + own;
-    if (words_fit(std::max(min_quads, 2ull * s->d.pool_quads), memory, max_quads())) {
-        const int rc = grow_pool(s, min_quads, st);
-        if (rc != REPT_E_NOMEM) return rc;
-    }
+    bool fits = false;
+    int rc = pool_may_hold_words(s, std::max(min_quads, 2ull * s->d.pool_quads), &fits);
+    if (!rc && fits) rc = grow_pool(s, min_quads, st);
+    if (rc ? rc != REPT_E_NOMEM : fits) return rc;
     return relayout(s, kColNone, s->d.pool_quads / 3ull * 4ull, st);
 }
 
@@ -827,14 +832,17 @@ int rept_restore(rept_state* s, const void* h_buf, uint64_t bytes, void* stream)
         h.c != s->cfg.c || h.seed != s->cfg.seed || h.n_nodes != s->cfg.n_nodes || h.flags != s->cfg.flags ||
         h.groups != s->groups || h.proc_begin != s->cfg.proc_begin || h.proc_end != s->cfg.proc_end)
         return REPT_E_INVAL;
-    if (pairs) h.colours = s->d.colours == kColMulti ? kColNone : s->d.colours;
+    // the blocks are taken as they are: in the handle's layout, or a several-group stream's with or without words
+    if (pairs) h.colours = s->wide == kColMulti ? kColNone : s->d.colours;
     else std::memcpy(&h.colours, static_cast<const char*>(h_buf) + kSnapHeader3, sizeof(h.colours));
-    // another layout can be taken over if its lists hold the stream indices
-    const bool convert = pairs || h.colours != s->d.colours;
-    if (convert && !pairs && (interleaved((uint32_t)h.colours) || interleaved(s->d.colours))) return REPT_E_INVAL;
+    const bool several = s->wide == kColMulti && (h.colours == kColNone || h.colours == kColMulti);
+    if (h.colours != s->d.colours && !several) return REPT_E_INVAL;
     int rc = rept_reset(s, stream);
     if (rc) return rc;
-    const size_t n = s->d.n_nodes;
+    const uint32_t wanted = s->d.colours;
+    s->d.colours = (uint32_t)h.colours;
+    if ((rc = set_intersect_grid(s))) return rc;
+    if (h.pool_top > s->d.pool_quads && (rc = grow_pool(s, h.pool_top, st))) return rc;
     s->next_t = h.next_t;
     if (s->d.local2 && (rc = ensure_pair_capacity(s, std::max<unsigned long long>(h.next_t, 1), st))) return rc;
     SnapPart parts[16];
@@ -844,64 +852,29 @@ int rept_restore(rept_state* s, const void* h_buf, uint64_t bytes, void* stream)
     for (int i = 0; i < np; ++i) total += parts[i].bytes;
     if (bytes < total) return REPT_E_INVAL;
     const char* in = static_cast<const char*>(h_buf) + header;
-    unsigned long long pool_top = h.pool_top;
-    std::vector<uint4> meta;
-    std::vector<uint32_t> old_off;
-    if (convert) {  // new block offsets, in node order
-        meta.resize(n);
-        old_off.resize(n);
-        std::memcpy(meta.data(), in, n * sizeof(uint4));
-        pool_top = 0;
-        for (size_t x = 0; x < n; ++x) {
-            old_off[x] = meta[x].x;
-            const uint32_t cnt = meta[x].y;
-            meta[x].x = cnt ? (uint32_t)pool_top : 0u;
-            if (cnt) pool_top += block_quads(table_lg(cnt), s->d.colours);
-        }
-    }
-    if (pool_top > s->d.pool_quads) {
-        if ((rc = grow_pool(s, pool_top, st))) return rc;
-        snap_parts(s, h.pool_top, parts, &np);  // the pool moved
-    }
-    void* old_pool = nullptr;
-    uint32_t* d_old_off = nullptr;
-    if (convert) {
-        if (cudaMalloc(&old_pool, std::max<size_t>(parts[3].bytes, 32)) != cudaSuccess ||
-            cudaMalloc((void**)&d_old_off, n * sizeof(uint32_t)) != cudaSuccess) {
-            (void)cudaGetLastError();
-            cudaFree(old_pool);
-            return REPT_E_NOMEM;
-        }
-        parts[3].ptr = old_pool;
-    }
-    cudaError_t err = cudaSuccess;
-    for (int i = 0; i < np && err == cudaSuccess; ++i) {
-        const void* src = convert && i == 0 ? (const void*)meta.data() : in;
-        if (parts[i].bytes) err = cudaMemcpyAsync(parts[i].ptr, src, parts[i].bytes, cudaMemcpyHostToDevice, st);
+    for (int i = 0; i < np; ++i) {
+        if (parts[i].bytes) REPT_CUDA(cudaMemcpyAsync(parts[i].ptr, in, parts[i].bytes, cudaMemcpyHostToDevice, st));
         in += parts[i].bytes;
     }
     // control block: the pool in use and the tallies; every per-batch counter starts at zero
     Ctrl c{};
-    c.pool_top = pool_top;
+    c.pool_top = h.pool_top;
     c.self_loops = h.self_loops;
     c.stored = h.stored;
     std::memcpy(s->h_ctrl, &c, sizeof(Ctrl));
-    if (err == cudaSuccess) err = cudaMemcpyAsync(s->d.ctrl, s->h_ctrl, sizeof(Ctrl), cudaMemcpyHostToDevice, st);
-    if (convert && err == cudaSuccess) {
-        err = cudaMemcpyAsync(d_old_off, old_off.data(), n * sizeof(uint32_t), cudaMemcpyHostToDevice, st);
-        if (err == cudaSuccess) {
-            k_convert<<<s->sm_count * 8, 256, 0, st>>>(s->d, static_cast<const uint2*>(old_pool), d_old_off,
-                                                       (uint32_t)h.colours, pairs);
-            g_launches.fetch_add(1, std::memory_order_relaxed);
-            err = cudaPeekAtLastError();
-        }
+    REPT_CUDA(cudaMemcpyAsync(s->d.ctrl, s->h_ctrl, sizeof(Ctrl), cudaMemcpyHostToDevice, st));
+    if (pairs) {
+        k_unpair<<<s->grid_stream, 256, 0, st>>>(s->d);
+        REPT_LAUNCHED();
     }
-    if (err == cudaSuccess) err = cudaStreamSynchronize(st);
-    cudaFree(old_pool);
-    cudaFree(d_old_off);
-    if (err != cudaSuccess) {
-        (void)cudaGetLastError();
-        return REPT_E_CUDA;
+    REPT_CUDA(cudaStreamSynchronize(st));
+    if (wanted == kColMulti && s->d.colours == kColNone) {
+        // with words (5/3 of the room at most, and half as much again) the rest of the stream counts faster;
+        // where they do not fit, it goes on without them
+        bool fits = false;
+        rc = pool_may_hold_words(s, std::max(h.pool_top / 2ull * 5ull + 1024, s->d.pool_quads), &fits);
+        if (!rc && fits) rc = relayout(s, kColMulti, s->d.pool_quads, st);
+        if (rc && rc != REPT_E_NOMEM && rc != REPT_E_CAPACITY) return rc;
     }
     return REPT_OK;
 }

@@ -2154,41 +2154,42 @@ __global__ void __launch_bounds__(256) k_relayout(StreamDev d, const uint2* __re
     }
 }
 
-// Rebuild every node's block from a pool of another layout: `from_colours`, with pair lists of version 3
-// when `pairs`.  meta holds the new block offsets, old_off those in `old`; a warp per node.
-__global__ void __launch_bounds__(256) k_convert(StreamDev d, const uint2* __restrict__ old,
-                                                 const uint32_t* __restrict__ old_off, uint32_t from_colours, bool pairs) {
-    const unsigned lane = threadIdx.x & 31u;
+// Turn the blocks of a version 3 snapshot, whose lists are {entry word, stream index} pairs, into lists of
+// entry words in place, a block of the grid per node: a list takes the same room in both, and its pairs
+// fill the table before the words close up.
+__global__ void __launch_bounds__(256) k_unpair(StreamDev d) {
+    __shared__ int s_bad;
     const uint32_t col = d.colours, mask = id_mask(d);
-    for (uint32_t x = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < d.n_nodes; x += (gridDim.x * blockDim.x) >> 5) {
+    for (unsigned long long x = blockIdx.x; x < d.n_nodes; x += gridDim.x) {
         const uint4 m = d.meta[x];
         const uint32_t cnt = m.y, lg = table_lg(cnt);
-        if (cnt == 0u || !block_fits(d, 10, m.x, lg)) continue;
-        const uint32_t* from = block_at(old, old_off[x]);
-        uint32_t* to = block_at(d.pool, m.x);
-        init_table_keys(to, lg, col, lane, 32u);
-        __syncwarp();
-        bool ok = true;
-        for (uint32_t j = lane; j < cnt; j += 32u) {
-            uint32_t word, t, cw = 0u;
-            if (pairs) {
-                word = from[(2u << lg) + 2u * j];
-                t = from[(2u << lg) + 2u * j + 1u];
-            } else {
-                word = list_of(from, lg, from_colours)[j];
-                t = aux_of(from, lg, from_colours)[from_colours == kColMulti ? 2ull * j : j];
+        if (cnt == 0u) continue;
+        const bool fits = (unsigned long long)m.x + block_quads(lg, col) <= d.pool_quads;
+        if (threadIdx.x == 0) s_bad = !fits;
+        if (fits) {
+            uint32_t* block = block_at(d.pool, m.x);
+            uint32_t* list = list_of(block, lg, col);
+            init_table_keys(block, lg, col, threadIdx.x, blockDim.x);
+            __syncthreads();
+            for (uint32_t j = threadIdx.x; j < cnt; j += blockDim.x)
+                if (!table_insert(block, lg, list[2ull * j] & mask, list[2ull * j + 1u], 0u, col)) s_bad = 1;
+            __syncthreads();
+            for (uint32_t j0 = 0; j0 < cnt; j0 += blockDim.x) {  // every word moves towards the front
+                const uint32_t j = j0 + threadIdx.x;
+                const uint32_t word = j < cnt ? list[2ull * j] : 0u;
+                __syncthreads();
+                if (j < cnt) list[j] = word;
+                __syncthreads();
             }
-            bool kept;
-            if (col == kColWords) cw = cw_of(from, lg)[j];
-            if (col == kColMulti) cw = colour_word(d, x, word, kept);
-            list_of(to, lg, col)[j] = word;
-            if (col == kColWords) cw_of(to, lg)[j] = cw;
-            if (col == kColNone) aux_of(to, lg, col)[j] = t;
-            if (col == kColMulti) reinterpret_cast<uint2*>(aux_of(to, lg, col))[j] = make_uint2(t, cw);
-            ok &= table_insert(to, lg, word & mask, t, cw, col);
+            if (col == kColNone) {
+                uint32_t ns;
+                for (uint32_t j = threadIdx.x; j < cnt; j += blockDim.x)
+                    aux_of(block, lg, col)[j] = table_find(block, lg, list[j], ns, col);
+            }
         }
-        if (!ok) atomicOr(&d.ctrl->status, kStInternal);
-        __syncwarp();
+        __syncthreads();
+        if (threadIdx.x == 0 && s_bad) atomicOr(&d.ctrl->status, kStInternal);
+        __syncthreads();
     }
 }
 

@@ -95,12 +95,14 @@ def main():
                     h.reset()
                     ingest(h, gg.EdgeStream(s.src[:E // 2], s.dst[:E // 2], s.n_nodes), batch)
                     half = h.snapshot()
-                limits()
-                with make(0, 1000) as h:
-                    h.restore(half)
-                    assert layout(h) == WORDS
-                    ingest(h, s, batch, E // 2)
-                    check(h, ref, f"{what}, restored")
+                for room, after in ((None, WORDS), (struct.unpack_from("<Q", half.tobytes(), 9 * 8)[0], PLAIN)):
+                    limits(quads=room)
+                    with make(0, 1000) as h:
+                        h.restore(half)
+                        assert layout(h) == after
+                        limits()
+                        ingest(h, s, batch, E // 2)
+                        check(h, ref, f"{what}, restored")
     # a group: streams that change their layout beside ones that do not
     streams = [s, gg.chung_lu(3000, 2.2, 9000, graph_seed=1, order_seed=2),
                gg.chung_lu(9000, 2.1, 70_000, graph_seed=3, order_seed=4)]
