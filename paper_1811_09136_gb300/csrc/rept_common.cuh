@@ -526,6 +526,18 @@ __host__ __device__ __forceinline__ int bin_of_cnt(uint32_t cnt) {
     return cnt <= 4u ? 0 : cnt <= 8u ? 1 : cnt <= 16u ? 2 : cnt <= 32u ? 3 : cnt <= 256u ? 4 : 5;
 }
 
+// Does a filter of the larger endpoint's list of n entries pay for a block unit's lists of `scanned` entries
+// together?  Building costs each of the n entries about as much as a test, and past one entry per bit or so the
+// filter lets most entries through.  Without it an entry costs a hash (one group's stored colours) or is looked
+// up at once (else), so that the line lies elsewhere.  Passes of a Chung-Lu graph with hubs of a million (40M
+// edges, m = c = 100; filter always, so): batches of 2^14 edges 798 and 312 ms, 2^16 283 and 116, 2^20 66 and 32;
+// five groups there, 2^18 165 and 160.  R-MAT scale 20: 10.86 and 10.92.  Half and twice the numbers: within
+// 2 %, but 65,536 for 24,576 347 ms at 2^14.  (In warp units too, the first three took 3 % less and the groups'
+// kernels spilled for it: 48 streams 47.3 and 48.6 ms.)
+__host__ __device__ __forceinline__ bool filter_pays(uint32_t colours, uint32_t n, unsigned long long scanned) {
+    return interleaved(colours) ? n <= 24576u && n <= 4ull * scanned : n <= 262144u && n <= 16ull * scanned;
+}
+
 // Home slot of neighbour w in a table of 2^lg slots: the first slot of a 4-slot (32-byte) bucket
 // chosen by Fibonacci hashing.  Probing is linear from there, so a lookup reads whole sectors.
 __device__ __forceinline__ uint32_t home_slot(uint32_t w, uint32_t lg) {

@@ -1251,6 +1251,40 @@ __device__ __forceinline__ void scan_rows(const S& st, uint32_t sid, const uint3
         });
     }
 }
+// The four entries of a quad without a filter, for an edge whose larger endpoint is l: bit i is set if entry i's
+// colour may agree with the hash of {l, entry i} (colour_may_match); without one group's stored colours every
+// entry passes.
+template <int MODE>
+__device__ __forceinline__ uint32_t hash_quad(const StreamDev& d, uint32_t l, const uint4& q, const uint4& cw) {
+    const uint32_t col = colours_of<MODE>(d), mask = id_mask(d);
+    if (!interleaved(col)) return 15u;
+    uint32_t m = 0;
+#pragma unroll
+    for (uint32_t i = 0; i < 4u; ++i) {
+        const uint32_t w = quad_word(q, i);
+        m |= (colour_may_match(d, l, w & mask, col == kColWords ? quad_word(cw, i) : w >> kIdBits) ? 1u : 0u) << i;
+    }
+    return m;
+}
+// ... and rows j0 .. j1 - 1 scanned so, one per step.
+template <bool WORK, int MODE, class S>
+__device__ __forceinline__ void hash_rows(const S& st, uint32_t sid, uint32_t l, uint32_t off_s, uint32_t n, uint32_t item,
+                                          uint32_t j0, uint32_t j1, WarpQueues& wq, Work& wk) {
+    const StreamDev& d = st.at(sid);
+    const unsigned lane = threadIdx.x & 31u;
+    const uint32_t col = colours_of<MODE>(d), lgs = table_lg(n), last = (n - 1u) >> 2;
+    const bool has_cw = MODE == (int)kColWords || (MODE == kColAny && col == kColWords);
+    const uint32_t* block = block_at(d.pool, off_s);
+    const uint4* list = reinterpret_cast<const uint4*>(list_of(block, lgs, col));
+    const uint4* words = reinterpret_cast<const uint4*>(cw_of(block, lgs));
+#pragma unroll 1
+    for (uint32_t j = j0; j < j1; ++j) {
+        const uint32_t at = min(32u * j + lane, last);
+        const uint4 q = list[at], cw = has_cw ? words[at] : make_uint4(0u, 0u, 0u, 0u);
+        queue_step<WORK, MODE>(st, wq, hash_quad<MODE>(d, l, q, cw), 4u * (32u * j + lane), n, item, sid, wk,
+                               [&](uint32_t b) { return quad_word(q, b); });
+    }
+}
 // Rows of a list of n entries.
 __device__ __forceinline__ uint32_t list_rows(uint32_t n) { return (n + 127u) >> 7; }
 
@@ -1310,21 +1344,21 @@ __device__ __forceinline__ void scan_short(const S& st, uint32_t sid, const uint
 }
 
 // A block unit as its first thread claims it: the edges order[first .. first + count) of stream sid and
-// the larger endpoint's block (n entries at off).
+// the larger endpoint l's block (n entries at off).  Before the scan: whether l's filter pays.
 struct UnitClaim {
-    uint32_t ok, sid, first, count, off, n;
+    uint32_t ok, sid, first, count, off, n, l, filter;
 };
 __device__ __forceinline__ UnitClaim claimed_unit(const StreamDev& d, uint32_t sid, unsigned long long at) {
     const Unit u = d.units[at];
     const WorkItem x = d.rec[d.order[u.first]];
     d.meta[x.l].w = 0u;  // the record's cursor has served
-    return UnitClaim{1u, sid, u.first, min(u.count, kUnitItems), x.off_l, x.cnt_l};
+    return UnitClaim{1u, sid, u.first, min(u.count, kUnitItems), x.off_l, x.cnt_l, x.l, 1u};
 }
 
 // Work through the block units: the block builds the larger endpoint's filter while its first warp cuts
 // the lists of the unit's edges into pieces of at most kPieceRows rows, which the warps then take in turn,
 // so that they finish together.  `claim` (first thread only) yields the next unit, while the other warps
-// scan.
+// scan; the first warp then adds up the unit's lists.
 constexpr uint32_t kPieceRows = 8u;  // 1,024 entries
 template <bool WORK, int MODE, class S, class Claim>
 __device__ __forceinline__ void run_block_units(const S& st, uint32_t* filter, uint4* items, WarpQueues& wq, Work& wk,
@@ -1332,14 +1366,30 @@ __device__ __forceinline__ void run_block_units(const S& st, uint32_t* filter, u
     __shared__ UnitClaim s_claim;
     __shared__ uint32_t s_taken;  // pieces taken
     const unsigned lane = threadIdx.x & 31u;
-    if (threadIdx.x == 0) s_claim = claim();
+    auto next = [&] {
+        if (threadIdx.x >= 32u) return;
+        UnitClaim u{};
+        if (lane == 0) u = claim();
+        const uint32_t sid = __shfl_sync(0xFFFFFFFFu, u.sid, 0), first = __shfl_sync(0xFFFFFFFFu, u.first, 0),
+                       count = __shfl_sync(0xFFFFFFFFu, u.count, 0);
+        const StreamDev& d = st.at(sid);
+        uint32_t sum = 0;  // (no line of filter_pays lies beyond 64 lists of 2^20 entries)
+        for (uint32_t i = lane; i < count; i += 32u) sum += min(d.rec[d.order[first + i]].cnt_s, 1u << 20);
+        sum = __reduce_add_sync(0xFFFFFFFFu, sum);
+        if (lane == 0) {
+            u.filter = filter_pays(colours_of<MODE>(d), u.n, sum);
+            s_claim = u;
+        }
+        __syncwarp();
+    };
+    next();
     __syncthreads();
     for (;;) {
         const UnitClaim u = s_claim;
         if (!u.ok) break;
         const StreamDev& d = st.at(u.sid);
         const uint32_t lg = filter_lg(2u * u.n, kFilterLg);
-        filter_clear(filter, lg, threadIdx.x, blockDim.x);
+        if (u.filter) filter_clear(filter, lg, threadIdx.x, blockDim.x);
         if (threadIdx.x == 0) s_taken = 0u;
         __syncthreads();
         if (threadIdx.x < 32u) {  // items[i] = {block offset, entries, edge, pieces of lists 0 .. i}
@@ -1371,10 +1421,9 @@ __device__ __forceinline__ void run_block_units(const S& st, uint32_t* filter, u
                 items[i] = x;
             }
         }
-        filter_build<MODE>(d, filter, lg, u.off, u.n, threadIdx.x, blockDim.x);
+        if (u.filter) filter_build<MODE>(d, filter, lg, u.off, u.n, threadIdx.x, blockDim.x);
         __syncthreads();
-        if (threadIdx.x == 0) s_claim = claim();
-        __syncwarp();
+        next();
         const uint32_t total = items[kUnitItems - 1u].w;
         for (;;) {
             uint32_t i = 0;
@@ -1387,7 +1436,9 @@ __device__ __forceinline__ void run_block_units(const S& st, uint32_t* filter, u
             const uint4 x = items[at];
             const uint32_t rows = list_rows(x.y), pieces = (rows + kPieceRows - 1u) / kPieceRows;
             const uint32_t j0 = (i + pieces - x.w) * kPieceRows;
-            scan_rows<WORK, MODE>(st, u.sid, filter, lg, x.x, x.y, x.z, j0, min(j0 + kPieceRows, rows), wq, wk);
+            const uint32_t j1 = min(j0 + kPieceRows, rows);
+            if (u.filter) scan_rows<WORK, MODE>(st, u.sid, filter, lg, x.x, x.y, x.z, j0, j1, wq, wk);
+            else hash_rows<WORK, MODE>(st, u.sid, u.l, x.x, x.y, x.z, j0, j1, wq, wk);
         }
         __syncthreads();
     }
@@ -1539,7 +1590,7 @@ __device__ __forceinline__ void k_intersect_body(const StreamDev& d, const Batch
                 const unsigned long long i = atomicAdd(&ct->bin_next[kind], 1ull);
                 if (i < ct->bin_count[kind]) return claimed_unit(d, 0u, kind == kBinBig ? i : d.unit_cap + i);
             }
-            return UnitClaim{0u, 0u, 0u, 0u, 0u, 0u};
+            return UnitClaim{};
         });
         mark(5);
 #pragma unroll 1
@@ -1674,7 +1725,7 @@ __device__ __forceinline__ void intersect_group_body(const StreamDev* __restrict
                 return claimed_unit(ds[sid], sid, i - pc[sid] + (kind == kBinBig ? 0ull : ds[sid].unit_cap));
             }
         }
-        return UnitClaim{0u, 0u, 0u, 0u, 0u, 0u};
+        return UnitClaim{};
     });
 #pragma unroll 1
     for (uint32_t part = 0; part < 2u; ++part) {
