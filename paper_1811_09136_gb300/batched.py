@@ -158,16 +158,28 @@ class StreamResult:
     local_hat: np.ndarray | None
 
 
-def _state_bytes(n_nodes: int, edges: int, batch: int) -> int:
+def _edge_bytes(n_nodes: int, edges: int, m: int, c: int) -> int:
+    """Pool bytes per edge of a REPT handle made for `edges` edges: 256, or 384 where every entry has a colour
+    word (one hash group whose colour does not fit the entry; several groups whose colours fit 32 bits
+    together, as far as 32-bit offsets reach)."""
+    groups = -(-c // m)
+    bits = (m - 1).bit_length() if m > 1 else 1
+    if groups == 1 and m > 1:
+        return 256 if m <= 256 and n_nodes <= 1 << 24 else 384
+    return 384 if groups * bits <= 32 and 12 * edges + 64 <= 0xFFFFFFFF else 256
+
+
+def _state_bytes(n_nodes: int, edges: int, batch: int, m: int = 2, c: int = 1) -> int:
     """Device bytes a stream's state needs: per-node arrays, per-batch scratch, and the pool at the
-    guaranteed bound (32 slots of 8 bytes per edge)."""
-    return 28 * n_nodes + 200_000 + 96 * batch + 256 * edges + (1 << 20)
+    guaranteed bound (_edge_bytes; by default that of streams without colour words)."""
+    return 28 * n_nodes + 200_000 + 96 * batch + _edge_bytes(n_nodes, edges, m, c) * edges + (1 << 20)
 
 
-def _waves(streams, batch, budget):
+def _waves(streams, batch, budget, params=None):
     wave, used = [], 0
     for i, s in enumerate(streams):
-        b = _state_bytes(s.n_nodes, len(s), min(batch, len(s))) + 8 * len(s)
+        m, c = params[i][:2] if params else (2, 1)
+        b = _state_bytes(s.n_nodes, len(s), min(batch, len(s)), m, c) + 8 * len(s)
         if wave and used + b > budget:
             yield wave
             wave, used = [], 0
@@ -217,7 +229,7 @@ def run_batched(streams, params, batch: int = 1 << 18, tile_max: int = 32, graph
     budget = budget or _device_budget()
     results = [None] * len(streams)
     total = 0.0
-    for wave in _waves(streams, batch, budget):
+    for wave in _waves(streams, batch, budget, params):
         handles, srcs, dsts, hsrc, hdst, outs = [], [], [], [], [], []
         for i in wave:
             s = streams[i]
@@ -267,7 +279,7 @@ def run_plain(streams, params, batch: int = 1 << 18, tile_max: int = 32, budget:
     budget = budget or _device_budget()
     results = [None] * len(streams)
     total = 0.0
-    for wave in _waves(streams, batch, budget):
+    for wave in _waves(streams, batch, budget, params):
         handles, srcs, dsts = [], [], []
         for i in wave:
             s = streams[i]

@@ -190,7 +190,7 @@ def serve(requests: list[Request], max_live: int = 256, budget_bytes: int | None
                 r.done = now
                 rep.cancelled.append(r)
                 continue
-            need = batched._state_bytes(r.stream.n_nodes, len(r.stream), feed(r)) + 8 * len(r.stream)
+            need = batched._state_bytes(r.stream.n_nodes, len(r.stream), feed(r), r.m, r.c) + 8 * len(r.stream)
             reuse = spare.get(shape(r))
             if reuse:
                 pending.pop()
