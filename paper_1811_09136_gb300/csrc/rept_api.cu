@@ -1353,7 +1353,7 @@ int rept_estimates_from_counts(uint32_t m, uint32_t c, uint32_t flags, const uin
     cfg.flags = flags & REPT_FLAG_MASCOT;
     const double f = estimate_factor(cfg);
     // the integer sum of the processors that enter the estimate, then one conversion, as
-    // k_global_estimate forms it
+    // k_estimates forms it
     const uint32_t c_used = mascot || c <= m ? c : (c / m) * m;
     unsigned long long sum = 0;
     for (uint32_t i = 0; i < c_used; ++i) sum += h_proc[i];

@@ -367,12 +367,6 @@ __device__ __forceinline__ uint32_t colour_of(uint32_t a, uint32_t b, uint64_t s
 
 __device__ __forceinline__ uint64_t group_seed(uint64_t seed, uint32_t k) { return seed + (uint64_t)k * kGoldenGamma; }
 
-// h_k({a, b}) == j, for m >= 2 and a colour j < m.
-__device__ __forceinline__ bool colour_is(uint32_t a, uint32_t b, uint64_t s_k, const FastMod& fm, uint32_t j) {
-    uint64_t lo = a < b ? a : b, hi = a < b ? b : a;
-    return mod_equals_in_range(splitmix64(((lo << 32) | hi) ^ s_k), j, fm);
-}
-
 // Do the wedge edges {s, w} and {l, w} have the same colour in the group of seed s_k?  Their hash
 // values are congruent modulo m exactly when m divides their (exact, non-negative) difference, which
 // the divisibility test decides without a remainder; only then is the colour j itself formed.

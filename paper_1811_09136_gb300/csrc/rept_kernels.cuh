@@ -422,14 +422,9 @@ __device__ __forceinline__ void k_rehash_big_body(const StreamDev& d, const Grid
          k += warps) {
         const Move mv = move_of(d, d.big[k], top);
         bool ok = true;
-        if (mv.fits && (1u << mv.lg_new) <= kMoveSlots && REPT_CHECK(d.ctrl, 14, wid, 32u))
+        if (mv.fits && REPT_CHECK(d.ctrl, 14, wid, 32u))
             ok = move_block_smem(mv.to, mv.from, mv.cnt_old, mv.lg_new, d.colours, smem + wid * 2u * kMoveSlots,
                                  smem + (wid * 2u + 1u) * kMoveSlots, lane, 32u);
-        else if (mv.fits) {
-            init_table_keys(mv.to, mv.lg_new, d.colours, lane, 32u);
-            __syncwarp();
-            ok = move_block(mv.to, mv.from, mv.cnt_old, mv.lg_new, d.colours, lane, 32u);
-        }
         if (!ok) atomicOr(&d.ctrl->status, kStInternal);
         __syncwarp();
         if (lane == 0) d.meta[mv.x] = make_uint4(mv.off_new, mv.cnt_new, 0u, 0u);
@@ -501,9 +496,9 @@ __device__ __forceinline__ bool move_block_index(uint32_t* to, const uint32_t* f
 }
 
 // Move the blocks listed by k_commit whose new table has more than kMoveSlots slots: thread blocks
-// claim pieces of the largest, then one node at a time, and build tables of at most max_slots slots in
+// claim pieces of the largest, then one node at a time, and build tables of at most kBlockMoveSlots slots in
 // shared memory (`smem`: as many 16-bit words), larger ones in place.
-__device__ __forceinline__ void k_rehash_huge_body(const StreamDev& d, const Grid g, uint32_t* smem, uint32_t max_slots) {
+__device__ __forceinline__ void k_rehash_huge_body(const StreamDev& d, const Grid g, uint32_t* smem) {
     __shared__ unsigned long long s_k;
     __shared__ int s_bad;
     const unsigned long long pieces = n_giants(d) * kGiantPieces;
@@ -522,7 +517,7 @@ __device__ __forceinline__ void k_rehash_huge_body(const StreamDev& d, const Gri
         if (mv.fits && k < pieces) {  // (uniform over the block)
             ok = move_block(mv.to, mv.from, mv.cnt_old, mv.lg_new, d.colours,
                             (uint32_t)(k % kGiantPieces) * blockDim.x + threadIdx.x, kGiantPieces * blockDim.x);
-        } else if (mv.fits && (1u << mv.lg_new) <= max_slots) {
+        } else if (mv.fits && (1u << mv.lg_new) <= kBlockMoveSlots) {
             ok = move_block_index(mv.to, mv.from, mv.cnt_old, mv.lg_new, d.colours, reinterpret_cast<uint16_t*>(smem));
         } else if (mv.fits) {  // built in place: empty keys first
             init_table_keys(mv.to, mv.lg_new, d.colours, threadIdx.x, blockDim.x);
@@ -1900,7 +1895,7 @@ __global__ void __launch_bounds__(256) k_rehash_big_multi(const StreamDev* __res
 __global__ void __launch_bounds__(1024, 2) k_rehash_huge(StreamDev d) {
     follow_previous();
     extern __shared__ __align__(16) uint32_t hsmem[];
-    k_rehash_huge_body(d, launch_grid(), hsmem, kBlockMoveSlots);
+    k_rehash_huge_body(d, launch_grid(), hsmem);
 }
 
 __global__ void __launch_bounds__(1024, 2) k_rehash_huge_multi(const StreamDev* __restrict__ ds,
@@ -1910,7 +1905,7 @@ __global__ void __launch_bounds__(1024, 2) k_rehash_huge_multi(const StreamDev* 
     __shared__ StreamDev sd;
     if (threadIdx.x == 0) sd = ds[blockIdx.y];
     __syncthreads();
-    k_rehash_huge_body(sd, launch_grid(), hsmem, kBlockMoveSlots);
+    k_rehash_huge_body(sd, launch_grid(), hsmem);
 }
 
 // 5 blocks of 256 threads per SM (48 registers).
@@ -1993,7 +1988,7 @@ __global__ void __cluster_dims__(kStateBlocks, 1, 1) __launch_bounds__(kStateThr
     // not meet, which a batch of 4,096 edges would pay with 3.7 us of 70
     if (n_giants(d)) cluster_barrier();
     else __syncthreads();
-    k_rehash_huge_body(d, g, hsmem, kBlockMoveSlots);
+    k_rehash_huge_body(d, g, hsmem);
     cluster_barrier();
     k_insert_body(d, b, g);
     cluster_barrier();
@@ -2098,7 +2093,7 @@ __global__ void __launch_bounds__(256, 3) k_group_persistent(const StreamDev* __
     ok = ok && grid_barrier(gs, wait_ns);
     if (ok) step(sh.x_big, [&](Grid g) { k_rehash_big_body(sd, g, psmem); });
     ok = ok && grid_barrier(gs, wait_ns);
-    if (ok) step(sh.x_huge, [&](Grid g) { k_rehash_huge_body(sd, g, psmem, kBlockMoveSlots); });
+    if (ok) step(sh.x_huge, [&](Grid g) { k_rehash_huge_body(sd, g, psmem); });
     ok = ok && grid_barrier(gs, wait_ns);
     if (ok) step(sh.x_edge, [&](Grid g) { k_insert_body(sd, sb, g); });
     ok = ok && grid_barrier(gs, wait_ns);

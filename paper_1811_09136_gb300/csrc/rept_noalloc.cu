@@ -129,11 +129,11 @@ extern "C" int rept_count_noalloc(const uint32_t* d_src, const uint32_t* d_dst, 
     d.local = reinterpret_cast<unsigned long long*>(d_local);
     d.proc = reinterpret_cast<unsigned long long*>(d_proc);
 
-    // the scratch keeps the previous call's contents: clear what must start empty
+    // the scratch keeps the previous call's contents: clear what must start empty (tables get their empty keys when
+    // their blocks are handed out)
     NA_CUDA(cudaMemsetAsync(d.meta, 0, (size_t)n_nodes * sizeof(uint4), st));
     NA_CUDA(cudaMemsetAsync(d.cnt_add, 0, (size_t)n_nodes * sizeof(uint32_t), st));
     NA_CUDA(cudaMemsetAsync(d.ctrl, 0, sizeof(Ctrl), st));
-    NA_CUDA(cudaMemsetAsync(d.pool, 0xFF, L.pool_quads * 32ull, st));
     NA_CUDA(cudaMemsetAsync(d_proc, 0, (size_t)c * sizeof(uint64_t), st));
     NA_CUDA(cudaMemsetAsync(d_local, 0, (size_t)n_nodes * sizeof(uint64_t), st));
 
@@ -158,7 +158,10 @@ extern "C" int rept_count_noalloc(const uint32_t* d_src, const uint32_t* d_dst, 
         const unsigned long long want_i = (n_edges + 31) / 32;
         const int grid_i = (int)(want_i < (unsigned long long)sms * 4 ? want_i : (unsigned long long)sms * 4);
         const size_t smem = ix_words((int)kColNone, false) * sizeof(uint32_t) + c * sizeof(unsigned long long);
-        NA_CUDA(cudaFuncSetAttribute(k_intersect_probe<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        // (the limit for the largest c, the same in every call: it belongs to the kernel, not to the call)
+        NA_CUDA(cudaFuncSetAttribute(k_intersect_probe<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)(ix_words((int)kColNone, false) * sizeof(uint32_t) +
+                                           kMaxProcessors * sizeof(unsigned long long))));
         k_intersect_probe<false><<<grid_i, kIxThreads, smem, st>>>(d, b);
         NA_CUDA(cudaPeekAtLastError());
     }
