@@ -62,7 +62,10 @@ extern "C" {
 
 #define REPT_FLAG_FIXED_POOL 1u /* never grow the adjacency pool; a full pool gives REPT_E_CAPACITY */
 #define REPT_FLAG_SYNC 2u       /* synchronise at the end of every ingest and report errors at once */
-#define REPT_FLAG_PROFILE 4u    /* time every kernel launch with CUDA events on its stream (rept_kernel_times) */
+#define REPT_FLAG_PROFILE 4u    /* time every kernel launch with CUDA events on its stream (rept_kernel_times).
+                                   Batches of at most 8,192 edges, whose steps before the intersection
+                                   otherwise run in one launch, then run a launch per step, as they do with
+                                   REPT_FLAG_CHECK_DUPS: their times are not those of the single launch */
 #define REPT_FLAG_WORK_COUNTERS 8u /* count the intersection's table reads into rept_stats (slower; not for timing) */
 #define REPT_FLAG_LOCAL_PER_PROCESSOR 16u /* also keep every tau_v^(i) (c * n_nodes uint64), read with
                                              rept_local_per_processor */
@@ -96,7 +99,8 @@ typedef struct rept_config {
     uint64_t max_batch;      /* sizing hint: largest batch passed to an ingest call (0: 2^20) */
     uint32_t tile_max;       /* tuning: edges whose smaller endpoint holds at most this many entries
                                 (4, 8, 16 or 32; 0: 32) share a warp with other edges, the others are
-                                grouped by their larger endpoint; results do not depend on it */
+                                grouped by their larger endpoint; without effect in batches below 2^15
+                                edges, which have a bound of their own; results do not depend on it */
     uint32_t proc_begin;     /* colour sharding: the handle keeps processors [proc_begin, proc_end) only
                                 (stores the edges they keep, counts their semi-triangles); 0, 0: all c.
                                 Processors are independent until the final sums (Algorithm 1), so
@@ -118,8 +122,8 @@ typedef struct rept_stats {
     uint64_t pool_used;      /* slots handed out to per-node tables so far */
     uint64_t device_bytes;   /* device memory held by the handle */
     /* with REPT_FLAG_WORK_COUNTERS, totals over the stream's intersection passes: */
-    uint64_t small_entries;  /* entries present in the smaller endpoint's table, summed over edges */
-    uint64_t small_slots;    /* slots of those tables read (entries plus empty slots) */
+    uint64_t small_entries;  /* entries present in the smaller endpoint's list, summed over edges */
+    uint64_t small_slots;    /* list words of those endpoints read: equal to small_entries (lists have no gaps) */
     uint64_t probes;         /* probes of the larger endpoint's table (small-side entries that its filter or
                                 their colours did not rule out) */
     uint64_t probe_slots;    /* slots read by those probes */

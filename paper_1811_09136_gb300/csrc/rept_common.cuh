@@ -1,18 +1,15 @@
 // Device-side data layout and helpers of the REPT streaming counter.
 //
 // HBM layout of one stream (one rept_state):
-//   meta[n_nodes]   uint4 {off, cnt, add, grp}: node x's block starts at slot
+//   meta[n_nodes]   uint4 {off, cnt, 0, grp}: node x's block starts at slot
 //                   4*off of the pool and holds cnt entries; its size is a
 //                   function of cnt alone (table_lg below), so a node's block
 //                   is re-allocated exactly when cnt crosses a power-of-two
-//                   boundary.  add counts the current batch's new entries of x
-//                   (zero between batches); it shares x's 16-byte record so
-//                   that the insert's position counter and the block's place
-//                   sit in one 32-byte sector.  grp counts the batch's
-//                   grouped edges whose larger endpoint is x (zero between
-//                   batches).  k_classify counts into the
-//                   compact array cnt_add[n_nodes] first; k_plan moves the
-//                   counts into the records.
+//                   boundary.  grp counts the batch's grouped edges whose
+//                   larger endpoint is x (zero between batches).
+//   cnt_add[n_nodes]  the current batch's new entries of x, as k_classify
+//                   counts them; k_plan takes each touched node's count and
+//                   clears it, so it is zero between batches.
 //   pool[]          32-byte quads: per node, an open-addressing (linear probing,
 //                   4-key buckets) table of 2^lg neighbour ids and their stream
 //                   indices (for single-group streams with stored colours
@@ -31,7 +28,7 @@
 //                   (Section III-A: processor i keeps colour i).
 //   local[n_nodes]  uint64 sum over processors of tau_v^(i)
 //   proc[c]         uint64 tau^(i)
-// Per-batch scratch: touched[] (nodes with add > 0), grow_rel[] (their new
+// Per-batch scratch: touched[] (nodes with new entries), grow_rel[] (their new
 // table's offset relative to this batch's allocation), the work records, and
 // the control block.
 #pragma once
@@ -54,12 +51,13 @@ constexpr uint32_t kMaxProcessors = 4096;  // per-block tau^(i) histogram lives 
 // small: warps take them straight from the batch, a chunk of edges at a time.  The others are grouped
 // by their larger endpoint l into units of edges of one l; a unit is worked on by a warp when l holds at
 // most kWarpUnitNodes entries, else by a thread block (those of the largest l's, above kBigUnitNodes
-// entries, first).
+// entries, first).  kWarpUnitNodes at 512: 1 to 4 % slower on 36 workloads; at 2,048: R-MAT scale 20 2 % faster in
+// batches of 2^17, 1 % slower at 2^20.  kBigUnitNodes at 2,048 or 16,384: no difference beyond 1 %.
 constexpr int kBins = 4;
 constexpr int kBinSmall = 0, kBinWarp = 1, kBinBlock = 2, kBinBig = 3;
 constexpr int kClasses = 6;  // work-counter classes (bin_of_cnt)
 constexpr unsigned long long kSmallBatch = 1ull << 15;  // smaller batches: make_batch
-constexpr uint32_t kSmallBatchMax = 256u;
+constexpr uint32_t kSmallBatchMax = 64u;
 constexpr uint32_t kWarpUnitItems = 32u;  // edges per warp unit: at most one per lane
 constexpr uint32_t kWarpUnitEntries = 8192u;
 constexpr uint32_t kUnitItems = 64u;      // ... and at most of a block unit
@@ -319,12 +317,15 @@ struct BatchDev {
     uint32_t unit_edges;    // edges of a block unit
 };
 
-// A batch of a stream.  Grouping pays through the lists that share a filter; in a small batch few do, and
-// what counts is the chain of dependent steps, so nearly all edges stay small (`tile_max`: the handle's
-// bound for the others) and are dealt out in smaller chunks.  Block units hold fewer edges in smaller
-// batches, so that there are units for every SM; the batches of a group's round (`round` edges together) fill
-// the GPU together and so share their filters among more (48 streams, 65,536 edges each a round: 48.3 ms with
-// units by the stream's own batch, 46.7 ms so).
+// A batch of a stream.  Grouping pays through the lists that share a filter; in a small batch few do, so lists
+// of up to kSmallBatchMax entries stay ungrouped there (`tile_max`: the handle's bound in other batches), and
+// the edges are dealt out in smaller chunks.  Bound 256 and so: R-MAT of 2M edges in batches of 2^13, 2^14 and 2^15
+// edges 23.3, 12.4, 8.2 ms and 22.1, 10.9, 6.5, five groups there 31.6, 18.6, 12.9 and 28.1, 14.6, 9.3; bound 32 the
+// same, but 1 % slower in batches of 4,096.  The line at 2^14 or 2^16 for 2^15, chunks of half the edges: within 3 %;
+// the other batches' chunk of 64 edges 1.2 to 2.5 times slower in batches of 4,096.  Block units hold fewer
+// edges in smaller batches, so that there are units for every SM; the batches of a group's round (`round` edges
+// together) fill the GPU together and so share their filters among more (48 streams, 65,536 edges each a round:
+// 48.3 ms with units by the stream's own batch, 46.7 ms so).
 inline BatchDev make_batch(const uint32_t* src, const uint32_t* dst, unsigned long long n, unsigned long long t0,
                            uint32_t tile_max, unsigned long long round) {
     const bool few = n < kSmallBatch;

@@ -911,7 +911,10 @@ __device__ __forceinline__ uint32_t count_groups(const StreamDev& d, uint32_t* h
 // dependent loads where many pass.
 
 constexpr int kIxThreads = 256;
-constexpr int kIxBlocks = 4;  // per SM: 4 x 48 KB of shared memory
+// Blocks per SM.  Shared memory of a block (ix_words): one stream 45 KB, 48 without stored colours, 54 with the
+// words of several groups, and 8 bytes per processor, of which four fit up to about 200 processors; a group's
+// kernels 51 KB, 54 and 60 (also for mixed layouts), of which the last fit three times.
+constexpr int kIxBlocks = 4;
 constexpr uint32_t kIxWarps = kIxThreads / 32;
 constexpr uint32_t kFilterLg = 13;  // words of a block's filter (32 KB); a warp's share serves warp units
 constexpr uint32_t kFilterWords = 1u << kFilterLg;
