@@ -1423,20 +1423,29 @@ __device__ __forceinline__ void run_block_units(const S& st, uint32_t* filter, u
         __syncthreads();
         next();
         const uint32_t total = items[kUnitItems - 1u].w;
-        for (;;) {
+        // (a loop for each kind of scan: with the choice inside one loop, R-MAT scale 20's scans took 0.8 % longer)
+        auto piece = [&](auto&& scan) {
             uint32_t i = 0;
             if (lane == 0) i = atomicAdd(&s_taken, 1u);
             i = __shfl_sync(0xFFFFFFFFu, i, 0);
-            if (i >= total) break;
+            if (i >= total) return false;
             // the list that piece i belongs to: as many lists end before it
             const uint32_t at = __popc(__ballot_sync(0xFFFFFFFFu, items[lane].w <= i)) +
                                 __popc(__ballot_sync(0xFFFFFFFFu, items[32u + lane].w <= i));
             const uint4 x = items[at];
             const uint32_t rows = list_rows(x.y), pieces = (rows + kPieceRows - 1u) / kPieceRows;
             const uint32_t j0 = (i + pieces - x.w) * kPieceRows;
-            const uint32_t j1 = min(j0 + kPieceRows, rows);
-            if (u.filter) scan_rows<WORK, MODE>(st, u.sid, filter, lg, x.x, x.y, x.z, j0, j1, wq, wk);
-            else hash_rows<WORK, MODE>(st, u.sid, u.l, x.x, x.y, x.z, j0, j1, wq, wk);
+            scan(x, j0, min(j0 + kPieceRows, rows));
+            return true;
+        };
+        if (u.filter) {
+            while (piece([&](const uint4& x, uint32_t j0, uint32_t j1) {
+                scan_rows<WORK, MODE>(st, u.sid, filter, lg, x.x, x.y, x.z, j0, j1, wq, wk);
+            })) {}
+        } else {
+            while (piece([&](const uint4& x, uint32_t j0, uint32_t j1) {
+                hash_rows<WORK, MODE>(st, u.sid, u.l, x.x, x.y, x.z, j0, j1, wq, wk);
+            })) {}
         }
         __syncthreads();
     }
